@@ -20,6 +20,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "fmg_strip.cuh"
 
 namespace fm {
 
@@ -90,11 +91,12 @@ __global__ void k_faces(int n, size_t S, int ns, const double* __restrict__ K, T
 // where they exist): the west face of a cell is its west neighbour's east
 // face, the same harmonic mean of the same two values, so D equals the sum
 // of four freshly formed faces bit for bit.  Boundary faces: 2K west, 2K
-// south when ns, else 0.
+// south when ns, else 0.  rD (FP64 grids): 1 / D for the smoothers, formed
+// once here (may be K's own buffer: a cell reads its K before it writes).
 template <typename T, typename C>
-__global__ void k_diagonal(int n, size_t S, int ns, const double* __restrict__ K, const T* __restrict__ Te,
+__global__ void k_diagonal(int n, size_t S, int ns, const double* K, const T* __restrict__ Te,
                            const T* __restrict__ Tn, const double* __restrict__ Te64,
-                           const double* __restrict__ Tn64, T* __restrict__ D, double* __restrict__ D64) {
+                           const double* __restrict__ Tn64, T* __restrict__ D, double* __restrict__ D64, T* rD) {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t cells = (size_t)n * n;
     if (t >= S * cells) return;
@@ -108,6 +110,7 @@ __global__ void k_diagonal(int n, size_t S, int ns, const double* __restrict__ K
     const C d = tw + fe(t) + ts + fn(t);
     D[t] = (T)d;
     if (D64) D64[t] = (double)d;
+    if (rD) rD[t] = T(1) / (T)d;
 }
 
 // Right-hand side of a stage problem: the Dirichlet data moved to the rhs.
@@ -167,12 +170,6 @@ __device__ __forceinline__ U coarse_ghost(int nc, const U* uc, int I, int J, con
 
 // (P u_c) at fine cell (i, j): bilinear cell-centred (9, 3, 3, 1) / 16 with
 // the ghosts above.  One expression for every kernel that prolongs.
-// The weights on the four coarse values: own cell (I, J), its x neighbour
-// Ix, its y neighbour Jy, and the diagonal one.
-template <typename U>
-__device__ __forceinline__ U prolong_vals(U own, U nx, U ny, U nxy) {
-    return (U(9) * own + U(3) * nx + U(3) * ny + U(1) * nxy) / U(16);
-}
 template <typename U>
 __device__ __forceinline__ U prolong_at(int nc, const U* u, int i, int j, const Ghost<U>& g) {
     const int I = i >> 1, J = j >> 1;
@@ -361,314 +358,6 @@ __global__ void __launch_bounds__((R / 2) * (R / RPT)) k_rbgs_tile_reg(int n, si
                 p_out[base + (size_t)gy * n + gx] = rp[k][j];
         }
     }
-}
-
-// Asynchronous global -> shared copies of B = 4, 8 or 16 bytes (cp.async, both
-// addresses B-aligned), commit groups, and the wait until at most N groups
-// of this thread are still in flight.
-template <int B>
-__device__ __forceinline__ void cp_async(void* smem, const void* gmem) {
-    static_assert(B == 4 || B == 8 || B == 16, "cp.async of 4, 8 or 16 bytes");
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)),
-                 "l"(gmem), "n"(B)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-// A product the compiler may not fuse into a neighbouring add.
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-
-// Column-strip wavefront smoother: nsweeps red-black sweeps (HS = 2 nsweeps
-// half-sweeps) by one warp over a window of 64 columns of one sample,
-// marching up the rows.  Lane l owns columns 2l, 2l+1 of the window, so in
-// every row it holds one cell of each colour; W / E neighbours in other
-// lanes come by warp shuffles, N / S neighbours from the rows the lane keeps
-// in registers.  At step y the warp takes in row y and runs half-sweep k on
-// row y - k for k = 1 .. HS: row y - k + 1 has just had half-sweep k - 1 and
-// row y - k - 1 had it one step earlier, so every update sees the values the
-// sweep order prescribes, and row y - HS is final and is written out.  The
-// HS + 2 rows being swept stay in registers (a ring whose slots are fixed by
-// the unrolled step index); the rows ahead of them arrive through a
-// per-warp shared-memory ring filled by cp.async (strip_depth rows deep:
-// each lane copies and later reads back only its own pairs).  A cell with an
-// in-domain neighbour outside the window (first or last column, first or
-// last row of a segment) is not updated, so after HS half-sweeps the window
-// minus HS columns and rows on each side is exact.  Every update is the
-// colour kernel's in the same order with the reciprocal of D, so the sweeps
-// are bit-identical to the other shapes (a missing face adds an exact zero).
-// Operands cross HBM once per call, as float2 / double2 pairs per lane.
-// p_in -> p_out as for the tiles; with ec the iterate is p_in + P ec: the
-// coarse row a fine row needs comes through the same ring (each lane's
-// coarse column, plus the columns left and right of the window), and the
-// three coarse rows in use stay in registers, so the correction adds no
-// dependent loads.
-//
-// With FUSE (pre-smoothing of a V-cycle) the warp also forms the residual
-// b - A p of each final row once the row above it is final, and the
-// restriction to the coarse grid: the lane's column pair is one coarse
-// column, so it sums its four fine residuals over two rows in
-// k_residual_restrict's order and writes b_c (and p_c = 0).  The residual
-// needs exact neighbours, so the strip and segment halos grow by two.
-// Strips overlap by 2 XH columns and row segments by 2 VH rows; one unit
-// (sample, row segment, strip) per warp, strip index fastest.
-constexpr int kStripWarps = 4;
-
-template <typename T>
-struct Pair;
-template <>
-struct Pair<float> {
-    using type = float2;
-};
-template <>
-struct Pair<double> {
-    using type = double2;
-};
-
-// Rows in flight per warp of the strip shapes (shared-memory ring of 40 KB per CTA).
-template <typename T>
-__host__ __device__ constexpr int strip_depth() { return sizeof(T) == 4 ? 8 : 4; }
-
-// Window offset (columns left of the output columns) and halo rows of the strip shapes.
-__host__ __device__ constexpr int strip_xh(int HS, bool fuse) { return fuse ? HS + 2 : HS; }
-__host__ __device__ constexpr int strip_ow(int HS, bool fuse) { return 64 - 2 * strip_xh(HS, fuse); }
-
-template <typename T, int HS, bool FUSE>
-__global__ void __launch_bounds__(32 * kStripWarps, sizeof(T) == 4 ? 4 : 1) k_rbgs_strip(int n, size_t S_all, int strips, int seg_all, int segs_all,
-                                                                 const T* __restrict__ b, const T* __restrict__ Te,
-                                                                 const T* __restrict__ Tn, const T* __restrict__ D,
-                                                                 const T* __restrict__ p_in, T* __restrict__ p_out,
-                                                                 const int32_t* __restrict__ active,
-                                                                 const T* __restrict__ ec, T* __restrict__ bc,
-                                                                 T* __restrict__ pc, const int32_t* __restrict__ order,
-                                                                 int ns, const int32_t* __restrict__ dcount,
-                                                                 int resident) {
-    using V2 = typename Pair<T>::type;
-    constexpr int R = HS + 2;                       // rows in registers: y - HS - 1 .. y
-    constexpr int XH = strip_xh(HS, FUSE), VH = XH;  // halo columns and rows (even)
-    constexpr int OW = strip_ow(HS, FUSE);          // output columns of a strip
-    constexpr int DEPTH = strip_depth<T>();         // rows in flight in the shared-memory ring
-    static_assert(HS % 2 == 0 && XH % 2 == 0, "even half-sweep count and halos");
-    // Each lane copies its own float2 / double2 of the five operands of a row
-    // into its own slot of the warp's ring (cp.async, one commit group per
-    // row) and reads back only what it copied, so no lane waits for another.
-    __shared__ V2 ring[kStripWarps][DEPTH][5][32];
-    __shared__ T cring[kStripWarps][DEPTH][34];   // with ec: [0] left of lane 0, [1 + l] lane l, [33] right of lane 31
-    constexpr unsigned kAll = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    // the samples enumerated and their row segments: as launched, or (dcount:
-    // inside a device-side refinement loop) the count of listed samples the
-    // last residual test left, with segments short enough to fill one wave
-    // of warps when those samples are few
-    size_t S = S_all;
-    int seg = seg_all, segs = segs_all;
-    if (dcount) {
-        S = (size_t)*dcount;
-        if (S * strips < (size_t)resident) {
-            int sg = n;
-            while (sg / 2 >= 16 && S * strips * (size_t)((n + sg / 2 - 1) / (sg / 2)) <= (size_t)resident) sg /= 2;
-            seg = sg;
-            segs = (n + sg - 1) / sg;
-        }
-    }
-    const size_t unit = (size_t)blockIdx.x * kStripWarps + (threadIdx.x >> 5);
-    if (unit >= S * (size_t)segs * strips) return;   // S: the samples enumerated (listed by order, if given)
-    const int sx = (int)(unit % strips);
-    const size_t rest = unit / strips;
-    const int sy = (int)(rest % segs);
-    const size_t s = order ? (size_t)order[rest / segs] : rest / segs;
-    if (inactive(active, s)) return;
-    const int ox = sx * OW, oy = sy * seg, oye = min(oy + seg, n);
-    const int gx = ox - XH + 2 * lane;   // even, so (n even) both cells are in the domain or neither
-    const bool in_x = gx >= 0 && gx < n;
-    const int ys = max(oy - VH, 0), ye = min(oye + VH, n);   // rows taken in; ys even
-    const bool updL = in_x && !(gx > 0 && lane == 0);
-    const bool updR = in_x && !(gx + 1 < n - 1 && lane == 31);
-    const bool out_x = in_x && gx >= ox && gx < ox + OW;
-    const size_t base = s * (size_t)n * n;
-    const T* ecs = ec ? ec + s * (size_t)(n / 2) * (n / 2) : nullptr;
-    const V2 zero2{T(0), T(0)}, one2{T(1), T(1)};
-
-    V2(*my)[5][32] = ring[threadIdx.x >> 5];
-    T(*myc)[34] = cring[threadIdx.x >> 5];
-    const int nc = n / 2, I = gx >> 1;   // the lane's coarse column
-    // row y into ring slot (y - ys) % DEPTH, with ec also coarse row
-    // min((y + 1) / 2, nc - 1), the highest one fine row y needs; every step
-    // commits one group
-    auto fetch = [&](int y) {
-        if (y < ye) {
-            const int slot = (y - ys) % DEPTH;
-            if (in_x) {
-                const size_t g = base + (size_t)y * n + gx;
-                V2* v = &my[slot][0][lane];
-                constexpr int B = (int)sizeof(V2);
-                cp_async<B>(v + 0 * 32, p_in + g);
-                cp_async<B>(v + 1 * 32, b + g);
-                cp_async<B>(v + 2 * 32, D + g);
-                cp_async<B>(v + 3 * 32, Te + g);
-                cp_async<B>(v + 4 * 32, Tn + g);
-            }
-            if (ecs) {
-                const T* crow = ecs + (size_t)min((y + 1) >> 1, nc - 1) * nc;
-                if (in_x) cp_async<(int)sizeof(T)>(&myc[slot][1 + lane], crow + I);
-                if (lane == 0 && I - 1 >= 0 && I - 1 < nc) cp_async<(int)sizeof(T)>(&myc[slot][0], crow + I - 1);
-                if (lane == 31 && I + 1 >= 0 && I + 1 < nc) cp_async<(int)sizeof(T)>(&myc[slot][33], crow + I + 1);
-            }
-        }
-        cp_async_commit();
-    };
-    // with ec: coarse values (own column, left and right neighbours with the
-    // Dirichlet ghosts of coarse_ghost) of the coarse rows taken in at the
-    // last three steps
-    T cs0[3] = {T(0), T(0), T(0)}, cs1[3] = {T(0), T(0), T(0)}, cs2[3] = {T(0), T(0), T(0)};
-    auto coarse3 = [&](T own, T left, T right, T (&dst)[3]) {
-        dst[0] = own;
-        dst[1] = I == 0 ? T(2) * T(0) - own : left;
-        dst[2] = I == nc - 1 ? T(2) * T(0) - own : right;
-    };
-    if (ecs && in_x && ys > 0) {   // coarse row ys / 2 - 1, the lower y neighbour of fine row ys
-        const T* crow = ecs + (size_t)(ys / 2 - 1) * nc;
-        coarse3(crow[I], I > 0 ? crow[I - 1] : T(0), I + 1 < nc ? crow[I + 1] : T(0), cs1);
-    }
-    T p[R][2], bb[R][2], rr[R][2], ee[R][2], nf[R][2], wl[R];
-#pragma unroll
-    for (int c = 0; c < R; ++c) {
-        p[c][0] = p[c][1] = bb[c][0] = bb[c][1] = ee[c][0] = ee[c][1] = nf[c][0] = nf[c][1] = wl[c] = T(0);
-        rr[c][0] = rr[c][1] = T(0);
-    }
-    // FUSE: the row leaving the ring (p and north faces) and the partial coarse sum
-    T pq[2] = {T(0), T(0)}, nq[2] = {T(0), T(0)}, rsum = T(0);
-    for (int q = 0; q < DEPTH; ++q) fetch(ys + q);
-    const int steps = ye - ys + HS + (FUSE ? 1 : 0);
-    for (int y0 = ys; y0 < ys + steps; y0 += R) {
-#pragma unroll
-        for (int J = 0; J < R; ++J) {
-            const int y = y0 + J;
-            if (FUSE) {   // keep row y - R (the S neighbour of the residual row y - HS - 1)
-                pq[0] = p[J][0];
-                pq[1] = p[J][1];
-                nq[0] = nf[J][0];
-                nq[1] = nf[J][1];
-            }
-            {   // take in row y (register slot J), then start the copy of row y + DEPTH
-                cp_async_wait<DEPTH - 1>();   // this lane's copies of row y have landed
-                V2 fp = zero2, fb = zero2, fd = one2, fe = zero2, fn = zero2;
-                if (in_x && y < ye) {
-                    const V2* slot = &my[(y - ys) % DEPTH][0][lane];
-                    fp = slot[0 * 32];
-                    fb = slot[1 * 32];
-                    fd = slot[2 * 32];
-                    fe = slot[3 * 32];
-                    fn = slot[4 * 32];
-                }
-                T a0 = fp.x, a1 = fp.y;
-                if (ecs) {   // the coarse-grid correction p + (P e) as k_prolong forms it
-                    __syncwarp();   // the neighbouring lanes' coarse copies have landed too
-#pragma unroll
-                    for (int q = 0; q < 3; ++q) {
-                        cs2[q] = cs1[q];
-                        cs1[q] = cs0[q];
-                    }
-                    if (in_x && y < ye) {
-                        const T* cv = myc[(y - ys) % DEPTH];
-                        coarse3(cv[1 + lane], cv[lane], cv[2 + lane], cs0);
-                        // fine row y: coarse row y / 2 and its y neighbour (one row down for
-                        // even y, one up for odd y); the step index J has the parity of y.
-                        // Past the south / north edge the neighbour is the ghost row: the
-                        // edge row itself across a no-flow edge, its negative across a
-                        // Dirichlet one (ns: -own, and -(the x ghosts) in the corners)
-                        const T* uJ = (J & 1) ? cs1 : cs0;
-                        const bool edge = (J & 1) ? y == n - 1 : y == 0;
-                        const T* uJy = (J & 1) ? (edge ? cs1 : cs0) : (edge ? cs0 : cs2);
-                        const T sg = (edge && ns) ? T(-1) : T(1);
-                        a0 = a0 + prolong_vals(uJ[0], uJ[1], sg * uJy[0], sg * uJy[1]);
-                        a1 = a1 + prolong_vals(uJ[0], uJ[2], sg * uJy[0], sg * uJy[2]);
-                    }
-                }
-                p[J][0] = a0;
-                p[J][1] = a1;
-                bb[J][0] = fb.x;
-                bb[J][1] = fb.y;
-                rr[J][0] = T(1) / fd.x;
-                rr[J][1] = T(1) / fd.y;
-                ee[J][0] = fe.x;
-                ee[J][1] = gx + 1 < n - 1 ? fe.y : T(0);
-                nf[J][0] = y < n - 1 ? fn.x : T(0);
-                nf[J][1] = y < n - 1 ? fn.y : T(0);
-                wl[J] = __shfl_up_sync(kAll, ee[J][1], 1);   // W face of the left cell
-                if (ecs) __syncwarp();   // every lane has read the coarse slot before it is refilled
-                fetch(y + DEPTH);
-            }
-#pragma unroll
-            for (int k = 1; k <= HS; ++k) {
-                // half-sweep k (colour (k - 1) & 1) on row r: the left cell
-                // (even column) has that colour iff y is odd
-                const int r = y - k;
-                const int c = (J - k + 4 * R) % R, lo = (J - k - 1 + 4 * R) % R, hi = (J - k + 1 + 4 * R) % R;
-                const bool row_ok = r >= ys && r < ye && (r > ys || ys == 0) && (r < ye - 1 || ye == n);
-                if (J & 1) {
-                    const T pw = __shfl_up_sync(kAll, p[c][1], 1);
-                    T acc = bb[c][0];
-                    acc += wl[c] * pw;
-                    acc += ee[c][0] * p[c][1];
-                    acc += nf[lo][0] * p[lo][0];
-                    acc += nf[c][0] * p[hi][0];
-                    const T v = acc * rr[c][0];
-                    p[c][0] = (row_ok && updL) ? v : p[c][0];
-                } else {
-                    const T pe = __shfl_down_sync(kAll, p[c][0], 1);
-                    T acc = bb[c][1];
-                    acc += ee[c][0] * p[c][0];
-                    acc += ee[c][1] * pe;
-                    acc += nf[lo][1] * p[lo][1];
-                    acc += nf[c][1] * p[hi][1];
-                    const T v = acc * rr[c][1];
-                    p[c][1] = (row_ok && updR) ? v : p[c][1];
-                }
-            }
-            {
-                const int r = y - HS;
-                if (out_x && r >= oy && r < oye) {
-                    const int c = (J - HS + 4 * R) % R;
-                    *reinterpret_cast<V2*>(p_out + base + (size_t)r * n + gx) = V2{p[c][0], p[c][1]};
-                }
-            }
-            if (FUSE) {
-                // residual of row q = y - HS - 1 (rows q - 1, q + 1 final), as residual_at forms it
-                const int q = y - HS - 1;
-                const int c = (J - HS - 1 + 4 * R) % R, hi = (J - HS + 4 * R) % R;
-                const T pw = __shfl_up_sync(kAll, p[c][1], 1);
-                const T pe = __shfl_down_sync(kAll, p[c][0], 1);
-                if (out_x && q >= oy && q < oye) {
-                    const V2 dq = *reinterpret_cast<const V2*>(D + base + (size_t)q * n + gx);
-                    T v0 = mul_rn(dq.x, p[c][0]);
-                    v0 = fma(-wl[c], pw, v0);
-                    v0 = fma(-ee[c][0], p[c][1], v0);
-                    v0 = fma(-nq[0], pq[0], v0);
-                    v0 = fma(-nf[c][0], p[hi][0], v0);
-                    const T r0 = bb[c][0] - v0;
-                    T v1 = mul_rn(dq.y, p[c][1]);
-                    v1 = fma(-ee[c][0], p[c][0], v1);
-                    v1 = fma(-ee[c][1], pe, v1);
-                    v1 = fma(-nq[1], pq[1], v1);
-                    v1 = fma(-nf[c][1], p[hi][1], v1);
-                    const T r1 = bb[c][1] - v1;
-                    if ((J & 1) == 0) {   // q odd: the coarse cell's upper row
-                        const size_t cc = s * (size_t)(n / 2) * (n / 2) + (size_t)(q / 2) * (n / 2) + gx / 2;
-                        bc[cc] = rsum + r0 + r1;
-                        pc[cc] = T(0);
-                    } else {
-                        rsum = r0 + r1;
-                    }
-                }
-            }
-        }
-    }
-    cp_async_wait<0>();
 }
 
 // r = b - A p at cell c: D p rounded, then one fused multiply-add per face
@@ -1012,7 +701,7 @@ __global__ void k_stage_partials(int n, size_t S, int chunks, const double* __re
                         r = -v;
                     }
                     bT[g] = (T)r;
-                    pT[g] = T(0);
+                    if (pT) pT[g] = T(0);
                 } else {
                     pv = (double)p[g];
                     r = (double)residual_at(n, g, i, j, b, Te, Tn, D, p);
@@ -1280,9 +969,10 @@ struct GridBufs {
     int n;
     const double* K;
     T *Te, *Tn, *D, *p, *b;
-    T* p2;                             // second iterate buffer of the tile smoother
+    T* p2;                             // second iterate buffer of the tile and strip smoothers
     double* Kc;                        // correction-grid coefficients (k < m)
     T *TeC, *TnC, *DC;                 // their faces and diagonal
+    T *rD, *rDC;                       // FP64: reciprocals of D and DC (DC's takes the place of Kc, k >= 1)
     double *p64, *Te64, *Tn64, *D64;   // refined grids of the mixed form only
 };
 
@@ -1318,8 +1008,16 @@ struct Hierarchy {
 // CTAs per sample of a residual test on grid n (about 8192 cells each).
 inline int check_chunks(int n) { return std::max(1, std::min(128, n * n / 8192)); }
 
-static size_t hierarchy_bytes(int n_fine, int n0, size_t S, size_t tsize, bool mixed, bool converged) {
+// Bytes of the reciprocal diagonals of one FP64 sample (grids below the
+// finest; the finest grid's takes the room counted for its K, the input).
+static size_t rdiag_bytes(int n_fine, int n0) {
     size_t total = 0;
+    for (int n = n0; n < n_fine; n *= 2) total += (size_t)n * n * 8 + 256;
+    return total;
+}
+
+static size_t hierarchy_bytes(int n_fine, int n0, size_t S, size_t tsize, bool mixed, bool converged) {
+    size_t total = tsize == 8 ? rdiag_bytes(n_fine, n0) : 0;
     int m = 0;
     while ((n0 << m) < n_fine) ++m;
     for (int k = 0; k <= m; ++k) {
@@ -1390,6 +1088,11 @@ static fm_status carve(fm_ctx* ctx, Arena& ar, Hierarchy<T>& H, int n_fine, int 
             g.TnC = (T*)take(cnt * sizeof(T));
             g.DC = (T*)take(cnt * sizeof(T));
         }
+        g.rD = g.rDC = nullptr;
+        if constexpr (sizeof(T) == 8) {
+            g.rD = (T*)take(cnt * 8);
+            if (k >= 1) g.rDC = (T*)g.Kc;
+        }
         g.p64 = g.Te64 = g.Tn64 = g.D64 = nullptr;
         if (mixed && k >= H.m - 1) {
             g.p64 = (double*)take(cnt * 8);
@@ -1412,19 +1115,6 @@ static fm_status carve(fm_ctx* ctx, Arena& ar, Hierarchy<T>& H, int n_fine, int 
 
 constexpr size_t kMaxSmem = 200 * 1024;   // dynamic shared memory of the tile smoother
 
-// Resident warps of the strip smoother on the whole GPU, [FP64, FP32][1 or 2 sweeps][fused residual].
-static int g_strip_warps[2][2][2] = {};
-
-template <typename T, int HS, bool FUSE>
-static void strip_occupancy(int sms) {
-    int blocks = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_rbgs_strip<T, HS, FUSE>, 32 * kStripWarps, 0) !=
-        cudaSuccess)
-        blocks = 1;
-    g_strip_warps[sizeof(T) == 4 ? 1 : 0][HS / 2 - 1][FUSE ? 1 : 0] =
-        std::max(1, blocks) * kStripWarps * std::max(1, sms);
-}
-
 // Kernel attributes and occupancies, set once per process before any launch
 // or capture.
 void fmg_init_attributes() {
@@ -1439,73 +1129,14 @@ void fmg_init_attributes() {
         int dev = 0, sms = 1;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        strip_occupancy<float, 2, false>(sms);
-        strip_occupancy<float, 4, false>(sms);
-        strip_occupancy<double, 2, false>(sms);
-        strip_occupancy<double, 4, false>(sms);
-        strip_occupancy<float, 2, true>(sms);
-        strip_occupancy<float, 4, true>(sms);
-        strip_occupancy<double, 2, true>(sms);
-        strip_occupancy<double, 4, true>(sms);
+        strip_init<float>(sms);
+        strip_init<double>(sms);
         cudaGetLastError();
     });
 }
 
-// Rows per segment of the strip smoother: the power-of-two fraction of n (at
-// least 16 rows) that minimises the waves of units over the resident warps
-// times the steps of one unit (segment plus 2 VH halo rows plus the steps
-// that drain the wavefront).
-static int strip_segment(int n, size_t S, int strips, int HS, int VH, int resident) {
-    int best = n;
-    double best_cost = 1e300;
-    for (int seg = n; seg >= 16; seg /= 2) {
-        const size_t units = S * (size_t)strips * ((n + seg - 1) / seg);
-        const double waves = std::ceil((double)units / std::max(1, resident));
-        const double cost = waves * (std::min(seg + (seg < n ? 2 * VH : 0), n) + HS + 1);
-        if (cost < best_cost * 0.999) {
-            best_cost = cost;
-            best = seg;
-        }
-    }
-    return best;
-}
-
-// One strip-smoother launch (bc, pc: with the fused residual and restriction
-// to the coarse grid).  nsweeps is 1 or 2 and n even (smooth_shape).
-template <typename T, int HS, bool FUSE>
-static void strip_launch(fm_ctx* ctx, int n, size_t S, const T* b, const T* Te, const T* Tn, const T* D,
-                         const T* p_in, T* p_out, const int32_t* active, const T* ec, T* bc, T* pc,
-                         cudaStream_t st, size_t busy, const int32_t* order, int ns, const int32_t* dcount) {
-    constexpr int OW = strip_ow(HS, FUSE), VH = strip_xh(HS, FUSE);
-    const int strips = (n + OW - 1) / OW;
-    const int resident = g_strip_warps[sizeof(T) == 4 ? 1 : 0][HS / 2 - 1][FUSE];
-    // with the host's count of active samples and their list, enumerate only
-    // those; with a device-side count (dcount, refinement loops inside a
-    // graph) the kernel enumerates the listed samples itself, and the grid
-    // covers the most units it can form (all samples, or one wave)
-    const bool dev = dcount && order;
-    const bool listed = !dev && order && busy > 0 && busy < S;
-    const size_t sb = listed ? busy : S;
-    const int seg = strip_segment(n, sb, strips, HS, VH, resident);
-    const int segs = (n + seg - 1) / seg;
-    size_t units = sb * (size_t)strips * segs;
-    if (dev) units = std::max(units, (size_t)resident);
-    const size_t cells = sb * (size_t)n * n;
-    const unsigned grid = (unsigned)((units + kStripWarps - 1) / kStripWarps);
-    const double bytes = (6.0 + (FUSE ? 0.5 : 0.0)) * sizeof(T) * cells;
-    const double flops = 5.0 * HS * cells + (FUSE ? 12.0 * cells : 0.0);
-    FM_TIMED(ctx, kFamSmootherStrip, st, bytes, flops,
-             k_rbgs_strip<T, HS, FUSE><<<grid, 32 * kStripWarps, 0, st>>>(
-                 n, sb, strips, seg, segs, b, Te, Tn, D, p_in, p_out, active, ec, bc, pc,
-                 (listed || dev) ? order : nullptr, ns, dev ? dcount : nullptr, resident));
-}
-
-// Launch shape code of the column-strip smoother (tile codes are > 0, colour
-// launches 0).  It runs 1 or 2 sweeps on even grids of at least 16 cells.
+// Launch shape code of the column-strip smoother (fmg_strip.cuh; tile codes are > 0, colour launches 0).
 constexpr int kShapeStrip = -1;
-static bool strip_fits(int n, int nu1, int nu2) {
-    return n >= 16 && n % 2 == 0 && nu1 >= 1 && nu1 <= 2 && nu2 >= 1 && nu2 <= 2;
-}
 
 static size_t tile_smem_bytes(int tile, int n, int nsweeps, size_t tsize) {
     const int TI = std::min(tile, n);
@@ -1522,19 +1153,9 @@ static size_t tile_smem_bytes(int tile, int n, int nsweeps, size_t tsize) {
 template <typename T>
 static T* smooth_with(fm_ctx* ctx, int tile, int threads, int n, size_t S, int nsweeps, const T* b, const T* Te,
                       const T* Tn, const T* D, T* p_in, T* p_out, const int32_t* active, cudaStream_t st,
-                      const T* ec = nullptr, size_t busy = 0, const int32_t* order = nullptr, int ns = 0,
-                      const int32_t* dcount = nullptr) {
+                      const T* ec = nullptr, int ns = 0) {
     if (nsweeps <= 0) return p_in;
     const size_t cells = S * (size_t)n * n;
-    if (tile == kShapeStrip) {
-        if (nsweeps == 2)
-            strip_launch<T, 4, false>(ctx, n, S, b, Te, Tn, D, p_in, p_out, active, ec, nullptr, nullptr, st, busy,
-                                      order, ns, dcount);
-        else
-            strip_launch<T, 2, false>(ctx, n, S, b, Te, Tn, D, p_in, p_out, active, ec, nullptr, nullptr, st, busy,
-                                      order, ns, dcount);
-        return p_out;
-    }
     if (tile > 0) {
         const int TI = std::min(tile, n);
         const int hh = TI >= n ? 0 : 2 * nsweeps;
@@ -1587,8 +1208,7 @@ static int tune_slot(int n) { return std::min(15, 31 - __builtin_clz((unsigned)n
 
 // Smoother launch shape of grid n.  Untuned defaults (fm_autotune's choices
 // on GB300 for two sweeps): register-blocked regions up to 32 x 32, then FP32
-// column strips; FP64 keeps one launch per colour up to 512 (its strips and
-// tiles are bound by the FP64 divide) and strips above.  An fm_autotune or
+// column strips; FP64 keeps one launch per colour up to 512 and strips above.  An fm_autotune or
 // fm_set_smoother_shape entry for this grid and precision replaces the
 // default.  Tiles and strips need both smoothing phases of the V-cycle (so
 // the iterate goes p -> p2 -> p); tiles need their staged region in shared
@@ -1644,11 +1264,59 @@ static void vcycle_tail(const Hierarchy<T>& H, int kt, const fm_solve_params& pr
              k_vcycle_tail<T><<<(unsigned)a.S, kTailThreads, smem, st>>>(a));
 }
 
-// One V(nu1, nu2) cycle on grid k; grid `top` carries the stage operator
-// (injected K), the grids below it the correction operators (child means).
+// Whether the smoother of correction grid k reads the zero iterate that the
+// restriction leaves there: the coarsest solve, the tail and the strips don't.
 template <typename T>
-static void vcycle(const Hierarchy<T>& H, int k, int top, const fm_solve_params& prm, const int32_t* active,
-                   cudaStream_t st) {
+static bool reads_zero(const Hierarchy<T>& H, int k, const fm_solve_params& prm) {
+    if (k == 0) return false;
+    if (H.g[k].n <= H.ctx->tail_max && !prm.energy_step) return false;
+    int tile, threads;
+    smooth_shape<T>(H.ctx, H.g[k].n, prm, &tile, &threads);
+    return tile != kShapeStrip;
+}
+
+// Where `count` V-cycles on grid k read their starting iterate: p, or p2
+// where merged strips (see vcycles) pass through the two buffers an odd
+// number of times; the result is always in p.
+template <typename T>
+static T* start_iterate(const Hierarchy<T>& H, int k, const fm_solve_params& prm, int count) {
+    int tile, threads;
+    smooth_shape<T>(H.ctx, H.g[k].n, prm, &tile, &threads);
+    const bool merged = k > 0 && tile == kShapeStrip && count > 1 && strip_merges<T>(prm.nu1, prm.nu2);
+    return merged && count % 2 == 0 ? H.g[k].p2 : H.g[k].p;
+}
+
+// The energy-optimal step of the correction on grid c.n onto iterate x of
+// grid k: partials, alpha per sample, x += alpha P e_c.
+template <typename T>
+static void energy_step(const Hierarchy<T>& H, int k, const T* Te, const T* Tn, const T* D, T* x, const int32_t* active,
+                        int ns, cudaStream_t st) {
+    fm_ctx* ctx = H.ctx;
+    const GridBufs<T>& g = H.g[k];
+    const GridBufs<T>& c = H.g[k - 1];
+    const size_t S = H.S, cells = S * (size_t)g.n * g.n;
+    const double ts = sizeof(T);
+    const int chunks = check_chunks(g.n);
+    const bool listed = H.listed();
+    const size_t nl = listed ? H.busy : S;
+    FM_TIMED(ctx, kFamProlong, st, (5.0 * ts + 1.25 * ts) * nl * g.n * g.n + 2.0 * ts * cells, 40.0 * nl * g.n * g.n,
+             k_energy_partials<T><<<(unsigned)(nl * chunks), kBlock, 0, st>>>(
+                 g.n, nl, chunks, g.b, Te, Tn, D, x, c.p, active, listed ? H.order : nullptr, H.partial, ns);
+             k_energy_alpha<<<blocks_for(S), kBlock, 0, st>>>(S, chunks, H.partial, H.alpha, active);
+             k_prolong_step<T><<<blocks_for(cells), kBlock, 0, st>>>(c.n, S, c.p, H.alpha, x, active, ns));
+}
+
+// `count` V(nu1, nu2) cycles on grid k, from start_iterate (zero: from a zero
+// iterate, which need not be in memory where the shape is the strip's) to
+// g.p; grid `top` carries the stage operator (injected K), the grids below
+// it the correction operators (child means).
+//
+// Strips with nu1 = nu2 run the post-smoothing of a cycle and the
+// pre-smoothing of the next as one call (the same sweeps in the same order):
+// count + 1 passes over the grid instead of 2 count.
+template <typename T>
+static void vcycles(const Hierarchy<T>& H, int k, int top, const fm_solve_params& prm, const int32_t* active,
+                    cudaStream_t st, int count, bool zero) {
     fm_ctx* ctx = H.ctx;
     const size_t S = H.S;
     const GridBufs<T>& g = H.g[k];
@@ -1658,6 +1326,7 @@ static void vcycle(const Hierarchy<T>& H, int k, int top, const fm_solve_params&
     const T* Te = stage_op ? g.Te : g.TeC;
     const T* Tn = stage_op ? g.Tn : g.TnC;
     const T* D = stage_op ? g.D : g.DC;
+    const T* rD = stage_op ? g.rD : g.rDC;
     if (k == 0) {
         const int m = H.n0 * H.n0;
         FM_TIMED(ctx, kFamCoarseSolve, st, (double)S * (m * m + 2 * m) * ts, 2.0 * S * m * m,
@@ -1667,68 +1336,82 @@ static void vcycle(const Hierarchy<T>& H, int k, int top, const fm_solve_params&
     }
     const int n = g.n;
     const size_t cells = S * (size_t)n * n;
+    const GridBufs<T>& c = H.g[k - 1];
     int tile, threads;
     smooth_shape<T>(ctx, n, prm, &tile, &threads);
-    // pre-smoothing p -> p2 (tiles, strips) or in place; post-smoothing back into p
-    const GridBufs<T>& c = H.g[k - 1];
-    T* cur;
+    T* const pc = reads_zero(H, k - 1, prm) ? c.p : nullptr;   // the coarse iterate, where it must be zeroed
+    // the V-cycle below: the resident tail for correction grids up to
+    // ctx->tail_max, else grid by grid
+    auto below = [&] {
+        if (k - 1 >= 1 && c.n <= ctx->tail_max && !prm.energy_step && S > 0) vcycle_tail(H, k - 1, prm, active, st);
+        else vcycles(H, k - 1, top, prm, active, st, 1, true);
+    };
     if (tile == kShapeStrip) {
-        // strips form the residual and its restriction in the same pass
-        if (prm.nu1 == 2)
-            strip_launch<T, 4, true>(ctx, n, S, g.b, Te, Tn, D, g.p, g.p2, active, nullptr, c.b, c.p, st, H.busy,
-                                     H.order, ns, H.dcount);
-        else
-            strip_launch<T, 2, true>(ctx, n, S, g.b, Te, Tn, D, g.p, g.p2, active, nullptr, c.b, c.p, st, H.busy,
-                                     H.order, ns, H.dcount);
-        cur = g.p2;
-    } else {
-        cur = smooth_with<T>(ctx, tile, threads, n, S, prm.nu1, g.b, Te, Tn, D, g.p, g.p2, active, st, nullptr,
-                             H.busy, H.order, ns, H.dcount);
+        const bool merge = count > 1 && strip_merges<T>(prm.nu1, prm.nu2);
+        T* cur = start_iterate(H, k, prm, count);
+        auto strip = [&](int sweeps, bool fuse, bool from_zero, bool correct) {
+            StripCall<T> s;
+            s.n = n;
+            s.S = S;
+            s.hs = 2 * sweeps;
+            s.fuse = fuse;
+            s.b = g.b;
+            s.Te = Te;
+            s.Tn = Tn;
+            s.D = D;
+            s.rD = rD;
+            s.p_in = from_zero ? nullptr : cur;
+            s.p_out = cur == g.p ? g.p2 : g.p;
+            s.active = active;
+            s.ec = correct ? c.p : nullptr;
+            s.bc = c.b;
+            s.pc = pc;
+            s.order = H.order;
+            s.busy = H.busy;
+            s.dcount = H.dcount;
+            s.ns = ns;
+            strip_launch(ctx, s, st);
+            cur = s.p_out;
+        };
+        for (int it = 0; it < count; ++it) {
+            // pre-smoothing with the residual and its restriction in the same pass
+            if (it == 0 || !merge) strip(prm.nu1, true, zero && it == 0, false);
+            below();
+            if (prm.energy_step) energy_step(H, k, Te, Tn, D, cur, active, ns, st);
+            const bool next = merge && it + 1 < count;
+            strip(next ? prm.nu1 + prm.nu2 : prm.nu2, next, false, !prm.energy_step);
+        }
+        return;
+    }
+    for (int it = 0; it < count; ++it) {
+        // pre-smoothing p -> p2 (tiles) or in place; post-smoothing back into p
+        T* cur = smooth_with<T>(ctx, tile, threads, n, S, prm.nu1, g.b, Te, Tn, D, g.p, g.p2, active, st, nullptr, ns);
         FM_TIMED(ctx, kFamResidualRestrict, st, 5.5 * ts * cells, 10.0 * cells,
                  k_residual_restrict<T><<<blocks_for(S * (size_t)c.n * c.n), kBlock, 0, st>>>(
                      c.n, S, g.b, Te, Tn, D, cur, c.b, c.p, active));
+        below();
+        if (prm.energy_step) {
+            // the stepped correction (converged mode: partials and alpha in the hierarchy)
+            energy_step(H, k, Te, Tn, D, cur, active, ns, st);
+            smooth_with<T>(ctx, tile, threads, n, S, prm.nu2, g.b, Te, Tn, D, cur, g.p, active, st, nullptr, ns);
+        } else if (tile == 0 && prm.nu2 >= 1) {
+            // colour launches: the correction rides in the first post-smoothing colour
+            FM_TIMED(ctx, kFamSmoother, st, 3.0 * ts * cells + ts * S * c.n * c.n, 5.0 * cells,
+                     k_rbgs_color0_prolong<T><<<blocks_for(cells / 2), kBlock, 0, st>>>(n, S, g.b, Te, Tn, D, cur,
+                                                                                        c.p, active, ns));
+            FM_TIMED(ctx, kFamSmoother, st, 3.0 * ts * cells, 5.0 * cells,
+                     k_rbgs_color<T><<<blocks_for(cells / 2), kBlock, 0, st>>>(n, S, 1, g.b, Te, Tn, D, cur, active));
+            smooth_with<T>(ctx, 0, 0, n, S, prm.nu2 - 1, g.b, Te, Tn, D, cur, g.p, active, st);
+        } else if (tile != 0 && prm.nu2 >= 1) {
+            // tiles: the correction is added as they load the iterate
+            smooth_with<T>(ctx, tile, threads, n, S, prm.nu2, g.b, Te, Tn, D, cur, g.p, active, st, c.p, ns);
+        } else {
+            const Ghost<T> zg{T(0), T(0), T(0), T(0), ns};
+            FM_TIMED(ctx, kFamProlong, st, 2.25 * ts * cells, 8.0 * cells,
+                     k_prolong<T><<<blocks_for(cells), kBlock, 0, st>>>(c.n, S, c.p, zg, 1, cur, active));
+            smooth_with<T>(ctx, tile, threads, n, S, prm.nu2, g.b, Te, Tn, D, cur, g.p, active, st, nullptr, ns);
+        }
     }
-    // the V-cycle below: the resident tail for correction grids up to
-    // ctx->tail_max, else grid by grid
-    if (k - 1 >= 1 && c.n <= ctx->tail_max && !prm.energy_step && S > 0)
-        vcycle_tail(H, k - 1, prm, active, st);
-    else
-        vcycle(H, k - 1, top, prm, active, st);
-    if (prm.energy_step) {
-        // the stepped correction (converged mode: partials and alpha in the hierarchy)
-        const int chunks = check_chunks(n);
-        const bool listed = H.listed();
-        const size_t nl = listed ? H.busy : S;
-        FM_TIMED(ctx, kFamProlong, st, (5.0 * ts + 1.25 * ts) * nl * n * n + 2.0 * ts * cells, 40.0 * nl * n * n,
-                 k_energy_partials<T><<<(unsigned)(nl * chunks), kBlock, 0, st>>>(
-                     n, nl, chunks, g.b, Te, Tn, D, cur, c.p, active, listed ? H.order : nullptr, H.partial, ns);
-                 k_energy_alpha<<<blocks_for(S), kBlock, 0, st>>>(S, chunks, H.partial, H.alpha, active);
-                 k_prolong_step<T><<<blocks_for(cells), kBlock, 0, st>>>(c.n, S, c.p, H.alpha, cur, active, ns));
-        smooth_with<T>(ctx, tile, threads, n, S, prm.nu2, g.b, Te, Tn, D, cur, g.p, active, st, nullptr, H.busy,
-                       H.order, ns, H.dcount);
-        return;
-    }
-    if (tile == 0 && prm.nu2 >= 1) {
-        // colour launches: the correction rides in the first post-smoothing colour
-        FM_TIMED(ctx, kFamSmoother, st, 3.0 * ts * cells + ts * S * c.n * c.n, 5.0 * cells,
-                 k_rbgs_color0_prolong<T><<<blocks_for(cells / 2), kBlock, 0, st>>>(n, S, g.b, Te, Tn, D, cur, c.p,
-                                                                                    active, ns));
-        FM_TIMED(ctx, kFamSmoother, st, 3.0 * ts * cells, 5.0 * cells,
-                 k_rbgs_color<T><<<blocks_for(cells / 2), kBlock, 0, st>>>(n, S, 1, g.b, Te, Tn, D, cur, active));
-        smooth_with<T>(ctx, 0, 0, n, S, prm.nu2 - 1, g.b, Te, Tn, D, cur, g.p, active, st);
-        return;
-    }
-    if (tile != 0 && prm.nu2 >= 1) {
-        // tiles and strips: the correction is added as they load the iterate
-        smooth_with<T>(ctx, tile, threads, n, S, prm.nu2, g.b, Te, Tn, D, cur, g.p, active, st, c.p, H.busy,
-                       H.order, ns, H.dcount);
-        return;
-    }
-    const Ghost<T> zero{T(0), T(0), T(0), T(0), ns};
-    FM_TIMED(ctx, kFamProlong, st, 2.25 * ts * cells, 8.0 * cells,
-             k_prolong<T><<<blocks_for(cells), kBlock, 0, st>>>(c.n, S, c.p, zero, 1, cur, active));
-    smooth_with<T>(ctx, tile, threads, n, S, prm.nu2, g.b, Te, Tn, D, cur, g.p, active, st, nullptr, H.busy,
-                   H.order, ns, H.dcount);
 }
 
 template <typename P>
@@ -1746,10 +1429,13 @@ static void stage_test(const Hierarchy<T>& H, int k, const fm_solve_params& prm,
     const size_t S = H.S, cells = (size_t)g.n * g.n;
     const int chunks = check_chunks(g.n);
     const size_t ns = H.listed() ? H.busy : S;
+    int tile, threads;
+    smooth_shape<T>(ctx, g.n, prm, &tile, &threads);
+    T* const pT = tile == kShapeStrip ? nullptr : g.p;   // strips start from zero without reading it
     FM_TIMED(ctx, kFamResidualRestrict, st, (mixed ? 48.0 : 40.0) * ns * cells, 12.0 * ns * cells,
              k_stage_partials<T><<<(unsigned)(ns * chunks), kBlock, 0, st>>>(
                  g.n, ns, chunks, g.K, bnd_of(prm), g.b, g.Te, g.Tn, g.D, g.p, g.p64, g.Te64, g.Tn64, g.D64, g.b,
-                 g.p, H.active, H.partial, H.listed() ? H.order : nullptr);
+                 pT, H.active, H.partial, H.listed() ? H.order : nullptr);
              k_stage_decide<<<blocks_for(S), kBlock, 0, st>>>(S, chunks, H.partial, prm.tol, prm.qtol, H.qprev,
                                                               H.active, H.left, H.order));
 }
@@ -1817,7 +1503,7 @@ static fm_status refine_stage_graph(const Hierarchy<T>& H, int k, const fm_solve
                                                    cudaStreamCaptureModeRelaxed));
     // the body's strips enumerate the samples the last test listed
     H.dcount = H.order ? H.left : nullptr;
-    for (int v = 0; v < cycles_per_test(prm); ++v) vcycle(H, k, k, prm, H.active, bs);
+    vcycles(H, k, k, prm, H.active, bs, cycles_per_test(prm), mixed);
     H.dcount = nullptr;
     if (mixed)
         k_ir_update<T><<<ir_update_blocks(ctx, S * cells), kBlock, 0, bs>>>(cells, S, g.p, g.p64, H.active,
@@ -1853,7 +1539,7 @@ static fm_status refine_stage(const Hierarchy<T>& H, int k, const fm_solve_param
             if (status) k_status<<<blocks_for(S), kBlock, 0, st>>>(S, H.active, status);
             break;
         }
-        for (int v = 0; v < cycles_per_test(prm); ++v) vcycle(H, k, k, prm, H.active, st);
+        vcycles(H, k, k, prm, H.active, st, cycles_per_test(prm), mixed);
         if (mixed)
             k_ir_update<T><<<ir_update_blocks(ctx, (H.listed() ? H.busy : S) * cells), kBlock, 0, st>>>(
                 cells, H.listed() ? H.busy : S, g.p, g.p64, H.active, H.listed() ? H.order : nullptr, nullptr);
@@ -1888,13 +1574,13 @@ static fm_status fmg_batch(const Hierarchy<T>& H, const fm_solve_params& prm, do
                      k_faces<T, double><<<blocks_for(cells), kBlock, 0, st>>>(g.n, S, bd.ns, g.K, g.Te, g.Tn,
                                                                               g.Te64, g.Tn64);
                      k_diagonal<T, double><<<blocks_for(cells), kBlock, 0, st>>>(g.n, S, bd.ns, g.K, g.Te, g.Tn,
-                                                                                 g.Te64, g.Tn64, g.D, g.D64));
+                                                                                 g.Te64, g.Tn64, g.D, g.D64, g.rD));
         else
             FM_TIMED(ctx, kFamCoefficients, st, (8.0 + 3.0 * ts) * cells, 16.0 * cells,
                      k_faces<T, T><<<blocks_for(cells), kBlock, 0, st>>>(g.n, S, bd.ns, g.K, g.Te, g.Tn, nullptr,
                                                                          nullptr);
                      k_diagonal<T, T><<<blocks_for(cells), kBlock, 0, st>>>(g.n, S, bd.ns, g.K, g.Te, g.Tn, nullptr,
-                                                                            nullptr, g.D, nullptr));
+                                                                            nullptr, g.D, nullptr, g.rD));
     }
     for (int k = 0; k < H.m; ++k) {
         const GridBufs<T>& g = H.g[k];
@@ -1904,7 +1590,7 @@ static fm_status fmg_batch(const Hierarchy<T>& H, const fm_solve_params& prm, do
                  k_faces<T, T><<<blocks_for(cells), kBlock, 0, st>>>(g.n, S, bd.ns, g.Kc, g.TeC, g.TnC, nullptr,
                                                                      nullptr);
                  k_diagonal<T, T><<<blocks_for(cells), kBlock, 0, st>>>(g.n, S, bd.ns, g.Kc, g.TeC, g.TnC, nullptr,
-                                                                        nullptr, g.DC, nullptr));
+                                                                        nullptr, g.DC, nullptr, g.rDC));
     }
     if (H.m >= 1) {
         const int m = H.n0 * H.n0;
@@ -1935,16 +1621,15 @@ static fm_status fmg_batch(const Hierarchy<T>& H, const fm_solve_params& prm, do
             } else {
                 FM_TIMED(ctx, kFamFmgInterp, st, 1.25 * ts * cells, 8.0 * cells,
                          k_prolong<T><<<blocks_for(cells), kBlock, 0, st>>>(
-                             c.n, S, c.p, Ghost<T>{(T)bd.g[0], (T)bd.g[1], (T)bd.g[2], (T)bd.g[3], bd.ns}, 0, g.p,
-                             nullptr));
+                             c.n, S, c.p, Ghost<T>{(T)bd.g[0], (T)bd.g[1], (T)bd.g[2], (T)bd.g[3], bd.ns}, 0,
+                             refined ? g.p : start_iterate(H, k, prm, prm.nu0), nullptr));
             }
         }
         FM_TIMED(ctx, kFamStageRhs, st, (8.0 + ts) * cells, 2.0 * cells,
                  k_stage_rhs<T><<<blocks_for(cells), kBlock, 0, st>>>(g.n, S, g.K, bd, g.b));
-        if (k == 0) vcycle(H, 0, 0, prm, nullptr, st);
+        if (k == 0) vcycles(H, 0, 0, prm, nullptr, st, 1, false);
         if (!refined) {
-            if (k > 0)
-                for (int it = 0; it < prm.nu0; ++it) vcycle(H, k, k, prm, nullptr, st);
+            if (k > 0) vcycles(H, k, k, prm, nullptr, st, prm.nu0, false);
         } else {
             if (mixed && !(k == H.m && H.m >= 1 && refine_c))
                 k_widen<T><<<blocks_for(cells), kBlock, 0, st>>>(cells, g.p, g.p64);
@@ -2045,8 +1730,10 @@ fm_status fmg_solve_with(fm_ctx* ctx, Arena& ar, int n_fine, uint32_t S, const d
 // ------------------------------------------------------------------ allocation-free variant
 // Scratch of fmg_solve_batch_static: one file-scope device array, present on
 // every device that loads the library for as long as the process lives.
+// What a batch may need, the reciprocal diagonals apart (at most a seventeenth
+// of it), and the array with room for those.
 constexpr size_t kStaticScratchBytes = (size_t)32 << 20;   // 32 MiB
-static __device__ __align__(256) char g_static_scratch[kStaticScratchBytes];
+static __device__ __align__(256) char g_static_scratch[kStaticScratchBytes + ((size_t)2 << 20)];
 
 // Device address of the array on the current device.  Host code only sees a
 // stand-in symbol, so the address is asked for once per device, with that
@@ -2110,6 +1797,8 @@ static void carve_into(fm_ctx* ctx, Hierarchy<double>& H, char* base, int n_fine
             g.TnC = (double*)take(cnt * 8);
             g.DC = (double*)take(cnt * 8);
         }
+        g.rD = (double*)take(cnt * 8);
+        g.rDC = k >= 1 ? g.Kc : nullptr;
         g.p64 = g.Te64 = g.Tn64 = g.D64 = nullptr;
     }
     H.Ainv = (double*)take(S * (size_t)n0 * n0 * n0 * n0 * 8);
@@ -2128,7 +1817,7 @@ static void carve_into(fm_ctx* ctx, Hierarchy<double>& H, char* base, int n_fine
 // that dominates them, rhs and iterate in (-1, 1) (a hash of the index).
 template <typename T>
 __global__ void k_tune_fill(size_t count, T* __restrict__ b, T* __restrict__ Te, T* __restrict__ Tn,
-                            T* __restrict__ D, T* __restrict__ p) {
+                            T* __restrict__ D, T* __restrict__ rD, T* __restrict__ p) {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= count) return;
     uint64_t h = t * 0x9E3779B97F4A7C15ULL;
@@ -2140,6 +1829,7 @@ __global__ void k_tune_fill(size_t count, T* __restrict__ b, T* __restrict__ Te,
     Te[t] = (T)(0.5 + u0);
     Tn[t] = (T)(0.5 + u1);
     D[t] = (T)(4.5 + u2);
+    rD[t] = T(1) / D[t];
     b[t] = (T)(2.0 * u2 - 1.0);
     p[t] = (T)(2.0 * u0 - 1.0);
 }
@@ -2150,9 +1840,9 @@ static fm_status autotune_grid(fm_ctx* ctx, int n, int nsweeps, fm_tune_entry* e
     const size_t S = std::max<size_t>(1, ((size_t)64 << 20) / ((size_t)n * n));
     const size_t cells = S * (size_t)n * n;
     T* buf = nullptr;
-    FM_CUDA_TRY(ctx, cudaMalloc((void**)&buf, 6 * cells * sizeof(T)));
-    T *b = buf, *Te = b + cells, *Tn = Te + cells, *D = Tn + cells, *p = D + cells, *p2 = p + cells;
-    k_tune_fill<T><<<blocks_for(cells), kBlock>>>(cells, b, Te, Tn, D, p);
+    FM_CUDA_TRY(ctx, cudaMalloc((void**)&buf, 7 * cells * sizeof(T)));
+    T *b = buf, *Te = b + cells, *Tn = Te + cells, *D = Tn + cells, *p = D + cells, *p2 = p + cells, *rD = p2 + cells;
+    k_tune_fill<T><<<blocks_for(cells), kBlock>>>(cells, b, Te, Tn, D, rD, p);
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -2160,11 +1850,27 @@ static fm_status autotune_grid(fm_ctx* ctx, int n, int nsweeps, fm_tune_entry* e
     ctx->prof.active = false;
     auto time_shape = [&](int tile, int threads) -> double {
         if (tile > 0 && tile_smem_bytes(tile, n, nsweeps, sizeof(T)) > kMaxSmem) return 1e30;
-        smooth_with<T>(ctx, tile, threads, n, S, nsweeps, b, Te, Tn, D, p, p2, nullptr, nullptr);   // warm-up
+        auto smooth = [&](T* in, T* out) {
+            if (tile != kShapeStrip) {
+                smooth_with<T>(ctx, tile, threads, n, S, nsweeps, b, Te, Tn, D, in, out, nullptr, nullptr);
+                return;
+            }
+            StripCall<T> c;
+            c.n = n;
+            c.S = S;
+            c.hs = 2 * nsweeps;
+            c.b = b;
+            c.Te = Te;
+            c.Tn = Tn;
+            c.D = D;
+            c.rD = rD;
+            c.p_in = in;
+            c.p_out = out;
+            strip_launch(ctx, c, nullptr);
+        };
+        smooth(p, p2);   // warm-up
         cudaEventRecord(e0);
-        for (int r = 0; r < 4; ++r)   // p -> p2 -> p for tiles
-            smooth_with<T>(ctx, tile, threads, n, S, nsweeps, b, Te, Tn, D, r & 1 ? p2 : p, r & 1 ? p : p2, nullptr,
-                           nullptr);
+        for (int r = 0; r < 4; ++r) smooth(r & 1 ? p2 : p, r & 1 ? p : p2);   // p -> p2 -> p for tiles and strips
         cudaEventRecord(e1);
         cudaEventSynchronize(e1);
         float ms = 0.0f;
@@ -2290,7 +1996,7 @@ extern "C" fm_status fmg_solve_batch_static(fm_ctx* ctx, int32_t n_fine, uint32_
                  "fmg_solve_batch_static: bc_case must be FM_CASE_I or FM_CASE_II");
     FM_CHECK_ARG(ctx, n == 0 || (d_K && d_qf), "fmg_solve_batch_static: null input or output");
     if (n == 0) return FM_OK;
-    const size_t need = hierarchy_bytes(n_fine, n0, n, 8, false, false);
+    const size_t need = hierarchy_bytes(n_fine, n0, n, 8, false, false) - n * rdiag_bytes(n_fine, n0);
     FM_CHECK_ARG(ctx, need <= kStaticScratchBytes,
                  "fmg_solve_batch_static: " + std::to_string(n) + " samples of " + std::to_string(n_fine) + "x" +
                      std::to_string(n_fine) + " need " + std::to_string(need) + " bytes of scratch; the static "
