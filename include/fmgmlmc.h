@@ -130,10 +130,10 @@ typedef struct {
 
 /* Kernel schedule of a batched FMG solve (same arithmetic, same result up
  * to rounding order). */
-#define FM_KERNEL_AUTO 0       /* resident where it is the faster schedule (up to 32 x 32 in
-                                  the mixed form, 16 x 16 in FP64, and a converged mixed
-                                  64 x 64 batch of at most two samples per SM; not with the
-                                  energy step), else levelwise */
+#define FM_KERNEL_AUTO 0       /* resident where it is the faster schedule (mixed form: up to
+                                  32 x 32, and a converged 64 x 64 batch of at most two samples
+                                  per SM; FP64: batches up to 64 x 64 of a few samples per SM; not
+                                  with the energy step), else levelwise */
 #define FM_KERNEL_LEVELWISE 1  /* one kernel per grid operation over all samples */
 #define FM_KERNEL_RESIDENT 2   /* one CTA per sample, hierarchy in shared memory
                                   (n_fine <= 64 in FP64) */
@@ -327,7 +327,7 @@ fm_status fmg_solve_batch(fm_ctx* ctx, int32_t n_fine, uint32_t n, const double*
  * memory pool owned by someone else, or on a path where a cudaMalloc would
  * stall the device or fail.  It allocates nothing (no cudaMalloc, cudaFree
  * or allocating library routine; profiling must be off): its scratch is one
- * static device array of 32 MiB that the library holds on every device that
+ * static device array of 34 MiB that the library holds on every device that
  * loads it until the process exits.  The paper has no counterpart; this is
  * an interface for callers that cannot allocate.
  *   - Inputs and outputs stay the caller's: d_K [n][n_fine][n_fine], d_qf

@@ -79,22 +79,29 @@ struct Ghost {
     int ns;
 };
 
-// The schedule FM_KERNEL_AUTO takes for a grid: the resident kernel where it
-// is the faster one on GB300 (up to 32 x 32 in the mixed form, 16 x 16 in
-// FP64), the level-wise schedule (with its V-cycle tail below 32 x 32) above
-// and for the energy-optimal step, which the resident kernel lacks.
-// Measured per grid, samples per second of resident over level-wise:
-// 16 x 16 2.0x (mixed), 1.1x (FP64, two cycles per stage), 1.2x (FP64
-// converged); 64 x 64 0.82x, 0.89x, 1.04x; 32 x 32 0.93x and 0.84x in FP64,
-// level in the mixed form (0.97x alone, ahead inside the five-level estimate).
-// The resident kernel for grids up to 32 x 32 in the mixed form (16 x 16 in
-// FP64); also for a converged mixed 64 x 64 batch of at most two samples per
-// SM: one CTA per sample then finishes in one or two waves, where the
-// level-wise schedule is a latency-bound chain of small launches.
+// The schedule FM_KERNEL_AUTO takes for S samples of a grid: the resident
+// kernel (one CTA or warp per sample) or the level-wise schedule; the latter
+// always for the energy-optimal step, which the resident kernel lacks.
+// FP64: the level-wise schedule has the higher throughput on every grid, the
+// resident kernel the shorter chain of launches, so it runs batches that it
+// takes in about one wave (fixed schedule) or a few (converged, where the
+// level-wise chain is several times longer).  Measured on GB300, ms level-wise
+// / resident, fixed: 16 x 16 0.35 / 0.32 at 1216 samples, 0.41 / 0.45 at 1824,
+// 6.6 / 14.6 at 60000; 32 x 32 0.59 / 0.43 at 608, 0.63 / 0.70 at 760; 64 x 64
+// 0.72 / 0.49 at 152, 0.88 / 0.96 at 200.  Converged: 16 x 16 4.95 / 4.20 at
+// 5000, 14.2 / 14.9 at 20000; 32 x 32 8.7 / 7.5 at 2432, 14.1 / 15.0 at 5000;
+// 64 x 64 13.4 / 12.4 at 608, 16.1 / 16.4 at 912.
+// Mixed: resident up to 32 x 32 (16 x 16 7.5 / 5.3 at 20000; 32 x 32 level
+// within 5%: 6.7 / 6.3 at 5000, 16.3 / 17.1 at 15000), and a converged 64 x 64
+// batch of at most two samples per SM (3.0 / 2.4 at 304, 3.2 / 3.5 at 380).
 inline bool auto_resident(int n_fine, size_t S, int sms, const fm_solve_params& prm) {
     if (prm.energy_step) return false;
-    if (prm.precision == FM_PREC_MIXED && prm.converged && n_fine == 64 && S <= 2 * (size_t)sms) return true;
-    return n_fine <= (prm.precision == FM_PREC_MIXED ? 32 : 16);
+    if (prm.precision == FM_PREC_MIXED)
+        return n_fine <= 32 || (prm.converged && n_fine == 64 && S <= 2 * (size_t)sms);
+    if (n_fine > 64) return false;
+    const size_t per_sm = prm.converged ? (n_fine <= 16 ? 32 : n_fine <= 32 ? 16 : 4)
+                                        : (n_fine <= 16 ? 8 : n_fine <= 32 ? 4 : 1);
+    return S <= per_sm * (size_t)sms;
 }
 
 // V-cycles between residual tests of a converged stage.

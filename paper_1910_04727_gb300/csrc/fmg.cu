@@ -28,8 +28,6 @@ constexpr int kBlock = 256;
 
 inline unsigned blocks_for(size_t threads) { return (unsigned)((threads + kBlock - 1) / kBlock); }
 
-template <typename C>
-__device__ __forceinline__ C harmonic(C a, C b) { return C(2) * a * b / (a + b); }
 
 // Sample of a flat thread index and whether it still iterates.
 __device__ __forceinline__ bool inactive(const int32_t* active, size_t s) { return active && !active[s]; }
@@ -58,7 +56,7 @@ __global__ void k_child_geomean(int nc, size_t S, const double* __restrict__ Kf,
     const int c = (int)(t % cells);
     const int I = c % nc, J = c / nc, nf = 2 * nc;
     const double* k = Kf + s * (size_t)nf * nf + (size_t)(2 * J) * nf + 2 * I;
-    Kc[t] = (double)exp(C(0.25) * (log((C)k[0]) + log((C)k[1]) + log((C)k[nf]) + log((C)k[nf + 1])));
+    Kc[t] = (double)geometric_mean4((C)k[0], (C)k[1], (C)k[nf], (C)k[nf + 1]);
 }
 
 // Face transmissibilities: harmonic mean inside, 2K on the Dirichlet edges
@@ -77,8 +75,8 @@ __global__ void k_faces(int n, size_t S, int ns, const double* __restrict__ K, T
     const int c = (int)(t % cells);
     const int i = c % n, j = c / n;
     const C k = (C)K[t];
-    const C te = (i < n - 1) ? harmonic<C>(k, (C)K[t + 1]) : C(2) * k;
-    const C tn = (j < n - 1) ? harmonic<C>(k, (C)K[t + n]) : (ns ? C(2) * k : C(0));
+    const C te = (i < n - 1) ? harmonic_mean(k, (C)K[t + 1]) : C(2) * k;
+    const C tn = (j < n - 1) ? harmonic_mean(k, (C)K[t + n]) : (ns ? C(2) * k : C(0));
     Te[t] = (T)te;
     Tn[t] = (T)tn;
     if (Te64) {
@@ -113,7 +111,8 @@ __global__ void k_diagonal(int n, size_t S, int ns, const double* K, const T* __
     if (rD) rD[t] = T(1) / (T)d;
 }
 
-// Right-hand side of a stage problem: the Dirichlet data moved to the rhs.
+// Right-hand side of a stage problem: the Dirichlet data moved to the rhs
+// (zero, without a read of K, off the edges).
 template <typename T>
 __global__ void k_stage_rhs(int n, size_t S, const double* __restrict__ K, Bnd bd, T* __restrict__ b) {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -121,14 +120,15 @@ __global__ void k_stage_rhs(int n, size_t S, const double* __restrict__ K, Bnd b
     if (t >= S * cells) return;
     const int c = (int)(t % cells);
     const int i = c % n, j = c / n;
-    b[t] = (T)dirichlet_rhs(bd, n, i, j, K[t]);
+    const bool edge = i == 0 || i == n - 1 || (bd.ns && (j == 0 || j == n - 1));
+    b[t] = edge ? (T)dirichlet_rhs(bd, n, i, j, K[t]) : T(0);
 }
 
 // One colour of a red-black Gauss-Seidel sweep: cells with (i + j) % 2 == color.
 template <typename T>
 __global__ void k_rbgs_color(int n, size_t S, int color, const T* __restrict__ b, const T* __restrict__ Te,
-                             const T* __restrict__ Tn, const T* __restrict__ D, T* __restrict__ p,
-                             const int32_t* __restrict__ active) {
+                             const T* __restrict__ Tn, const T* __restrict__ D, const T* __restrict__ rD,
+                             T* __restrict__ p, const int32_t* __restrict__ active) {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t half = (size_t)n * n / 2;
     if (t >= S * half) return;
@@ -143,40 +143,36 @@ __global__ void k_rbgs_color(int n, size_t S, int color, const T* __restrict__ b
     if (i < n - 1) acc += Te[c] * p[c + 1];
     if (j > 0) acc += Tn[c - n] * p[c - n];
     if (j < n - 1) acc += Tn[c] * p[c + n];
-    p[c] = acc * (T(1) / D[c]);
+    p[c] = acc * (rD ? rD[c] : T(1) / D[c]);
 }
 
-// Coarse value with ghosts: 2g - u across the Dirichlet edges (g = 0 for an
-// error), the edge value mirrored across the no-flow edges; a corner ghost
-// takes the x rule on the y ghost.
-template <typename U>
-__device__ __forceinline__ U coarse_ghost_x(int nc, const U* uc, int I, int J, const Ghost<U>& g) {
-    if (I < 0) return U(2) * g.w - uc[(size_t)J * nc];
-    if (I > nc - 1) return U(2) * g.e - uc[(size_t)J * nc + nc - 1];
-    return uc[(size_t)J * nc + I];
-}
-template <typename U>
-__device__ __forceinline__ U coarse_ghost(int nc, const U* uc, int I, int J, const Ghost<U>& g) {
-    if (J < 0) {
-        const U edge = coarse_ghost_x(nc, uc, I, 0, g);
-        return g.ns ? U(2) * g.s - edge : edge;
-    }
-    if (J > nc - 1) {
-        const U edge = coarse_ghost_x(nc, uc, I, nc - 1, g);
-        return g.ns ? U(2) * g.n - edge : edge;
-    }
-    return coarse_ghost_x(nc, uc, I, J, g);
-}
-
-// (P u_c) at fine cell (i, j): bilinear cell-centred (9, 3, 3, 1) / 16 with
-// the ghosts above.  One expression for every kernel that prolongs.
+// (P u_c) at fine cell (i, j): bilinear cell-centred (9, 3, 3, 1) / 16
+// (prolong_vals, one expression for every kernel that prolongs), with ghosts
+// 2g - u across the Dirichlet edges (g = 0 for an error) and the edge value
+// mirrored across the no-flow edges; a corner ghost takes the x rule on the
+// y ghost.  The ghosts are formed only where a cell needs them: formed for
+// every cell and selected, they were two thirds of an FP64 prolongation.
 template <typename U>
 __device__ __forceinline__ U prolong_at(int nc, const U* u, int i, int j, const Ghost<U>& g) {
     const int I = i >> 1, J = j >> 1;
     const int Ix = (i & 1) ? I + 1 : I - 1;
     const int Jy = (j & 1) ? J + 1 : J - 1;
-    return prolong_vals(coarse_ghost(nc, u, I, J, g), coarse_ghost(nc, u, Ix, J, g), coarse_ghost(nc, u, I, Jy, g),
-                        coarse_ghost(nc, u, Ix, Jy, g));
+    const bool xe = Ix < 0 || Ix > nc - 1, ye = Jy < 0 || Jy > nc - 1;
+    const int Ic = xe ? I : Ix, Jc = ye ? J : Jy;
+    const U* row = u + (size_t)J * nc;
+    const U* other = u + (size_t)Jc * nc;
+    U nx = row[Ic], ny = other[I], nxy = other[Ic];
+    if (xe) {
+        const U b = Ix < 0 ? g.w : g.e;
+        nx = fma(U(2), b, -nx);
+        nxy = fma(U(2), b, -nxy);
+    }
+    if (ye && g.ns) {
+        const U b = Jy < 0 ? g.s : g.n;
+        ny = fma(U(2), b, -ny);
+        nxy = fma(U(2), b, -nxy);
+    }
+    return prolong_vals(row[I], nx, ny, nxy);
 }
 // an error's ghosts: zero boundary data
 template <typename U>
@@ -199,9 +195,9 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_rbgs_tile(int n, size_t S, int TI, int hh, int nsweeps,
                                                    const T* __restrict__ b, const T* __restrict__ Te,
                                                    const T* __restrict__ Tn, const T* __restrict__ D,
-                                                   const T* __restrict__ p_in, T* __restrict__ p_out,
-                                                   const int32_t* __restrict__ active, const T* __restrict__ ec,
-                                                   int ns) {
+                                                   const T* __restrict__ rD, const T* __restrict__ p_in,
+                                                   T* __restrict__ p_out, const int32_t* __restrict__ active,
+                                                   const T* __restrict__ ec, int ns) {
     extern __shared__ __align__(16) unsigned char tile_smem[];
     const int tiles = (n + TI - 1) / TI;
     const size_t s = blockIdx.x / ((unsigned)tiles * tiles);
@@ -226,7 +222,7 @@ __global__ void __launch_bounds__(256) k_rbgs_tile(int n, size_t S, int TI, int 
         sb[e] = b[g];
         se[e] = Te[g];
         sn[e] = Tn[g];
-        sd[e] = D[g];
+        sd[e] = rD ? rD[g] : T(1) / D[g];
     }
     __syncthreads();
     const int W2 = (RW + 1) / 2;
@@ -246,7 +242,7 @@ __global__ void __launch_bounds__(256) k_rbgs_tile(int n, size_t S, int TI, int 
             if (i < n - 1) acc += se[e] * sp[e + 1];
             if (j > 0) acc += sn[e - RW] * sp[e - RW];
             if (j < n - 1) acc += sn[e] * sp[e + RW];
-            sp[e] = acc * (T(1) / sd[e]);
+            sp[e] = acc * sd[e];
         }
         __syncthreads();
     }
@@ -275,6 +271,7 @@ __global__ void __launch_bounds__((R / 2) * (R / RPT)) k_rbgs_tile_reg(int n, si
                                                                       const T* __restrict__ Te,
                                                                       const T* __restrict__ Tn,
                                                                       const T* __restrict__ D,
+                                                                      const T* __restrict__ rD,
                                                                       const T* __restrict__ p_in, T* __restrict__ p_out,
                                                                       const int32_t* __restrict__ active,
                                                                       const T* __restrict__ ec, int ns) {
@@ -307,7 +304,7 @@ __global__ void __launch_bounds__((R / 2) * (R / RPT)) k_rbgs_tile_reg(int n, si
                 rp[k][j] = ec ? p_in[g] + prolong_err(n / 2, ec + s * (size_t)(n / 2) * (n / 2), gx, gy, ns)
                               : p_in[g];
                 rb[k][j] = b[g];
-                rr[k][j] = T(1) / D[g];
+                rr[k][j] = rD ? rD[g] : T(1) / D[g];
                 if (gx < n - 1) re[k][j] = Te[g];
                 if (gy < n - 1) rn[k][j] = Tn[g];
                 if (gx > 0) rw[k][j] = Te[g - 1];
@@ -510,7 +507,8 @@ __global__ void k_prolong_step(int nc, size_t S, const T* __restrict__ uc, const
 // bit-identical to a prolongation pass followed by the colour launches.
 template <typename T>
 __global__ void k_rbgs_color0_prolong(int n, size_t S, const T* __restrict__ b, const T* __restrict__ Te,
-                                      const T* __restrict__ Tn, const T* __restrict__ D, T* __restrict__ p,
+                                      const T* __restrict__ Tn, const T* __restrict__ D, const T* __restrict__ rD,
+                                      T* __restrict__ p,
                                       const T* __restrict__ ec, const int32_t* __restrict__ active, int ns) {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t half = (size_t)n * n / 2;
@@ -529,66 +527,100 @@ __global__ void k_rbgs_color0_prolong(int n, size_t S, const T* __restrict__ b, 
     if (i < n - 1) acc += Te[c] * (p[c + 1] + prolong_err(nc, e, i + 1, j, ns));
     if (j > 0) acc += Tn[c - n] * (p[c - n] + prolong_err(nc, e, i, j - 1, ns));
     if (j < n - 1) acc += Tn[c] * (p[c + n] + prolong_err(nc, e, i, j + 1, ns));
-    p[c] = acc * (T(1) / D[c]);
+    p[c] = acc * (rD ? rD[c] : T(1) / D[c]);
 }
 
-// Inverse of the dense operator of the coarsest grid (m = n0^2 <= 16
-// unknowns), Gauss-Jordan on [A | I] in FP64 (A is SPD, so no pivoting).
-// One warp per sample with [A | X] in shared memory: lane c < 16 owns column
-// c of A, lane 16 + c column c of X.
-constexpr int kInvWarps = 8;
+// Inverse of the operator of the coarsest grid (m = n0^2 <= 16 unknowns) in
+// FP64, 32 samples per CTA: the faces by all threads, the banded L D L^T
+// factors (half bandwidth n0) of a sample by one thread, then one column of
+// the inverse per thread (forward and backward substitution of a unit
+// vector).  Faces and factors lie in shared memory with the samples fastest,
+// so a warp reads them without conflicts.  About 150 FP64 operations a column
+// and 200 a sample, and chains of some 300 dependent ones; the dense
+// Gauss-Jordan elimination of [A | I] by a warp per sample that this replaces
+// took 83 us for 256 samples and 393 us for 5304.
+constexpr int kInvSamples = 32;
+
+template <typename T, int N0>
+__global__ void __launch_bounds__(kInvSamples* N0* N0) k_coarse_inverse(size_t S, const double* __restrict__ K,
+                                                                         T* __restrict__ Ainv, int ns) {
+    constexpr int M = N0 * N0;
+    __shared__ double se[M][kInvSamples], sn[M][kInvSamples];   // east and north faces
+    __shared__ double sk[M][kInvSamples];                       // coefficients; then 1 / D(r)
+    __shared__ double sl[M * N0][kInvSamples];                  // L(r, r - k) at r N0 + k - 1
+    const int u = threadIdx.x % kInvSamples, c = threadIdx.x / kInvSamples;
+    const size_t s = (size_t)blockIdx.x * kInvSamples + u;
+    {   // cell c of sample u
+        const double* k = K + s * M;
+        const int i = c % N0, j = c / N0;
+        const double kc = s < S ? k[c] : 1.0;
+        const double ke = s < S && i < N0 - 1 ? k[c + 1] : kc, kn = s < S && j < N0 - 1 ? k[c + N0] : kc;
+        sk[c][u] = kc;
+        se[c][u] = i < N0 - 1 ? harmonic_mean(kc, ke) : 2.0 * kc;
+        sn[c][u] = j < N0 - 1 ? harmonic_mean(kc, kn) : (ns ? 2.0 * kc : 0.0);
+    }
+    __syncthreads();
+    if (threadIdx.x < kInvSamples) {
+        double L[M][N0 + 1], rd[M];   // indexed by constants once unrolled
+#pragma unroll
+        for (int r = 0; r < M; ++r) {
+            const int i = r % N0, j = r / N0;
+            const double tw = i > 0 ? se[i > 0 ? r - 1 : r][u] : 2.0 * sk[r][u];
+            const double ts = j > 0 ? sn[j > 0 ? r - N0 : r][u] : (ns ? 2.0 * sk[r][u] : 0.0);
+            double d = tw + se[r][u] + ts + sn[r][u];
+            double mr[N0 + 1];                // L(r, r - k) D(r - k)
+#pragma unroll
+            for (int q = N0; q >= 1; --q) {
+                mr[q] = 0.0;
+                L[r][q] = 0.0;
+                if (r - q < 0) continue;
+                double v = q == N0 ? -ts : ((q == 1 && i > 0) ? -tw : 0.0);
+#pragma unroll
+                for (int t = q + 1; t <= N0; ++t)
+                    if (r - t >= 0) v = fma(-mr[t], L[r - q][t - q], v);
+                mr[q] = v;
+                L[r][q] = v * rd[r - q];
+                d = fma(-v, L[r][q], d);
+            }
+            rd[r] = 1.0 / d;
+#pragma unroll
+            for (int q = 1; q <= N0; ++q) sl[r * N0 + q - 1][u] = L[r][q];
+        }
+#pragma unroll
+        for (int r = 0; r < M; ++r) sk[r][u] = rd[r];
+    }
+    __syncthreads();
+    if (s >= S) return;
+    double x[M];
+#pragma unroll
+    for (int r = 0; r < M; ++r) {
+        double v = r == c ? 1.0 : 0.0;
+#pragma unroll
+        for (int q = N0; q >= 1; --q)
+            if (r - q >= 0) v = fma(-sl[r * N0 + q - 1][u], x[r - q], v);
+        x[r] = v;
+    }
+#pragma unroll
+    for (int r = M - 1; r >= 0; --r) {
+        double v = x[r] * sk[r][u];
+#pragma unroll
+        for (int q = N0; q >= 1; --q)
+            if (r + q < M) v = fma(-sl[(r + q) * N0 + q - 1][u], x[r + q], v);
+        x[r] = v;
+    }
+    T* out = Ainv + (s * M + c) * M;   // column c as row c: the inverse is symmetric
+#pragma unroll
+    for (int r = 0; r < M; ++r) out[r] = (T)x[r];
+}
 
 template <typename T>
-__global__ void __launch_bounds__(32 * kInvWarps) k_coarse_inverse(int n0, size_t S, const double* __restrict__ K,
-                                                                   T* __restrict__ Ainv, int ns) {
-    __shared__ double sh[kInvWarps][2][16][16];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const size_t s = (size_t)blockIdx.x * kInvWarps + warp;
-    if (s >= S) return;   // whole warps leave together
+static void coarse_inverse(fm_ctx* ctx, int n0, size_t S, const double* K, T* Ainv, int ns, cudaStream_t st) {
     const int m = n0 * n0;
-    double(*A)[16] = sh[warp][0];
-    double(*X)[16] = sh[warp][1];
-    const double* k = K + s * m;
-    for (int r = lane; r < m; r += 32) {   // row r: the equation of cell r
-        for (int c = 0; c < m; ++c) {
-            A[r][c] = 0.0;
-            X[r][c] = (r == c) ? 1.0 : 0.0;
-        }
-        const int i = r % n0, j = r / n0;
-        const double tw = (i > 0) ? harmonic(k[r - 1], k[r]) : 2.0 * k[r];
-        const double te = (i < n0 - 1) ? harmonic(k[r], k[r + 1]) : 2.0 * k[r];
-        const double tb = ns ? 2.0 * k[r] : 0.0;   // north / south boundary face
-        const double ts = (j > 0) ? harmonic(k[r - n0], k[r]) : tb;
-        const double tn = (j < n0 - 1) ? harmonic(k[r], k[r + n0]) : tb;
-        A[r][r] = tw + te + ts + tn;
-        if (i > 0) A[r][r - 1] = -tw;
-        if (i < n0 - 1) A[r][r + 1] = -te;
-        if (j > 0) A[r][r - n0] = -ts;
-        if (j < n0 - 1) A[r][r + n0] = -tn;
-    }
-    __syncwarp();
-    const bool ownA = lane < m, ownX = lane >= 16 && lane - 16 < m;
-    const int col = lane & 15;
-    for (int p = 0; p < m; ++p) {
-        const double piv = A[p][p];
-        double f[16];
-#pragma unroll
-        for (int r = 0; r < 16; ++r) f[r] = (r < m) ? A[r][p] : 0.0;
-        __syncwarp();
-        // scale row p, then eliminate column p from every other row
-        if (ownA) A[p][col] /= piv;
-        if (ownX) X[p][col] /= piv;
-        __syncwarp();
-#pragma unroll
-        for (int r = 0; r < 16; ++r) {
-            if (r >= m || r == p) continue;
-            if (ownA) A[r][col] -= f[r] * A[p][col];
-            if (ownX) X[r][col] -= f[r] * X[p][col];
-        }
-        __syncwarp();
-    }
-    T* out = Ainv + s * (size_t)m * m;
-    for (int e = lane; e < m * m; e += 32) out[e] = (T)X[e / m][e % m];
+    const unsigned grid = (unsigned)((S + kInvSamples - 1) / kInvSamples);
+    FM_TIMED(ctx, kFamCoarseInverse, st, (double)S * (8 * m + sizeof(T) * m * m), 2.0 * S * m * m * (2 * n0 + 1),
+             if (n0 == 2) k_coarse_inverse<T, 2><<<grid, kInvSamples * m, 0, st>>>(S, K, Ainv, ns);
+             else if (n0 == 3) k_coarse_inverse<T, 3><<<grid, kInvSamples * m, 0, st>>>(S, K, Ainv, ns);
+             else k_coarse_inverse<T, 4><<<grid, kInvSamples * m, 0, st>>>(S, K, Ainv, ns));
 }
 
 // p = A^{-1} b on the coarsest grid; one thread per (sample, unknown).
@@ -819,6 +851,7 @@ struct TailArgs {
     const T* Te[8];                         // correction operators of grids 0 .. kt
     const T* Tn[8];
     const T* D[8];
+    const T* rD[8];                         // their reciprocals, where the hierarchy holds them (FP64)
     const T* b;                             // rhs of grid kt [..][n_kt^2]
     T* p;                                   // out: the correction on grid kt
     const T* Ainv;                          // coarsest correction operator's inverse [..][m][m]
@@ -866,6 +899,7 @@ __global__ void __launch_bounds__(kTailThreads) k_vcycle_tail(TailArgs<T> a) {
         const T* gte = a.Te[j] + s * (size_t)c;
         const T* gtn = a.Tn[j] + s * (size_t)c;
         const T* gd = a.D[j] + s * (size_t)c;
+        const T* gr = a.rD[j] ? a.rD[j] + s * (size_t)c : nullptr;
         T* te = arr(j, 0);
         T* tn = arr(j, 1);
         T* dd = arr(j, 2);
@@ -876,7 +910,7 @@ __global__ void __launch_bounds__(kTailThreads) k_vcycle_tail(TailArgs<T> a) {
             te[e] = gte[e];
             tn[e] = gtn[e];
             dd[e] = d;
-            rd[e] = T(1) / d;
+            rd[e] = gr ? gr[e] : T(1) / d;
         }
     }
     T* const ainv = arr(a.kt + 1, 0);
@@ -1152,8 +1186,8 @@ static size_t tile_smem_bytes(int tile, int n, int nsweeps, size_t tsize) {
 // the tiles load.
 template <typename T>
 static T* smooth_with(fm_ctx* ctx, int tile, int threads, int n, size_t S, int nsweeps, const T* b, const T* Te,
-                      const T* Tn, const T* D, T* p_in, T* p_out, const int32_t* active, cudaStream_t st,
-                      const T* ec = nullptr, int ns = 0) {
+                      const T* Tn, const T* D, const T* rD, T* p_in, T* p_out, const int32_t* active,
+                      cudaStream_t st, const T* ec = nullptr, int ns = 0) {
     if (nsweeps <= 0) return p_in;
     const size_t cells = S * (size_t)n * n;
     if (tile > 0) {
@@ -1169,30 +1203,30 @@ static T* smooth_with(fm_ctx* ctx, int tile, int threads, int n, size_t S, int n
         if (threads == 0 && hh == 0 && (n == 8 || n == 16 || n == 32 || (f32 && n == 64))) {
             if (n == 8)
                 FM_TIMED(ctx, kFamSmootherTile, st, bytes, flops, k_rbgs_tile_reg<T, 8, 1><<<grid, 4 * 8, 0, st>>>(
-                    n, S, TI, hh, nsweeps, b, Te, Tn, D, p_in, p_out, active, ec, ns));
+                    n, S, TI, hh, nsweeps, b, Te, Tn, D, rD, p_in, p_out, active, ec, ns));
             else if (n == 16)
                 FM_TIMED(ctx, kFamSmootherTile, st, bytes, flops, k_rbgs_tile_reg<T, 16, 2><<<grid, 8 * 8, 0, st>>>(
-                    n, S, TI, hh, nsweeps, b, Te, Tn, D, p_in, p_out, active, ec, ns));
+                    n, S, TI, hh, nsweeps, b, Te, Tn, D, rD, p_in, p_out, active, ec, ns));
             else if (n == 32)
                 FM_TIMED(ctx, kFamSmootherTile, st, bytes, flops, k_rbgs_tile_reg<T, 32, 4><<<grid, 16 * 8, 0, st>>>(
-                    n, S, TI, hh, nsweeps, b, Te, Tn, D, p_in, p_out, active, ec, ns));
+                    n, S, TI, hh, nsweeps, b, Te, Tn, D, rD, p_in, p_out, active, ec, ns));
             else if constexpr (f32)
                 FM_TIMED(ctx, kFamSmootherTile, st, bytes, flops, k_rbgs_tile_reg<T, 64, 8><<<grid, 32 * 8, 0, st>>>(
-                    n, S, TI, hh, nsweeps, b, Te, Tn, D, p_in, p_out, active, ec, ns));
+                    n, S, TI, hh, nsweeps, b, Te, Tn, D, rD, p_in, p_out, active, ec, ns));
             return p_out;
         }
         if (threads == 0 && hh > 0 && hh <= 4 && (TI == 32 || (f32 && TI == 64))) {
             if (TI == 32)
                 FM_TIMED(ctx, kFamSmootherTile, st, bytes, flops, k_rbgs_tile_reg<T, 40, 5><<<grid, 20 * 8, 0, st>>>(
-                    n, S, TI, hh, nsweeps, b, Te, Tn, D, p_in, p_out, active, ec, ns));
+                    n, S, TI, hh, nsweeps, b, Te, Tn, D, rD, p_in, p_out, active, ec, ns));
             else if constexpr (f32)
                 FM_TIMED(ctx, kFamSmootherTile, st, bytes, flops, k_rbgs_tile_reg<T, 72, 9><<<grid, 36 * 8, 0, st>>>(
-                    n, S, TI, hh, nsweeps, b, Te, Tn, D, p_in, p_out, active, ec, ns));
+                    n, S, TI, hh, nsweeps, b, Te, Tn, D, rD, p_in, p_out, active, ec, ns));
             return p_out;
         }
         FM_TIMED(ctx, kFamSmootherTile, st, bytes, flops,
                  k_rbgs_tile<T><<<grid, threads > 0 ? threads : 256, tile_smem_bytes(tile, n, nsweeps, sizeof(T)),
-                                  st>>>(n, S, TI, hh, nsweeps, b, Te, Tn, D, p_in, p_out, active, ec, ns));
+                                  st>>>(n, S, TI, hh, nsweeps, b, Te, Tn, D, rD, p_in, p_out, active, ec, ns));
         return p_out;
     }
     T* p = p_in;
@@ -1200,15 +1234,19 @@ static T* smooth_with(fm_ctx* ctx, int tile, int threads, int n, size_t S, int n
     for (int it = 0; it < nsweeps; ++it)
         for (int color = 0; color < 2; ++color)
             FM_TIMED(ctx, kFamSmoother, st, 3.0 * sizeof(T) * cells, 5.0 * cells,
-                     k_rbgs_color<T><<<blocks_for(half), kBlock, 0, st>>>(n, S, color, b, Te, Tn, D, p, active));
+                     k_rbgs_color<T><<<blocks_for(half), kBlock, 0, st>>>(n, S, color, b, Te, Tn, D, rD, p, active));
     return p;
 }
 
 static int tune_slot(int n) { return std::min(15, 31 - __builtin_clz((unsigned)n)); }
 
-// Smoother launch shape of grid n.  Untuned defaults (fm_autotune's choices
-// on GB300 for two sweeps): register-blocked regions up to 32 x 32, then FP32
-// column strips; FP64 keeps one launch per colour up to 512 and strips above.  An fm_autotune or
+// Smoother launch shape of grid n.  Untuned defaults (fastest on GB300 for two
+// sweeps): register-blocked regions up to 32 x 32 (FP64 solves of 5000 32 x 32
+// samples 2.37 ms against 2.48 with packed strips), then column strips.  FP64
+// strips against one launch per colour, fixed schedule: 64 x 64, 5000 samples
+// 12.0 / 14.0 ms; 128 x 128, 1000 samples 8.9 / 11.5; 256 x 256, 250 samples
+// 9.2 / 11.8 (before the strips read 1 / D instead of forming it, the FP64
+// divide made colour launches the faster ones).  An fm_autotune or
 // fm_set_smoother_shape entry for this grid and precision replaces the
 // default.  Tiles and strips need both smoothing phases of the V-cycle (so
 // the iterate goes p -> p2 -> p); tiles need their staged region in shared
@@ -1216,11 +1254,8 @@ static int tune_slot(int n) { return std::min(15, 31 - __builtin_clz((unsigned)n
 template <typename T>
 static void smooth_shape(const fm_ctx* ctx, int n, const fm_solve_params& prm, int* tile, int* threads) {
     const int pi = sizeof(T) == 4 ? 1 : 0, slot = tune_slot(n);
-    const bool f32 = sizeof(T) == 4;
-    *tile = 0;
     *threads = 0;
-    if (n <= 32) *tile = 32;   // one register-blocked region per sample
-    else if (f32 || n > 512) *tile = kShapeStrip;
+    *tile = n <= 32 ? 32 : kShapeStrip;   // 32: one register-blocked region per sample
     if (ctx->tune.n[pi][slot] == n) {
         *tile = ctx->tune.tile[pi][slot];
         *threads = ctx->tune.threads[pi][slot];
@@ -1250,6 +1285,7 @@ static void vcycle_tail(const Hierarchy<T>& H, int kt, const fm_solve_params& pr
         a.Te[j] = H.g[j].TeC;
         a.Tn[j] = H.g[j].TnC;
         a.D[j] = H.g[j].DC;
+        a.rD[j] = H.g[j].rDC;
         cells += (double)H.g[j].n * H.g[j].n;
     }
     a.b = H.g[kt].b;
@@ -1385,7 +1421,7 @@ static void vcycles(const Hierarchy<T>& H, int k, int top, const fm_solve_params
     }
     for (int it = 0; it < count; ++it) {
         // pre-smoothing p -> p2 (tiles) or in place; post-smoothing back into p
-        T* cur = smooth_with<T>(ctx, tile, threads, n, S, prm.nu1, g.b, Te, Tn, D, g.p, g.p2, active, st, nullptr, ns);
+        T* cur = smooth_with<T>(ctx, tile, threads, n, S, prm.nu1, g.b, Te, Tn, D, rD, g.p, g.p2, active, st, nullptr, ns);
         FM_TIMED(ctx, kFamResidualRestrict, st, 5.5 * ts * cells, 10.0 * cells,
                  k_residual_restrict<T><<<blocks_for(S * (size_t)c.n * c.n), kBlock, 0, st>>>(
                      c.n, S, g.b, Te, Tn, D, cur, c.b, c.p, active));
@@ -1393,23 +1429,24 @@ static void vcycles(const Hierarchy<T>& H, int k, int top, const fm_solve_params
         if (prm.energy_step) {
             // the stepped correction (converged mode: partials and alpha in the hierarchy)
             energy_step(H, k, Te, Tn, D, cur, active, ns, st);
-            smooth_with<T>(ctx, tile, threads, n, S, prm.nu2, g.b, Te, Tn, D, cur, g.p, active, st, nullptr, ns);
+            smooth_with<T>(ctx, tile, threads, n, S, prm.nu2, g.b, Te, Tn, D, rD, cur, g.p, active, st, nullptr, ns);
         } else if (tile == 0 && prm.nu2 >= 1) {
             // colour launches: the correction rides in the first post-smoothing colour
             FM_TIMED(ctx, kFamSmoother, st, 3.0 * ts * cells + ts * S * c.n * c.n, 5.0 * cells,
-                     k_rbgs_color0_prolong<T><<<blocks_for(cells / 2), kBlock, 0, st>>>(n, S, g.b, Te, Tn, D, cur,
-                                                                                        c.p, active, ns));
+                     k_rbgs_color0_prolong<T><<<blocks_for(cells / 2), kBlock, 0, st>>>(n, S, g.b, Te, Tn, D, rD,
+                                                                                        cur, c.p, active, ns));
             FM_TIMED(ctx, kFamSmoother, st, 3.0 * ts * cells, 5.0 * cells,
-                     k_rbgs_color<T><<<blocks_for(cells / 2), kBlock, 0, st>>>(n, S, 1, g.b, Te, Tn, D, cur, active));
-            smooth_with<T>(ctx, 0, 0, n, S, prm.nu2 - 1, g.b, Te, Tn, D, cur, g.p, active, st);
+                     k_rbgs_color<T><<<blocks_for(cells / 2), kBlock, 0, st>>>(n, S, 1, g.b, Te, Tn, D, rD, cur,
+                                                                               active));
+            smooth_with<T>(ctx, 0, 0, n, S, prm.nu2 - 1, g.b, Te, Tn, D, rD, cur, g.p, active, st);
         } else if (tile != 0 && prm.nu2 >= 1) {
             // tiles: the correction is added as they load the iterate
-            smooth_with<T>(ctx, tile, threads, n, S, prm.nu2, g.b, Te, Tn, D, cur, g.p, active, st, c.p, ns);
+            smooth_with<T>(ctx, tile, threads, n, S, prm.nu2, g.b, Te, Tn, D, rD, cur, g.p, active, st, c.p, ns);
         } else {
             const Ghost<T> zg{T(0), T(0), T(0), T(0), ns};
             FM_TIMED(ctx, kFamProlong, st, 2.25 * ts * cells, 8.0 * cells,
                      k_prolong<T><<<blocks_for(cells), kBlock, 0, st>>>(c.n, S, c.p, zg, 1, cur, active));
-            smooth_with<T>(ctx, tile, threads, n, S, prm.nu2, g.b, Te, Tn, D, cur, g.p, active, st, nullptr, ns);
+            smooth_with<T>(ctx, tile, threads, n, S, prm.nu2, g.b, Te, Tn, D, rD, cur, g.p, active, st, nullptr, ns);
         }
     }
 }
@@ -1592,18 +1629,8 @@ static fm_status fmg_batch(const Hierarchy<T>& H, const fm_solve_params& prm, do
                  k_diagonal<T, T><<<blocks_for(cells), kBlock, 0, st>>>(g.n, S, bd.ns, g.Kc, g.TeC, g.TnC, nullptr,
                                                                         nullptr, g.DC, nullptr, g.rDC));
     }
-    if (H.m >= 1) {
-        const int m = H.n0 * H.n0;
-        FM_TIMED(ctx, kFamCoarseInverse, st, (double)S * (8 * m + ts * m * m), 2.0 * S * m * m * m,
-                 k_coarse_inverse<T><<<(unsigned)((S + kInvWarps - 1) / kInvWarps), 32 * kInvWarps, 0, st>>>(
-                     H.n0, S, H.g[0].Kc, H.AinvC, bd.ns));
-    }
-    {
-        const int m = H.n0 * H.n0;
-        FM_TIMED(ctx, kFamCoarseInverse, st, (double)S * (8 * m + ts * m * m), 2.0 * S * m * m * m,
-                 k_coarse_inverse<T><<<(unsigned)((S + kInvWarps - 1) / kInvWarps), 32 * kInvWarps, 0, st>>>(H.n0, S, H.g[0].K, H.Ainv,
-                                                                                                 bd.ns));
-    }
+    if (H.m >= 1) coarse_inverse<T>(ctx, H.n0, S, H.g[0].Kc, H.AinvC, bd.ns, st);
+    coarse_inverse<T>(ctx, H.n0, S, H.g[0].K, H.Ainv, bd.ns, st);
     // the stage one grid coarser is refined only where its QoI is asked for:
     // otherwise it just gives the finest stage its starting guess
     const bool refine_c = conv && qc != nullptr;
@@ -1625,8 +1652,11 @@ static fm_status fmg_batch(const Hierarchy<T>& H, const fm_solve_params& prm, do
                              refined ? g.p : start_iterate(H, k, prm, prm.nu0), nullptr));
             }
         }
-        FM_TIMED(ctx, kFamStageRhs, st, (8.0 + ts) * cells, 2.0 * cells,
-                 k_stage_rhs<T><<<blocks_for(cells), kBlock, 0, st>>>(g.n, S, g.K, bd, g.b));
+        // (a refined stage of the mixed form has its first residual written there instead;
+        // the coarsest grid is solved first)
+        if (!(mixed && refined && k > 0))
+            FM_TIMED(ctx, kFamStageRhs, st, ts * cells, 2.0 * cells,
+                     k_stage_rhs<T><<<blocks_for(cells), kBlock, 0, st>>>(g.n, S, g.K, bd, g.b));
         if (k == 0) vcycles(H, 0, 0, prm, nullptr, st, 1, false);
         if (!refined) {
             if (k > 0) vcycles(H, k, k, prm, nullptr, st, prm.nu0, false);
@@ -1852,7 +1882,8 @@ static fm_status autotune_grid(fm_ctx* ctx, int n, int nsweeps, fm_tune_entry* e
         if (tile > 0 && tile_smem_bytes(tile, n, nsweeps, sizeof(T)) > kMaxSmem) return 1e30;
         auto smooth = [&](T* in, T* out) {
             if (tile != kShapeStrip) {
-                smooth_with<T>(ctx, tile, threads, n, S, nsweeps, b, Te, Tn, D, in, out, nullptr, nullptr);
+                smooth_with<T>(ctx, tile, threads, n, S, nsweeps, b, Te, Tn, D, sizeof(T) == 8 ? rD : nullptr, in, out,
+                               nullptr, nullptr);
                 return;
             }
             StripCall<T> c;

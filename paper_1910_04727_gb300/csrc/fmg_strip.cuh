@@ -12,6 +12,36 @@ __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(
 __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
 
+// Harmonic mean 2ab / (a + b) of two coefficients, the face between them.
+// FP64: the divide of the FP64 pipe (a 58th of the FP32 rate) bounds the
+// set-up of every operator, so the quotient is formed with six operations
+// instead of nine: the hardware's approximate reciprocal (outside that pipe),
+// one third-order Newton step r += r (e + e^2), e = 1 - d r, and the
+// quotient corrected by its own remainder (Markstein), within an ulp of the
+// IEEE quotient for results in the normal range.
+__device__ __forceinline__ float harmonic_mean(float a, float b) { return 2.0f * a * b / (a + b); }
+__device__ __forceinline__ double harmonic_mean(double a, double b) {
+    const double n = (a + a) * b, d = a + b;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+    const double e = fma(-d, r, 1.0);
+    r = fma(r, fma(e, e, e), r);
+    const double q = n * r;
+    return fma(fma(-d, q, n), r, q);
+}
+
+// Geometric mean of four positive coefficients.  FP64: two square roots (25
+// operations of the FP64 pipe, against 157 for four logarithms and an
+// exponential) where no product leaves the range, else by logarithms.
+__device__ __forceinline__ float geometric_mean4(float a, float b, float c, float d) {
+    return expf(0.25f * (logf(a) + logf(b) + logf(c) + logf(d)));
+}
+__device__ __forceinline__ double geometric_mean4(double a, double b, double c, double d) {
+    const double p = a * b, q = c * d;
+    if (p > 1e-140 && p < 1e140 && q > 1e-140 && q < 1e140) return sqrt(sqrt(p * q));
+    return exp(0.25 * (log(a) + log(b) + log(c) + log(d)));
+}
+
 // The bilinear cell-centred prolongation (9, 3, 3, 1) / 16 of four coarse
 // values: own cell, its x neighbour, its y neighbour, the diagonal one.  The
 // roundings are spelled out, so every kernel that prolongs rounds the same
