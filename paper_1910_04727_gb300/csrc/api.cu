@@ -66,7 +66,10 @@ extern "C" fm_status fm_create(const fm_config* cfg, fm_ctx** out) {
     const size_t vbytes = ctx->h_sobol_V.size() * sizeof(uint32_t);
     const size_t sums = (size_t)(cfg->n_levels + 1) * (cfg->n_shifts > 0 ? cfg->n_shifts : 1);
     if (cudaMalloc((void**)&ctx->d_sobol_V, vbytes) != cudaSuccess ||
-        cudaMalloc((void**)&ctx->d_sums, sums * sizeof(fm_level_sums)) != cudaSuccess) {
+        cudaMalloc((void**)&ctx->d_sums, sums * sizeof(fm_level_sums)) != cudaSuccess ||
+        // the flag of the bounded device-side waits stays set until fm_sync reports it
+        cudaMalloc((void**)&ctx->tc.err, sizeof(int)) != cudaSuccess ||
+        cudaMemset(ctx->tc.err, 0, sizeof(int)) != cudaSuccess) {
         fm_destroy(ctx);
         set_error(nullptr, "fm_create: device allocation failed");
         return FM_ENOMEM;
@@ -100,6 +103,7 @@ extern "C" fm_status fm_create(const fm_config* cfg, fm_ctx** out) {
     }
     fmg_init_attributes();
     resident_init_attributes();
+    kl_split_init_attributes();
     *out = ctx;
     return FM_OK;
 }
@@ -125,6 +129,7 @@ extern "C" void fm_destroy(fm_ctx* ctx) {
     for (int l = 0; l < FM_MAX_LEVELS; ++l) cudaFree(ctx->tc.basis[l]);
     cudaFree(ctx->tc.xi);
     cudaFree(ctx->tc.err);
+    kl_split_free(ctx);
     delete ctx;
 }
 

@@ -262,6 +262,23 @@ struct TcState {
     int* err = nullptr;                // device flag: a bounded wait ran out
 };
 
+// FP64 KL synthesis by exact digit products on the tensor cores (kl_split.cu).
+struct OzState {
+    int Mpad = 0;
+    bool have[FM_MAX_LEVELS] = {};
+    void* basis[FM_MAX_LEVELS] = {};   // BF16 digits [cells][9 Mpad] per level
+    int* ec[FM_MAX_LEVELS] = {};       // scale exponents of the basis rows
+    CUtensorMap mapA[FM_MAX_LEVELS];
+    static constexpr int kStreams = 4;
+    struct Xi {                        // digits of a batch's coefficients, one buffer per stream
+        unsigned long long id = 0;
+        size_t cap = 0;
+        void* digits = nullptr;
+        int* ex = nullptr;
+        CUtensorMap map;
+    } xi[kStreams];
+};
+
 }  // namespace fm
 
 struct fm_ctx {
@@ -291,6 +308,7 @@ struct fm_ctx {
     size_t partial_capacity = 0;
     fm::Profiler prof;
     fm::TcState tc;
+    fm::OzState oz;
     void* mlp = nullptr;             // surrogate network state (mlp.cu)
     int surrogate_on = 0;            // level -1 = S(xi), level 0 = Q_0 - S(xi)
     // Streams that capture the bodies of device-side refinement loops, one
@@ -377,6 +395,12 @@ bool fmg_resident_launch(fm_ctx* ctx, int n_fine, int n0, size_t S, const double
 // Tensor-core KL synthesis (kl_tc.cu): install the BF16 basis, then fields.
 fm_status kl_tc_install(fm_ctx* ctx, int split);
 fm_status kl_tc_field(fm_ctx* ctx, int level, uint32_t n, const double* d_xi, double* d_K, cudaStream_t st);
+// FP64 KL synthesis by exact digit products (kl_split.cu).
+fm_status kl_split_install(fm_ctx* ctx);
+bool kl_split_field(fm_ctx* ctx, int level, uint32_t n, const double* d_xi, double* d_K, cudaStream_t st,
+                    fm_status* status);
+void kl_split_free(fm_ctx* ctx);
+void kl_split_init_attributes();
 // Nystrom interpolation of the KL basis on the tensor cores (kl_tc.cu).
 fm_status kl_tc_nystrom(fm_ctx* ctx, int q, const double* dVt, const double* d_inv_sqrt_theta, double* d_out);
 

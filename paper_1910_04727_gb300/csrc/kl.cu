@@ -1,8 +1,9 @@
 // Karhunen-Loeve field synthesis (Sec. 3.1) and the one-time basis setup.
 //
 // kl_field_batch is the contraction K[s][c] = exp(sum_k B[c][k] xi[s][k]):
-// cells x modes by modes x samples.  The FP64 form below is a register-tiled
-// SIMT GEMM (FP64 has no fast tensor-core path on this part) with the
+// cells x modes by modes x samples.  The FP64 form is a split product on the
+// tensor cores (kl_split.cu) up to 512 modes; above, and where a call cannot
+// take it, the register-tiled SIMT GEMM below, in the FP64 pipe, with the
 // exponential fused into the epilogue, so g is never written to memory.
 #include <cublas_v2.h>
 #include <cusolverDn.h>
@@ -128,6 +129,7 @@ static fm_status install_basis(fm_ctx* ctx, const double* d_Bref) {
     FM_CUDA_TRY(ctx, cudaDeviceSynchronize());
     const int mode = kl_mode_of(ctx);
     if (mode == FM_KL_BF16 || mode == FM_KL_BF16X3) FM_TRY(kl_tc_install(ctx, mode == FM_KL_BF16X3));
+    else FM_TRY(kl_split_install(ctx));
     ctx->basis_ready = true;
     return FM_OK;
 }
@@ -328,10 +330,12 @@ extern "C" fm_status kl_field_batch(fm_ctx* ctx, int32_t level, uint32_t n, cons
     const int mode = kl_mode_of(ctx);
     if (mode == FM_KL_BF16 || mode == FM_KL_BF16X3)
         return kl_tc_field(ctx, level, n, d_xi, d_K, as_stream(stream));
+    FM_CHECK_ARG(ctx, (n + kTS - 1) / kTS <= 65535, "kl_field_batch: too many samples in one call");
+    fm_status fs = FM_OK;
+    if (kl_split_field(ctx, level, n, d_xi, d_K, as_stream(stream), &fs)) return fs;
     const int N = grid_of_level(ctx, level);
     const int cells = N * N;
     dim3 grid((cells + kTC - 1) / kTC, (n + kTS - 1) / kTS);
-    FM_CHECK_ARG(ctx, grid.y <= 65535, "kl_field_batch: too many samples in one call");
     const double M = ctx->cfg.M;
     FM_TIMED(ctx, kFamKlGemm, as_stream(stream), 8.0 * ((double)n * M + (double)cells * M + (double)n * cells),
              2.0 * n * (double)cells * M,

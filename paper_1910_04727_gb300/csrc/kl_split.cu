@@ -1,0 +1,411 @@
+// FP64 KL field synthesis (Sec. 3.1) on the tensor cores:
+//   K[s][c] = exp( sum_k B[c][k] xi[s][k] )
+// by the error-free splitting of Ozaki, Ogita, Oishi & Rump (Numer. Algorithms
+// 59, 2012).  A row of B (or xi) is scaled by a power of two to magnitudes
+// below 1/2 and cut into nine signed digits of seven bits, |d| <= 64, which
+// BF16 holds exactly (digit i as d 2^(-7 i)): 63 bits below the row's scale,
+// where FP64 has 53 below each entry.  The product of two digits is at most
+// 2^12 units, so the sum of the products of all digit pairs (i, j) with i + j
+// = t over up to 512 modes stays within 2^24 units: the FP32 accumulators of
+// the tensor cores hold it exactly, in whatever order they add.  Pairs with i +
+// j <= 8 (from 0) are kept: t = 0 .. 7 in accumulators of their own, t = 8, whose
+// place value is 2^-70 of the row scales, rounded into the eighth; the rest
+// are below 2^-65.  The epilogue joins the accumulators in integers, rounds
+// twice, and takes the exponential.  (Eight digits and t <= 7 would do for
+// rows of even size; a row with one entry thousands of times the others,
+// against a small coefficient, was then less accurate than the plain sum.)
+//
+// Bound: the FP64 pipe, two operations per clock and SM.  A contraction in it
+// takes M operations per field value and its exponential 21; here the
+// conversion takes 3 and the exponential 11 (fm_exp below), and the 45 M
+// tensor-core products per value run beside it (two CTAs per SM, one's
+// epilogue under the other's loads and products).  2000 fields of 64 x 64
+// cells from 128 modes: 396 us, 2035 by the FP64 contraction (95% of that
+// pipe), with errors against 128-bit arithmetic of 8.2e-17 (rms; at most
+// 4.9e-16) against its 6.9e-16 (6.2e-15).
+//
+// One CTA: 128 cells x 32 samples, eight 128 x 32 accumulators in 256 columns
+// of tensor memory.  Warp 0 (one thread) brings all digits of 32 modes into
+// shared memory by TMA (64-byte swizzle, 90 KB), warp 1 (one thread) issues
+// the 45 products, all eight warps drain.
+#include <cuda_bf16.h>
+#include <cudaTypedefs.h>
+
+#include <algorithm>
+
+#include "common.cuh"
+#include "tc.cuh"
+
+namespace fm {
+
+constexpr int kOzDigits = 9, kOzBits = 7, kOzAcc = 8;   // digits a row, bits a digit, accumulators
+constexpr int kOzM = 128;      // cells per tile (MMA M)
+constexpr int kOzN = 32;       // samples per tile (MMA N)
+constexpr int kOzK = 32;       // modes per stage (one 64-byte swizzle row)
+constexpr int kOzThreads = 256;
+constexpr int kOzMaxM = 512;   // 512 modes x 8 pairs x 2^12 = 2^24
+constexpr uint32_t kOzABytes = kOzM * kOzK * 2, kOzBBytes = kOzN * kOzK * 2;
+constexpr size_t kOzSmem = 1024 + kOzDigits * (kOzABytes + kOzBBytes) + 64 * 16 + 64;
+constexpr int kOzNoScale = -(1 << 28);   // exponent of a row that is not split (a value that is not finite, or far out)
+constexpr size_t kOzMaxBytes = (size_t)4 << 30;   // most digits kept per level
+
+// 2^(j / 64) as the sum of two doubles.
+__device__ const double2 kExpTable[64] = {
+    {0x1.0000000000000p+0, 0x0.0p+0}, {0x1.02c9a3e778061p+0, -0x1.19083535b085dp-56},
+    {0x1.059b0d3158574p+0, 0x1.d73e2a475b465p-55}, {0x1.0874518759bc8p+0, 0x1.186be4bb284ffp-57},
+    {0x1.0b5586cf9890fp+0, 0x1.8a62e4adc610bp-54}, {0x1.0e3ec32d3d1a2p+0, 0x1.03a1727c57b53p-59},
+    {0x1.11301d0125b51p+0, -0x1.6c51039449b3ap-54}, {0x1.1429aaea92de0p+0, -0x1.32fbf9af1369ep-54},
+    {0x1.172b83c7d517bp+0, -0x1.19041b9d78a76p-55}, {0x1.1a35beb6fcb75p+0, 0x1.e5b4c7b4968e4p-55},
+    {0x1.1d4873168b9aap+0, 0x1.e016e00a2643cp-54}, {0x1.2063b88628cd6p+0, 0x1.dc775814a8495p-55},
+    {0x1.2387a6e756238p+0, 0x1.9b07eb6c70573p-54}, {0x1.26b4565e27cddp+0, 0x1.2bd339940e9d9p-55},
+    {0x1.29e9df51fdee1p+0, 0x1.612e8afad1255p-55}, {0x1.2d285a6e4030bp+0, 0x1.0024754db41d5p-54},
+    {0x1.306fe0a31b715p+0, 0x1.6f46ad23182e4p-55}, {0x1.33c08b26416ffp+0, 0x1.32721843659a6p-54},
+    {0x1.371a7373aa9cbp+0, -0x1.63aeabf42eae2p-54}, {0x1.3a7db34e59ff7p+0, -0x1.5e436d661f5e3p-56},
+    {0x1.3dea64c123422p+0, 0x1.ada0911f09ebcp-55}, {0x1.4160a21f72e2ap+0, -0x1.ef3691c309278p-58},
+    {0x1.44e086061892dp+0, 0x1.89b7a04ef80d0p-59}, {0x1.486a2b5c13cd0p+0, 0x1.3c1a3b69062f0p-56},
+    {0x1.4bfdad5362a27p+0, 0x1.d4397afec42e2p-56}, {0x1.4f9b2769d2ca7p+0, -0x1.4b309d25957e3p-54},
+    {0x1.5342b569d4f82p+0, -0x1.07abe1db13cadp-55}, {0x1.56f4736b527dap+0, 0x1.9bb2c011d93adp-54},
+    {0x1.5ab07dd485429p+0, 0x1.6324c054647adp-54}, {0x1.5e76f15ad2148p+0, 0x1.ba6f93080e65ep-54},
+    {0x1.6247eb03a5585p+0, -0x1.383c17e40b497p-54}, {0x1.6623882552225p+0, -0x1.bb60987591c34p-54},
+    {0x1.6a09e667f3bcdp+0, -0x1.bdd3413b26456p-54}, {0x1.6dfb23c651a2fp+0, -0x1.bbe3a683c88abp-57},
+    {0x1.71f75e8ec5f74p+0, -0x1.16e4786887a99p-55}, {0x1.75feb564267c9p+0, -0x1.0245957316dd3p-54},
+    {0x1.7a11473eb0187p+0, -0x1.41577ee04992fp-55}, {0x1.7e2f336cf4e62p+0, 0x1.05d02ba15797ep-56},
+    {0x1.82589994cce13p+0, -0x1.d4c1dd41532d8p-54}, {0x1.868d99b4492edp+0, -0x1.fc6f89bd4f6bap-54},
+    {0x1.8ace5422aa0dbp+0, 0x1.6e9f156864b27p-54}, {0x1.8f1ae99157736p+0, 0x1.5cc13a2e3976cp-55},
+    {0x1.93737b0cdc5e5p+0, -0x1.75fc781b57ebcp-57}, {0x1.97d829fde4e50p+0, -0x1.d185b7c1b85d1p-54},
+    {0x1.9c49182a3f090p+0, 0x1.c7c46b071f2bep-56}, {0x1.a0c667b5de565p+0, -0x1.359495d1cd533p-54},
+    {0x1.a5503b23e255dp+0, -0x1.d2f6edb8d41e1p-54}, {0x1.a9e6b5579fdbfp+0, 0x1.0fac90ef7fd31p-54},
+    {0x1.ae89f995ad3adp+0, 0x1.7a1cd345dcc81p-54}, {0x1.b33a2b84f15fbp+0, -0x1.2805e3084d708p-57},
+    {0x1.b7f76f2fb5e47p+0, -0x1.5584f7e54ac3bp-56}, {0x1.bcc1e904bc1d2p+0, 0x1.23dd07a2d9e84p-55},
+    {0x1.c199bdd85529cp+0, 0x1.11065895048ddp-55}, {0x1.c67f12e57d14bp+0, 0x1.2884dff483cadp-54},
+    {0x1.cb720dcef9069p+0, 0x1.503cbd1e949dbp-56}, {0x1.d072d4a07897cp+0, -0x1.cbc3743797a9cp-54},
+    {0x1.d5818dcfba487p+0, 0x1.2ed02d75b3707p-55}, {0x1.da9e603db3285p+0, 0x1.c2300696db532p-54},
+    {0x1.dfc97337b9b5fp+0, -0x1.1a5cd4f184b5cp-54}, {0x1.e502ee78b3ff6p+0, 0x1.39e8980a9cc8fp-55},
+    {0x1.ea4afa2a490dap+0, -0x1.e9c23179c2893p-54}, {0x1.efa1bee615a27p+0, 0x1.dc7f486a4b6b0p-54},
+    {0x1.f50765b6e4540p+0, 0x1.9d3e12dd8a18bp-54}, {0x1.fa7c1819e90d8p+0, 0x1.74853f3a5931ep-55},
+};
+
+// e^x to within 0.53 ulp (table-driven: Tang, ACM TOMS 15, 1989): x = n ln 2 / 64
+// + r, e^x = 2^(n / 64) (1 + p(r)), |r| <= ln 2 / 128, p the Taylor polynomial
+// of degree 5 (its remainder below 2^-54.6), the table value in two parts.
+// Eleven FP64 operations; the exponent is added in integers.
+__device__ __forceinline__ double fm_exp(double x, const double2* tab) {
+    if (!(fabs(x) < 700.0)) return exp(x);   // over- and underflow, NaN
+    constexpr double kMagic = 6755399441055744.0;   // 1.5 2^52
+    const double t = fma(x, 0x1.71547652b82fep+6, kMagic);
+    const int n = __double2loint(t);
+    const double tn = t - kMagic;
+    const double r = fma(tn, -0x1.9ef35793c7673p-47, fma(tn, -0x1.62e42fefa2000p-7, x));
+    const double r2 = r * r;
+    double q = fma(r, 1.0 / 120, 1.0 / 24);
+    q = fma(q, r, 1.0 / 6);
+    q = fma(q, r, 0.5);
+    const double p = fma(q, r2, r);
+    const double2 e = tab[n & 63];
+    const double v = e.x + fma(e.x, p, e.y);
+    return __hiloint2double(__double2hiint(v) + ((n >> 6) << 20), __double2loint(v));
+}
+
+// The sum of the eight accumulators (of d d 2^(-7 t)), in units of 2^-14, scaled
+// by 2^e.
+__device__ __forceinline__ double oz_join(const uint32_t (&acc)[kOzAcc][8], int i, int e) {
+    long long h = 0, l = 0;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        const float uh = __uint_as_float(acc[t][i]) * (float)(1LL << (kOzBits * t));
+        const float ul = __uint_as_float(acc[t + 4][i]) * (float)(1LL << (kOzBits * (t + 4)));
+        h += (long long)__float2int_rn(uh) * (1LL << (kOzBits * (3 - t)));
+        l += (long long)__float2int_rn(ul) * (1LL << (kOzBits * (3 - t)));
+    }
+    // |h|, |l| < 2^51: the bits of 1.5 2^52 + h, less 1.5 2^52
+    constexpr long long kBits = 0x4338000000000000LL;
+    constexpr double kMagic = 6755399441055744.0;
+    const double dh = __longlong_as_double(kBits + h) - kMagic, dl = __longlong_as_double(kBits + l) - kMagic;
+    const double g = fma(dl, 0x1p-28, dh);
+    const int hi = __double2hiint(g);
+    // times 2^(e - 35) in the exponent field (g is 0 or between 2^-28 and 2^47)
+    return (hi << 1) == 0 ? 0.0 : __hiloint2double(hi + ((e - 5 * kOzBits) << 20), __double2loint(g));
+}
+
+__device__ __forceinline__ void tmem_ld_32x32b_x8(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+}
+
+// Shared-memory matrix descriptor of a K-major tile written by TMA with
+// 64-byte swizzling: rows of 64 B, 8-row groups 512 B apart.
+__device__ __forceinline__ uint64_t sdesc_kmajor_sw64(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);   // start address
+    d |= (uint64_t)1 << 16;                     // leading-dimension offset (unused here)
+    d |= (uint64_t)(512 >> 4) << 32;            // stride between 8-row groups
+    d |= (uint64_t)1 << 46;                     // descriptor version of tcgen05
+    d |= (uint64_t)4 << 61;                     // 64-byte swizzle
+    return d;
+}
+
+__global__ void __launch_bounds__(kOzThreads, 2)
+    k_kl_split(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int cells, int S,
+               int M, int Mpad, const int* __restrict__ ec, const int* __restrict__ ex, const double* __restrict__ B,
+               const double* __restrict__ xi, double* __restrict__ K, int* __restrict__ err) {
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = tc::smem_u32(smem_raw);
+    uint8_t* sA = smem_raw + ((1024 - (raw & 1023)) & 1023);   // digit i at i kOzABytes
+    uint8_t* sB = sA + kOzDigits * kOzABytes;
+    double2* tab = reinterpret_cast<double2*>(sB + kOzDigits * kOzBBytes);
+    uint64_t* full = reinterpret_cast<uint64_t*>(tab + 64);
+    uint64_t* empty = full + 1;
+    uint64_t* done = full + 2;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(full + 3);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int s0 = blockIdx.x * kOzN, c0 = blockIdx.y * kOzM;
+    if (threadIdx.x < 64) tab[threadIdx.x] = kExpTable[threadIdx.x];
+    if (threadIdx.x == 0) {
+        tc::mbar_init(full, 1);
+        tc::mbar_init(empty, 1);
+        tc::mbar_init(done, 1);
+        tc::fence_barrier_init();
+        tc::prefetch_tensormap(&mapA);
+        tc::prefetch_tensormap(&mapB);
+    }
+    if (warp == 0) tc::tmem_alloc(tmem_slot, kOzAcc * kOzN);
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = *tmem_slot;
+    const int kblocks = Mpad / kOzK;
+    if (warp == 0 && lane == 0) {
+        int issued = 0;
+        for (int kb = 0; kb < kblocks; ++kb) {
+            if (kb > 0 && !tc::mbar_wait(empty, (kb - 1) & 1, err)) break;
+            tc::mbar_arrive_expect_tx(full, kOzDigits * (kOzABytes + kOzBBytes));
+            for (int i = 0; i < kOzDigits; ++i) {
+                tc::tma_load_2d(sA + i * kOzABytes, &mapA, full, i * Mpad + kb * kOzK, c0);
+                tc::tma_load_2d(sB + i * kOzBBytes, &mapB, full, i * Mpad + kb * kOzK, s0);
+            }
+            ++issued;
+        }
+        tc::drain_loads(full, 1, issued, err);
+    } else if (warp == 1 && lane == 0) {
+        constexpr uint32_t idesc = tc::idesc_bf16_f32(kOzM, kOzN);
+        for (int kb = 0; kb < kblocks; ++kb) {
+            if (!tc::mbar_wait(full, kb & 1, err)) break;
+            tc::fence_after_sync();
+            for (int i = 0; i < kOzDigits; ++i)
+                for (int j = 0; i + j < kOzDigits; ++j) {
+                    const int t = i + j < kOzAcc ? i + j : kOzAcc - 1;
+                    const uint32_t a = tc::smem_u32(sA + i * kOzABytes), b = tc::smem_u32(sB + j * kOzBBytes);
+#pragma unroll
+                    for (int k = 0; k < kOzK / 16; ++k)
+                        tc::mma_bf16(tmem + t * kOzN, sdesc_kmajor_sw64(a + 32 * k), sdesc_kmajor_sw64(b + 32 * k),
+                                     idesc, (kb | i | k) != 0 || j >= kOzAcc);
+                }
+            tc::mma_commit(empty);
+        }
+        tc::mma_commit(done);
+    }
+    __syncwarp();
+    const bool ok = tc::mbar_wait(done, 0, err);
+    __syncwarp();
+    tc::fence_after_sync();
+    if (ok) {
+        const int c = c0 + 32 * (warp & 3) + lane;
+        const int e_c = c < cells ? ec[c] : 0;
+        const uint32_t row = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            const int col = 16 * (warp >> 2) + 8 * h;
+            uint32_t acc[kOzAcc][8];
+#pragma unroll
+            for (int t = 0; t < kOzAcc; ++t) tmem_ld_32x32b_x8(row + t * kOzN + col, acc[t]);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int s = s0 + col + i;
+                if (c >= cells || s >= S) continue;
+                const int e = e_c + ex[s];
+                double g;
+                if (e > -(1 << 20)) {
+                    g = oz_join(acc, i, e);
+                } else {   // a row that is not split: the plain sum
+                    g = 0.0;
+                    for (int k = 0; k < M; ++k) g = fma(xi[(size_t)s * M + k], B[(size_t)c * M + k], g);
+                }
+                K[(size_t)s * cells + c] = fm_exp(g, tab);
+            }
+        }
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    if (warp == 0) tc::tmem_dealloc(tmem, kOzAcc * kOzN);
+}
+
+// Rows of x (FP64 [rows][M]) -> digits out [rows][9 Mpad] BF16, digit i of mode
+// k at i Mpad + k (zero beyond M), and the rows' scale exponents: x = 2^(e - 7)
+// sum_i d_i 2^(-7 i).  One warp per row.  In integers: the value below the scale
+// as a 63-bit fixed-point number, cut from the low end into balanced digits.
+__global__ void k_split_rows(size_t rows, int M, int Mpad, const double* __restrict__ x,
+                             __nv_bfloat16* __restrict__ out, int* __restrict__ exps) {
+    const size_t r = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (r >= rows) return;
+    const double* row = x + r * M;
+    int top = 0;   // largest biased exponent of the row
+    for (int k = lane; k < M; k += 32) top = max(top, (__double2hiint(row[k]) >> 20) & 0x7FF);
+    top = __reduce_max_sync(0xffffffffu, top);
+    // 2^e is at least twice the largest magnitude; rows with values that are
+    // not finite, or with scales far from 1, are left to the plain sum
+    const int e = top - 1023 + 2;
+    const bool split = top != 0x7FF && e < 200 && (e > -200 || top == 0);
+    if (lane == 0) exps[r] = split ? (top == 0 ? 0 : e) : kOzNoScale;
+    __nv_bfloat16* o = out + r * (size_t)(kOzDigits * Mpad);
+    for (int k = lane; k < Mpad; k += 32) {
+        long long v = 0;
+        if (k < M && split && top != 0) {
+            const long long bits = __double_as_longlong(row[k]);
+            const int be = (int)(bits >> 52) & 0x7FF;
+            if (be != 0) {
+                // mantissa 2^52 .. 2^53 at exponent be - 1075; in units of 2^(e - 63)
+                const long long m = (bits & 0xFFFFFFFFFFFFFLL) | (1LL << 52);
+                const int sh = be - 1075 - (e - kOzDigits * kOzBits);   // at most 9
+                if (sh >= 0) v = m << sh;
+                else if (sh > -54) v = (m + (1LL << (-sh - 1))) >> -sh;
+                if (bits < 0) v = -v;
+            }
+        }
+#pragma unroll
+        for (int i = kOzDigits - 1; i >= 0; --i) {
+            const int d = i > 0 ? ((int)(v + 64) & 127) - 64 : (int)v;
+            v = (v - d) >> kOzBits;
+            o[(size_t)i * Mpad + k] = __float2bfloat16_rn((float)d * (1.0f / (float)(1LL << (kOzBits * i))));
+        }
+    }
+}
+
+// ------------------------------------------------------------------ host
+static bool oz_map(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t width, uint32_t box_rows) {
+    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+    if (!fn) {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) !=
+                cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            return false;
+        fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+    }
+    cuuint64_t dims[2] = {width, rows};
+    cuuint64_t strides[1] = {width * 2};
+    cuuint32_t box[2] = {(cuuint32_t)kOzK, box_rows};
+    cuuint32_t estr[2] = {1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+static unsigned warps_grid(size_t rows) { return (unsigned)((rows + 7) / 8); }
+
+// Digits of the installed basis, level by level (levels whose digits would
+// take more than kOzMaxBytes, and bases of more than 512 modes, keep the FP64
+// contraction).
+fm_status kl_split_install(fm_ctx* ctx) {
+    const int M = ctx->cfg.M;
+    OzState& z = ctx->oz;
+    z.Mpad = (M + kOzK - 1) / kOzK * kOzK;
+    for (int l = 0; l < ctx->cfg.n_levels; ++l) {
+        const int n = grid_of_level(ctx, l);
+        const size_t cells = (size_t)n * n, bytes = cells * kOzDigits * z.Mpad * 2;
+        z.have[l] = false;
+        if (M > kOzMaxM || bytes > kOzMaxBytes || (cells + kOzM - 1) / kOzM > 65535) continue;
+        if (!z.basis[l] && (cudaMalloc(&z.basis[l], bytes) != cudaSuccess ||
+                            cudaMalloc((void**)&z.ec[l], cells * sizeof(int)) != cudaSuccess)) {
+            cudaGetLastError();   // no room for the digits: the FP64 contraction serves this level
+            cudaFree(z.basis[l]);
+            z.basis[l] = nullptr;
+            continue;
+        }
+        k_split_rows<<<warps_grid(cells), 256>>>(cells, M, z.Mpad, ctx->d_basis[l], (__nv_bfloat16*)z.basis[l],
+                                                 z.ec[l]);
+        z.have[l] = oz_map(&z.mapA[l], z.basis[l], cells, (uint64_t)kOzDigits * z.Mpad, kOzM);
+    }
+    FM_CUDA_TRY(ctx, cudaDeviceSynchronize());
+    return FM_OK;
+}
+
+void kl_split_free(fm_ctx* ctx) {
+    for (int l = 0; l < FM_MAX_LEVELS; ++l) {
+        cudaFree(ctx->oz.basis[l]);
+        cudaFree(ctx->oz.ec[l]);
+    }
+    for (OzState::Xi& x : ctx->oz.xi) {
+        cudaFree(x.digits);
+        cudaFree(x.ex);
+    }
+}
+
+// Fields of n samples of `level` into d_K; false: the caller's FP64
+// contraction serves this call (no digits of this level, a stream beyond the
+// kept buffers, or a stream capture, whose graph would keep a buffer's address).
+bool kl_split_field(fm_ctx* ctx, int level, uint32_t n, const double* d_xi, double* d_K, cudaStream_t st,
+                    fm_status* status) {
+    OzState& z = ctx->oz;
+    *status = FM_OK;
+    if (!z.have[level]) return false;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone ||
+        cudaStreamGetId(st, &id) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    // the digits of xi: one buffer per stream (calls on other streams may
+    // overlap this one), up to kStreams of them
+    OzState::Xi* x = nullptr;
+    for (OzState::Xi& c : z.xi)
+        if (c.cap && c.id == id) x = &c;
+    for (OzState::Xi& c : z.xi)
+        if (!x && !c.cap) x = &c;
+    if (!x) return false;
+    if (x->cap < n) {
+        cudaFree(x->digits);
+        cudaFree(x->ex);
+        x->digits = nullptr;
+        x->ex = nullptr;
+        x->cap = 0;
+        if (cudaMalloc(&x->digits, (size_t)n * kOzDigits * z.Mpad * 2) != cudaSuccess ||
+            cudaMalloc((void**)&x->ex, (size_t)n * sizeof(int)) != cudaSuccess ||
+            !oz_map(&x->map, x->digits, n, (uint64_t)kOzDigits * z.Mpad, kOzN)) {
+            cudaGetLastError();
+            cudaFree(x->digits);
+            cudaFree(x->ex);
+            x->digits = nullptr;
+            x->ex = nullptr;
+            return false;
+        }
+        x->cap = n;
+        x->id = id;
+    }
+    const int N = grid_of_level(ctx, level), cells = N * N, M = ctx->cfg.M;
+    k_split_rows<<<warps_grid(n), 256, 0, st>>>(n, M, z.Mpad, d_xi, (__nv_bfloat16*)x->digits, x->ex);
+    const dim3 grid((n + kOzN - 1) / kOzN, (cells + kOzM - 1) / kOzM);
+    FM_TIMED(ctx, kFamKlGemm, st, 8.0 * ((double)n * M + (double)cells * M + (double)n * cells),
+             2.0 * n * (double)cells * M,
+             k_kl_split<<<grid, kOzThreads, kOzSmem, st>>>(z.mapA[level], x->map, cells, (int)n, M, z.Mpad,
+                                                           z.ec[level], x->ex, ctx->d_basis[level], d_xi, d_K,
+                                                           ctx->tc.err));
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) {
+        set_error(ctx, std::string("kl_field_batch: ") + cudaGetErrorString(e));
+        *status = FM_ECUDA;
+    }
+    return true;
+}
+
+void kl_split_init_attributes() {
+    cudaFuncSetAttribute(k_kl_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzSmem);
+    cudaGetLastError();
+}
+
+}  // namespace fm
