@@ -18,16 +18,14 @@
 // Bound: the FP64 pipe, two operations per clock and SM.  A contraction in it
 // takes M operations per field value and its exponential 21; here the
 // conversion takes 3 and the exponential 11 (fm_exp below), and the 45 M
-// tensor-core products per value run beside it (two CTAs per SM, one's
-// epilogue under the other's loads and products).  2000 fields of 64 x 64
-// cells from 128 modes: 396 us, 2035 by the FP64 contraction (95% of that
+// tensor-core products per value run beside it, a tile ahead.  2000 fields of
+// 64 x 64 cells from 128 modes: 283 us (388 with a tile per CTA and two CTAs an
+// SM, whose loads and products were not hidden), 2035 by the FP64 contraction (95% of that
 // pipe), with errors against 128-bit arithmetic of 8.2e-17 (rms; at most
 // 4.9e-16) against its 6.9e-16 (6.2e-15).
 //
-// One CTA: 128 cells x 32 samples, eight 128 x 32 accumulators in 256 columns
-// of tensor memory.  Warp 0 (one thread) brings all digits of 32 modes into
-// shared memory by TMA (64-byte swizzle, 90 KB), warp 1 (one thread) issues
-// the 45 products, all eight warps drain.
+// A tile is 128 cells x 32 samples: eight 128 x 32 accumulators in 256 columns
+// of tensor memory, the digits of 32 modes per stage (64-byte swizzle, 90 KB).
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
@@ -42,10 +40,13 @@ constexpr int kOzDigits = 9, kOzBits = 7, kOzAcc = 8;   // digits a row, bits a 
 constexpr int kOzM = 128;      // cells per tile (MMA M)
 constexpr int kOzN = 32;       // samples per tile (MMA N)
 constexpr int kOzK = 32;       // modes per stage (one 64-byte swizzle row)
-constexpr int kOzThreads = 256;
+constexpr int kOzEpi = 256;          // threads that drain and store
+constexpr int kOzThreads = kOzEpi + 64;
+constexpr int kOzStages = 2;
 constexpr int kOzMaxM = 512;   // 512 modes x 8 pairs x 2^12 = 2^24
 constexpr uint32_t kOzABytes = kOzM * kOzK * 2, kOzBBytes = kOzN * kOzK * 2;
-constexpr size_t kOzSmem = 1024 + kOzDigits * (kOzABytes + kOzBBytes) + 64 * 16 + 64;
+constexpr uint32_t kOzStage = kOzDigits * (kOzABytes + kOzBBytes);
+constexpr size_t kOzSmem = 1024 + kOzStages * kOzStage + 64 * 16 + 128;
 constexpr int kOzNoScale = -(1 << 28);   // exponent of a row that is not split (a value that is not finite, or far out)
 constexpr size_t kOzMaxBytes = (size_t)4 << 30;   // most digits kept per level
 
@@ -90,7 +91,8 @@ __device__ const double2 kExpTable[64] = {
 // of degree 5 (its remainder below 2^-54.6), the table value in two parts.
 // Eleven FP64 operations; the exponent is added in integers.
 __device__ __forceinline__ double fm_exp(double x, const double2* tab) {
-    if (!(fabs(x) < 700.0)) return exp(x);   // over- and underflow, NaN
+    // (compared in integers: a comparison is an operation of the FP64 pipe too)
+    if ((unsigned)(__double2hiint(x) & 0x7FFFFFFF) >= 0x4085E000u) return exp(x);   // |x| >= 700, NaN
     constexpr double kMagic = 6755399441055744.0;   // 1.5 2^52
     const double t = fma(x, 0x1.71547652b82fep+6, kMagic);
     const int n = __double2loint(t);
@@ -146,100 +148,138 @@ __device__ __forceinline__ uint64_t sdesc_kmajor_sw64(uint32_t saddr) {
     return d;
 }
 
-__global__ void __launch_bounds__(kOzThreads, 2)
+// Persistent: CTA b takes tiles b, b + gridDim.x, ... (sample tiles fastest).
+// Warps 0 .. 7 drain, warp 8 (one thread) loads, warp 9 (one thread) issues the
+// products; two stages of operands and two sets of accumulators, so the next
+// tile's products run under this one's epilogue.
+__global__ void __launch_bounds__(kOzThreads, 1)
     k_kl_split(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int cells, int S,
                int M, int Mpad, const int* __restrict__ ec, const int* __restrict__ ex, const double* __restrict__ B,
                const double* __restrict__ xi, double* __restrict__ K, int* __restrict__ err) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = tc::smem_u32(smem_raw);
-    uint8_t* sA = smem_raw + ((1024 - (raw & 1023)) & 1023);   // digit i at i kOzABytes
-    uint8_t* sB = sA + kOzDigits * kOzABytes;
-    double2* tab = reinterpret_cast<double2*>(sB + kOzDigits * kOzBBytes);
+    uint8_t* stage = smem_raw + ((1024 - (raw & 1023)) & 1023);   // per stage: A digits, then B digits
+    double2* tab = reinterpret_cast<double2*>(stage + kOzStages * kOzStage);
     uint64_t* full = reinterpret_cast<uint64_t*>(tab + 64);
-    uint64_t* empty = full + 1;
-    uint64_t* done = full + 2;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(full + 3);
+    uint64_t* empty = full + kOzStages;
+    uint64_t* tfull = empty + kOzStages;    // accumulators ready, by set
+    uint64_t* tempty = tfull + 2;           // accumulators drained
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int s0 = blockIdx.x * kOzN, c0 = blockIdx.y * kOzM;
+    const unsigned stiles = (unsigned)(S + kOzN - 1) / kOzN, tiles = stiles * ((unsigned)(cells + kOzM - 1) / kOzM);
     if (threadIdx.x < 64) tab[threadIdx.x] = kExpTable[threadIdx.x];
     if (threadIdx.x == 0) {
-        tc::mbar_init(full, 1);
-        tc::mbar_init(empty, 1);
-        tc::mbar_init(done, 1);
+        for (int i = 0; i < kOzStages; ++i) {
+            tc::mbar_init(&full[i], 1);
+            tc::mbar_init(&empty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            tc::mbar_init(&tfull[i], 1);
+            tc::mbar_init(&tempty[i], kOzEpi);
+        }
         tc::fence_barrier_init();
         tc::prefetch_tensormap(&mapA);
         tc::prefetch_tensormap(&mapB);
     }
-    if (warp == 0) tc::tmem_alloc(tmem_slot, kOzAcc * kOzN);
+    if (warp == 0) tc::tmem_alloc(tmem_slot, 2 * kOzAcc * kOzN);
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
     const int kblocks = Mpad / kOzK;
-    if (warp == 0 && lane == 0) {
-        int issued = 0;
-        for (int kb = 0; kb < kblocks; ++kb) {
-            if (kb > 0 && !tc::mbar_wait(empty, (kb - 1) & 1, err)) break;
-            tc::mbar_arrive_expect_tx(full, kOzDigits * (kOzABytes + kOzBBytes));
-            for (int i = 0; i < kOzDigits; ++i) {
-                tc::tma_load_2d(sA + i * kOzABytes, &mapA, full, i * Mpad + kb * kOzK, c0);
-                tc::tma_load_2d(sB + i * kOzBBytes, &mapB, full, i * Mpad + kb * kOzK, s0);
+    if (warp == 8) {
+        if (lane == 0) {
+            int q = 0;   // stage loads so far
+            bool ok = true;
+            for (unsigned tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x) {
+                const int s0 = (int)(tile % stiles) * kOzN, c0 = (int)(tile / stiles) * kOzM;
+                for (int kb = 0; kb < kblocks; ++kb) {
+                    const int st = q % kOzStages, round = q / kOzStages;
+                    if (round > 0 && !(ok = tc::mbar_wait(&empty[st], (round - 1) & 1, err))) break;
+                    uint8_t* a = stage + st * kOzStage;
+                    uint8_t* b = a + kOzDigits * kOzABytes;
+                    tc::mbar_arrive_expect_tx(&full[st], kOzStage);
+                    for (int i = 0; i < kOzDigits; ++i) {
+                        tc::tma_load_2d(a + i * kOzABytes, &mapA, &full[st], i * Mpad + kb * kOzK, c0);
+                        tc::tma_load_2d(b + i * kOzBBytes, &mapB, &full[st], i * Mpad + kb * kOzK, s0);
+                    }
+                    ++q;
+                }
             }
-            ++issued;
+            tc::drain_loads(full, kOzStages, q, err);
         }
-        tc::drain_loads(full, 1, issued, err);
-    } else if (warp == 1 && lane == 0) {
-        constexpr uint32_t idesc = tc::idesc_bf16_f32(kOzM, kOzN);
-        for (int kb = 0; kb < kblocks; ++kb) {
-            if (!tc::mbar_wait(full, kb & 1, err)) break;
+    } else if (warp == 9) {
+        if (lane == 0) {
+            constexpr uint32_t idesc = tc::idesc_bf16_f32(kOzM, kOzN);
+            int q = 0, it = 0;
+            bool ok = true;
+            for (unsigned tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x, ++it) {
+                const int set = it & 1;
+                if (it >= 2 && !(ok = tc::mbar_wait(&tempty[set], ((it >> 1) - 1) & 1, err))) break;
+                tc::fence_after_sync();
+                const uint32_t acc = tmem + set * (kOzAcc * kOzN);
+                for (int kb = 0; kb < kblocks; ++kb, ++q) {
+                    const int st = q % kOzStages;
+                    if (!(ok = tc::mbar_wait(&full[st], (q / kOzStages) & 1, err))) break;
+                    tc::fence_after_sync();
+                    const uint32_t sa = tc::smem_u32(stage + st * kOzStage), sb = sa + kOzDigits * kOzABytes;
+                    for (int i = 0; i < kOzDigits; ++i)
+                        for (int j = 0; i + j < kOzDigits; ++j) {
+                            const int t = i + j < kOzAcc ? i + j : kOzAcc - 1;
+                            const uint32_t a = sa + i * kOzABytes, b = sb + j * kOzBBytes;
+#pragma unroll
+                            for (int k = 0; k < kOzK / 16; ++k)
+                                tc::mma_bf16(acc + t * kOzN, sdesc_kmajor_sw64(a + 32 * k),
+                                             sdesc_kmajor_sw64(b + 32 * k), idesc, (kb | i | k) != 0 || j >= kOzAcc);
+                        }
+                    tc::mma_commit(&empty[st]);
+                }
+                tc::mma_commit(&tfull[set]);
+            }
+        }
+    } else {
+        int it = 0;
+        for (unsigned tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++it) {
+            const int set = it & 1;
+            const int s0 = (int)(tile % stiles) * kOzN, c0 = (int)(tile / stiles) * kOzM;
+            const int c = c0 + 32 * (warp & 3) + lane;
+            const int e_c = c < cells ? ec[c] : 0;
+            // all lanes or none (the loads below are warp-wide)
+            const bool ok = __all_sync(0xffffffffu, tc::mbar_wait(&tfull[set], (it >> 1) & 1, err));
+            if (!ok) break;
             tc::fence_after_sync();
-            for (int i = 0; i < kOzDigits; ++i)
-                for (int j = 0; i + j < kOzDigits; ++j) {
-                    const int t = i + j < kOzAcc ? i + j : kOzAcc - 1;
-                    const uint32_t a = tc::smem_u32(sA + i * kOzABytes), b = tc::smem_u32(sB + j * kOzBBytes);
-#pragma unroll
-                    for (int k = 0; k < kOzK / 16; ++k)
-                        tc::mma_bf16(tmem + t * kOzN, sdesc_kmajor_sw64(a + 32 * k), sdesc_kmajor_sw64(b + 32 * k),
-                                     idesc, (kb | i | k) != 0 || j >= kOzAcc);
-                }
-            tc::mma_commit(empty);
-        }
-        tc::mma_commit(done);
-    }
-    __syncwarp();
-    const bool ok = tc::mbar_wait(done, 0, err);
-    __syncwarp();
-    tc::fence_after_sync();
-    if (ok) {
-        const int c = c0 + 32 * (warp & 3) + lane;
-        const int e_c = c < cells ? ec[c] : 0;
-        const uint32_t row = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+            const uint32_t row = tmem + set * (kOzAcc * kOzN) + ((uint32_t)(32 * (warp & 3)) << 16);
 #pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-            const int col = 16 * (warp >> 2) + 8 * h;
-            uint32_t acc[kOzAcc][8];
+            for (int h = 0; h < 2; ++h) {
+                const int col = 16 * (warp >> 2) + 8 * h;
+                uint32_t acc[kOzAcc][8];
 #pragma unroll
-            for (int t = 0; t < kOzAcc; ++t) tmem_ld_32x32b_x8(row + t * kOzN + col, acc[t]);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int s = s0 + col + i;
-                if (c >= cells || s >= S) continue;
-                const int e = e_c + ex[s];
-                double g;
-                if (e > -(1 << 20)) {
-                    g = oz_join(acc, i, e);
-                } else {   // a row that is not split: the plain sum
-                    g = 0.0;
-                    for (int k = 0; k < M; ++k) g = fma(xi[(size_t)s * M + k], B[(size_t)c * M + k], g);
+                for (int t = 0; t < kOzAcc; ++t) tmem_ld_32x32b_x8(row + t * kOzN + col, acc[t]);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if (h == 1) {   // this thread has read the set
+                    tc::fence_before_sync();
+                    tc::mbar_arrive(&tempty[set]);
                 }
-                K[(size_t)s * cells + c] = fm_exp(g, tab);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int s = s0 + col + i;
+                    if (c >= cells || s >= S) continue;
+                    const int e = e_c + ex[s];
+                    double g;
+                    if (e > -(1 << 20)) {
+                        g = oz_join(acc, i, e);
+                    } else {   // a row that is not split: the plain sum
+                        g = 0.0;
+                        for (int k = 0; k < M; ++k) g = fma(xi[(size_t)s * M + k], B[(size_t)c * M + k], g);
+                    }
+                    K[(size_t)s * cells + c] = fm_exp(g, tab);
+                }
             }
         }
     }
     tc::fence_before_sync();
     __syncthreads();
-    if (warp == 0) tc::tmem_dealloc(tmem, kOzAcc * kOzN);
+    if (warp == 0) tc::tmem_dealloc(tmem, 2 * kOzAcc * kOzN);
 }
 
 // Rows of x (FP64 [rows][M]) -> digits out [rows][9 Mpad] BF16, digit i of mode
@@ -318,7 +358,7 @@ fm_status kl_split_install(fm_ctx* ctx) {
         const int n = grid_of_level(ctx, l);
         const size_t cells = (size_t)n * n, bytes = cells * kOzDigits * z.Mpad * 2;
         z.have[l] = false;
-        if (M > kOzMaxM || bytes > kOzMaxBytes || (cells + kOzM - 1) / kOzM > 65535) continue;
+        if (M > kOzMaxM || bytes > kOzMaxBytes || cells > ((size_t)1 << 30)) continue;
         if (!z.basis[l] && (cudaMalloc(&z.basis[l], bytes) != cudaSuccess ||
                             cudaMalloc((void**)&z.ec[l], cells * sizeof(int)) != cudaSuccess)) {
             cudaGetLastError();   // no room for the digits: the FP64 contraction serves this level
@@ -389,7 +429,8 @@ bool kl_split_field(fm_ctx* ctx, int level, uint32_t n, const double* d_xi, doub
     }
     const int N = grid_of_level(ctx, level), cells = N * N, M = ctx->cfg.M;
     k_split_rows<<<warps_grid(n), 256, 0, st>>>(n, M, z.Mpad, d_xi, (__nv_bfloat16*)x->digits, x->ex);
-    const dim3 grid((n + kOzN - 1) / kOzN, (cells + kOzM - 1) / kOzM);
+    const size_t tiles = (size_t)((n + kOzN - 1) / kOzN) * ((cells + kOzM - 1) / kOzM);
+    const unsigned grid = (unsigned)std::min<size_t>(tiles, (size_t)std::max(ctx->sms, 1));
     FM_TIMED(ctx, kFamKlGemm, st, 8.0 * ((double)n * M + (double)cells * M + (double)n * cells),
              2.0 * n * (double)cells * M,
              k_kl_split<<<grid, kOzThreads, kOzSmem, st>>>(z.mapA[level], x->map, cells, (int)n, M, z.Mpad,
