@@ -34,10 +34,15 @@ namespace fm {
 constexpr int kH = 256;          // hidden width
 constexpr int kGm = 128;         // GEMM tile rows (MMA M)
 constexpr int kGk = 64;          // K per stage
-constexpr int kGStages = 2;
+// Operand stages of a GEMM: the training GEMMs (N tile 64) are chains of
+// latencies, so all four K blocks of a 256-wide layer are in flight at once
+// (with two stages the weight gradients' 16 blocks cost a round trip to L2
+// each pair); the inference GEMMs keep two, for two CTAs an SM.
+template <int BN>
+constexpr int gemm_stages() { return BN <= 64 ? 4 : 2; }
 constexpr int kMaxBatch = 4096;  // training mini-batch capacity (leading dimension of transposed operands)
 constexpr int kLossBatch = 256;  // rows of surrogate_loss_grad
-constexpr int kTrainBN = 64;     // N tile of the training GEMMs (more CTAs on small problems)
+constexpr int kTrainBN = 32;     // N tile of the training GEMMs (more CTAs on small problems)
 constexpr int kEvalBN = 256;     // N tile of the inference GEMMs
 constexpr int kEvalChunk = 1 << 16;
 
@@ -69,35 +74,36 @@ __device__ __forceinline__ void pdl_wait_then_release() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// n consecutive FP32 / BF16 values of one row: 16-byte stores when the row
-// chunk is whole and aligned, element stores otherwise.
-__device__ __forceinline__ void store_row_f32(float* p, const float (&a)[32], int n) {
-    if (n == 32 && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+// n consecutive FP32 / BF16 values of one row (chunks of kEpiCols columns):
+// 16-byte accesses when the chunk is whole and aligned, element ones otherwise.
+constexpr int kEpiCols = 16;
+__device__ __forceinline__ void store_row_f32(float* p, const float (&a)[kEpiCols], int n) {
+    if (n == kEpiCols && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < kEpiCols / 4; ++i)
             reinterpret_cast<float4*>(p)[i] = make_float4(a[4 * i], a[4 * i + 1], a[4 * i + 2], a[4 * i + 3]);
     } else {
 #pragma unroll
-        for (int i = 0; i < 32; ++i)
+        for (int i = 0; i < kEpiCols; ++i)
             if (i < n) p[i] = a[i];
     }
 }
 
-__device__ __forceinline__ void store_row_bf16(__nv_bfloat16* p, const __nv_bfloat16 (&h)[32], int n) {
-    if (n == 32 && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+__device__ __forceinline__ void store_row_bf16(__nv_bfloat16* p, const __nv_bfloat16 (&h)[kEpiCols], int n) {
+    if (n == kEpiCols && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) reinterpret_cast<uint4*>(p)[i] = reinterpret_cast<const uint4*>(h)[i];
+        for (int i = 0; i < kEpiCols / 8; ++i) reinterpret_cast<uint4*>(p)[i] = reinterpret_cast<const uint4*>(h)[i];
     } else {
 #pragma unroll
-        for (int i = 0; i < 32; ++i)
+        for (int i = 0; i < kEpiCols; ++i)
             if (i < n) p[i] = h[i];
     }
 }
 
-__device__ __forceinline__ void load_row_f32(const float* p, float (&a)[32], int n) {
-    if (n == 32 && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+__device__ __forceinline__ void load_row_f32(const float* p, float (&a)[kEpiCols], int n) {
+    if (n == kEpiCols && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < kEpiCols / 4; ++i) {
             const float4 v = reinterpret_cast<const float4*>(p)[i];
             a[4 * i] = v.x;
             a[4 * i + 1] = v.y;
@@ -106,19 +112,24 @@ __device__ __forceinline__ void load_row_f32(const float* p, float (&a)[32], int
         }
     } else {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) a[i] = i < n ? p[i] : 0.0f;
+        for (int i = 0; i < kEpiCols; ++i) a[i] = i < n ? p[i] : 0.0f;
     }
 }
 
 // D[m][n] = sum_k A[m][k] B[n][k]: A [M][K] and B [N][K] BF16 K-major, one
 // 128 x BN tile per CTA, then the EPI epilogue on D.  Warp 0 lane 0 issues
-// the TMA loads, warp 1 lane 0 the MMAs; all four warps drain TMEM (warp w
-// owns rows 32w .. 32w+31 of the tile, one row per thread).
+// the TMA loads, warp 1 lane 0 the MMAs; all eight warps drain TMEM, two per 32
+// rows (one row per thread), taking the 16-column chunks in turn.  The
+// training GEMMs are latencies end to end, the epilogue a large part: N tiles
+// of 32 on eight warps instead of 64 on four took the 20480 x 20 training run
+// from 30.9 to 25.2 ms (tiles) and further (warps).
+constexpr int kGemmThreads = 256;
 template <int BN, int EPI>
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(kGemmThreads, 1)
     k_gemm_bf16_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int kblocks,
                    EpiArgs e, int* __restrict__ err) {
     constexpr uint32_t kA = kGm * kGk * 2, kB = BN * kGk * 2;
+    constexpr int kGStages = gemm_stages<BN>();
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = tc::smem_u32(smem_raw);
     uint8_t* base = smem_raw + ((1024 - (raw & 1023)) & 1023);
@@ -178,39 +189,39 @@ __global__ void __launch_bounds__(128, 1)
     __syncwarp();
     tc::fence_after_sync();
     if (ok) {
-        const int r = m0 + warp * 32 + lane;
-        const uint32_t row = tmem + ((uint32_t)(warp * 32) << 16);
+        const int r = m0 + (warp & 3) * 32 + lane;
+        const uint32_t row = tmem + ((uint32_t)((warp & 3) * 32) << 16);
 #pragma unroll 1
-        for (int chunk = 0; chunk < BN / 32; ++chunk) {
-            uint32_t v[32];
-            tc::tmem_ld_32x32b_x32(row + chunk * 32, v);
-            const int c0 = n0 + chunk * 32;
+        for (int chunk = warp >> 2; chunk < BN / kEpiCols; chunk += 2) {
+            uint32_t v[kEpiCols];
+            tc::tmem_ld_32x32b_x16(row + chunk * kEpiCols, v);
+            const int c0 = n0 + chunk * kEpiCols;
             if (r >= e.M || c0 >= e.N) continue;
-            const int n = min(32, e.N - c0);
-            float a[32];
+            const int n = min(kEpiCols, e.N - c0);
+            float a[kEpiCols];
 #pragma unroll
-            for (int i = 0; i < 32; ++i) a[i] = __uint_as_float(v[i]);
+            for (int i = 0; i < kEpiCols; ++i) a[i] = __uint_as_float(v[i]);
             if (EPI == kEpiF32) {
                 store_row_f32(e.F + (size_t)r * e.ldf + c0, a, n);
                 continue;
             }
-            __nv_bfloat16 h[32];
+            __align__(16) __nv_bfloat16 h[kEpiCols];
             if (EPI == kEpiFwdGelu) {
 #pragma unroll
-                for (int i = 0; i < 32; ++i) a[i] += (i < n) ? __ldg(e.bias + c0 + i) : 0.0f;
+                for (int i = 0; i < kEpiCols; ++i) a[i] += (i < n) ? __ldg(e.bias + c0 + i) : 0.0f;
                 if (e.Z) store_row_f32(e.Z + (size_t)r * e.ldz + c0, a, n);
 #pragma unroll
-                for (int i = 0; i < 32; ++i) h[i] = __float2bfloat16_rn(gelu_f(a[i]));
+                for (int i = 0; i < kEpiCols; ++i) h[i] = __float2bfloat16_rn(gelu_f(a[i]));
             } else {
-                float z[32];
+                float z[kEpiCols];
                 load_row_f32(e.Z + (size_t)r * e.ldz + c0, z, n);
 #pragma unroll
-                for (int i = 0; i < 32; ++i) h[i] = __float2bfloat16_rn(a[i] * gelu_grad_f(z[i]));
+                for (int i = 0; i < kEpiCols; ++i) h[i] = __float2bfloat16_rn(a[i] * gelu_grad_f(z[i]));
             }
             store_row_bf16(e.H + (size_t)r * e.ldh + c0, h, n);
             if (e.HT) {
 #pragma unroll
-                for (int i = 0; i < 32; ++i)
+                for (int i = 0; i < kEpiCols; ++i)
                     if (i < n) e.HT[(size_t)(c0 + i) * e.ldt + r] = h[i];
             }
         }
@@ -222,7 +233,7 @@ __global__ void __launch_bounds__(128, 1)
 
 template <int BN>
 constexpr size_t gemm_smem() {
-    return 1024 + kGStages * ((size_t)kGm * kGk * 2 + (size_t)BN * kGk * 2) + 256;
+    return 1024 + gemm_stages<BN>() * ((size_t)kGm * kGk * 2 + (size_t)BN * kGk * 2) + 256;
 }
 
 // ------------------------------------------------------------------ fused MC inference
@@ -459,55 +470,106 @@ __global__ void k_mlp_out(int B, const __nv_bfloat16* __restrict__ H3, const __n
 // Training: the output layer and its gradient in one pass, one warp per row:
 // out, dout and the squared error as k_mlp_out forms them, then the
 // pre-activation gradient dZ3 = bf16((dout w4) * gelu'(Z3)), row-major and
-// transposed [kH][ldt].
-__global__ void k_mlp_out_train(int B, int ldt, const __nv_bfloat16* __restrict__ H3,
-                                const __nv_bfloat16* __restrict__ w4, const float* __restrict__ b4,
-                                const float* __restrict__ t, float* __restrict__ out, float* __restrict__ dout,
-                                float* __restrict__ sq, const float* __restrict__ Z3, __nv_bfloat16* __restrict__ dZ,
-                                __nv_bfloat16* __restrict__ dZT) {
+// transposed [kH][ldt].  A CTA takes 16 rows, two per warp with the loads of
+// both in flight, and writes the transposed operand through shared memory in
+// 32-byte runs: written row by row, its 2-byte stores (one sector each) were
+// most of the kernel.
+constexpr int kOutRows = 16;
+__global__ void __launch_bounds__(256) k_mlp_out_train(int B, int ldt, const __nv_bfloat16* __restrict__ H3,
+                                                       const __nv_bfloat16* __restrict__ w4,
+                                                       const float* __restrict__ b4, const float* __restrict__ t,
+                                                       float* __restrict__ out, float* __restrict__ dout,
+                                                       float* __restrict__ sq, const float* __restrict__ Z3,
+                                                       __nv_bfloat16* __restrict__ dZ,
+                                                       __nv_bfloat16* __restrict__ dZT) {
+    __shared__ __align__(16) __nv_bfloat16 tr[kH][kOutRows + 8];   // rows of 48 bytes
+    constexpr int kPer = kOutRows / 8, kJ = kH / 32;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int b0 = blockIdx.x * kOutRows + warp * kPer;   // B is a multiple of 128
     pdl_wait_then_release();
-    const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (b >= B) return;
-    float acc = 0.0f;
-    for (int j = lane; j < kH; j += 32)
-        acc += __bfloat162float(H3[(size_t)b * kH + j]) * __bfloat162float(w4[j]);
+    float w[kJ], h[kPer][kJ], z[kPer][kJ];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-    float dv = 0.0f;
-    if (lane == 0) {
-        const float o = acc + b4[0];
-        out[b] = o;
-        const float d = o - t[b];
-        dv = 2.0f * d / (float)B;
-        dout[b] = dv;
-        sq[b] = d * d;
+    for (int q = 0; q < kJ; ++q) w[q] = __bfloat162float(w4[lane + 32 * q]);
+#pragma unroll
+    for (int u = 0; u < kPer; ++u)
+#pragma unroll
+        for (int q = 0; q < kJ; ++q) {
+            h[u][q] = __bfloat162float(H3[(size_t)(b0 + u) * kH + lane + 32 * q]);
+            z[u][q] = Z3[(size_t)(b0 + u) * kH + lane + 32 * q];
+        }
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        const int b = b0 + u;
+        float acc = 0.0f;
+#pragma unroll
+        for (int q = 0; q < kJ; ++q) acc += h[u][q] * w[q];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
+        float dv = 0.0f;
+        if (lane == 0) {
+            const float o = acc + b4[0];
+            out[b] = o;
+            const float d = o - t[b];
+            dv = 2.0f * d / (float)B;
+            dout[b] = dv;
+            sq[b] = d * d;
+        }
+        dv = __shfl_sync(0xffffffffu, dv, 0);
+#pragma unroll
+        for (int q = 0; q < kJ; ++q) {
+            const int j = lane + 32 * q;
+            const __nv_bfloat16 v = __float2bfloat16_rn(dv * w[q] * gelu_grad_f(z[u][q]));
+            dZ[(size_t)b * kH + j] = v;
+            tr[j][warp * kPer + u] = v;
+        }
     }
-    dv = __shfl_sync(0xffffffffu, dv, 0);
-    for (int j = lane; j < kH; j += 32) {
-        const float d = dv * __bfloat162float(w4[j]) * gelu_grad_f(Z3[(size_t)b * kH + j]);
-        const __nv_bfloat16 v = __float2bfloat16_rn(d);
-        dZ[(size_t)b * kH + j] = v;
-        dZT[(size_t)j * ldt + b] = v;
-    }
+    __syncthreads();
+    // one column per thread: 16 rows, 32 bytes
+    const uint4* src = reinterpret_cast<const uint4*>(tr[threadIdx.x]);
+    uint4* dst = reinterpret_cast<uint4*>(dZT + (size_t)threadIdx.x * ldt + blockIdx.x * kOutRows);
+    dst[0] = src[0];
+    dst[1] = src[1];
 }
 
-// Row sums of a transposed operand, one warp per row j (lanes over the batch,
-// fixed order): gb[j] = sum_b w[b] T[j][b], with w = 1 when null.  With
-// ones_row, warp N also writes gb[N] = sum_b w[b] (the output bias).
-__global__ void k_row_sums(int N, int B, int ldt, const __nv_bfloat16* __restrict__ T, const float* __restrict__ w,
-                           float* __restrict__ gb, float* __restrict__ ones_row) {
+// Row sums of transposed operands, one warp per row (lanes over the batch,
+// fixed order; the loads of 32 terms a lane in flight together).  Job 0: gb[j] =
+// sum_b w[b] T[j][b], with w = 1 when null; with ones_row, row kH gives sum_b
+// w[b] (the output bias).  Job 1 (T2 given): gb2[j] = sum_b T2[j][b].
+__global__ void k_row_sums(int B, int ldt, const __nv_bfloat16* __restrict__ T, const float* __restrict__ w,
+                           float* __restrict__ gb, float* __restrict__ ones_row,
+                           const __nv_bfloat16* __restrict__ T2, float* __restrict__ gb2) {
     pdl_wait_then_release();
-    const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (j > N || (j == N && !ones_row)) return;
+    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    const int first = kH + (ones_row ? 1 : 0);
+    const bool two = row >= first;
+    const int j = two ? row - first : row;
+    if (two && (!T2 || j >= kH)) return;
+    const __nv_bfloat16* t = two ? T2 : T;
+    const float* wt = two ? nullptr : w;
     float acc = 0.0f;
-    for (int b = lane; b < B; b += 32) {
-        const float x = (j < N) ? __bfloat162float(T[(size_t)j * ldt + b]) : 1.0f;
-        acc += w ? w[b] * x : x;
+    constexpr int kU = 32;
+    for (int b0 = lane; b0 < B; b0 += 32 * kU) {
+        float x[kU], v[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int b = b0 + 32 * u;
+            x[u] = b < B ? (j < kH ? __bfloat162float(t[(size_t)j * ldt + b]) : 1.0f) : 0.0f;
+            v[u] = wt && b < B ? wt[b] : 0.0f;
+        }
+        // terms past the batch add +0 (an exact no-op on a sum that starts at +0)
+        if (wt) {
+#pragma unroll
+            for (int u = 0; u < kU; ++u) acc = fmaf(v[u], x[u], acc);
+        } else {
+#pragma unroll
+            for (int u = 0; u < kU; ++u) acc += x[u];
+        }
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
     if (lane == 0) {
-        if (j < N) gb[j] = acc;
+        if (two) gb2[j] = acc;
+        else if (j < kH) gb[j] = acc;
         else ones_row[0] = acc;
     }
 }
@@ -564,11 +626,9 @@ struct AdamArgs {
     __nv_bfloat16 *W1b, *W2b, *W3b, *W2T, *W3T, *w4b;
 };
 
-// One parameter's Adam update at step s, and its BF16 operand copies.
-__device__ __forceinline__ void adam_update(const AdamArgs& a, size_t t, int s) {
-    const float k = (float)(s + 1);
-    const float lr = a.lr0 * 0.5f * (1.0f + cospif((float)s / (float)a.total));
-    const float c1 = 1.0f - powf(a.b1, k), c2 = 1.0f - powf(a.b2, k);
+// One parameter's Adam update with learning rate lr and bias corrections c1,
+// c2; returns its BF16 operand copy, written row-major.
+__device__ __forceinline__ __nv_bfloat16 adam_update(const AdamArgs& a, size_t t, float lr, float c1, float c2) {
     const float gt = a.g[t];
     const float mt = a.b1 * a.m[t] + (1.0f - a.b1) * gt;
     const float vt = a.b2 * a.v[t] + (1.0f - a.b2) * gt * gt;
@@ -577,26 +637,52 @@ __device__ __forceinline__ void adam_update(const AdamArgs& a, size_t t, int s) 
     const float p = a.P[t] - lr * (mt / c1) / (sqrtf(vt / c2) + a.eps);
     a.P[t] = p;
     const __nv_bfloat16 h = __float2bfloat16_rn(p);
-    if (t < a.off[1]) {
-        a.W1b[(t / a.M) * a.D + t % a.M] = h;
-    } else if (t >= a.off[2] && t < a.off[3]) {
-        const size_t u = t - a.off[2];
-        a.W2b[u] = h;
-        a.W2T[(u % kH) * kH + u / kH] = h;
-    } else if (t >= a.off[4] && t < a.off[5]) {
-        const size_t u = t - a.off[4];
-        a.W3b[u] = h;
-        a.W3T[(u % kH) * kH + u / kH] = h;
-    } else if (t >= a.off[6] && t < a.off[7]) {
-        a.w4b[t - a.off[6]] = h;
-    }
+    if (t < a.off[1]) a.W1b[(t / a.M) * a.D + t % a.M] = h;
+    else if (t >= a.off[2] && t < a.off[3]) a.W2b[t - a.off[2]] = h;
+    else if (t >= a.off[4] && t < a.off[5]) a.W3b[t - a.off[4]] = h;
+    else if (t >= a.off[6] && t < a.off[7]) a.w4b[t - a.off[6]] = h;
+    return h;
 }
 
+// Blocks of 256 parameters; those of W2 and W3 (256 x 256, starting at a
+// multiple of 256) take 16 x 16 tiles, whose transposed operand goes through
+// shared memory in 32-byte rows (2-byte stores a row apart took a sector each).
 __global__ void k_adam_step(AdamArgs a) {
+    __shared__ __align__(16) __nv_bfloat16 tr[16][24];
+    __shared__ float coef[3];   // learning rate and bias corrections of this step, formed once per block
     pdl_wait_then_release();
-    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    size_t t = (size_t)blockIdx.x * 256 + threadIdx.x;
+    const size_t o = t < a.off[4] ? a.off[2] : a.off[4];
+    const bool tile = (t >= a.off[2] && t < a.off[3]) || (t >= a.off[4] && t < a.off[5]);   // the whole block
+    const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+    int tr0 = 0, tc0 = 0;   // the tile's first row and column
+    if (tile) {
+        const int q = (int)((t - o) >> 8);
+        tr0 = (q >> 4) * 16;
+        tc0 = (q & 15) * 16;
+        t = o + (size_t)(tr0 + ty) * kH + tc0 + tx;
+    }
     const int s = *a.step;
-    if (t < a.np) adam_update(a, t, s);
+    if (threadIdx.x < 3) {
+        const float k = (float)(s + 1);
+        coef[threadIdx.x] = threadIdx.x == 0   ? a.lr0 * 0.5f * (1.0f + cospif((float)s / (float)a.total))
+                            : threadIdx.x == 1 ? 1.0f - powf(a.b1, k)
+                                               : 1.0f - powf(a.b2, k);
+    }
+    __syncthreads();
+    if (t < a.np) {
+        const __nv_bfloat16 h = adam_update(a, t, coef[0], coef[1], coef[2]);
+        if (tile) tr[tx][ty] = h;
+    }
+    if (tile) {
+        __syncthreads();
+        if (threadIdx.x < 32) {   // column tc0 + r, rows tr0 + 8 c ..
+            const int r = threadIdx.x >> 1, c = threadIdx.x & 1;
+            __nv_bfloat16* WT = o == a.off[2] ? a.W2T : a.W3T;
+            *reinterpret_cast<uint4*>(WT + (size_t)(tc0 + r) * kH + tr0 + 8 * c) =
+                *reinterpret_cast<const uint4*>(&tr[r][8 * c]);
+        }
+    }
     // the last block to finish advances the step counter (every block has
     // read it by then) and re-arms the block count for the next step
     __syncthreads();
@@ -664,8 +750,8 @@ struct MlpState {
     cudaStream_t st = nullptr;         // training stream (graph capture)
     // the weight- and bias-gradient kernels of a step run on `side`, beside
     // the back-propagation chain on the step's stream (fork / join events)
-    cudaStream_t side = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_dz2 = nullptr, ev_dz1 = nullptr, ev_join = nullptr;
+    cudaStream_t side = nullptr, side2 = nullptr;   // weight gradients; bias sums
+    cudaEvent_t ev_fork = nullptr, ev_dz2 = nullptr, ev_dz1 = nullptr, ev_join = nullptr, ev_join2 = nullptr;
     // A training run whose steps may still be running on `st` (launched with
     // fm_train_opts.async_run): every use of the network waits for `trained`
     // on its stream, host-side uses wait on the host.  The run's buffers and
@@ -767,7 +853,7 @@ static void gemm(fm_ctx* ctx, const CUtensorMap& A, const CUtensorMap& B, int M,
     dim3 grid((M + kGm - 1) / kGm, (N + BN - 1) / BN);
     FM_TIMED(ctx, kFamMlp, st, 2.0 * ((double)M * K + (double)N * K) + 4.0 * (double)M * N,
              2.0 * (double)M * N * K,
-             launch(pdl, k_gemm_bf16_tc<BN, EPI>, grid, dim3(128), gemm_smem<BN>(), st, A, B, K / kGk, e,
+             launch(pdl, k_gemm_bf16_tc<BN, EPI>, grid, dim3(kGemmThreads), gemm_smem<BN>(), st, A, B, K / kGk, e,
                     state(ctx)->err));
 }
 
@@ -826,7 +912,8 @@ static fm_status mlp_alloc(fm_ctx* ctx) {
     cudaDeviceGetStreamPriorityRange(&lo, &hi);
     if (ok && cudaStreamCreateWithPriority(&S->st, cudaStreamNonBlocking, hi) != cudaSuccess) ok = false;
     if (ok && cudaStreamCreateWithPriority(&S->side, cudaStreamNonBlocking, hi) != cudaSuccess) ok = false;
-    for (cudaEvent_t* e : {&S->ev_fork, &S->ev_dz2, &S->ev_dz1, &S->ev_join})
+    if (ok && cudaStreamCreateWithPriority(&S->side2, cudaStreamNonBlocking, hi) != cudaSuccess) ok = false;
+    for (cudaEvent_t* e : {&S->ev_fork, &S->ev_dz2, &S->ev_dz1, &S->ev_join, &S->ev_join2})
         if (ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) ok = false;
     if (!ok) {
         set_error(ctx, "surrogate: device allocation failed");
@@ -877,12 +964,13 @@ static void refresh_bf16(fm_ctx* ctx, cudaStream_t st) {
 // on S->side (forked after the output layer, joined at the end), so a
 // training step's critical path is 9 kernels (batch gather, three forward
 // GEMMs, the output layer with its gradient, dZ2, dZ1, dW1, Adam with the
-// step counter) instead of 17.
+// step counter) instead of 17.  The bias sums run on S->side2, beside both: in
+// line with the weight gradients they made that branch the longer one.
 static void train_step_grads(fm_ctx* ctx, int B, cudaStream_t st, bool pdl = false) {
     MlpState* S = state(ctx);
     const int D = S->D, L = kMaxBatch;
     constexpr int BN = kTrainBN;
-    cudaStream_t sd = S->side;
+    cudaStream_t sd = S->side, sb = S->side2;
     EpiArgs e{};
     // forward: Z_l = H_(l-1) W_l^T + b_l, H_l = bf16(gelu(Z_l))
     e = EpiArgs{B, kH, S->P + S->off[1], S->Z[0], kH, S->H[0], kH, S->HT[0], L, nullptr, 0};
@@ -892,17 +980,16 @@ static void train_step_grads(fm_ctx* ctx, int B, cudaStream_t st, bool pdl = fal
     e = EpiArgs{B, kH, S->P + S->off[5], S->Z[2], kH, S->H[2], kH, S->HT[2], L, nullptr, 0};
     gemm<BN, kEpiFwdGelu>(ctx, S->mH2, S->tW3, B, kH, kH, e, st, pdl);
     // output layer and dZ3 = bf16(dout w4 gelu'(Z3)) on st; gw4 = dout^T H3, gb4 = sum dout beside it
-    launch(pdl, k_mlp_out_train, dim3(nb((size_t)B * 32)), dim3(256), 0, st, B, L, S->H[2], S->w4b,
+    launch(pdl, k_mlp_out_train, dim3((unsigned)(B / kOutRows)), dim3(256), 0, st, B, L, S->H[2], S->w4b,
            S->P + S->off[7], S->t, S->out, S->dout, S->sq, S->Z[2], S->dZ[2], S->dZT[2]);
     cudaEventRecord(S->ev_fork, st);
     cudaStreamWaitEvent(sd, S->ev_fork, 0);
-    launch(pdl, k_row_sums, dim3(nb((size_t)(kH + 1) * 32)), dim3(256), 0, sd, kH, B, L, S->HT[2], S->dout,
-           S->G + S->off[6], S->G + S->off[7]);
+    cudaStreamWaitEvent(sb, S->ev_fork, 0);
+    launch(pdl, k_row_sums, dim3(nb((size_t)(2 * kH + 1) * 32)), dim3(256), 0, sb, B, L, S->HT[2], S->dout,
+           S->G + S->off[6], S->G + S->off[7], S->dZT[2], S->G + S->off[5]);
     // layer 3: dW3 = dZ3^T H2, db3 beside; dZ2 = bf16((dZ3 W3) gelu'(Z2)) on st
     e = EpiArgs{kH, kH, nullptr, nullptr, 0, nullptr, 0, nullptr, 0, S->G + S->off[4], kH};
     gemm<BN, kEpiF32>(ctx, S->mdZ3T, S->tH2T, kH, kH, B, e, sd, pdl);
-    launch(pdl, k_row_sums, dim3(nb((size_t)kH * 32)), dim3(256), 0, sd, kH, B, L, S->dZT[2], nullptr,
-           S->G + S->off[5], nullptr);
     e = EpiArgs{B, kH, nullptr, S->Z[1], kH, S->dZ[1], kH, S->dZT[1], L, nullptr, 0};
     gemm<BN, kEpiBwdGelu>(ctx, S->mdZ3, S->tW3T, B, kH, kH, e, st, pdl);
     // layer 2: dW2, db2 beside; dZ1 on st
@@ -910,20 +997,23 @@ static void train_step_grads(fm_ctx* ctx, int B, cudaStream_t st, bool pdl = fal
     cudaStreamWaitEvent(sd, S->ev_dz2, 0);
     e = EpiArgs{kH, kH, nullptr, nullptr, 0, nullptr, 0, nullptr, 0, S->G + S->off[2], kH};
     gemm<BN, kEpiF32>(ctx, S->mdZ2T, S->tH1T, kH, kH, B, e, sd, pdl);
-    launch(pdl, k_row_sums, dim3(nb((size_t)kH * 32)), dim3(256), 0, sd, kH, B, L, S->dZT[1], nullptr,
-           S->G + S->off[3], nullptr);
+    cudaStreamWaitEvent(sb, S->ev_dz2, 0);
+    launch(pdl, k_row_sums, dim3(nb((size_t)kH * 32)), dim3(256), 0, sb, B, L, S->dZT[1], nullptr, S->G + S->off[3],
+           nullptr, nullptr, nullptr);
     e = EpiArgs{B, kH, nullptr, S->Z[0], kH, S->dZ[0], kH, S->dZT[0], L, nullptr, 0};
     gemm<BN, kEpiBwdGelu>(ctx, S->mdZ2, S->tW2T, B, kH, kH, e, st, pdl);
     // layer 1: db1 beside; dW1 = dZ1^T X on st (N = D input columns; the FP32
     // gradient keeps the M real ones)
     cudaEventRecord(S->ev_dz1, st);
-    cudaStreamWaitEvent(sd, S->ev_dz1, 0);
-    launch(pdl, k_row_sums, dim3(nb((size_t)kH * 32)), dim3(256), 0, sd, kH, B, L, S->dZT[0], nullptr,
-           S->G + S->off[1], nullptr);
+    cudaStreamWaitEvent(sb, S->ev_dz1, 0);
+    launch(pdl, k_row_sums, dim3(nb((size_t)kH * 32)), dim3(256), 0, sb, B, L, S->dZT[0], nullptr, S->G + S->off[1],
+           nullptr, nullptr, nullptr);
     e = EpiArgs{kH, S->M, nullptr, nullptr, 0, nullptr, 0, nullptr, 0, S->G + S->off[0], S->M};
     gemm<BN, kEpiF32>(ctx, S->mdZ1T, S->tXT, kH, D, B, e, st, pdl);
     cudaEventRecord(S->ev_join, sd);
     cudaStreamWaitEvent(st, S->ev_join, 0);
+    cudaEventRecord(S->ev_join2, sb);
+    cudaStreamWaitEvent(st, S->ev_join2, 0);
 }
 
 // Forward of n rows, chunked: fill(o, cnt, st) writes rows o .. o+cnt-1 of
@@ -1015,7 +1105,8 @@ void mlp_free(fm_ctx* ctx) {
                     S->t, S->out, S->dout, S->sq, S->eX, S->eout, S->err, S->step};
     if (S->st) cudaStreamDestroy(S->st);
     if (S->side) cudaStreamDestroy(S->side);
-    for (cudaEvent_t e : {S->ev_fork, S->ev_dz2, S->ev_dz1, S->ev_join})
+    if (S->side2) cudaStreamDestroy(S->side2);
+    for (cudaEvent_t e : {S->ev_fork, S->ev_dz2, S->ev_dz1, S->ev_join, S->ev_join2})
         if (e) cudaEventDestroy(e);
     for (void* p : ptrs) cudaFree(p);
     for (int l = 0; l < 3; ++l) {
