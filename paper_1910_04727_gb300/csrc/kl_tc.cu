@@ -3,11 +3,17 @@
 // A = the level's basis sqrt(theta_k) phi_k(x_c) and B = the KL coefficients,
 // both BF16 and K-major, FP32 accumulation in tensor memory.
 //
-// One CTA computes a 128-cell x 256-sample tile: warp 0 (one thread) streams
-// 64-wide K blocks of A and B into shared memory with TMA (128-byte
-// swizzle), warp 1 (one thread) issues tcgen05.mma into a 128 x 256 FP32
-// accumulator in TMEM, and all four warps drain TMEM with tcgen05.ld, apply
-// exp and store FP64 fields (consecutive cells across a warp: coalesced).
+// A tile is 128 cells x 256 samples, a 128 x 256 FP32 accumulator in tensor
+// memory.  Persistent CTAs: warp 8 (one thread) streams 64-wide K blocks of A
+// and B through four stages of shared memory with TMA (128-byte swizzle), warp 9
+// (one thread) issues tcgen05.mma into one of two accumulators, and warps 0 .. 7
+// drain the other with tcgen05.ld, apply exp and store FP64 fields (consecutive
+// cells across a warp: coalesced), so the next tile's products run under this
+// one's epilogue.  Bound: HBM (the FP64 fields out, the BF16 basis in).  The
+// conversion of exp to FP64 is done in integers: the FP64 pipe, where F2F runs,
+// takes 1.7 us per million.  500 fields of 256 x 256 cells from 256 modes: 85 us
+// (4.7 TB/s of field, basis and coefficients), 126 with a CTA per tile, two K
+// stages and F2F.
 //
 // Split precision ("bf16x3"): the host lays out A' = [A_hi | A_hi | A_lo] and
 // B' = [B_hi | B_lo | B_hi] along an extended K, so one GEMM gives
@@ -26,16 +32,26 @@ namespace fm {
 constexpr int kTcM = 128;     // cells per tile (MMA M)
 constexpr int kTcN = 256;     // samples per tile (MMA N)
 constexpr int kTcK = 64;      // K elements per stage (one 128-byte swizzle row)
-constexpr int kTcStages = 2;
+constexpr int kTcStages = 4;
+constexpr int kTcEpi = 256;                // threads that drain and store
+constexpr int kTcThreads = kTcEpi + 64;
 constexpr uint32_t kTcABytes = kTcM * kTcK * 2;   // 16 KiB
 constexpr uint32_t kTcBBytes = kTcN * kTcK * 2;   // 32 KiB
 constexpr size_t kTcSmem = 1024 + kTcStages * (kTcABytes + kTcBBytes) + 256;
 
+// x (not negative) to FP64: in integers where x is a normal number.
+__device__ __forceinline__ double widen_positive(float x) {
+    const uint32_t u = __float_as_uint(x);
+    if (u - 0x00800000u < 0x7F000000u) return __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29));
+    return (double)x;   // zero, denormal, infinity, NaN
+}
+
 // EPI 0 (field synthesis): K[s][c] = exp(D[c][s]).  EPI 1 (Nystrom
 // interpolation of the KL basis): K[c][s] = D[c][s] colscale[s], row-major
-// [cells][S] in FP64.
+// [cells][S] in FP64.  CTA b takes tiles b, b + gridDim.x, ... (sample tiles
+// fastest).
 template <int EPI>
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(kTcThreads, 1)
     k_kl_gemm_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int cells,
                  int S, int kblocks, double* __restrict__ K, int* __restrict__ err,
                  const double* __restrict__ colscale) {
@@ -46,80 +62,110 @@ __global__ void __launch_bounds__(128, 1)
     uint8_t* sB = base + kTcStages * kTcABytes;
     uint64_t* full = reinterpret_cast<uint64_t*>(sB + kTcStages * kTcBBytes);
     uint64_t* empty = full + kTcStages;
-    uint64_t* done = empty + kTcStages;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+    uint64_t* tfull = empty + kTcStages;    // accumulator ready, by set
+    uint64_t* tempty = tfull + 2;           // accumulator drained
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int c0 = blockIdx.x * kTcM, s0 = blockIdx.y * kTcN;
+    const unsigned stiles = (unsigned)(S + kTcN - 1) / kTcN, tiles = stiles * ((unsigned)(cells + kTcM - 1) / kTcM);
     if (threadIdx.x == 0) {
         for (int i = 0; i < kTcStages; ++i) {
             tc::mbar_init(&full[i], 1);
             tc::mbar_init(&empty[i], 1);
         }
-        tc::mbar_init(done, 1);
+        for (int i = 0; i < 2; ++i) {
+            tc::mbar_init(&tfull[i], 1);
+            tc::mbar_init(&tempty[i], kTcEpi);
+        }
         tc::fence_barrier_init();
         tc::prefetch_tensormap(&mapA);
         tc::prefetch_tensormap(&mapB);
     }
-    if (warp == 0) tc::tmem_alloc(tmem_slot, kTcN);
+    if (warp == 0) tc::tmem_alloc(tmem_slot, 2 * kTcN);
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
 
-    if (warp == 0 && lane == 0) {
-        // producer: K blocks through a kTcStages-deep ring
-        int issued = 0;
-        for (int kb = 0; kb < kblocks; ++kb) {
-            const int st = kb % kTcStages, round = kb / kTcStages;
-            if (round > 0 && !tc::mbar_wait(&empty[st], (round - 1) & 1, err)) break;
-            tc::mbar_arrive_expect_tx(&full[st], kTcABytes + kTcBBytes);
-            tc::tma_load_2d(sA + st * kTcABytes, &mapA, &full[st], kb * kTcK, c0);
-            tc::tma_load_2d(sB + st * kTcBBytes, &mapB, &full[st], kb * kTcK, s0);
-            ++issued;
+    if (warp == 8) {
+        if (lane == 0) {
+            int q = 0;   // stage loads so far
+            bool ok = true;
+            for (unsigned tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x) {
+                const int s0 = (int)(tile % stiles) * kTcN, c0 = (int)(tile / stiles) * kTcM;
+                for (int kb = 0; kb < kblocks; ++kb) {
+                    const int st = q % kTcStages, round = q / kTcStages;
+                    if (round > 0 && !(ok = tc::mbar_wait(&empty[st], (round - 1) & 1, err))) break;
+                    tc::mbar_arrive_expect_tx(&full[st], kTcABytes + kTcBBytes);
+                    tc::tma_load_2d(sA + st * kTcABytes, &mapA, &full[st], kb * kTcK, c0);
+                    tc::tma_load_2d(sB + st * kTcBBytes, &mapB, &full[st], kb * kTcK, s0);
+                    ++q;
+                }
+            }
+            tc::drain_loads(full, kTcStages, q, err);
         }
-        tc::drain_loads(full, kTcStages, issued, err);
-    } else if (warp == 1 && lane == 0) {
-        // MMA issuer: four K=16 steps per stage, accumulate after the first
-        constexpr uint32_t idesc = tc::idesc_bf16_f32(kTcM, kTcN);
-        for (int kb = 0; kb < kblocks; ++kb) {
-            const int st = kb % kTcStages, round = kb / kTcStages;
-            if (!tc::mbar_wait(&full[st], round & 1, err)) break;
+    } else if (warp == 9) {
+        if (lane == 0) {
+            // four K = 16 steps per stage, accumulate after the first
+            constexpr uint32_t idesc = tc::idesc_bf16_f32(kTcM, kTcN);
+            int q = 0, it = 0;
+            bool ok = true;
+            for (unsigned tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x, ++it) {
+                const int set = it & 1;
+                if (it >= 2 && !(ok = tc::mbar_wait(&tempty[set], ((it >> 1) - 1) & 1, err))) break;
+                tc::fence_after_sync();
+                for (int kb = 0; kb < kblocks; ++kb, ++q) {
+                    const int st = q % kTcStages;
+                    if (!(ok = tc::mbar_wait(&full[st], (q / kTcStages) & 1, err))) break;
+                    tc::fence_after_sync();
+                    const uint32_t a = tc::smem_u32(sA + st * kTcABytes), b = tc::smem_u32(sB + st * kTcBBytes);
+#pragma unroll
+                    for (int j = 0; j < kTcK / 16; ++j)
+                        tc::mma_bf16(tmem + set * kTcN, tc::sdesc_kmajor_sw128(a + 32 * j),
+                                     tc::sdesc_kmajor_sw128(b + 32 * j), idesc, (kb | j) != 0);
+                    tc::mma_commit(&empty[st]);   // frees the stage once these MMAs have read it
+                }
+                tc::mma_commit(&tfull[set]);
+            }
+        }
+    } else {
+        int it = 0;
+        for (unsigned tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++it) {
+            const int set = it & 1;
+            const int s0 = (int)(tile % stiles) * kTcN, c0 = (int)(tile / stiles) * kTcM;
+            const int c = c0 + (warp & 3) * 32 + lane;
+            // all lanes or none (the loads below are warp-wide)
+            if (!__all_sync(0xffffffffu, tc::mbar_wait(&tfull[set], (it >> 1) & 1, err))) break;
             tc::fence_after_sync();
-            const uint32_t a = tc::smem_u32(sA + st * kTcABytes), b = tc::smem_u32(sB + st * kTcBBytes);
-#pragma unroll
-            for (int j = 0; j < kTcK / 16; ++j)
-                tc::mma_bf16(tmem, tc::sdesc_kmajor_sw128(a + 32 * j), tc::sdesc_kmajor_sw128(b + 32 * j), idesc,
-                             (kb | j) != 0);
-            tc::mma_commit(&empty[st]);   // frees the stage once these MMAs have read it
-        }
-        tc::mma_commit(done);
-    }
-    __syncwarp();
-    const bool ok = tc::mbar_wait(done, 0, err);
-    __syncwarp();
-    tc::fence_after_sync();
-    if (ok) {
-        const int c = c0 + warp * 32 + lane;
-        const uint32_t row = tmem + ((uint32_t)(warp * 32) << 16);
+            const uint32_t row = tmem + set * kTcN + ((uint32_t)((warp & 3) * 32) << 16);
+            constexpr int kChunks = kTcN / 64;   // chunks of 32 columns, two warps per 32 rows
 #pragma unroll 1
-        for (int chunk = 0; chunk < kTcN / 32; ++chunk) {
-            uint32_t r[32];
-            tc::tmem_ld_32x32b_x32(row + chunk * 32, r);
-            if (c < cells) {
+            for (int h = 0; h < kChunks; ++h) {
+                const int chunk = (warp >> 2) * kChunks + h;
+                uint32_t r[32];
+                tc::tmem_ld_32x32b_x32(row + chunk * 32, r);
+                if (h == kChunks - 1) {   // this thread has read the accumulator
+                    tc::fence_before_sync();
+                    tc::mbar_arrive(&tempty[set]);
+                }
+                if (c < cells) {
+                    const int sc = s0 + chunk * 32;
+                    double* out = EPI == 0 ? K + (size_t)sc * cells + c : K + (size_t)c * S + sc;
+                    const size_t step = EPI == 0 ? (size_t)cells : 1;
 #pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    const int s = s0 + chunk * 32 + i;
-                    if (s >= S) continue;
-                    if (EPI == 0) K[(size_t)s * cells + c] = (double)expf(__uint_as_float(r[i]));
-                    else K[(size_t)c * S + s] = (double)__uint_as_float(r[i]) * colscale[s];
+                    for (int i = 0; i < 32; ++i) {
+                        if (sc + i >= S) break;
+                        const float d = __uint_as_float(r[i]);
+                        *out = EPI == 0 ? widen_positive(expf(d)) : (double)d * colscale[sc + i];
+                        out += step;
+                    }
                 }
             }
         }
     }
     tc::fence_before_sync();
     __syncthreads();
-    if (warp == 0) tc::tmem_dealloc(tmem, kTcN);
+    if (warp == 0) tc::tmem_dealloc(tmem, 2 * kTcN);
 }
 
 // One CTA waits, with the bounded wait of the kernels above, on an mbarrier
@@ -223,6 +269,13 @@ static bool make_map(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t 
 
 static unsigned nblk(size_t threads) { return (unsigned)((threads + 255) / 256); }
 
+// Persistent CTAs of a GEMM over cells x n: one per SM (shared memory and
+// tensor memory allow one), no more than there are tiles.
+static unsigned gemm_grid(const fm_ctx* ctx, int cells, uint32_t n) {
+    const size_t tiles = (size_t)((cells + kTcM - 1) / kTcM) * ((n + kTcN - 1) / kTcN);
+    return (unsigned)std::min<size_t>(tiles, (size_t)std::max(ctx->sms, 1));
+}
+
 fm_status kl_tc_install(fm_ctx* ctx, int split) {
     const int M = ctx->cfg.M, Mpad = (M + kTcK - 1) / kTcK * kTcK, Kp = split ? 3 * Mpad : Mpad;
     ctx->tc.split = split;
@@ -283,11 +336,11 @@ fm_status kl_tc_field(fm_ctx* ctx, int level, uint32_t n, const double* d_xi, do
     k_xi_to_bf16<<<nblk((size_t)n * Mpad), 256, 0, st>>>(n, M, Mpad, ctx->tc.split, d_xi,
                                                         (__nv_bfloat16*)ctx->tc.xi);
     // the coefficient map covers the buffer's capacity; rows >= n are never stored
-    dim3 grid((cells + kTcM - 1) / kTcM, (n + kTcN - 1) / kTcN);
+    const unsigned grid = gemm_grid(ctx, cells, n);
     const double flops = 2.0 * (double)n * cells * Kp;
     const double bytes = 2.0 * ((double)cells * Kp + (double)n * Kp) + 8.0 * (double)n * cells;
     FM_TIMED(ctx, kFamKlGemm, st, bytes, flops,
-             k_kl_gemm_tc<0><<<grid, 128, kTcSmem, st>>>(ctx->tc.mapA[level],
+             k_kl_gemm_tc<0><<<grid, kTcThreads, kTcSmem, st>>>(ctx->tc.mapA[level],
                                                         ctx->tc.mapB, cells, (int)n,
                                                         Kp / kTcK, d_K, ctx->tc.err, nullptr));
     FM_CUDA_TRY(ctx, cudaGetLastError());
@@ -341,8 +394,8 @@ fm_status kl_tc_nystrom(fm_ctx* ctx, int q, const double* dVt, const double* d_i
             const size_t nr = std::min(chunk, rows - r0);
             k_nystrom_cross_bf16<<<nblk(nr * Kpad), 256>>>(n_ref, r0, nr, q, Kpad, nu, sigma2, lambda,
                                                            (__nv_bfloat16*)A);
-            dim3 grid((unsigned)((nr + kTcM - 1) / kTcM), (unsigned)((M + kTcN - 1) / kTcN));
-            k_kl_gemm_tc<1><<<grid, 128, kTcSmem>>>(mapA, mapB, (int)nr, M, Kp / kTcK, d_out + r0 * M, ctx->tc.err,
+            const unsigned grid = gemm_grid(ctx, (int)nr, (uint32_t)M);
+            k_kl_gemm_tc<1><<<grid, kTcThreads, kTcSmem>>>(mapA, mapB, (int)nr, M, Kp / kTcK, d_out + r0 * M, ctx->tc.err,
                                                    d_inv_sqrt_theta);
         }
         if (cudaDeviceSynchronize() != cudaSuccess || cudaGetLastError() != cudaSuccess) {
