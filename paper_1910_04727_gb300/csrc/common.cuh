@@ -36,8 +36,32 @@ struct u64x4 {
 
 __host__ __device__ inline void mulhilo64(uint64_t a, uint64_t b, uint64_t& hi, uint64_t& lo) {
 #ifdef __CUDA_ARCH__
-    hi = __umul64hi(a, b);
-    lo = a * b;
+    // four 32-bit wide products and two carry chains (the high and the low half
+    // formed apart took nearly twice the instructions)
+    const uint32_t a0 = (uint32_t)a, a1 = (uint32_t)(a >> 32), b0 = (uint32_t)b, b1 = (uint32_t)(b >> 32);
+    uint32_t l0, l1, h0, h1;
+    asm("{\n"
+        " .reg .u64 p, t, q, s;\n"
+        " .reg .u32 p1, t0, t1, q0, q1, s0, s1, c;\n"
+        " mul.wide.u32 p, %4, %6;\n"
+        " mul.wide.u32 t, %4, %7;\n"
+        " mul.wide.u32 q, %5, %6;\n"
+        " mul.wide.u32 s, %5, %7;\n"
+        " mov.b64 {%0, p1}, p;\n"
+        " mov.b64 {t0, t1}, t;\n"
+        " mov.b64 {q0, q1}, q;\n"
+        " mov.b64 {s0, s1}, s;\n"
+        " add.cc.u32 t0, t0, q0;\n"
+        " addc.cc.u32 t1, t1, q1;\n"
+        " addc.u32 c, s1, 0;\n"
+        " add.cc.u32 %1, t0, p1;\n"
+        " addc.cc.u32 %2, t1, s0;\n"
+        " addc.u32 %3, c, 0;\n"
+        "}\n"
+        : "=r"(l0), "=r"(l1), "=r"(h0), "=r"(h1)
+        : "r"(a0), "r"(a1), "r"(b0), "r"(b1));
+    lo = ((uint64_t)l1 << 32) | l0;
+    hi = ((uint64_t)h1 << 32) | h0;
 #else
     unsigned __int128 p = (unsigned __int128)a * b;
     hi = (uint64_t)(p >> 64);
@@ -45,19 +69,35 @@ __host__ __device__ inline void mulhilo64(uint64_t a, uint64_t b, uint64_t& hi, 
 #endif
 }
 
+__host__ __device__ inline void philox_round(u64x4& c, uint64_t k0, uint64_t k1) {
+    uint64_t hi0, lo0, hi1, lo1;
+    mulhilo64(kPhiloxM0, c.v[0], hi0, lo0);
+    mulhilo64(kPhiloxM1, c.v[2], hi1, lo1);
+    c = u64x4{{hi1 ^ c.v[1] ^ k0, lo1, hi0 ^ c.v[3] ^ k1, lo0}};
+}
+
 __host__ __device__ inline u64x4 philox4x64(u64x4 c, uint64_t k0, uint64_t k1) {
 #pragma unroll
+    for (int r = 0; r < 10; ++r) philox_round(c, k0 + (uint64_t)r * kPhiloxW0, k1 + (uint64_t)r * kPhiloxW1);
+    return c;
+}
+
+// The round keys of one stream, formed on the host: as kernel parameters they
+// are operands in constant memory, not additions of every thread.
+struct PhiloxKeys {
+    uint64_t k[10][2];
+};
+inline PhiloxKeys philox_keys(uint64_t k0, uint64_t k1) {
+    PhiloxKeys p;
     for (int r = 0; r < 10; ++r) {
-        if (r) {
-            k0 += kPhiloxW0;
-            k1 += kPhiloxW1;
-        }
-        uint64_t hi0, lo0, hi1, lo1;
-        mulhilo64(kPhiloxM0, c.v[0], hi0, lo0);
-        mulhilo64(kPhiloxM1, c.v[2], hi1, lo1);
-        u64x4 n = {{hi1 ^ c.v[1] ^ k0, lo1, hi0 ^ c.v[3] ^ k1, lo0}};
-        c = n;
+        p.k[r][0] = k0 + (uint64_t)r * kPhiloxW0;
+        p.k[r][1] = k1 + (uint64_t)r * kPhiloxW1;
     }
+    return p;
+}
+__device__ __forceinline__ u64x4 philox4x64(u64x4 c, const PhiloxKeys& p) {
+#pragma unroll
+    for (int r = 0; r < 10; ++r) philox_round(c, p.k[r][0], p.k[r][1]);
     return c;
 }
 

@@ -62,8 +62,90 @@ struct EpiArgs {
 };
 
 __device__ __forceinline__ float gelu_f(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
+// bf16(gelu_f(z)) of two values, packed (z0 in the low half): the same bits as
+// rounding gelu_f, at half its instructions.  1 + erf(z / sqrt 2) to about 2e-7
+// by Hastings' rational form (Abramowitz & Stegun 7.1.26), g = max(z, 0) - |z| E
+// / 2; where g - d and g + d, d = 4e-7 |z| (both sides' errors), round to the same
+// BF16 number, gelu_f rounds to it too; else (a few pairs in ten thousand), and
+// beyond |z| = 64 and for NaN, gelu_f itself.  Checked against gelu_f over all
+// 2^32 FP32 numbers.
+__device__ __forceinline__ float gelu_fast(float z, float az) {
+    float t, e;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(az, 0.3275911f * 0.70710678f, 1.0f)));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(z * z * (-0.5f * 1.44269504f)));
+    float q = fmaf(t, 0.5f * 1.061405429f, 0.5f * -1.453152027f);
+    q = fmaf(q, t, 0.5f * 1.421413741f);
+    q = fmaf(q, t, 0.5f * -0.284496736f);
+    q = fmaf(q, t, 0.5f * 0.254829592f);
+    return fmaf(-az, q * t * e, fmaxf(z, -0.0f));   // -0.0f: keeps the sign of a zero
+}
+__device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&v);
+}
+__device__ __noinline__ uint32_t gelu_bf16x2_slow(float z0, float z1) { return bf16x2_bits(gelu_f(z0), gelu_f(z1)); }
+__device__ __forceinline__ uint32_t gelu_bf16x2(float z0, float z1) {
+    const float a0 = fabsf(z0), a1 = fabsf(z1);
+    const float g0 = gelu_fast(z0, a0), g1 = gelu_fast(z1, a1);
+    constexpr float d = 4e-7f;
+    const uint32_t up = bf16x2_bits(fmaf(a0, d, g0), fmaf(a1, d, g1));
+    const uint32_t dn = bf16x2_bits(fmaf(a0, -d, g0), fmaf(a1, -d, g1));
+    if (up == dn && a0 < 64.0f && a1 < 64.0f) return up;
+    return gelu_bf16x2_slow(z0, z1);   // a call: inlined at every use, it made the epilogues outgrow the instruction cache
+}
+
+// bf16(Phi^-1(u)) of two MC input words, packed: u = (k + 1/2) 2^-23, k < 2^23 the
+// top bits of a Philox word, the same bits as rounding normcdfinvf(u), at half
+// its instructions.  Phi^-1(u) = (2u - 1) f(t), t = -log2(4 u (1 - u)), f a
+// polynomial of degree 8 fitted for t <= 7 (2e-7 relative); u and 1 - u are exact.
+// Where r (1 - d) and r (1 + d), d = 1e-6, round to the same BF16 number,
+// normcdfinvf rounds to it too; else, and in the tails (0.4% of the words),
+// normcdfinvf itself.  Checked over all 2^23 words.
+__device__ __forceinline__ float word_uniform(uint32_t k) { return ((float)k + 0.5f) * 0x1p-23f; }
+__device__ __noinline__ uint32_t normal_bf16x2_slow(uint32_t k0, uint32_t k1) {
+    return bf16x2_bits(normcdfinvf(word_uniform(k0)), normcdfinvf(word_uniform(k1)));
+}
+__device__ __forceinline__ float normal_fast(uint32_t k, float* t) {
+    const float x = (float)k;
+    const float u = fmaf(x, 0x1p-23f, 0x1p-24f), v = fmaf(x, -0x1p-23f, 1.0f - 0x1p-24f);
+    float l;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(4.0f * u * v));
+    *t = -l;
+    const float s = -3.5f - l;
+    float q = fmaf(s, 2.547130506513895e-09f, 3.641305568180542e-08f);
+    q = fmaf(q, s, -5.891061505280959e-07f);
+    q = fmaf(q, s, -6.486233132818597e-07f);
+    q = fmaf(q, s, 7.1850219683256e-05f);
+    q = fmaf(q, s, -0.0006209334242157638f);
+    q = fmaf(q, s, -0.002644734922796488f);
+    q = fmaf(q, s, 0.24235691130161285f);
+    q = fmaf(q, s, 2.09747576713562f);
+    return q * (u - v);
+}
+__device__ __forceinline__ uint32_t normal_bf16x2(uint32_t k0, uint32_t k1) {
+    float t0, t1;
+    const float r0 = normal_fast(k0, &t0), r1 = normal_fast(k1, &t1);
+    constexpr float d = 1e-6f;
+    const uint32_t up = bf16x2_bits(r0 * (1.0f + d), r1 * (1.0f + d));
+    const uint32_t dn = bf16x2_bits(r0 * (1.0f - d), r1 * (1.0f - d));
+    if (up == dn && t0 < 7.0f && t1 < 7.0f) return up;
+    return normal_bf16x2_slow(k0, k1);
+}
 __device__ __forceinline__ float gelu_grad_f(float z) {
     return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * expf(-0.5f * z * z) * 0.39894228040143268f;
+}
+
+// The BF16 inputs of four words (left: columns left in the row, the rest zero).
+// 23 bits keep (k + 1/2) exact in FP32, so 0 < u < 1 strictly.
+__device__ __forceinline__ uint2 mc_inputs(const u64x4& w, int left) {
+    uint2 h;
+    h.x = normal_bf16x2((uint32_t)(w.v[0] >> 41), (uint32_t)(w.v[1] >> 41));
+    h.y = normal_bf16x2((uint32_t)(w.v[2] >> 41), (uint32_t)(w.v[3] >> 41));
+    if (left < 4) {
+        if (left < 2) h.x &= 0xFFFFu;
+        h.y = left < 3 ? 0u : h.y & 0xFFFFu;
+    }
+    return h;
 }
 
 // Programmatic dependent launch: wait until the preceding kernel of the
@@ -211,7 +293,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                 for (int i = 0; i < kEpiCols; ++i) a[i] += (i < n) ? __ldg(e.bias + c0 + i) : 0.0f;
                 if (e.Z) store_row_f32(e.Z + (size_t)r * e.ldz + c0, a, n);
 #pragma unroll
-                for (int i = 0; i < kEpiCols; ++i) h[i] = __float2bfloat16_rn(gelu_f(a[i]));
+                for (int i = 0; i < kEpiCols; i += 2)
+                    reinterpret_cast<uint32_t*>(h)[i / 2] = gelu_bf16x2(a[i], a[i + 1]);
             } else {
                 float z[kEpiCols];
                 load_row_f32(e.Z + (size_t)r * e.ldz + c0, z, n);
@@ -237,7 +320,7 @@ constexpr size_t gemm_smem() {
 }
 
 // ------------------------------------------------------------------ fused MC inference
-// S for MC samples in one kernel, one 128-row tile per CTA (eight warps):
+// S for MC samples in one kernel, one 128-row tile per CTA (sixteen warps):
 // the tile's BF16 inputs are formed from the samples' Philox words straight
 // into shared memory (k_surrogate_x_mc's map), the three hidden layers run
 // back to back on the tensor cores with the activations kept in shared
@@ -250,8 +333,14 @@ constexpr size_t gemm_smem() {
 // Weights stream in blocks of 64 inputs x 128 outputs (16 KB, two MMAs of
 // N = 128 per 64-input block), so a CTA takes 97 KB of shared memory and two
 // CTAs share an SM: one's epilogue runs beside the other's loads and MMAs.
+// Bound: instruction issue (input generation two fifths, GELU three): 1000003
+// samples of 128 inputs 1.26 ms; 1.59 with eight warps a CTA, erff and
+// normcdfinvf in full for every value (inlined, the loops outgrew the
+// instruction cache), a 64-bit high product per Philox multiplication and round
+// keys formed by every thread.
 constexpr int kFusedRows = 128;
-constexpr int kFusedThreads = 256;
+constexpr int kFusedThreads = 512;
+constexpr int kFusedCols = kH / (kFusedThreads / 128);    // columns a warp drains per layer
 constexpr uint32_t kFusedKBlock = kFusedRows * kGk * 2;   // 16 KB: 128 rows x 64 columns BF16
 constexpr uint32_t kFusedWStage = (kH / 2) * kGk * 2;     // 16 KB: half the rows (128 outputs) x 64 columns BF16
 constexpr int kFusedH3Stride = kH * 2 + 16;               // bytes per row of the staged last layer
@@ -270,8 +359,8 @@ __device__ __forceinline__ uint32_t fused_a_offset(int r, int k) {
 }
 
 struct FusedArgs {
-    uint64_t seed, first;
-    uint32_t level;
+    PhiloxKeys keys;
+    uint64_t first;
     int n, M, D;
     const float *b1, *b2, *b3, *b4;
     const __nv_bfloat16* w4;
@@ -308,23 +397,15 @@ __global__ void __launch_bounds__(kFusedThreads, 2)
     if (warp == 0) tc::tmem_alloc(tmem_slot, kH);
     // the tile's inputs: 4 columns per Philox call, as k_surrogate_x_mc forms them
     {
-        const int groups = a.D / 4;
-        for (int t = threadIdx.x; t < kFusedRows * groups; t += kFusedThreads) {
-            const int r = t / groups, g = t % groups;
-            __align__(8) __nv_bfloat16 h[4];
+        const int lg = a.D == 128 ? 5 : 6;   // D is 128 or 256: 32 or 64 groups of 4 columns a row
+        for (int t = threadIdx.x; t < kFusedRows << lg; t += kFusedThreads) {
+            const int r = t >> lg, g = t & ((1 << lg) - 1);
+            uint2 h = make_uint2(0u, 0u);
             if (r0 + r < a.n && 4 * g < a.M) {
                 u64x4 c = {{(uint64_t)g, a.first + (uint64_t)(r0 + r), 0, 0}};
-                const u64x4 w = philox4x64(c, a.seed, (kPurposeMC << 32) | a.level);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float u = ((float)(w.v[q] >> 41) + 0.5f) * 0x1p-23f;
-                    h[q] = __float2bfloat16_rn(4 * g + q < a.M ? normcdfinvf(u) : 0.0f);
-                }
-            } else {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) h[q] = __float2bfloat16_rn(0.0f);
+                h = mc_inputs(philox4x64(c, a.keys), a.M - 4 * g);
             }
-            *reinterpret_cast<uint2*>(sAct + fused_a_offset(r, 4 * g)) = *reinterpret_cast<const uint2*>(h);
+            *reinterpret_cast<uint2*>(sAct + fused_a_offset(r, 4 * g)) = h;
         }
     }
     tc::fence_proxy_async_smem();
@@ -342,7 +423,7 @@ __global__ void __launch_bounds__(kFusedThreads, 2)
     constexpr uint32_t idesc = tc::idesc_bf16_f32(kFusedRows, kH / 2);
     int issued = 0;   // producer (warp 0 lane 0): weight blocks issued so far
     bool ok = true;
-    const int qd = warp & 3, ch = warp >> 2;   // TMEM lane quadrant, column half of the epilogue
+    const int qd = warp & 3, ch = warp >> 2;   // TMEM lane quadrant, column part of the epilogue
     const int r = 32 * qd + lane;               // the tile row this thread drains
     for (int L = 0; L < 3 && ok; ++L) {
         if (warp == 0 && lane == 0) {
@@ -375,34 +456,37 @@ __global__ void __launch_bounds__(kFusedThreads, 2)
         __syncwarp();
         // every thread goes on alike: a wait that ran out anywhere ends the
         // layers for the whole CTA (the error flag is already set)
-        ok = __syncthreads_and(tc::mbar_wait(done, L & 1, a.err)) != 0;
+        // (one thread waits for the products, the others at the barrier: 512
+        // threads polling took issue slots from the CTA beside this one)
+        bool arrived = true;
+        if (threadIdx.x == kFusedThreads - 1) {
+            arrived = tc::mbar_wait(done, L & 1, a.err);
+            tc::fence_after_sync();
+            tc::fence_before_sync();
+        }
+        ok = __syncthreads_and(arrived) != 0;
         tc::fence_after_sync();
         if (ok) {
             // bias + GELU + BF16, as the layer-by-layer epilogue forms it: the
             // next layer's A operand in place, the last layer's rows plainly
             const uint32_t trow = tmem + ((uint32_t)(32 * qd) << 16);
 #pragma unroll 1
-            for (int c = 0; c < 4; ++c) {
-                const int c0 = ch * 128 + c * 32;
-                uint32_t v[32];
-                tc::tmem_ld_32x32b_x32(trow + c0, v);
-                float x[32];
-                __align__(16) __nv_bfloat16 h[32];
+            for (int c = 0; c < kFusedCols / 16; ++c) {   // 16 columns at a time: the loop body stays in the instruction cache
+                const int c0 = ch * kFusedCols + c * 16;
+                uint32_t v[16];
+                tc::tmem_ld_32x32b_x16(trow + c0, v);
+                uint32_t h[8];
 #pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    x[i] = __uint_as_float(v[i]) + __ldg(biases[L] + c0 + i);
-                    h[i] = __float2bfloat16_rn(gelu_f(x[i]));
+                for (int i = 0; i < 16; i += 4) {
+                    const float4 b4 = __ldg(reinterpret_cast<const float4*>(biases[L] + c0 + i));
+                    h[i / 2] = gelu_bf16x2(__uint_as_float(v[i]) + b4.x, __uint_as_float(v[i + 1]) + b4.y);
+                    h[i / 2 + 1] = gelu_bf16x2(__uint_as_float(v[i + 2]) + b4.z, __uint_as_float(v[i + 3]) + b4.w);
                 }
-                if (L < 2) {
 #pragma unroll
-                    for (int m = 0; m < 4; ++m)
-                        *reinterpret_cast<uint4*>(sAct + fused_a_offset(r, c0 + 8 * m)) =
-                            reinterpret_cast<const uint4*>(h)[m];
-                } else {
-#pragma unroll
-                    for (int m = 0; m < 4; ++m)
-                        *reinterpret_cast<uint4*>(base + (size_t)r * kFusedH3Stride + (c0 + 8 * m) * 2) =
-                            reinterpret_cast<const uint4*>(h)[m];
+                for (int m = 0; m < 2; ++m) {
+                    uint8_t* dst = L < 2 ? sAct + fused_a_offset(r, c0 + 8 * m)
+                                         : base + (size_t)r * kFusedH3Stride + (c0 + 8 * m) * 2;
+                    *reinterpret_cast<uint4*>(dst) = make_uint4(h[4 * m], h[4 * m + 1], h[4 * m + 2], h[4 * m + 3]);
                 }
             }
         }
@@ -706,21 +790,12 @@ __global__ void k_surrogate_x_mc(uint64_t seed, uint32_t level, uint64_t first, 
     const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (uint64_t)n * blocks) return;
     const int s = (int)(t / blocks), b = (int)(t % blocks);
-    __align__(8) __nv_bfloat16 h[4];
+    uint2 h = make_uint2(0u, 0u);
     if (4 * b < M) {
         u64x4 c = {{(uint64_t)b, first + s, 0, 0}};
-        const u64x4 w = philox4x64(c, seed, (kPurposeMC << 32) | level);
-#pragma unroll
-        for (int lane = 0; lane < 4; ++lane) {
-            // 23 bits keep (k + 1/2) exact in FP32, so 0 < u < 1 strictly
-            const float u = ((float)(w.v[lane] >> 41) + 0.5f) * 0x1p-23f;
-            h[lane] = __float2bfloat16_rn(4 * b + lane < M ? normcdfinvf(u) : 0.0f);
-        }
-    } else {
-#pragma unroll
-        for (int lane = 0; lane < 4; ++lane) h[lane] = __float2bfloat16_rn(0.0f);
+        h = mc_inputs(philox4x64(c, seed, (kPurposeMC << 32) | level), M - 4 * b);
     }
-    *reinterpret_cast<uint2*>(X + (size_t)s * D + 4 * b) = *reinterpret_cast<const uint2*>(h);
+    *reinterpret_cast<uint2*>(X + (size_t)s * D + 4 * b) = h;
 }
 
 // ------------------------------------------------------------------ host state
@@ -1055,7 +1130,7 @@ fm_status surrogate_eval_mc_impl(fm_ctx* ctx, uint32_t level, uint64_t first, ui
     if (S->D <= kH && ctx->fused_infer) {
         // inputs up to 256 wide: the whole network in one kernel per 128 rows
         wait_trained(S, st);
-        FusedArgs fa{seed, first, level, (int)n, S->M, S->D, S->P + S->off[1], S->P + S->off[3], S->P + S->off[5],
+        FusedArgs fa{philox_keys(seed, (kPurposeMC << 32) | level), first, (int)n, S->M, S->D, S->P + S->off[1], S->P + S->off[3], S->P + S->off[5],
                      S->P + S->off[7], S->w4b, S->mu, S->sd, d_s, S->err};
         const double flops = 2.0 * n * ((double)S->D * kH + 2.0 * kH * kH + kH);
         FM_TIMED(ctx, kFamMlp, st, 8.0 * n, flops,
