@@ -32,14 +32,39 @@ inline unsigned blocks_for(size_t threads) { return (unsigned)((threads + kBlock
 // Sample of a flat thread index and whether it still iterates.
 __device__ __forceinline__ bool inactive(const int32_t* active, size_t s) { return active && !active[s]; }
 
+// Sample, cell and column / row of a flat index over n x n grids.  By shifts
+// where n is a power of two: the four divisions (64-bit ones for the sample) took
+// longer than the arithmetic of the kernels that move a few bytes a cell.
+struct CellAt {
+    size_t s;
+    int c, i, j;
+};
+__device__ __forceinline__ CellAt cell_at(size_t t, int n) {
+    CellAt a;
+    if ((n & (n - 1)) == 0) {
+        const int lg = __ffs(n) - 1;
+        a.s = t >> (2 * lg);
+        a.c = (int)t & (n * n - 1);
+        a.i = a.c & (n - 1);
+        a.j = a.c >> lg;
+    } else {
+        const size_t cells = (size_t)n * n;
+        a.s = t / cells;
+        a.c = (int)(t % cells);
+        a.i = a.c % n;
+        a.j = a.c / n;
+    }
+    return a;
+}
+
 // K_c[J][I] = K_f[2J][2I] (Sec. 2.5, the lower-left child in 0-indexed form).
 __global__ void k_inject(int nc, size_t S, const double* __restrict__ Kf, double* __restrict__ Kc) {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t cells = (size_t)nc * nc;
     if (t >= S * cells) return;
-    const size_t s = t / cells;
-    const int c = (int)(t % cells);
-    const int I = c % nc, J = c / nc, nf = 2 * nc;
+    const CellAt at = cell_at(t, nc);
+    const size_t s = at.s;
+    const int I = at.i, J = at.j, nf = 2 * nc;
     Kc[t] = Kf[s * (size_t)nf * nf + (size_t)(2 * J) * nf + 2 * I];
 }
 
@@ -52,11 +77,11 @@ __global__ void k_child_geomean(int nc, size_t S, const double* __restrict__ Kf,
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t cells = (size_t)nc * nc;
     if (t >= S * cells) return;
-    const size_t s = t / cells;
-    const int c = (int)(t % cells);
-    const int I = c % nc, J = c / nc, nf = 2 * nc;
+    const CellAt at = cell_at(t, nc);
+    const size_t s = at.s;
+    const int I = at.i, J = at.j, nf = 2 * nc;
     const double* k = Kf + s * (size_t)nf * nf + (size_t)(2 * J) * nf + 2 * I;
-    Kc[t] = (double)geometric_mean4((C)k[0], (C)k[1], (C)k[nf], (C)k[nf + 1]);
+    Kc[t] = widen(geometric_mean4(rounded<C>(k[0]), rounded<C>(k[1]), rounded<C>(k[nf]), rounded<C>(k[nf + 1])));
 }
 
 // Face transmissibilities: harmonic mean inside, 2K on the Dirichlet edges
@@ -72,13 +97,13 @@ __global__ void k_faces(int n, size_t S, int ns, const double* __restrict__ K, T
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t cells = (size_t)n * n;
     if (t >= S * cells) return;
-    const int c = (int)(t % cells);
-    const int i = c % n, j = c / n;
-    const C k = (C)K[t];
-    const C te = (i < n - 1) ? harmonic_mean(k, (C)K[t + 1]) : C(2) * k;
-    const C tn = (j < n - 1) ? harmonic_mean(k, (C)K[t + n]) : (ns ? C(2) * k : C(0));
-    Te[t] = (T)te;
-    Tn[t] = (T)tn;
+    const CellAt at = cell_at(t, n);
+    const int i = at.i, j = at.j;
+    const C k = rounded<C>(K[t]);
+    const C te = (i < n - 1) ? harmonic_mean(k, rounded<C>(K[t + 1])) : C(2) * k;
+    const C tn = (j < n - 1) ? harmonic_mean(k, rounded<C>(K[t + n])) : (ns ? C(2) * k : C(0));
+    Te[t] = rounded<T>(te);
+    Tn[t] = rounded<T>(tn);
     if (Te64) {
         Te64[t] = (double)te;
         Tn64[t] = (double)tn;
@@ -98,15 +123,21 @@ __global__ void k_diagonal(int n, size_t S, int ns, const double* K, const T* __
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t cells = (size_t)n * n;
     if (t >= S * cells) return;
-    const int c = (int)(t % cells);
-    const int i = c % n, j = c / n;
-    auto fe = [&](size_t u) { return Te64 ? (C)Te64[u] : (C)Te[u]; };
-    auto fn = [&](size_t u) { return Tn64 ? (C)Tn64[u] : (C)Tn[u]; };
-    const C k = (C)K[t];
-    const C tw = (i > 0) ? fe(t - 1) : C(2) * k;
-    const C ts = (j > 0) ? fn(t - n) : (ns ? C(2) * k : C(0));
+    const CellAt at = cell_at(t, n);
+    const int i = at.i, j = at.j;
+    // (a test for the copies here converted every face, in the FP64 pipe: 0.6 ms
+    // where 0.3 do, 1000 grids of 256 x 256)
+    auto face = [&](const T* f, const double* f64, size_t u) {
+        if constexpr (sizeof(C) != sizeof(T)) return f64[u];
+        else return f[u];
+    };
+    auto fe = [&](size_t u) { return face(Te, Te64, u); };
+    auto fn = [&](size_t u) { return face(Tn, Tn64, u); };
+    auto edge = [&] { return C(2) * rounded<C>(K[t]); };
+    const C tw = (i > 0) ? fe(t - 1) : edge();
+    const C ts = (j > 0) ? fn(t - n) : (ns ? edge() : C(0));
     const C d = tw + fe(t) + ts + fn(t);
-    D[t] = (T)d;
+    D[t] = rounded<T>(d);
     if (D64) D64[t] = (double)d;
     if (rD) rD[t] = T(1) / (T)d;
 }
@@ -118,8 +149,8 @@ __global__ void k_stage_rhs(int n, size_t S, const double* __restrict__ K, Bnd b
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t cells = (size_t)n * n;
     if (t >= S * cells) return;
-    const int c = (int)(t % cells);
-    const int i = c % n, j = c / n;
+    const CellAt at = cell_at(t, n);
+    const int i = at.i, j = at.j;
     const bool edge = i == 0 || i == n - 1 || (bd.ns && (j == 0 || j == n - 1));
     b[t] = edge ? (T)dirichlet_rhs(bd, n, i, j, K[t]) : T(0);
 }
@@ -395,72 +426,188 @@ __global__ void k_residual_restrict(int nc, size_t S, const T* __restrict__ bf, 
 }
 
 // p_f += P e_c (add = 1, boundary values 0) or p_f = P u_c (add = 0, FMG start,
-// the Dirichlet data as ghost values).
+// the Dirichlet data as ghost values).  Cells off the edges first, then the edge
+// cells on threads of their own: the ghosts' FP64 operations take the FP64 pipe
+// from every warp that holds them, predicated off or not (1000 grids of
+// 256 x 256: nine operations a cell for five).
 template <typename U>
 __global__ void k_prolong(int nc, size_t S, const U* __restrict__ uc, Ghost<U> gh, int add, U* __restrict__ pf,
                           const int32_t* __restrict__ active) {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int nf = 2 * nc;
+    const int nf = 2 * nc, ring = 4 * (nf - 1);
     const size_t cells = (size_t)nf * nf;
-    if (t >= S * cells) return;
-    const size_t s = t / cells;
-    if (inactive(active, s)) return;
-    const int c = (int)(t % cells);
-    const int i = c % nf, j = c / nf;
-    const U v = prolong_at(nc, uc + s * (size_t)nc * nc, i, j, gh);
-    pf[t] = add ? pf[t] + v : v;
+    size_t s;
+    int i, j;
+    U v;
+    if (t < S * cells) {
+        const CellAt at = cell_at(t, nf);
+        s = at.s;
+        i = at.i;
+        j = at.j;
+        if (i == 0 || i == nf - 1 || j == 0 || j == nf - 1 || inactive(active, s)) return;
+        const U* row = uc + s * (size_t)nc * nc + (size_t)(j >> 1) * nc + (i >> 1);
+        const int x = (i & 1) ? 1 : -1, y = (j & 1) ? nc : -nc;
+        v = prolong_vals(row[0], row[x], row[y], row[y + x]);
+    } else {
+        const size_t r = t - S * cells;
+        s = r / ring;
+        if (s >= S || inactive(active, s)) return;
+        const int e = (int)(r % ring), q = e / (nf - 1), o = e % (nf - 1);   // side, position along it
+        i = q == 0 ? o : q == 1 ? nf - 1 : q == 2 ? nf - 1 - o : 0;
+        j = q == 0 ? 0 : q == 1 ? o : q == 2 ? nf - 1 : nf - 1 - o;
+        v = prolong_at(nc, uc + s * (size_t)nc * nc, i, j, gh);
+    }
+    const size_t g = s * cells + (size_t)j * nf + i;
+    pf[g] = add ? pf[g] + v : v;
 }
+
+inline size_t prolong_threads(size_t S, int n) { return S * ((size_t)n * n + 4 * (size_t)(n - 1)); }
+
+// Three neighbouring values of a coarse row around column I: its own, west and
+// east; past the Dirichlet edges the error's ghosts, minus its own.
+template <typename T>
+struct CoarseRow {
+    T o, w, e;
+};
+template <typename T>
+__device__ __forceinline__ CoarseRow<T> ghost_row(const CoarseRow<T>& r, int ns) {
+    return ns ? CoarseRow<T>{-r.o, -r.w, -r.e} : r;
+}
+// (P e) at the two fine columns of a coarse cell, in the fine row next to row `other`.
+template <typename T, typename V2>
+__device__ __forceinline__ V2 prolong_pair(const CoarseRow<T>& own, const CoarseRow<T>& other) {
+    V2 d;
+    d.x = prolong_vals(own.o, own.w, other.o, other.w);
+    d.y = prolong_vals(own.o, own.e, other.o, other.e);
+    return d;
+}
+
+template <typename T>
+struct PairOf;
+template <>
+struct PairOf<float> {
+    using type = float2;
+};
+template <>
+struct PairOf<double> {
+    using type = double2;
+};
 
 // Energy-optimal step of a coarse-grid correction: the correction d = P e_c
 // is added as alpha d with alpha = (r, d) / (d, A d), r = b - A x the
 // residual it answers, the exact line minimum of the energy error for the
 // symmetric positive definite A (so a cycle never raises the energy error,
 // whatever the correction operators).  Per (sample, chunk) of grid n: the
-// partial sums of (r, d) and (d, A d) in FP64, with d formed on the fly by
-// the prolongation (A d takes it at the four neighbours too); entries 0 and
-// 1 of the sample's 3-double slots in partial.
+// partial sums of (r, d) and (d, A d) in FP64; entries 0 and 1 of the
+// sample's 3-double slots in partial.
+//
+// A lane owns a coarse column (two fine ones) and walks up its band of rows:
+// d of each cell is formed once, x and Tn of the row below stay in registers,
+// and values of the next columns come by shuffle (windows of 30 columns with
+// one more at each end, or 32 where the grid is no wider).  A thread per cell,
+// forming d at the cell and its four neighbours, took 9.3 ms of a solve of seven
+// fields of 1024 x 1024 (312 launches of 30 us on average); the walk takes 3.6
+// (67 us on five fields of the finest grid, where the FP64 pipe's two FMAs a cell
+// are 18 us and the instructions issued most of the rest).
 template <typename T>
-__global__ void k_energy_partials(int n, size_t S, int chunks, const T* __restrict__ b, const T* __restrict__ Te,
-                                  const T* __restrict__ Tn, const T* __restrict__ D, const T* __restrict__ x,
-                                  const T* __restrict__ ec, const int32_t* __restrict__ active,
-                                  const int32_t* __restrict__ order, double* __restrict__ partial, int ns) {
+__global__ void __launch_bounds__(256) k_energy_partials(
+    int n, size_t S, int chunks, const T* __restrict__ b, const T* __restrict__ Te, const T* __restrict__ Tn,
+    const T* __restrict__ D, const T* __restrict__ x, const T* __restrict__ ec, const int32_t* __restrict__ active,
+    const int32_t* __restrict__ order, double* __restrict__ partial, int ns) {
+    using V2 = typename PairOf<T>::type;
+    constexpr unsigned all = 0xffffffffu;
     __shared__ double red[2][32];
     if (blockIdx.x / chunks >= S) return;   // S: the samples enumerated (listed by order, if given)
     const size_t s = order ? (size_t)order[blockIdx.x / chunks] : blockIdx.x / chunks;
     const int ch = (int)(blockIdx.x % chunks);
     if (inactive(active, s)) return;
-    const int nc = n / 2;
+    const int nc = n / 2, lane = threadIdx.x & 31, warps = (int)(blockDim.x >> 5);
     const size_t base = s * (size_t)n * n;
     const T* e = ec + s * (size_t)nc * nc;
-    const int cells = n * n, per = (cells + chunks - 1) / chunks;
-    const int c0 = ch * per, c1 = min(cells, c0 + per);
+    // the chunk's coarse rows, as tasks of (window, part of the rows)
+    const int cr = (nc + chunks - 1) / chunks, J0 = min(nc, ch * cr), J1 = min(nc, J0 + cr);
+    const bool whole = nc <= 32;
+    const int windows = whole ? 1 : (nc + 29) / 30;
+    const int parts = max(1, min(cr, warps / windows)), pr = (cr + parts - 1) / parts;
     double rd = 0.0, dad = 0.0;
-    for (int c = c0 + threadIdx.x; c < c1; c += blockDim.x) {
-        const int i = c % n, j = c / n;
-        const size_t g = base + c;
-        const T r = residual_at(n, g, i, j, b, Te, Tn, D, x);
-        const T d = prolong_err(nc, e, i, j, ns);
-        T ad = mul_rn(D[g], d);
-        if (i > 0) ad = fma(-Te[g - 1], prolong_err(nc, e, i - 1, j, ns), ad);
-        if (i < n - 1) ad = fma(-Te[g], prolong_err(nc, e, i + 1, j, ns), ad);
-        if (j > 0) ad = fma(-Tn[g - n], prolong_err(nc, e, i, j - 1, ns), ad);
-        if (j < n - 1) ad = fma(-Tn[g], prolong_err(nc, e, i, j + 1, ns), ad);
-        rd += (double)r * (double)d;
-        dad += (double)d * (double)ad;
+    for (int t = (int)(threadIdx.x >> 5); t < windows * parts; t += warps) {
+        const int I = whole ? lane : 30 * (t % windows) - 1 + lane, Ic = min(max(I, 0), nc - 1);
+        const bool mine = I >= 0 && I < nc && (whole || (lane >= 1 && lane <= 30));
+        const int Ja = J0 + (t / windows) * pr, Jb = min(J1, Ja + pr);
+        if (Ja >= Jb) continue;
+        auto coarse = [&](int J) {
+            CoarseRow<T> r;
+            r.o = e[(size_t)J * nc + Ic];
+            r.w = __shfl_up_sync(all, r.o, 1);
+            r.e = __shfl_down_sync(all, r.o, 1);
+            if (I <= 0) r.w = -r.o;
+            if (I >= nc - 1) r.e = -r.o;
+            return r;
+        };
+        auto fine = [&](const T* a, int j) { return *reinterpret_cast<const V2*>(a + base + (size_t)j * n + 2 * Ic); };
+        CoarseRow<T> cur = coarse(Ja);
+        const CoarseRow<T> below = Ja > 0 ? coarse(Ja - 1) : ghost_row(cur, ns);
+        V2 dm = prolong_pair<T, V2>(below, cur), dc = prolong_pair<T, V2>(cur, below);
+        const int jm = max(2 * Ja - 1, 0);
+        V2 xm = fine(x, jm), tm = fine(Tn, jm), xc = fine(x, 2 * Ja);
+        // row j: its values, those of the rows below and above
+        auto row = [&](int j, const V2& dl, const V2& d, const V2& dh, const V2& xl, const V2& xv, const V2& xh,
+                       const V2& tl, const V2& tn) {
+            const V2 bv = fine(b, j), te = fine(Te, j), dd = fine(D, j);
+            const T tw = __shfl_up_sync(all, te.y, 1);
+            const T xw = __shfl_up_sync(all, xv.y, 1), xe = __shfl_down_sync(all, xv.x, 1);
+            const T dw = __shfl_up_sync(all, d.y, 1), de = __shfl_down_sync(all, d.x, 1);
+            const bool in_w = I > 0, in_e = I < nc - 1, in_s = j > 0, in_n = j < n - 1;
+            auto apply = [&](T diag, T c, T fw, T vw, bool w, T fe, T ve, bool ee, T fs, T vs, T fn, T vn) {
+                T v = mul_rn(diag, c);   // as residual_at forms A x
+                if (w) v = fma(-fw, vw, v);
+                if (ee) v = fma(-fe, ve, v);
+                if (in_s) v = fma(-fs, vs, v);
+                if (in_n) v = fma(-fn, vn, v);
+                return v;
+            };
+            const T r0 = bv.x - apply(dd.x, xv.x, tw, xw, in_w, te.x, xv.y, true, tl.x, xl.x, tn.x, xh.x);
+            const T r1 = bv.y - apply(dd.y, xv.y, te.x, xv.x, true, te.y, xe, in_e, tl.y, xl.y, tn.y, xh.y);
+            const T a0 = apply(dd.x, d.x, tw, dw, in_w, te.x, d.y, true, tl.x, dl.x, tn.x, dh.x);
+            const T a1 = apply(dd.y, d.y, te.x, d.x, true, te.y, de, in_e, tl.y, dl.y, tn.y, dh.y);
+            if (mine) {
+                const double d0 = widen(d.x), d1 = widen(d.y);
+                rd = fma(widen(r0), d0, rd);
+                dad = fma(d0, widen(a0), dad);
+                rd = fma(widen(r1), d1, rd);
+                dad = fma(d1, widen(a1), dad);
+            }
+        };
+#pragma unroll 1
+        for (int J = Ja; J < Jb; ++J) {
+            const CoarseRow<T> up = J + 1 < nc ? coarse(J + 1) : ghost_row(cur, ns);
+            const int j = 2 * J;
+            const V2 d1 = prolong_pair<T, V2>(cur, up), d2 = prolong_pair<T, V2>(up, cur);
+            const V2 x1 = fine(x, j + 1), x2 = fine(x, min(j + 2, n - 1));
+            const V2 t0 = fine(Tn, j), t1 = fine(Tn, j + 1);
+            row(j, dm, dc, d1, xm, xc, x1, tm, t0);
+            row(j + 1, dc, d1, d2, xc, x1, x2, t0, t1);
+            dm = d1;
+            dc = d2;
+            xm = x1;
+            xc = x2;
+            tm = t1;
+            cur = up;
+        }
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
-        rd += __shfl_down_sync(0xffffffffu, rd, off);
-        dad += __shfl_down_sync(0xffffffffu, dad, off);
+        rd += __shfl_down_sync(all, rd, off);
+        dad += __shfl_down_sync(all, dad, off);
     }
-    if ((threadIdx.x & 31) == 0) {
+    if (lane == 0) {
         red[0][threadIdx.x >> 5] = rd;
         red[1][threadIdx.x >> 5] = dad;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         double a = 0.0, q = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+        for (int w = 0; w < warps; ++w) {
             a += red[0][w];
             q += red[1][w];
         }
@@ -470,32 +617,64 @@ __global__ void k_energy_partials(int n, size_t S, int chunks, const T* __restri
     }
 }
 
-// alpha[s] = (r, d) / (d, A d) from the chunks' partial sums (0 when d = 0).
-__global__ void k_energy_alpha(size_t S, int chunks, const double* __restrict__ partial, double* __restrict__ alpha,
-                               const int32_t* __restrict__ active) {
-    const size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= S || inactive(active, s)) return;
-    double rd = 0.0, dad = 0.0;
-    for (int ch = 0; ch < chunks; ++ch) {
-        rd += partial[((size_t)s * chunks + ch) * 3];
-        dad += partial[((size_t)s * chunks + ch) * 3 + 1];
-    }
-    alpha[s] = dad > 0.0 ? rd / dad : 0.0;
-}
-
-// p_f += alpha[s] P e_c, the stepped correction (in FP64, rounded once to T).
+// p_f += alpha P e_c, the stepped correction (in FP64, rounded once to T), with
+// alpha = (r, d) / (d, A d) of the sample from its chunks' partial sums (0 when
+// d = 0), summed by the first warp of each block: a launch of its own cost 4 us
+// a cycle and grid.  Threads take coarse cells, so four fine cells share the nine
+// coarse values (seven fields of 1024 x 1024: 3.5 ms a solve for both, now 2.4);
+// S, order as in k_energy_partials.
+constexpr int kStepCells = 4;   // coarse cells a thread
 template <typename T>
-__global__ void k_prolong_step(int nc, size_t S, const T* __restrict__ uc, const double* __restrict__ alpha,
-                               T* __restrict__ pf, const int32_t* __restrict__ active, int ns) {
-    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int nf = 2 * nc;
-    const size_t cells = (size_t)nf * nf;
-    if (t >= S * cells) return;
-    const size_t s = t / cells;
+__global__ void __launch_bounds__(256) k_energy_apply(int nc, size_t S, int chunks, int blocks,
+                                                      const T* __restrict__ uc, const double* __restrict__ partial,
+                                                      T* __restrict__ pf, const int32_t* __restrict__ active,
+                                                      const int32_t* __restrict__ order, int ns) {
+    using V2 = typename PairOf<T>::type;
+    __shared__ double alpha_s;
+    if (blockIdx.x / blocks >= S) return;
+    const size_t s = order ? (size_t)order[blockIdx.x / blocks] : blockIdx.x / blocks;
     if (inactive(active, s)) return;
-    const int c = (int)(t % cells);
-    const T v = prolong_err(nc, uc + s * (size_t)nc * nc, c % nf, c / nf, ns);
-    pf[t] = (T)((double)pf[t] + alpha[s] * (double)v);
+    if (threadIdx.x < 32) {
+        double rd = 0.0, dad = 0.0;
+        for (int ch = (int)threadIdx.x; ch < chunks; ch += 32) {
+            rd += partial[((size_t)s * chunks + ch) * 3];
+            dad += partial[((size_t)s * chunks + ch) * 3 + 1];
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            rd += __shfl_down_sync(0xffffffffu, rd, off);
+            dad += __shfl_down_sync(0xffffffffu, dad, off);
+        }
+        if (threadIdx.x == 0) alpha_s = dad > 0.0 ? rd / dad : 0.0;
+    }
+    __syncthreads();
+    const double alpha = alpha_s;
+    const int nf = 2 * nc, cells = nc * nc;
+    const T* u = uc + s * (size_t)cells;
+    T* p = pf + s * (size_t)nf * nf;
+    for (int c = (int)(blockIdx.x % blocks) * 256 + (int)threadIdx.x; c < cells; c += blocks * 256) {
+        const int I = c % nc, J = c / nc;
+        auto coarse = [&](int j) {
+            const T* r = u + (size_t)j * nc + I;
+            CoarseRow<T> v;
+            v.o = r[0];
+            v.w = I > 0 ? r[-1] : -v.o;
+            v.e = I < nc - 1 ? r[1] : -v.o;
+            return v;
+        };
+        const CoarseRow<T> own = coarse(J);
+        const CoarseRow<T> lo = J > 0 ? coarse(J - 1) : ghost_row(own, ns);
+        const CoarseRow<T> hi = J < nc - 1 ? coarse(J + 1) : ghost_row(own, ns);
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+            const V2 d = prolong_pair<T, V2>(own, y ? hi : lo);
+            V2* q = reinterpret_cast<V2*>(p + (size_t)(2 * J + y) * nf + 2 * I);
+            V2 v = *q;
+            v.x = rounded<T>(fma(alpha, widen(d.x), widen(v.x)));
+            v.y = rounded<T>(fma(alpha, widen(d.y), widen(v.y)));
+            *q = v;
+        }
+    }
 }
 
 // The first colour (0) of post-smoothing fused with the coarse-grid
@@ -679,12 +858,15 @@ __global__ void k_fill(size_t count, double v, double* __restrict__ x) {
 // zeroed.  k_stage_decide then folds the partials in chunk order.  b / bT
 // and p / pT are the same arrays, hence no __restrict__ on them.
 // Threads walk rows (a column each, or several rows per pass on grids
-// narrower than the block), so no cell index is divided.  The rhs of a stage
-// problem is zero off the Dirichlet edges: interior cells take r = -A p with
-// no K load, and only edge cells form the Dirichlet term and add to ||b||^2.
-// On GB300 the FP64 pipe (1/58 of the FP32 rate) bounds this kernel, so the
-// interior FP64 work is the residual's product and four FMAs, the square
-// and one rounding.
+// narrower than the block), so no cell index is divided.  The FP64 pipe (1/58 of
+// the FP32 rate) bounds this kernel, so a cell off the Dirichlet edges, whose
+// rhs is zero (r = -A p, no K load), takes six operations: the residual's
+// product and four FMAs, and the square.  Cells on an edge, whose Dirichlet
+// term and QoI share any warp that met one would wait for, come after them,
+// one a thread.  An instruction of the FP64 pipe takes its turn also where its
+// predicate is off for the whole warp, so there are none beside those six: 1000
+// samples of 256 x 256 from 546 us a test on average to 319 (an eighth of the
+// time: the sums across the warp).
 template <typename T>
 __global__ void k_stage_partials(int n, size_t S, int chunks, const double* __restrict__ K, Bnd bd,
                                  const T* b, const T* __restrict__ Te, const T* __restrict__ Tn,
@@ -708,54 +890,58 @@ __global__ void k_stage_partials(int n, size_t S, int chunks, const double* __re
     const int i0 = wide ? (int)threadIdx.x : (int)threadIdx.x % n;
     const int jo = wide ? 0 : (int)threadIdx.x / n;
     const int istep = wide ? nt : n;
-    const int h0 = n / 2 - 1, h1 = n / 2;   // Case I: the four centre cells
     double rr = 0.0, bb = 0.0, qq = 0.0;
-    if (jo < rpi) {
-        for (int j = j0 + jo; j < j1; j += rpi) {
-            const bool row_edge = bd.ns && (j == 0 || j == n - 1);
-            const bool row_centre = bd.ns && (j == h0 || j == h1);
-            for (int i = i0; i < n; i += istep) {
-                const size_t g = base + (size_t)j * n + i;
-                const bool edge = row_edge || i == 0 || i == n - 1;
-                double r, pv;
-                if (p64) {
-                    pv = p64[g];
-                    double v = D64[g] * pv;
-                    if (i > 0) v -= Te64[g - 1] * p64[g - 1];
-                    if (i < n - 1) v -= Te64[g] * p64[g + 1];
-                    if (j > 0) v -= Tn64[g - n] * p64[g - n];
-                    if (j < n - 1) v -= Tn64[g] * p64[g + n];
-                    if (edge) {
-                        const double f = dirichlet_rhs(bd, n, i, j, K[g]);
-                        r = f - v;
-                        bb += f * f;
-                    } else {
-                        r = -v;
-                    }
-                    bT[g] = (T)r;
-                    if (pT) pT[g] = T(0);
-                } else {
-                    pv = (double)p[g];
-                    r = (double)residual_at(n, g, i, j, b, Te, Tn, D, p);
-                    if (edge) {
-                        const double f = dirichlet_rhs(bd, n, i, j, K[g]);
-                        bb += f * f;
-                    }
-                }
-                rr += r * r;
-                if (bd.ns) {
-                    if (row_centre && (i == h0 || i == h1)) qq += 0.25 * pv;
-                } else if (i == n - 1) {
-                    qq += 2.0 * K[g] * (pv - bd.g[1]);
-                }
-            }
+    // the residual at cell (i, j) (interior: rhs zero), rounded into bT in the mixed form
+    auto residual = [&](int i, int j, bool interior, double f) {
+        const size_t g = base + (size_t)j * n + i;
+        double r;
+        if (p64) {
+            double v = D64[g] * p64[g];
+            if (interior || i > 0) v = fma(-Te64[g - 1], p64[g - 1], v);
+            if (interior || i < n - 1) v = fma(-Te64[g], p64[g + 1], v);
+            if (j > 0) v = fma(-Tn64[g - n], p64[g - n], v);
+            if (j < n - 1) v = fma(-Tn64[g], p64[g + n], v);
+            // (the sign changes in FP32: negated in FP64 it was an addition more a cell)
+            r = interior ? v : f - v;
+            bT[g] = interior ? -rounded<T>(r) : rounded<T>(r);
+            if (pT) pT[g] = T(0);
+        } else {
+            r = widen(residual_at(n, g, i, j, b, Te, Tn, D, p));
         }
+        rr = fma(r, r, rr);
+    };
+    const int ja = max(j0, bd.ns ? 1 : 0), jb = min(j1, bd.ns ? n - 1 : n);   // rows with interior cells
+    if (jo < rpi) {
+        for (int j = ja + jo; j < jb; j += rpi)
+            for (int i = i0; i < n; i += istep)
+                if (i > 0 && i < n - 1) residual(i, j, true, 0.0);
+    }
+    // the chunk's west and east columns, and in Case I what is left of its south and north rows
+    const int cols = 2 * max(0, j1 - j0);
+    const int south = bd.ns && j0 == 0 ? n - 2 : 0, north = bd.ns && j1 == n && j0 < n ? n - 2 : 0;
+    for (int t = (int)threadIdx.x; t < cols + south + north; t += nt) {
+        const int i = t < cols ? (t & 1) * (n - 1) : 1 + (t - cols) % (n - 2);
+        const int j = t < cols ? j0 + (t >> 1) : (t - cols < south ? 0 : n - 1);
+        const size_t g = base + (size_t)j * n + i;
+        const double f = dirichlet_rhs(bd, n, i, j, K[g]);
+        residual(i, j, false, f);
+        bb = fma(f, f, bb);
+        if (!bd.ns && i == n - 1) qq += 2.0 * K[g] * ((p64 ? p64[g] : widen(p[g])) - bd.g[1]);
+    }
+    if (bd.ns && threadIdx.x < 4) {   // Case I: the four centre cells
+        const int i = n / 2 - 1 + (threadIdx.x & 1), j = n / 2 - 1 + (threadIdx.x >> 1);
+        const size_t g = base + (size_t)j * n + i;
+        if (j >= j0 && j < j1) qq = 0.25 * (p64 ? p64[g] : widen(p[g]));
     }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        rr += __shfl_down_sync(0xffffffffu, rr, off);
-        bb += __shfl_down_sync(0xffffffffu, bb, off);
-        qq += __shfl_down_sync(0xffffffffu, qq, off);
+    for (int off = 16; off > 0; off >>= 1) rr += __shfl_down_sync(0xffffffffu, rr, off);
+    // most warps met no edge (bits: an FP64 comparison costs as much as an addition)
+    if (__any_sync(0xffffffffu, (__double_as_longlong(bb) | __double_as_longlong(qq)) != 0)) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            bb += __shfl_down_sync(0xffffffffu, bb, off);
+            qq += __shfl_down_sync(0xffffffffu, qq, off);
+        }
     }
     if ((threadIdx.x & 31) == 0) {
         red[0][threadIdx.x >> 5] = rr;
@@ -777,20 +963,27 @@ __global__ void k_stage_partials(int n, size_t S, int chunks, const double* __re
     }
 }
 
-// The test itself, one thread per sample: active[s] = ||b - A p|| > tol ||b||
+// The test itself, one warp per sample: active[s] = ||b - A p|| > tol ||b||
 // and the last pass moved the outflux by more than qtol |Q|; counted in *left.
 __global__ void k_stage_decide(size_t S, int chunks, const double* __restrict__ partial, double tol, double qtol,
                                double* __restrict__ qprev, int32_t* __restrict__ active, int32_t* __restrict__ left,
                                int32_t* __restrict__ order) {
-    const size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t s = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (s >= S || inactive(active, s)) return;
     double a = 0.0, b2 = 0.0, q = 0.0;
-    for (int ch = 0; ch < chunks; ++ch) {
+    for (int ch = (int)(threadIdx.x & 31); ch < chunks; ch += 32) {
         const double* v = partial + ((size_t)s * chunks + ch) * 3;
         a += v[0];
         b2 += v[1];
         q += v[2];
     }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        a += __shfl_down_sync(0xffffffffu, a, off);
+        b2 += __shfl_down_sync(0xffffffffu, b2, off);
+        q += __shfl_down_sync(0xffffffffu, q, off);
+    }
+    if (threadIdx.x & 31) return;
     const bool done = a <= tol * tol * b2 || (qtol > 0 && fabs(q - qprev[s]) <= qtol * fabs(q));
     qprev[s] = q;
     active[s] = done ? 0 : 1;
@@ -801,27 +994,40 @@ __global__ void k_stage_decide(size_t S, int chunks, const double* __restrict__ 
 }
 
 // Mixed form: the FP64 refinement update p64 += e (the FP32 correction).
-template <typename T>
 // Grid-stride over the enumerated cells: S samples (listed by order, if
 // given), or with dcount (inside a graph's refinement loop) the count the
 // last residual test left, so a launch sized for every sample does little
-// work once few of them still iterate.
-__global__ void k_ir_update(size_t cells, size_t S, const T* __restrict__ e, double* __restrict__ p64,
+// work once few of them still iterate.  Cells go by pairs where a grid has an
+// even number of them.
+template <typename T>
+__global__ void k_ir_update(int n, size_t S, const T* __restrict__ e, double* __restrict__ p64,
                             const int32_t* __restrict__ active, const int32_t* __restrict__ order,
                             const int32_t* __restrict__ dcount) {
-    const size_t total = (dcount ? (size_t)*dcount : S) * cells;
-    for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-        const size_t s = order ? (size_t)order[t / cells] : t / cells;
+    using V2 = typename PairOf<T>::type;
+    const size_t cells = (size_t)n * n, total = (dcount ? (size_t)*dcount : S) * cells;
+    const int w = cells % 2 == 0 ? 2 : 1;
+    for (size_t t = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * w; t < total;
+         t += (size_t)gridDim.x * blockDim.x * w) {
+        const CellAt at = cell_at(t, n);
+        const size_t s = order ? (size_t)order[at.s] : at.s;
         if (inactive(active, s)) continue;
-        const size_t g = s * cells + t % cells;
-        p64[g] += (double)e[g];
+        const size_t g = s * cells + at.c;
+        if (w == 1) {
+            p64[g] += widen(e[g]);
+            continue;
+        }
+        const V2 v = *reinterpret_cast<const V2*>(e + g);
+        double2 p = *reinterpret_cast<const double2*>(p64 + g);
+        p.x += widen(v.x);
+        p.y += widen(v.y);
+        *reinterpret_cast<double2*>(p64 + g) = p;
     }
 }
 
 template <typename T>
 __global__ void k_widen(size_t count, const T* __restrict__ x, double* __restrict__ y) {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < count) y[t] = (double)x[t];
+    if (t < count) y[t] = widen(x[t]);
 }
 
 __global__ void k_status(size_t S, const int32_t* __restrict__ active, int32_t* __restrict__ status) {
@@ -1025,7 +1231,6 @@ struct Hierarchy {
     double* qprev;     // outflux of the previous iteration per sample
     double* partial;   // per-(sample, chunk) partial sums of the residual tests
     int32_t* order;    // the samples still iterating, as listed by the last residual test
-    double* alpha;     // per-sample step of the energy-optimal coarse-grid correction
     // Host-side count of the samples still iterating in a refined stage (the
     // host loop reads it after every test; S otherwise): the strip smoother
     // sizes its row segments for it, so that a launch with few active samples
@@ -1041,6 +1246,15 @@ struct Hierarchy {
 
 // CTAs per sample of a residual test on grid n (about 8192 cells each).
 inline int check_chunks(int n) { return std::max(1, std::min(128, n * n / 8192)); }
+
+// Chunks of a residual test (and of the energy step's sums): four times those,
+// eight cells a thread, so that the last tests of a stage, with a few samples
+// left, still spread over the SMs (200 fields of 128 x 128, 7 left: 78 us with 2
+// chunks a sample).  48 more at most: hierarchy_bytes counts check_chunks and 1.8 KB
+// a sample besides.
+inline int test_chunks(int n) {
+    return std::min(std::max(1, std::min(128, n * n / 2048)), check_chunks(n) + 48);
+}
 
 // Bytes of the reciprocal diagonals of one FP64 sample (grids below the
 // finest; the finest grid's takes the room counted for its K, the input).
@@ -1141,9 +1355,8 @@ static fm_status carve(fm_ctx* ctx, Arena& ar, Hierarchy<T>& H, int n_fine, int 
     H.left = converged ? (int32_t*)take(4) : nullptr;
     H.iter = converged ? (int32_t*)take(4) : nullptr;
     H.qprev = converged ? (double*)take(S * 8) : nullptr;
-    H.partial = converged ? (double*)take(S * (size_t)check_chunks(n_fine) * 24) : nullptr;
+    H.partial = converged ? (double*)take(S * (size_t)test_chunks(n_fine) * 24) : nullptr;
     H.order = converged ? (int32_t*)take(S * 4) : nullptr;
-    H.alpha = converged ? (double*)take(S * 8) : nullptr;
     return FM_OK;
 }
 
@@ -1323,23 +1536,25 @@ static T* start_iterate(const Hierarchy<T>& H, int k, const fm_solve_params& prm
 }
 
 // The energy-optimal step of the correction on grid c.n onto iterate x of
-// grid k: partials, alpha per sample, x += alpha P e_c.
+// grid k: partial sums, then alpha and x += alpha P e_c.
 template <typename T>
 static void energy_step(const Hierarchy<T>& H, int k, const T* Te, const T* Tn, const T* D, T* x, const int32_t* active,
                         int ns, cudaStream_t st) {
     fm_ctx* ctx = H.ctx;
     const GridBufs<T>& g = H.g[k];
     const GridBufs<T>& c = H.g[k - 1];
-    const size_t S = H.S, cells = S * (size_t)g.n * g.n;
     const double ts = sizeof(T);
-    const int chunks = check_chunks(g.n);
+    // bands of four coarse rows at least, as many as the sample's slots hold: few
+    // large fields leave the coarser grids' launches with a few warps otherwise
+    const int chunks = std::max(1, std::min(test_chunks(H.g[H.m].n), c.n / 4));
     const bool listed = H.listed();
-    const size_t nl = listed ? H.busy : S;
-    FM_TIMED(ctx, kFamProlong, st, (5.0 * ts + 1.25 * ts) * nl * g.n * g.n + 2.0 * ts * cells, 40.0 * nl * g.n * g.n,
-             k_energy_partials<T><<<(unsigned)(nl * chunks), kBlock, 0, st>>>(
+    const size_t nl = listed ? H.busy : H.S;
+    const int blocks = std::max(1, (int)(((size_t)c.n * c.n + 256 * kStepCells - 1) / (256 * kStepCells)));
+    FM_TIMED(ctx, kFamProlong, st, (5.0 * ts + 1.25 * ts) * nl * g.n * g.n + 2.0 * ts * nl * g.n * g.n, 40.0 * nl * g.n * g.n,
+             k_energy_partials<T><<<(unsigned)(nl * chunks), 256, 0, st>>>(
                  g.n, nl, chunks, g.b, Te, Tn, D, x, c.p, active, listed ? H.order : nullptr, H.partial, ns);
-             k_energy_alpha<<<blocks_for(S), kBlock, 0, st>>>(S, chunks, H.partial, H.alpha, active);
-             k_prolong_step<T><<<blocks_for(cells), kBlock, 0, st>>>(c.n, S, c.p, H.alpha, x, active, ns));
+             k_energy_apply<T><<<(unsigned)(nl * blocks), 256, 0, st>>>(c.n, nl, chunks, blocks, c.p, H.partial, x,
+                                                                        active, listed ? H.order : nullptr, ns));
 }
 
 // `count` V(nu1, nu2) cycles on grid k, from start_iterate (zero: from a zero
@@ -1427,7 +1642,7 @@ static void vcycles(const Hierarchy<T>& H, int k, int top, const fm_solve_params
                      c.n, S, g.b, Te, Tn, D, cur, c.b, c.p, active));
         below();
         if (prm.energy_step) {
-            // the stepped correction (converged mode: partials and alpha in the hierarchy)
+            // the stepped correction (converged mode: partial sums in the hierarchy)
             energy_step(H, k, Te, Tn, D, cur, active, ns, st);
             smooth_with<T>(ctx, tile, threads, n, S, prm.nu2, g.b, Te, Tn, D, rD, cur, g.p, active, st, nullptr, ns);
         } else if (tile == 0 && prm.nu2 >= 1) {
@@ -1445,7 +1660,8 @@ static void vcycles(const Hierarchy<T>& H, int k, int top, const fm_solve_params
         } else {
             const Ghost<T> zg{T(0), T(0), T(0), T(0), ns};
             FM_TIMED(ctx, kFamProlong, st, 2.25 * ts * cells, 8.0 * cells,
-                     k_prolong<T><<<blocks_for(cells), kBlock, 0, st>>>(c.n, S, c.p, zg, 1, cur, active));
+                     k_prolong<T><<<blocks_for(prolong_threads(S, n)), kBlock, 0, st>>>(c.n, S, c.p, zg, 1, cur,
+                                                                                        active));
             smooth_with<T>(ctx, tile, threads, n, S, prm.nu2, g.b, Te, Tn, D, rD, cur, g.p, active, st, nullptr, ns);
         }
     }
@@ -1464,7 +1680,7 @@ static void stage_test(const Hierarchy<T>& H, int k, const fm_solve_params& prm,
     fm_ctx* ctx = H.ctx;
     const GridBufs<T>& g = H.g[k];
     const size_t S = H.S, cells = (size_t)g.n * g.n;
-    const int chunks = check_chunks(g.n);
+    const int chunks = test_chunks(g.n);
     const size_t ns = H.listed() ? H.busy : S;
     int tile, threads;
     smooth_shape<T>(ctx, g.n, prm, &tile, &threads);
@@ -1473,7 +1689,7 @@ static void stage_test(const Hierarchy<T>& H, int k, const fm_solve_params& prm,
              k_stage_partials<T><<<(unsigned)(ns * chunks), kBlock, 0, st>>>(
                  g.n, ns, chunks, g.K, bnd_of(prm), g.b, g.Te, g.Tn, g.D, g.p, g.p64, g.Te64, g.Tn64, g.D64, g.b,
                  pT, H.active, H.partial, H.listed() ? H.order : nullptr);
-             k_stage_decide<<<blocks_for(S), kBlock, 0, st>>>(S, chunks, H.partial, prm.tol, prm.qtol, H.qprev,
+             k_stage_decide<<<blocks_for(S * 32), kBlock, 0, st>>>(S, chunks, H.partial, prm.tol, prm.qtol, H.qprev,
                                                               H.active, H.left, H.order));
 }
 
@@ -1543,7 +1759,7 @@ static fm_status refine_stage_graph(const Hierarchy<T>& H, int k, const fm_solve
     vcycles(H, k, k, prm, H.active, bs, cycles_per_test(prm), mixed);
     H.dcount = nullptr;
     if (mixed)
-        k_ir_update<T><<<ir_update_blocks(ctx, S * cells), kBlock, 0, bs>>>(cells, S, g.p, g.p64, H.active,
+        k_ir_update<T><<<ir_update_blocks(ctx, S * cells), kBlock, 0, bs>>>(g.n, S, g.p, g.p64, H.active,
                                                                               H.order, H.order ? H.left : nullptr);
     test(bs);
     cudaGraph_t body = nullptr;
@@ -1579,7 +1795,7 @@ static fm_status refine_stage(const Hierarchy<T>& H, int k, const fm_solve_param
         vcycles(H, k, k, prm, H.active, st, cycles_per_test(prm), mixed);
         if (mixed)
             k_ir_update<T><<<ir_update_blocks(ctx, (H.listed() ? H.busy : S) * cells), kBlock, 0, st>>>(
-                cells, H.listed() ? H.busy : S, g.p, g.p64, H.active, H.listed() ? H.order : nullptr, nullptr);
+                g.n, H.listed() ? H.busy : S, g.p, g.p64, H.active, H.listed() ? H.order : nullptr, nullptr);
     }
     H.busy = 0;   // later stages run every sample
     return FM_OK;
@@ -1642,12 +1858,12 @@ static fm_status fmg_batch(const Hierarchy<T>& H, const fm_solve_params& prm, do
             const GridBufs<T>& c = H.g[k - 1];
             if (mixed && refined && k == H.m && H.m >= 1 && refine_c) {
                 FM_TIMED(ctx, kFamFmgInterp, st, 10.0 * cells, 8.0 * cells,
-                         k_prolong<double><<<blocks_for(cells), kBlock, 0, st>>>(
+                         k_prolong<double><<<blocks_for(prolong_threads(S, g.n)), kBlock, 0, st>>>(
                              c.n, S, c.p64, Ghost<double>{bd.g[0], bd.g[1], bd.g[2], bd.g[3], bd.ns}, 0, g.p64,
                              nullptr));
             } else {
                 FM_TIMED(ctx, kFamFmgInterp, st, 1.25 * ts * cells, 8.0 * cells,
-                         k_prolong<T><<<blocks_for(cells), kBlock, 0, st>>>(
+                         k_prolong<T><<<blocks_for(prolong_threads(S, g.n)), kBlock, 0, st>>>(
                              c.n, S, c.p, Ghost<T>{(T)bd.g[0], (T)bd.g[1], (T)bd.g[2], (T)bd.g[3], bd.ns}, 0,
                              refined ? g.p : start_iterate(H, k, prm, prm.nu0), nullptr));
             }
@@ -1839,7 +2055,6 @@ static void carve_into(fm_ctx* ctx, Hierarchy<double>& H, char* base, int n_fine
     H.qprev = nullptr;
     H.partial = nullptr;
     H.order = nullptr;
-    H.alpha = nullptr;
 }
 
 // ------------------------------------------------------------------ autotuning

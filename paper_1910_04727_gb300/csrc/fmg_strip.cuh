@@ -15,19 +15,50 @@ __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(
 // FP64 -> FP32 (round to nearest even) and back in integers.  The conversion
 // instructions run in the FP64 pipe (two lanes a clock and SM), which bounds
 // every kernel that refines: ten and seven integer operations cost a sixth of
-// one conversion.  Zeros, and what is not a normal number of both types, take
-// the instruction.
+// one conversion.  What is not a normal number of both types goes by integers
+// too: a conversion there would take its turn in the pipe in every warp,
+// predicated off or not.
+static __device__ __noinline__ float narrow_rare(unsigned hi, unsigned lo) {
+    const unsigned e = (hi >> 20) & 0x7ffu;
+    const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+    unsigned r = 0;
+    if (e >= 1151u) {
+        if (e == 2047u && (m & 0xfffffffffffffull)) return __uint_as_float(0x7fffffffu);
+        r = 0x7f800000u;
+    } else if (e >= 873u) {   // a subnormal: units of 2^-149
+        const unsigned shift = 926u - e;
+        r = (unsigned)((m + ((1ull << (shift - 1)) - 1) + ((m >> shift) & 1)) >> shift);
+    }
+    return __uint_as_float(r | (hi & 0x80000000u));
+}
 __device__ __forceinline__ float narrow(double x) {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    if (((hi >> 20) & 0x7ffu) - 897u > 253u) return __double2float_rn(x);
+    if (((hi >> 20) & 0x7ffu) - 897u > 253u) return narrow_rare(hi, lo);
     const unsigned long long t = (((unsigned long long)hi << 32) | lo) + (0x0fffffffu + ((lo >> 29) & 1u));
     const unsigned u = __funnelshift_l((unsigned)t, (unsigned)(t >> 32), 3) - 0xc0000000u;
     return __uint_as_float((u & 0x7fffffffu) | (hi & 0x80000000u));
 }
+static __device__ __noinline__ double widen_rare(unsigned u) {
+    const unsigned m = u & 0x7fffffffu, sign = u & 0x80000000u;
+    if (m == 0) return __hiloint2double((int)sign, 0);
+    if (m >= 0x7f800000u) return __hiloint2double((int)(sign | 0x7ff00000u | ((m & 0x7fffffu) >> 3)), (int)(u << 29));
+    const unsigned shift = __clz(m) - 8, f = (m << shift) & 0x7fffffu;
+    return __hiloint2double((int)(sign | ((897u - shift) << 20) | (f >> 3)), (int)(f << 29));
+}
 __device__ __forceinline__ double widen(float x) {
     const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
-    if (m - 0x00800000u >= 0x7f000000u) return (double)x;
+    if (m - 0x00800000u >= 0x7f000000u) return widen_rare(u);
     return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+template <typename T>
+__device__ __forceinline__ T rounded(float x) {
+    return (T)x;
+}
+template <typename T>
+__device__ __forceinline__ T rounded(double x) {
+    if constexpr (sizeof(T) == 4) return narrow(x);
+    else return x;
 }
 
 // Harmonic mean 2ab / (a + b) of two coefficients, the face between them.
