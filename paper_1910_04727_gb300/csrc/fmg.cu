@@ -205,11 +205,17 @@ __device__ __forceinline__ U prolong_at(int nc, const U* u, int i, int j, const 
     }
     return prolong_vals(row[I], nx, ny, nxy);
 }
-// an error's ghosts: zero boundary data
+// The same of an error, whose boundary data are zero: the ghosts change sign.
 template <typename U>
 __device__ __forceinline__ U prolong_err(int nc, const U* u, int i, int j, int ns) {
-    const Ghost<U> g{U(0), U(0), U(0), U(0), ns};
-    return prolong_at(nc, u, i, j, g);
+    const int I = i >> 1, J = j >> 1;
+    const int Ix = (i & 1) ? I + 1 : I - 1;
+    const int Jy = (j & 1) ? J + 1 : J - 1;
+    const bool xe = Ix < 0 || Ix > nc - 1, ye = Jy < 0 || Jy > nc - 1, fy = ye && ns;
+    const int Ic = xe ? I : Ix;
+    const U* row = u + (size_t)J * nc;
+    const U* other = u + (size_t)(ye ? J : Jy) * nc;
+    return prolong_vals(row[I], flip_if(xe, row[Ic]), flip_if(fy, other[I]), flip_if(xe != fy, other[Ic]));
 }
 
 // nsweeps red-black sweeps (colour 0 then 1) on tiles of TI x TI cells of
@@ -247,9 +253,11 @@ __global__ void __launch_bounds__(256) k_rbgs_tile(int n, size_t S, int TI, int 
     for (int e = threadIdx.x; e < R; e += blockDim.x) {
         const int r = e / RW, q = e % RW;
         const size_t g = base + (size_t)(ya + r) * n + xa + q;
-        // with ec: the coarse-grid correction p + (P e) as k_prolong forms it
-        sp[e] = ec ? p_in[g] + prolong_err(n / 2, ec + s * (size_t)(n / 2) * (n / 2), xa + q, ya + r, ns)
-                   : p_in[g];
+        // with ec: the coarse-grid correction p + (P e) as k_prolong forms it, on black
+        // cells only (the first half-sweep replaces the red ones)
+        const bool corr = ec && ((xa + q + ya + r) & 1);
+        sp[e] = corr ? p_in[g] + prolong_err(n / 2, ec + s * (size_t)(n / 2) * (n / 2), xa + q, ya + r, ns)
+                     : p_in[g];
         sb[e] = b[g];
         se[e] = Te[g];
         sn[e] = Tn[g];
@@ -331,9 +339,11 @@ __global__ void __launch_bounds__((R / 2) * (R / RPT)) k_rbgs_tile_reg(int n, si
             up[k][j] = false;
             if (x < RW && y < RH) {
                 const size_t g = base + (size_t)gy * n + gx;
-                // with ec: the coarse-grid correction p + (P e) as k_prolong forms it
-                rp[k][j] = ec ? p_in[g] + prolong_err(n / 2, ec + s * (size_t)(n / 2) * (n / 2), gx, gy, ns)
-                              : p_in[g];
+                // with ec: the coarse-grid correction p + (P e) as k_prolong forms it, on
+                // black cells only (the first half-sweep replaces the red ones)
+                rp[k][j] = ec && ((gx + gy) & 1)
+                               ? p_in[g] + prolong_err(n / 2, ec + s * (size_t)(n / 2) * (n / 2), gx, gy, ns)
+                               : p_in[g];
                 rb[k][j] = b[g];
                 rr[k][j] = rD ? rD[g] : T(1) / D[g];
                 if (gx < n - 1) re[k][j] = Te[g];
@@ -402,26 +412,34 @@ __device__ __forceinline__ T residual_at(int n, size_t c, int i, int j, const T*
     return b[c] - v;
 }
 
+// Residuals of the four children of coarse cell (I, J), summed (kRedOnly: smoothed
+// = the last half-sweep has zeroed the black ones').
+template <typename T>
+__device__ __forceinline__ T restricted_at(int nf, size_t c00, int I, int J, const T* b, const T* Te, const T* Tn,
+                                           const T* D, const T* p, bool smoothed) {
+    const int i = 2 * I, j = 2 * J;
+    const T r00 = residual_at(nf, c00, i, j, b, Te, Tn, D, p);
+    if (kRedOnly<T> && smoothed) return r00 + residual_at(nf, c00 + nf + 1, i + 1, j + 1, b, Te, Tn, D, p);
+    const T r10 = residual_at(nf, c00 + 1, i + 1, j, b, Te, Tn, D, p);
+    const T r01 = residual_at(nf, c00 + nf, i, j + 1, b, Te, Tn, D, p);
+    const T r11 = residual_at(nf, c00 + nf + 1, i + 1, j + 1, b, Te, Tn, D, p);
+    return r00 + r10 + r01 + r11;
+}
+
 // Fused residual + restriction: b_c = sum of the four fine residuals; p_c = 0.
 template <typename T>
 __global__ void k_residual_restrict(int nc, size_t S, const T* __restrict__ bf, const T* __restrict__ Te,
                                     const T* __restrict__ Tn, const T* __restrict__ D, const T* __restrict__ pf,
-                                    T* __restrict__ bc, T* __restrict__ pc, const int32_t* __restrict__ active) {
+                                    T* __restrict__ bc, T* __restrict__ pc, const int32_t* __restrict__ active,
+                                    int smoothed) {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t cells = (size_t)nc * nc;
     if (t >= S * cells) return;
-    const size_t s = t / cells;
-    if (inactive(active, s)) return;
-    const int C = (int)(t % cells);
-    const int I = C % nc, J = C / nc, nf = 2 * nc;
-    const size_t base = s * (size_t)nf * nf;
-    const int i0 = 2 * I, j0 = 2 * J;
-    const size_t c00 = base + (size_t)j0 * nf + i0;
-    const T r00 = residual_at(nf, c00, i0, j0, bf, Te, Tn, D, pf);
-    const T r10 = residual_at(nf, c00 + 1, i0 + 1, j0, bf, Te, Tn, D, pf);
-    const T r01 = residual_at(nf, c00 + nf, i0, j0 + 1, bf, Te, Tn, D, pf);
-    const T r11 = residual_at(nf, c00 + nf + 1, i0 + 1, j0 + 1, bf, Te, Tn, D, pf);
-    bc[t] = r00 + r10 + r01 + r11;
+    const CellAt at = cell_at(t, nc);
+    if (inactive(active, at.s)) return;
+    const int nf = 2 * nc;
+    const size_t c00 = at.s * (size_t)nf * nf + (size_t)(2 * at.j) * nf + 2 * at.i;
+    bc[t] = restricted_at(nf, c00, at.i, at.j, bf, Te, Tn, D, pf, smoothed != 0);
     pc[t] = T(0);
 }
 
@@ -471,7 +489,7 @@ struct CoarseRow {
 };
 template <typename T>
 __device__ __forceinline__ CoarseRow<T> ghost_row(const CoarseRow<T>& r, int ns) {
-    return ns ? CoarseRow<T>{-r.o, -r.w, -r.e} : r;
+    return CoarseRow<T>{flip_if(ns, r.o), flip_if(ns, r.w), flip_if(ns, r.e)};
 }
 // (P e) at the two fine columns of a coarse cell, in the fine row next to row `other`.
 template <typename T, typename V2>
@@ -540,8 +558,8 @@ __global__ void __launch_bounds__(256) k_energy_partials(
             r.o = e[(size_t)J * nc + Ic];
             r.w = __shfl_up_sync(all, r.o, 1);
             r.e = __shfl_down_sync(all, r.o, 1);
-            if (I <= 0) r.w = -r.o;
-            if (I >= nc - 1) r.e = -r.o;
+            if (I <= 0) r.w = flip_if(true, r.o);
+            if (I >= nc - 1) r.e = flip_if(true, r.o);
             return r;
         };
         auto fine = [&](const T* a, int j) { return *reinterpret_cast<const V2*>(a + base + (size_t)j * n + 2 * Ic); };
@@ -658,8 +676,8 @@ __global__ void __launch_bounds__(256) k_energy_apply(int nc, size_t S, int chun
             const T* r = u + (size_t)j * nc + I;
             CoarseRow<T> v;
             v.o = r[0];
-            v.w = I > 0 ? r[-1] : -v.o;
-            v.e = I < nc - 1 ? r[1] : -v.o;
+            v.w = I > 0 ? r[-1] : flip_if(true, v.o);
+            v.e = I < nc - 1 ? r[1] : flip_if(true, v.o);
             return v;
         };
         const CoarseRow<T> own = coarse(J);
@@ -1135,7 +1153,8 @@ __global__ void __launch_bounds__(kTailThreads) k_vcycle_tail(TailArgs<T> a) {
     }
     __syncthreads();
     // Red-black sweeps on grid j: thread -> column pair xh of rows y0, y0 + ry, ...
-    auto sweeps = [&](int j, int nsw) {
+    // (zero: from a zero iterate, which the first red half-sweep need not read).
+    auto sweeps = [&](int j, int nsw, bool zero) {
         const int n = a.n0 << j, hn = n >> 1, ry = nt / hn;
         const int xh = tid % hn, y0 = tid / hn;
         const T* te = arr(j, 0);
@@ -1148,17 +1167,19 @@ __global__ void __launch_bounds__(kTailThreads) k_vcycle_tail(TailArgs<T> a) {
                 for (int y = y0; y < n && y0 < ry; y += ry) {
                     const int x = 2 * xh + ((y + color) & 1), c = y * n + x;
                     T acc = bb[c];
-                    if (x > 0) acc = fma(te[c - 1], pp[c - 1], acc);
-                    if (x < n - 1) acc = fma(te[c], pp[c + 1], acc);
-                    if (y > 0) acc = fma(tn[c - n], pp[c - n], acc);
-                    if (y < n - 1) acc = fma(tn[c], pp[c + n], acc);
+                    if (!(zero && it == 0 && color == 0)) {
+                        if (x > 0) acc = fma(te[c - 1], pp[c - 1], acc);
+                        if (x < n - 1) acc = fma(te[c], pp[c + 1], acc);
+                        if (y > 0) acc = fma(tn[c - n], pp[c - n], acc);
+                        if (y < n - 1) acc = fma(tn[c], pp[c + n], acc);
+                    }
                     pp[c] = acc * rd[c];
                 }
                 __syncthreads();
             }
     };
     for (int j = a.kt; j >= 1; --j) {
-        sweeps(j, a.nu1);
+        sweeps(j, a.nu1, true);
         const int nf = a.n0 << j, nc = nf / 2, rc = nt / nc;
         const int I = tid % nc, J0 = tid / nc;
         const T* te = arr(j, 0);
@@ -1169,13 +1190,7 @@ __global__ void __launch_bounds__(kTailThreads) k_vcycle_tail(TailArgs<T> a) {
         T* bc = arr(j - 1, 4);
         T* pc = arr(j - 1, 5);
         for (int J = J0; J < nc && J0 < rc; J += rc) {
-            const int i0 = 2 * I, j0 = 2 * J;
-            const size_t c00 = (size_t)j0 * nf + i0;
-            const T r00 = residual_at(nf, c00, i0, j0, bf, te, tn, dd, pf);
-            const T r10 = residual_at(nf, c00 + 1, i0 + 1, j0, bf, te, tn, dd, pf);
-            const T r01 = residual_at(nf, c00 + nf, i0, j0 + 1, bf, te, tn, dd, pf);
-            const T r11 = residual_at(nf, c00 + nf + 1, i0 + 1, j0 + 1, bf, te, tn, dd, pf);
-            bc[J * nc + I] = r00 + r10 + r01 + r11;
+            bc[J * nc + I] = restricted_at(nf, (size_t)(2 * J) * nf + 2 * I, I, J, bf, te, tn, dd, pf, a.nu1 > 0);
             pc[J * nc + I] = T(0);
         }
         __syncthreads();
@@ -1188,13 +1203,19 @@ __global__ void __launch_bounds__(kTailThreads) k_vcycle_tail(TailArgs<T> a) {
     }
     __syncthreads();
     for (int j = 1; j <= a.kt; ++j) {
-        const int nf = a.n0 << j, nc = nf / 2, rf = nt / nf;
-        const int i = tid % nf, y0 = tid / nf;
+        // black cells (column pairs as in the sweeps), which post-smoothing starts
+        // from; the red ones too where there is none
+        const int nf = a.n0 << j, nc = nf / 2, ry = nt / nc;
+        const int xh = tid % nc, y0 = tid / nc;
         const T* pc = arr(j - 1, 5);
         T* pf = arr(j, 5);
-        for (int y = y0; y < nf && y0 < rf; y += rf) pf[y * nf + i] = pf[y * nf + i] + prolong_err(nc, pc, i, y, a.ns);
+        for (int color = 1; color >= (a.nu2 > 0 ? 1 : 0); --color)
+            for (int y = y0; y < nf && y0 < ry; y += ry) {
+                const int x = 2 * xh + ((y + color) & 1);
+                pf[y * nf + x] = pf[y * nf + x] + prolong_err(nc, pc, x, y, a.ns);
+            }
         __syncthreads();
-        sweeps(j, a.nu2);
+        sweeps(j, a.nu2, false);
     }
     const int c = m0 << (2 * a.kt);
     const T* pt = arr(a.kt, 5);
@@ -1639,7 +1660,7 @@ static void vcycles(const Hierarchy<T>& H, int k, int top, const fm_solve_params
         T* cur = smooth_with<T>(ctx, tile, threads, n, S, prm.nu1, g.b, Te, Tn, D, rD, g.p, g.p2, active, st, nullptr, ns);
         FM_TIMED(ctx, kFamResidualRestrict, st, 5.5 * ts * cells, 10.0 * cells,
                  k_residual_restrict<T><<<blocks_for(S * (size_t)c.n * c.n), kBlock, 0, st>>>(
-                     c.n, S, g.b, Te, Tn, D, cur, c.b, c.p, active));
+                     c.n, S, g.b, Te, Tn, D, cur, c.b, c.p, active, prm.nu1 > 0));
         below();
         if (prm.energy_step) {
             // the stepped correction (converged mode: partial sums in the hierarchy)

@@ -28,6 +28,7 @@
 
 #include "common.cuh"
 #include "fmg_resident.cuh"
+#include "fmg_strip.cuh"
 
 namespace fm {
 
@@ -338,16 +339,22 @@ static __device__ __forceinline__ T resident_residual(const RGrid<T>& g, int c, 
     return rhs_at(g, c, i, j, d) - v;
 }
 
-static __device__ __forceinline__ void resident_restrict(const RGrid<T>& f, const RGrid<T>& cg, const Ghost<T>& d) {
+// smoothed: after a sweep (FP64: the red residuals only, kRedOnly).
+static __device__ __forceinline__ void resident_restrict(const RGrid<T>& f, const RGrid<T>& cg, const Ghost<T>& d,
+                                                         bool smoothed) {
     const int nc = cg.n, nf = f.n;
     for (int C = rank(); C < nc * nc; C += size()) {
         const int I = C & (nc - 1), J = C >> cg.lg, i0 = 2 * I, j0 = 2 * J, c0 = j0 * nf + i0;
         const T r00 = resident_residual(f, c0, i0, j0, d);
+        cg.p[C] = T(0);
+        if (kRedOnly<T> && smoothed) {
+            cg.b[C] = r00 + resident_residual(f, c0 + nf + 1, i0 + 1, j0 + 1, d);
+            continue;
+        }
         const T r10 = resident_residual(f, c0 + 1, i0 + 1, j0, d);
         const T r01 = resident_residual(f, c0 + nf, i0, j0 + 1, d);
         const T r11 = resident_residual(f, c0 + nf + 1, i0 + 1, j0 + 1, d);
         cg.b[C] = r00 + r10 + r01 + r11;
-        cg.p[C] = T(0);
     }
     sync();
 }
@@ -397,7 +404,7 @@ static __device__ __forceinline__ void resident_prolong(const U* uc, int nc, U* 
 static __device__ void resident_vcycle(const RLayout<T>& L, int k, int nu1, int nu2, const Ghost<T>& d) {
     for (int l = k; l >= 1; --l) {
         for (int s = 0; s < nu1; ++s) resident_rbgs(L.g[l], d);
-        resident_restrict(L.g[l], L.g[l - 1], d);
+        resident_restrict(L.g[l], L.g[l - 1], d, nu1 > 0);
     }
     resident_coarse_solve(L.g[0], L.ainv, d);
     const Ghost<T> zero{T(0), T(0), T(0), T(0), d.ns};

@@ -91,6 +91,14 @@ __device__ __forceinline__ double geometric_mean4(double a, double b, double c, 
     return exp(0.25 * (log(a) + log(b) + log(c) + log(d)));
 }
 
+// -x where flip, by the sign bit (a negation is an addition of the FP64 pipe).
+__device__ __forceinline__ float flip_if(bool flip, float x) {
+    return __uint_as_float(__float_as_uint(x) ^ (flip ? 0x80000000u : 0u));
+}
+__device__ __forceinline__ double flip_if(bool flip, double x) {
+    return __hiloint2double((int)((unsigned)__double2hiint(x) ^ (flip ? 0x80000000u : 0u)), __double2loint(x));
+}
+
 // The bilinear cell-centred prolongation (9, 3, 3, 1) / 16 of four coarse
 // values: own cell, its x neighbour, its y neighbour, the diagonal one.  The
 // roundings are spelled out, so every kernel that prolongs rounds the same
@@ -99,6 +107,14 @@ template <typename U>
 __device__ __forceinline__ U prolong_vals(U own, U nx, U ny, U nxy) {
     return mul_rn(add_rn(fma(U(3), ny, fma(U(9), own, mul_rn(U(3), nx))), nxy), U(0.0625));
 }
+
+// Restriction after red-black sweeps in FP64: a sweep ends on black, whose cells
+// then satisfy their equations to rounding, so their residuals are taken as zero
+// and half the residuals, three FP64 operations a cell, are never formed.  (In
+// FP32 the rounding is not far below what the correction still has to resolve,
+// and the pipe is not the bound: all four.)
+template <typename T>
+constexpr bool kRedOnly = sizeof(T) == 8;
 
 // One smoothing call of the strip shape on grid n x n: hs half-sweeps
 // (red first) on p_in -> p_out.

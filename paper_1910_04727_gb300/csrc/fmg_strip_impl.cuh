@@ -241,17 +241,17 @@ __global__ void __launch_bounds__(32 * kStripMaxWarps, (strip_min_blocks<T, HS, 
     // Dirichlet edges; past the south / north edge the edge row itself across a
     // no-flow edge, its negative across a Dirichlet one (ns)
     T cm[3] = {T(0), T(0), T(0)}, c0[3] = {T(0), T(0), T(0)}, cp[3] = {T(0), T(0), T(0)};
-    const T sg = a.ns ? T(-1) : T(1);
+    const bool sg = a.ns != 0;
     auto coarse3 = [&](T own, T lf, T rt, T (&dst)[3]) {
         dst[0] = own;
-        dst[1] = I == 0 ? -own : lf;
-        dst[2] = I == nc - 1 ? -own : rt;
+        dst[1] = I == 0 ? flip_if(true, own) : lf;
+        dst[2] = I == nc - 1 ? flip_if(true, own) : rt;
     };
     if (EC && in_x) {   // coarse rows ys / 2 - 1 and ys / 2 around fine row ys
         const T* crow = ecs + (size_t)(ys / 2) * nc;
         coarse3(crow[0], I > 0 ? crow[-1] : T(0), I + 1 < nc ? crow[1] : T(0), c0);
 #pragma unroll
-        for (int q = 0; q < 3; ++q) cm[q] = sg * c0[q];
+        for (int q = 0; q < 3; ++q) cm[q] = flip_if(sg, c0[q]);
         if (ys > 0) {
             crow -= nc;
             coarse3(crow[0], I > 0 ? crow[-1] : T(0), I + 1 < nc ? crow[1] : T(0), cm);
@@ -346,15 +346,15 @@ __global__ void __launch_bounds__(32 * kStripMaxWarps, (strip_min_blocks<T, HS, 
                         __syncwarp();   // every lane has read the slot before it is refilled
                         if (y == n - 1) {
 #pragma unroll
-                            for (int q = 0; q < 3; ++q) cp[q] = sg * c0[q];
+                            for (int q = 0; q < 3; ++q) cp[q] = flip_if(sg, c0[q]);
                         }
                     }
                     // fine row y: coarse row y / 2 and its y neighbour, one row down for
-                    // even y, one up for odd y
+                    // even y, one up for odd y.  Black cells only: the first half-sweep
+                    // replaces the red ones from their black neighbours.
                     if (in_x && y < ye) {
-                        const T* const u = (J & 1) ? cp : cm;
-                        a0 = add_rn(a0, prolong_vals(c0[0], c0[1], u[0], u[1]));
-                        a1 = add_rn(a1, prolong_vals(c0[0], c0[2], u[0], u[2]));
+                        if (J & 1) a0 = add_rn(a0, prolong_vals(c0[0], c0[1], cp[0], cp[1]));
+                        else a1 = add_rn(a1, prolong_vals(c0[0], c0[2], cm[0], cm[2]));
                     }
                     if (J & 1) {
 #pragma unroll
@@ -420,24 +420,30 @@ __global__ void __launch_bounds__(32 * kStripMaxWarps, (strip_min_blocks<T, HS, 
                 const int c = (J - HS - 1 + 4 * R) % R, hi = (J - HS + 4 * R) % R;
                 if (out_x && q >= oy && q < oye) {
                     const V2 dq = sm.dring[(J + 1 < R ? (half ^ 1) * R : half * R) + (J + 1) % R][lane];
-                    T v0 = mul_rn(dq.x, p[c][0]);
-                    v0 = fma(-wl[c], qw, v0);
-                    v0 = fma(-ee[c][0], p[c][1], v0);
-                    v0 = fma(-nq[0], pq[0], v0);
-                    v0 = fma(-nf[c][0], p[hi][0], v0);
-                    const T r0 = bb[c][0] - v0;
-                    T v1 = mul_rn(dq.y, p[c][1]);
-                    v1 = fma(-ee[c][0], p[c][0], v1);
-                    v1 = fma(-ee[c][1], qe, v1);
-                    v1 = fma(-nq[1], pq[1], v1);
-                    v1 = fma(-nf[c][1], p[hi][1], v1);
-                    const T r1 = bb[c][1] - v1;
+                    // FP64: red cells only, a row's left one on even q (kRedOnly)
+                    T r0 = T(0), r1 = T(0);
+                    if (!kRedOnly<T> || (J & 1)) {
+                        T v0 = mul_rn(dq.x, p[c][0]);
+                        v0 = fma(-wl[c], qw, v0);
+                        v0 = fma(-ee[c][0], p[c][1], v0);
+                        v0 = fma(-nq[0], pq[0], v0);
+                        v0 = fma(-nf[c][0], p[hi][0], v0);
+                        r0 = bb[c][0] - v0;
+                    }
+                    if (!kRedOnly<T> || !(J & 1)) {
+                        T v1 = mul_rn(dq.y, p[c][1]);
+                        v1 = fma(-ee[c][0], p[c][0], v1);
+                        v1 = fma(-ee[c][1], qe, v1);
+                        v1 = fma(-nq[1], pq[1], v1);
+                        v1 = fma(-nf[c][1], p[hi][1], v1);
+                        r1 = bb[c][1] - v1;
+                    }
                     if ((J & 1) == 0) {   // q odd: the coarse cell's upper row
                         const size_t cc = s * (size_t)nc * nc + (size_t)(q / 2) * nc + I;
-                        a.bc[cc] = rsum + r0 + r1;
+                        a.bc[cc] = kRedOnly<T> ? rsum + r1 : rsum + r0 + r1;
                         if (a.pc) a.pc[cc] = T(0);
                     } else {
-                        rsum = r0 + r1;
+                        rsum = kRedOnly<T> ? r0 : r0 + r1;
                     }
                 }
             }
