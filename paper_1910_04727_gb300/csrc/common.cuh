@@ -131,9 +131,9 @@ struct Ghost {
 // 0.72 / 0.49 at 152, 0.88 / 0.96 at 200.  Converged: 16 x 16 4.95 / 4.20 at
 // 5000, 14.2 / 14.9 at 20000; 32 x 32 8.7 / 7.5 at 2432, 14.1 / 15.0 at 5000;
 // 64 x 64 13.4 / 12.4 at 608, 16.1 / 16.4 at 912.
-// Mixed: resident up to 32 x 32 (16 x 16 7.5 / 5.3 at 20000; 32 x 32 level
-// within 5%: 6.7 / 6.3 at 5000, 16.3 / 17.1 at 15000), and a converged 64 x 64
-// batch of at most two samples per SM (3.0 / 2.4 at 304, 3.2 / 3.5 at 380).
+// Mixed: resident up to 32 x 32 (grids in registers: 16 x 16 2.2 / 0.27 at 4000,
+// 12.2 / 2.2 at 40000; 32 x 32 2.8 / 0.47 at 1000, 8.6 / 2.5 at 8000), and a converged
+// 64 x 64 batch of at most two samples per SM (2.8 / 2.4 at 300).
 inline bool auto_resident(int n_fine, size_t S, int sms, const fm_solve_params& prm) {
     if (prm.energy_step) return false;
     if (prm.precision == FM_PREC_MIXED)

@@ -21,7 +21,10 @@
 // Mixed form (T = float): the grids of the two refined stages (n_fine/2 and
 // n_fine, which give Q^c and Q^f) also hold FP64 p, te, tn, tw; the FP64
 // residual of the stage problem is the right-hand side of an FP32 V-cycle
-// for the correction, which is added to the FP64 iterate.
+// for the correction, which is added to the FP64 iterate.  Hierarchies from 4 x 4 to
+// 16 x 16 and 32 x 32 take the same arithmetic with their grids in registers
+// (fmg_warp16.cu, fmg_team32.cu); this form then runs the samples that met an
+// infinity or a NaN there.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -556,6 +559,7 @@ __global__ void __launch_bounds__(512, 1) k_fmg_resident(ResidentArgs a) {
     const int m = L.m;
     const size_t stride = (size_t)gridDim.x * groups;
     for (size_t s = (size_t)blockIdx.x * groups + grp; s < a.S; s += stride) {
+        if (a.again && __double_as_longlong(a.qf[s]) != kAgain) continue;
         const double* Kf = a.K + s * (size_t)a.n_fine * a.n_fine;
         for (int k = 0; k <= m; ++k) {
             const HGrid* h = (MIXED && k >= m - 1) ? &L.h[k - (m - 1)] : nullptr;
@@ -712,6 +716,12 @@ static bool launch_resident(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st)
     const int pi = prof_start(ctx, kFamResidentFmg, st);
     ResidentArgs b = a;
     b.flops = prof_counter(ctx, pi);
+    if (MIXED && a.converged && a.n0 == 4 && (a.n_fine == 16 || a.n_fine == 32)) {
+        // grids in registers; then, here, the samples that met an infinity or a NaN
+        if (a.n_fine == 16) launch_warp16(ctx, b, st);
+        else launch_team32(ctx, b, st);
+        b.again = true;
+    }
     k_fmg_resident<T, MIXED, WARP><<<(unsigned)grid, threads, smem, st>>>(b);
     prof_stop(ctx, pi, st, 8.0 * cells + 16.0 * a.S, 0.0);
     return true;
@@ -757,11 +767,9 @@ bool fmg_resident_launch(fm_ctx* ctx, int n_fine, int n0, size_t S, const double
     a.qc = qc;
     a.p_out = p_out;
     a.status = status;
+    a.again = false;
     a.flops = nullptr;
-    if (prm.precision == FM_PREC_MIXED) {
-        if (n_fine == 16 && n0 == 4 && prm.converged) return launch_warp16(ctx, a, st);   // 4, 8, 16: in registers
-        return launch_resident<float, true>(ctx, a, st);
-    }
+    if (prm.precision == FM_PREC_MIXED) return launch_resident<float, true>(ctx, a, st);
     return launch_resident<double, false>(ctx, a, st);
 }
 

@@ -5,6 +5,10 @@
 
 namespace fm {
 
+// A sample whose V-cycles left the finite numbers: its QoI until a second launch has
+// solved it again by the shared-memory form (a payload no arithmetic makes).
+constexpr long long kAgain = 0x7ff8000057313641ll;
+
 struct ResidentArgs {
     int n_fine, n0;
     size_t S;
@@ -16,6 +20,7 @@ struct ResidentArgs {
     double tol, qtol;
     double *qf, *qc, *p_out;
     int32_t* status;
+    bool again;      // only the samples whose qf is kAgain
     double* flops;   // nullable (profiling): [0] solver flops, [1] their FP64 part, [2] model bytes
 };
 
@@ -45,7 +50,10 @@ __device__ __forceinline__ double vcycle_bytes(int n0, int k, int nu1, int nu2, 
     return b;
 }
 
-// The 16 x 16 mixed form, one sample per warp in registers (fmg_warp16.cu).
-bool launch_warp16(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st);
+// The converged mixed form with grids in registers: 16 x 16, one sample per warp
+// (fmg_warp16.cu), and 32 x 32, one per five warps (fmg_team32.cu), coarsest grid
+// 4 x 4.  Samples that leave the finite numbers come back as kAgain in qf.
+void launch_warp16(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st);
+void launch_team32(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st);
 
 }  // namespace fm

@@ -22,845 +22,61 @@
 #include <cmath>
 #include <mutex>
 
-#include "fmg_resident.cuh"
-#include "fmg_strip.cuh"
+#include "fmg_warp.cuh"
 
 namespace fm {
 
-namespace {
-
 constexpr int kW16Warps = 4;
-constexpr unsigned kAll = 0xffffffffu;
-
-// FP32 faces of an n x n operator: east and north of each cell, west of each row,
-// south of each column.
-struct FacesF {
-    float te[256], tn[256], tw[16], ts[16];
-};
-
-// FP64 faces likewise, diagonal and iterate of the refined grid (16 x 16, or 8 x 8
-// with a pitch of 8), and the rhs of its stage problem on the edges.
-struct W16Smem {
-    double p[256], d[256], te[256], tn[256];
-    double tw[16], ts[16];
-    double f[4][16];         // west, east column, south, north row
-    double c[64];            // scratch of the interpolation, and of the coefficients
-    union {
-        FacesF faces;
-        float r[256];        // residual, then correction, of the refined grid
-    };
-    float df[8][32];         // FP32 diagonal of the 16 x 16 grid, by lane
-    float ainv[16][20];      // inverse of the coarsest operator, row-major
-    float rhs[16];           // coarsest rhs
-};
-
-__device__ __forceinline__ float up1(float v) { return __shfl_up_sync(kAll, v, 1); }
-__device__ __forceinline__ float dn1(float v) { return __shfl_down_sync(kAll, v, 1); }
-
-// The sides on which a lane's cells have neighbours.
-struct Inner {
-    bool w, e, s, n;
-};
-
-// acc + f p where the neighbour exists.  Where it does not, f is zero and p another
-// cell's value, which changes nothing while that is finite; a sample that meets
-// an infinity or a NaN runs again with SAFE, the terms left out (seven predicates
-// for eight sides: selecting in every sweep cost a tenth of the time).
-template <bool SAFE>
-__device__ __forceinline__ float add_if(bool in, float f, float p, float acc) {
-    return !SAFE || in ? fmaf(f, p, acc) : acc;
-}
-
-// The 16 x 16 grid: faces, 1 / D, rhs, iterate.
-struct G16 {
-    float w[4], ei[4], ee[4];   // west face of column 0, face between the columns, east face of column 1
-    float sf[2], nf[4][2];      // south faces of row 0, north faces of every cell
-    float rd[4][2], b[4][2], p[4][2];
-};
-
-// The 8 x 8 grid, a 2 x 2 block per lane.
-struct G8 {
-    float w[2], ei[2], ee[2], sf[2], ni[2], nn[2];
-    float rd[2][2], d[2][2], b[2][2], p[2][2];
-};
-
-template <bool SAFE, int C>
-__device__ __forceinline__ void half_sweep16(G16& g, const Inner& in) {
-    float nb[4];
-#pragma unroll
-    for (int y = 0; y < 4; ++y) nb[y] = ((y + C) & 1) == 0 ? up1(g.p[y][1]) : dn1(g.p[y][0]);
-    const float lo = __shfl_up_sync(kAll, g.p[3][C & 1], 8), hi = __shfl_down_sync(kAll, g.p[0][(3 + C) & 1], 8);
-#pragma unroll
-    for (int y = 0; y < 4; ++y) {
-        const int x = (y + C) & 1;
-        float acc = g.b[y][x];
-        acc = x == 0 ? add_if<SAFE>(in.w, g.w[y], nb[y], acc) : fmaf(g.ei[y], g.p[y][0], acc);
-        acc = x == 0 ? fmaf(g.ei[y], g.p[y][1], acc) : add_if<SAFE>(in.e, g.ee[y], nb[y], acc);
-        acc = y == 0 ? add_if<SAFE>(in.s, g.sf[x], lo, acc) : fmaf(g.nf[y > 0 ? y - 1 : 0][x], g.p[y > 0 ? y - 1 : 0][x], acc);
-        acc = y == 3 ? add_if<SAFE>(in.n, g.nf[3][x], hi, acc) : fmaf(g.nf[y][x], g.p[y < 3 ? y + 1 : 3][x], acc);
-        g.p[y][x] = __fmul_rn(acc, g.rd[y][x]);
-    }
-}
-
-template <bool SAFE>
-__device__ __forceinline__ void sweeps16(G16& g, const Inner& in, int n) {
-#pragma unroll 1
-    for (int s = 0; s < n; ++s) {
-        half_sweep16<SAFE, 0>(g, in);
-        half_sweep16<SAFE, 1>(g, in);
-    }
-}
-
-// The north and south neighbours of a block are the lanes four up and down.
-__device__ __forceinline__ float lf(float v) { return __shfl_up_sync(kAll, v, 1, 16); }
-__device__ __forceinline__ float rt(float v) { return __shfl_down_sync(kAll, v, 1, 16); }
-__device__ __forceinline__ float be(float v) { return __shfl_up_sync(kAll, v, 4, 16); }
-__device__ __forceinline__ float ab(float v) { return __shfl_down_sync(kAll, v, 4, 16); }
-
-template <bool SAFE>
-__device__ __forceinline__ void sweeps8(G8& g, const Inner& in, int n) {
-#pragma unroll 1
-    for (int s = 0; s < n; ++s) {
-        {   // colour 0: cells (0, 0) and (1, 1) of the block
-            const float W = lf(g.p[0][1]), S = be(g.p[1][0]), E = rt(g.p[1][0]), N = ab(g.p[0][1]);
-            float a = add_if<SAFE>(in.w, g.w[0], W, g.b[0][0]), c = fmaf(g.ei[1], g.p[1][0], g.b[1][1]);
-            a = fmaf(g.ei[0], g.p[0][1], a);
-            c = add_if<SAFE>(in.e, g.ee[1], E, c);
-            a = add_if<SAFE>(in.s, g.sf[0], S, a);
-            c = fmaf(g.ni[1], g.p[0][1], c);
-            a = fmaf(g.ni[0], g.p[1][0], a);
-            c = add_if<SAFE>(in.n, g.nn[1], N, c);
-            g.p[0][0] = __fmul_rn(a, g.rd[0][0]);
-            g.p[1][1] = __fmul_rn(c, g.rd[1][1]);
-        }
-        {   // colour 1: cells (0, 1) and (1, 0)  ([row][column])
-            const float E = rt(g.p[0][0]), S = be(g.p[1][1]), W = lf(g.p[1][1]), N = ab(g.p[0][0]);
-            float a = fmaf(g.ei[0], g.p[0][0], g.b[0][1]), c = add_if<SAFE>(in.w, g.w[1], W, g.b[1][0]);
-            a = add_if<SAFE>(in.e, g.ee[0], E, a);
-            c = fmaf(g.ei[1], g.p[1][1], c);
-            a = add_if<SAFE>(in.s, g.sf[1], S, a);
-            c = fmaf(g.ni[0], g.p[0][0], c);
-            a = fmaf(g.ni[1], g.p[1][1], a);
-            c = add_if<SAFE>(in.n, g.nn[0], N, c);
-            g.p[0][1] = __fmul_rn(a, g.rd[0][1]);
-            g.p[1][0] = __fmul_rn(c, g.rd[1][0]);
-        }
-    }
-}
-
-// b - A p at column X of a lane's pair (the first product of the sum differs: in
-// column 1 the west term is always there).
-template <bool SAFE, int X>
-__device__ __forceinline__ float residual(float d, float p, float b, bool w, float tw, float pw, bool e, float te,
-                                          float pe, bool s, float ts, float ps, bool n, float tn, float pn) {
-    float v = X == 0 ? add_if<SAFE>(w, -tw, pw, __fmul_rn(d, p)) : fmaf(d, p, -__fmul_rn(tw, pw));
-    v = add_if<SAFE>(e, -te, pe, v);
-    v = add_if<SAFE>(s, -ts, ps, v);
-    v = add_if<SAFE>(n, -tn, pn, v);
-    return __fsub_rn(b, v);
-}
-
-// Residual of the 16 x 16 grid restricted to the 8 x 8 rhs, zero iterate there.
-template <bool SAFE>
-__device__ __forceinline__ void restrict16(const G16& g, G8& c, const Inner& in, const W16Smem& sm, int lane) {
-    float W[4], E[4], S[2], N[2];
-#pragma unroll
-    for (int y = 0; y < 4; ++y) {
-        W[y] = up1(g.p[y][1]);
-        E[y] = dn1(g.p[y][0]);
-    }
-#pragma unroll
-    for (int x = 0; x < 2; ++x) {
-        S[x] = __shfl_up_sync(kAll, g.p[3][x], 8);
-        N[x] = __shfl_down_sync(kAll, g.p[0][x], 8);
-    }
-    float sum[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        float r[2][2];
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int y = 2 * h + q, ys = y > 0 ? y - 1 : 0, yn = y < 3 ? y + 1 : 3;
-            const bool s = y > 0 || in.s, n = y < 3 || in.n;
-            r[q][0] = residual<SAFE, 0>(sm.df[2 * y][lane], g.p[y][0], g.b[y][0], in.w, g.w[y], W[y], true, g.ei[y],
-                                  g.p[y][1], s, y == 0 ? g.sf[0] : g.nf[ys][0], y == 0 ? S[0] : g.p[ys][0], n,
-                                  g.nf[y][0], y == 3 ? N[0] : g.p[yn][0]);
-            r[q][1] = residual<SAFE, 1>(sm.df[2 * y + 1][lane], g.p[y][1], g.b[y][1], true, g.ei[y], g.p[y][0], in.e,
-                                  g.ee[y], E[y], s, y == 0 ? g.sf[1] : g.nf[ys][1], y == 0 ? S[1] : g.p[ys][1], n,
-                                  g.nf[y][1], y == 3 ? N[1] : g.p[yn][1]);
-        }
-        sum[h] = r[0][0] + r[0][1] + r[1][0] + r[1][1];
-    }
-    // coarse column l mod 8, rows 2 (l / 8) + h  ->  blocks
-    const int src = ((lane & 15) >> 2) * 8 + 2 * (lane & 3);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        c.b[h][0] = __shfl_sync(kAll, sum[h], src);
-        c.b[h][1] = __shfl_sync(kAll, sum[h], src + 1);
-        c.p[h][0] = c.p[h][1] = 0.0f;
-    }
-}
-
-// p (+)= P u: 2 x 2 values at the lane's coarse cell from the coarse value of
-// every block lane (coarse grid 4 x 4).
-__device__ __forceinline__ void prolong8(float u, G8& g, const Ghost<float>& gh, bool add, int lane) {
-    const int I = lane & 3, J = (lane >> 2) & 3;
-    float L = lf(u), R = rt(u);
-    if (I == 0) L = fmaf(2.0f, gh.w, -u);
-    if (I == 3) R = fmaf(2.0f, gh.e, -u);
-    float s[3] = {be(L), be(u), be(R)}, n[3] = {ab(L), ab(u), ab(R)};   // the edge rows keep their own
-    if (gh.ns) {
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            if (J == 0) s[q] = fmaf(2.0f, gh.s, -s[q]);
-            if (J == 3) n[q] = fmaf(2.0f, gh.n, -n[q]);
-        }
-    }
-    const float v00 = prolong_vals(u, L, s[1], s[0]), v01 = prolong_vals(u, R, s[1], s[2]);
-    const float v10 = prolong_vals(u, L, n[1], n[0]), v11 = prolong_vals(u, R, n[1], n[2]);
-    g.p[0][0] = add ? __fadd_rn(g.p[0][0], v00) : v00;
-    g.p[0][1] = add ? __fadd_rn(g.p[0][1], v01) : v01;
-    g.p[1][0] = add ? __fadd_rn(g.p[1][0], v10) : v10;
-    g.p[1][1] = add ? __fadd_rn(g.p[1][1], v11) : v11;
-}
-
-// The same from the 8 x 8 grid (blocks) to the 16 x 16 grid.
-__device__ __forceinline__ void prolong16(const G8& c, G16& g, const Ghost<float>& gh, bool add, int lane) {
-    const int I = lane & 7, ry = lane >> 3, src = ry * 4 + (I >> 1);
-    // the lane's coarse column at rows 2 ry - 1 .. 2 ry + 2: [1], [2] own, then its neighbours
-    float o[4], l[4], r[4];
-    {
-        const float a0 = __shfl_sync(kAll, c.p[0][0], src), a1 = __shfl_sync(kAll, c.p[0][1], src);
-        const float b0 = __shfl_sync(kAll, c.p[1][0], src), b1 = __shfl_sync(kAll, c.p[1][1], src);
-        o[1] = (I & 1) ? a1 : a0;
-        o[2] = (I & 1) ? b1 : b0;
-    }
-#pragma unroll
-    for (int q = 1; q < 3; ++q) {
-        l[q] = up1(o[q]);
-        r[q] = dn1(o[q]);
-        if (I == 0) l[q] = fmaf(2.0f, gh.w, -o[q]);
-        if (I == 7) r[q] = fmaf(2.0f, gh.e, -o[q]);
-    }
-    auto rows = [&](float (&v)[4]) {   // rows of the lanes below and above; past the edges the edge row's ghost
-        v[0] = __shfl_up_sync(kAll, v[2], 8);
-        v[3] = __shfl_down_sync(kAll, v[1], 8);
-        if (ry == 0) v[0] = gh.ns ? fmaf(2.0f, gh.s, -v[1]) : v[1];
-        if (ry == 3) v[3] = gh.ns ? fmaf(2.0f, gh.n, -v[2]) : v[2];
-    };
-    rows(o);
-    rows(l);
-    rows(r);
-#pragma unroll
-    for (int y = 0; y < 4; ++y) {
-        const int J = 1 + (y >> 1), K = (y & 1) ? J + 1 : J - 1;
-        const float v0 = prolong_vals(o[J], l[J], o[K], l[K]), v1 = prolong_vals(o[J], r[J], o[K], r[K]);
-        g.p[y][0] = add ? __fadd_rn(g.p[y][0], v0) : v0;
-        g.p[y][1] = add ? __fadd_rn(g.p[y][1], v1) : v1;
-    }
-}
-
-// The 8 x 8 iterate to FP64, in shared memory.
-__device__ __forceinline__ void store8(const G8& g, W16Smem& sm, int lane) {
-    if (lane >= 16) return;
-#pragma unroll
-    for (int y = 0; y < 2; ++y)
-#pragma unroll
-        for (int x = 0; x < 2; ++x) sm.p[8 * (2 * (lane >> 2) + y) + 2 * (lane & 3) + x] = widen(g.p[y][x]);
-}
-
-// Coarsest solve of the block lanes' right-hand sides: A^-1 b, row (l mod 16).
-__device__ __forceinline__ float coarse_solve(float b, W16Smem& sm, int lane) {
-    if (lane < 16) sm.rhs[lane] = b;
-    __syncwarp();
-    float acc = 0.0f;
-    const float* row = sm.ainv[lane & 15];
-#pragma unroll
-    for (int c = 0; c < 16; c += 4) {
-        const float4 a = *reinterpret_cast<const float4*>(row + c);
-        const float4 v = *reinterpret_cast<const float4*>(sm.rhs + c);
-        acc = fmaf(a.x, v.x, acc);
-        acc = fmaf(a.y, v.y, acc);
-        acc = fmaf(a.z, v.z, acc);
-        acc = fmaf(a.w, v.w, acc);
-    }
-    __syncwarp();
-    return acc;
-}
-
-// Correction of the 8 x 8 grid from the 4 x 4 grid: residual, exact solve, prolongation.
-template <bool SAFE>
-__device__ __forceinline__ void coarse_correction(G8& g, const Inner& in, W16Smem& sm, const Ghost<float>& zero,
-                                                  int lane) {
-    const float W0 = lf(g.p[0][1]), W1 = lf(g.p[1][1]), E0 = rt(g.p[0][0]), E1 = rt(g.p[1][0]);
-    const float S0 = be(g.p[1][0]), S1 = be(g.p[1][1]), N0 = ab(g.p[0][0]), N1 = ab(g.p[0][1]);
-    const float r00 = residual<SAFE, 0>(g.d[0][0], g.p[0][0], g.b[0][0], in.w, g.w[0], W0, true, g.ei[0], g.p[0][1],
-                                        in.s, g.sf[0], S0, true, g.ni[0], g.p[1][0]);
-    const float r10 = residual<SAFE, 1>(g.d[0][1], g.p[0][1], g.b[0][1], true, g.ei[0], g.p[0][0], in.e, g.ee[0], E0,
-                                        in.s, g.sf[1], S1, true, g.ni[1], g.p[1][1]);
-    const float r01 = residual<SAFE, 0>(g.d[1][0], g.p[1][0], g.b[1][0], in.w, g.w[1], W1, true, g.ei[1], g.p[1][1],
-                                        true, g.ni[0], g.p[0][0], in.n, g.nn[0], N0);
-    const float r11 = residual<SAFE, 1>(g.d[1][1], g.p[1][1], g.b[1][1], true, g.ei[1], g.p[1][0], in.e, g.ee[1], E1,
-                                        true, g.ni[1], g.p[0][1], in.n, g.nn[1], N1);
-    prolong8(coarse_solve(r00 + r10 + r01 + r11, sm, lane), g, zero, true, lane);
-}
-
-// One V-cycle on the 16 x 16 grid (fine) or the 8 x 8 grid.  Loops of two passes
-// (smoothing, then the correction and smoothing) hold one copy of each piece, as
-// everywhere below: with the pieces inlined where they are used the code took
-// 340 KB, and two issue slots of three waited for instructions.
-template <bool SAFE>
-__device__ __forceinline__ void vcycle(bool fine, G16& g, G8& c, const Inner& in, const Inner& in8, W16Smem& sm,
-                                       int nu1, int nu2, const Ghost<float>& zero, int lane) {
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-        if (h) {
-            if (fine) restrict16<SAFE>(g, c, in, sm, lane);
-#pragma unroll 1
-            for (int q = 0; q < 2; ++q) {
-                if (q) coarse_correction<SAFE>(c, in8, sm, zero, lane);
-                sweeps8<SAFE>(c, in8, q ? nu2 : nu1);
-            }
-            if (fine) prolong16(c, g, zero, true, lane);
-        }
-        if (fine) sweeps16<SAFE>(g, in, h ? nu2 : nu1);
-    }
-}
-
-// The 4 x 4 operator of cell coefficients k (block lanes) and its inverse into
-// sm.ainv: Gauss-Jordan on [A | I], lane c < 16 owning column c of A, lane 16 + c
-// column c of the inverse.  Returns the stage problem's Dirichlet data on the rhs.
-__device__ __forceinline__ float coarse_inverse(float k, const Ghost<float>& gh, W16Smem& sm, int lane) {
-    const int c = lane & 15, I = c & 3, J = c >> 2;
-    const float kr = rt(k), ka = ab(k);
-    const float tb = gh.ns ? 2.0f * k : 0.0f;
-    const float te = I < 3 ? harmonic_mean(k, kr) : 2.0f * k;
-    const float tn = J < 3 ? harmonic_mean(k, ka) : tb;
-    const float tel = lf(te), tnb = be(tn);
-    const float tw = I > 0 ? tel : 2.0f * k;
-    const float ts = J > 0 ? tnb : tb;
-    const float d = tw + te + ts + tn;
-    // step q works on row 0 of columns rotated q times: the rotation is in the
-    // destination registers
-    float col[16];
-#pragma unroll
-    for (int r = 0; r < 16; ++r) {
-        float v = 0.0f;
-        if (r == c) v = d;
-        if (r == c - 1 && I > 0) v = -tw;
-        if (r == c + 1 && I < 3) v = -te;
-        if (r == c - 4) v = -ts;
-        if (r == c + 4) v = -tn;
-        col[r] = lane < 16 ? v : (r == c ? 1.0f : 0.0f);
-    }
-#pragma unroll 1
-    for (int q = 0; q < 16; ++q) {
-        const float p = col[0] / __shfl_sync(kAll, col[0], q);
-#pragma unroll
-        for (int r = 1; r < 16; ++r) {
-            const float f = __shfl_sync(kAll, col[r], q);   // column q of A
-            const float v = fmaf(-f, p, col[r]);
-            col[r - 1] = lane == q ? 0.0f : v;
-        }
-        col[15] = p;
-    }
-    __syncwarp();
-    if (lane >= 16) {
-#pragma unroll
-        for (int r = 0; r < 16; ++r) sm.ainv[r][c] = col[r];
-    }
-    __syncwarp();
-    float v = 0.0f;
-    if (I == 0) v = fmaf(tw, gh.w, v);
-    if (I == 3) v = fmaf(te, gh.e, v);
-    if (gh.ns && J == 0) v = fmaf(ts, gh.s, v);
-    if (gh.ns && J == 3) v = fmaf(tn, gh.n, v);
-    return v;
-}
-
-// FP64 faces of the n x n stage grid (n = 2^lg; every (16 / n)-th cell of the field
-// K), its diagonal, and the faces in FP32, in shared memory; a cell's face beyond
-// the edge is 2K, or 0 on a no-flow edge.
-__device__ __forceinline__ void stage_faces(const double* __restrict__ K, int lg, int ns, W16Smem& sm, int lane) {
-    const int n = 1 << lg, s = 16 >> lg, last = n - 1;
-    __syncwarp();
-#pragma unroll 1
-    for (int c = lane; c < n * n; c += 32) {
-        const int i = c & last, j = c >> lg;
-        const double* f = K + 16 * s * j + s * i;
-        const double k = __ldg(f);
-        sm.te[c] = harmonic_mean(k, __ldg(f + (i < last ? s : 0)));
-        sm.tn[c] = harmonic_mean(k, __ldg(f + (j < last ? 16 * s : 0)));
-    }
-    __syncwarp();
-    if (lane < n) {   // the four edges: row / column `lane`
-        const double tw = 2.0 * __ldg(K + 16 * s * lane), ts = ns ? 2.0 * __ldg(K + s * lane) : 0.0;
-        sm.tw[lane] = tw;
-        sm.ts[lane] = ts;
-        sm.te[n * lane + last] = 2.0 * __ldg(K + 16 * s * lane + s * last);
-        sm.tn[n * last + lane] = ns ? 2.0 * __ldg(K + 16 * s * last + s * lane) : 0.0;
-        sm.faces.tw[lane] = narrow(tw);
-        sm.faces.ts[lane] = narrow(ts);
-    }
-    __syncwarp();
-#pragma unroll 1
-    for (int c = lane; c < n * n; c += 32) {
-        const int i = c & last, j = c >> lg;
-        const double te = sm.te[c], tn = sm.tn[c];
-        const double tw = *(i > 0 ? sm.te + c - 1 : sm.tw + j), ts = *(j > 0 ? sm.tn + c - n : sm.ts + i);
-        sm.d[c] = tw + te + ts + tn;
-        sm.faces.te[c] = narrow(te);
-        sm.faces.tn[c] = narrow(tn);
-    }
-    __syncwarp();
-}
-
-// 1 / d: the approximation and a Newton step give the IEEE quotient where both
-// are normal numbers.
-__device__ __forceinline__ float recip(float d) {
-    if (((__float_as_uint(d) >> 23) & 0xffu) - 1u > 251u) return 1.0f / d;
-    float r;
-    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(d));
-    return fmaf(r, fmaf(-d, r, 1.0f), r);
-}
-
-// FP32 operators from their faces in shared memory: 8 x 8 and 16 x 16.
-__device__ __forceinline__ void load8(const FacesF& f, G8& g, int lane) {
-    const int bx = lane & 3, by = (lane >> 2) & 3, c = 16 * by + 2 * bx;
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        const float2 e = *reinterpret_cast<const float2*>(f.te + c + 8 * q);
-        g.ei[q] = e.x;
-        g.ee[q] = bx < 3 ? e.y : 0.0f;
-        g.ni[q] = f.tn[c + q];
-        g.nn[q] = by < 3 ? f.tn[c + 8 + q] : 0.0f;
-        g.w[q] = bx > 0 ? f.te[c + 8 * q - 1] : 0.0f;
-        g.sf[q] = by > 0 ? f.tn[c - 8 + q] : 0.0f;
-    }
-#pragma unroll
-    for (int y = 0; y < 2; ++y)
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-            const int i = 2 * bx + x, j = 2 * by + y, o = c + 8 * y + x;
-            const float w = *(i > 0 ? f.te + o - 1 : f.tw + j), s = *(j > 0 ? f.tn + o - 8 : f.ts + i);
-            g.d[y][x] = w + f.te[o] + s + f.tn[o];
-            g.rd[y][x] = recip(g.d[y][x]);
-        }
-}
-
-__device__ __forceinline__ void load16(const FacesF& f, G16& g, W16Smem& sm, int lane) {
-    const int cx = lane & 7, ry = lane >> 3;
-#pragma unroll
-    for (int y = 0; y < 4; ++y) {
-        const int j = 4 * ry + y, c = 16 * j + 2 * cx;
-        const float2 e = *reinterpret_cast<const float2*>(f.te + c), t = *reinterpret_cast<const float2*>(f.tn + c);
-        const float w = *(cx > 0 ? f.te + c - 1 : f.tw + j);
-        const float2 s = *reinterpret_cast<const float2*>(j > 0 ? f.tn + c - 16 : f.ts + 2 * cx);
-        const float d0 = w + e.x + s.x + t.x, d1 = e.x + e.y + s.y + t.y;
-        sm.df[2 * y][lane] = d0;
-        sm.df[2 * y + 1][lane] = d1;
-        g.rd[y][0] = recip(d0);
-        g.rd[y][1] = recip(d1);
-        // no cells past the edges
-        g.w[y] = cx > 0 ? w : 0.0f;
-        g.ei[y] = e.x;
-        g.ee[y] = cx < 7 ? e.y : 0.0f;
-        g.nf[y][0] = j < 15 ? t.x : 0.0f;
-        g.nf[y][1] = j < 15 ? t.y : 0.0f;
-        if (y == 0) {
-            g.sf[0] = j > 0 ? s.x : 0.0f;
-            g.sf[1] = j > 0 ? s.y : 0.0f;
-        }
-    }
-}
-
-// FP32 rhs of the 8 x 8 stage problem.
-__device__ __forceinline__ void stage_rhs8(const FacesF& f, G8& g, const Ghost<float>& gh, int lane) {
-#pragma unroll
-    for (int y = 0; y < 2; ++y)
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-            const int i = 2 * (lane & 3) + x, j = 2 * ((lane >> 2) & 3) + y;
-            float v = 0.0f;
-            if (i == 0) v = fmaf(f.tw[j], gh.w, v);
-            if (i == 7) v = fmaf(f.te[8 * j + 7], gh.e, v);
-            if (gh.ns && j == 0) v = fmaf(f.ts[i], gh.s, v);
-            if (gh.ns && j == 7) v = fmaf(f.tn[56 + i], gh.n, v);
-            g.b[y][x] = v;
-        }
-}
-
-// Geometric mean of a cell of the field at stride h and its neighbours (geometric_mean4).
-__device__ __forceinline__ float children_mean(const double* __restrict__ K, int h) {
-    float a = 0.0f;
-#pragma unroll 1
-    for (int t = 0; t < 4; ++t) {
-        const float l = logf(narrow(__ldg(K + h * ((t & 1) + 16 * (t >> 1)))));
-        a = t ? a + l : l;
-    }
-    return expf(0.25f * a);
-}
-
-// The 8 x 8 correction operator: faces of the geometric means of the children.
-__device__ __forceinline__ void correction8(const double* __restrict__ K, int ns, W16Smem& sm, int lane) {
-    FacesF& f = sm.faces;
-    float* k = reinterpret_cast<float*>(sm.c);
-    __syncwarp();
-#pragma unroll 1
-    for (int c = lane; c < 64; c += 32) k[c] = children_mean(K + 32 * (c >> 3) + 2 * (c & 7), 1);
-    __syncwarp();
-#pragma unroll 1
-    for (int c = lane; c < 64; c += 32) {
-        const int i = c & 7, j = c >> 3;
-        const float v = k[c], tb = ns ? 2.0f * v : 0.0f;
-        f.te[c] = i < 7 ? harmonic_mean(v, k[c + 1]) : 2.0f * v;
-        f.tn[c] = j < 7 ? harmonic_mean(v, k[c + 8]) : tb;
-        if (i == 0) f.tw[j] = 2.0f * v;
-        if (j == 0) f.ts[i] = tb;
-    }
-    __syncwarp();
-}
-
-// Dirichlet data of cell (i, j) on the rhs of the n x n stage problem.
-__device__ __forceinline__ double rhs64(const W16Smem& sm, int n, int i, int j, const Ghost<double>& gh) {
-    double r = 0.0;
-    if (i == 0) r = fma(sm.tw[j], gh.w, r);
-    if (i == n - 1) r = fma(sm.te[j * n + i], gh.e, r);
-    if (gh.ns && j == 0) r = fma(sm.ts[i], gh.s, r);
-    if (gh.ns && j == n - 1) r = fma(sm.tn[j * n + i], gh.n, r);
-    return r;
-}
-
-__device__ __forceinline__ double warp_sum(double a) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(kAll, a, off);
-    return __shfl_sync(kAll, a, 0);
-}
-
-// The QoI of the refined grid (every lane).
-__device__ __forceinline__ double qoi(const W16Smem& sm, int n, const Ghost<double>& gh, int lane) {
-    if (gh.ns) {
-        const int c = (n / 2 - 1) * n + n / 2 - 1;
-        return 0.25 * ((sm.p[c] + sm.p[c + 1]) + (sm.p[c + n] + sm.p[c + n + 1]));
-    }
-    const int c = (lane & (n - 1)) * n + n - 1;
-    double acc = __dmul_rn(sm.te[c], sm.p[c] - gh.e);
-#pragma unroll 1
-    for (int off = n >> 1; off > 0; off >>= 1) acc += __shfl_down_sync(kAll, acc, off);
-    return __shfl_sync(kAll, acc, 0);
-}
-
-// ||r||^2 <= tol^2 ||b||^2 of a refined stage.  The FP32 sum of the rounded
-// residuals is within 1e-5 of ||r||^2, so it decides except next to the limit
-// (or the ends of its range), where the FP64 sum is formed: the decisions are
-// those of FP64 sums, without their operations in the FP64 pipe.
-struct Stop {
-    double limit;
-    float below, above;   // an FP32 sum under / over these decides
-};
-
-__device__ __forceinline__ Stop stop_at(double limit) {
-    const float t = (float)limit;
-    return {limit, t > 1e-30f ? t * 0.99999f : -1.0f, fmaxf(t * 1.00001f, 1e-30f)};
-}
-
-__device__ __forceinline__ float warp_sum(float a) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(kAll, a, off);
-    return a;
-}
-
-// The rhs of the stage problem (zero off the edges) into sm.f; returns the stop
-// rule's limits.
-__device__ __forceinline__ Stop stage_limit(W16Smem& sm, int n, const Ghost<double>& gh, double tol, int lane) {
-    double bb = 0.0;
-    if (lane < n) {
-#pragma unroll 1
-        for (int q = 0; q < 2; ++q) {
-            const double v = rhs64(sm, n, q * (n - 1), lane, gh);
-            sm.f[q][lane] = v;
-            bb = fma(v, v, bb);
-        }
-        if (gh.ns) {
-#pragma unroll 1
-            for (int q = 0; q < 2; ++q) {
-                const double v = rhs64(sm, n, lane, q * (n - 1), gh);
-                sm.f[2 + q][lane] = v;
-                if (lane > 0 && lane < n - 1) bb = fma(v, v, bb);
-            }
-        }
-    }
-    const Stop stop = stop_at(tol * tol * warp_sum(bb));
-    __syncwarp();
-    return stop;
-}
-
-// FP64 residual of the stage problem at cell c of the refined grid.
-__device__ __forceinline__ double residual64(const W16Smem& sm, int lg, int c, int ns) {
-    const int n = 1 << lg, last = n - 1, i = c & last, j = c >> lg;
-    double v = __dmul_rn(sm.d[c], sm.p[c]);
-    if (i > 0) v = fma(-sm.te[c - 1], sm.p[c - 1], v);
-    if (i < last) v = fma(-sm.te[c], sm.p[c + 1], v);
-    if (j > 0) v = fma(-sm.tn[c - n], sm.p[c - n], v);
-    if (j < last) v = fma(-sm.tn[c], sm.p[c + n], v);
-    double f = 0.0;
-    if (ns && j == 0) f = sm.f[2][i];
-    if (ns && j == last) f = sm.f[3][i];
-    if (i == 0) f = sm.f[0][j];
-    if (i == last) f = sm.f[1][j];
-    return f - v;
-}
-
-// Residuals of the refined grid, rounded to FP32, and the residual test.
-__device__ __forceinline__ bool residual_test(W16Smem& sm, int lg, int ns, const Stop& stop, int lane) {
-    float rr = 0.0f;
-    const int cells = 1 << 2 * lg;
-#pragma unroll 2
-    for (int c = lane; c < cells; c += 32) {
-        const float r = narrow(residual64(sm, lg, c, ns));
-        sm.r[c] = r;
-        rr = fmaf(r, r, rr);
-    }
-    rr = warp_sum(rr);
-    if (rr > stop.above) return false;
-    if (rr < stop.below) return true;
-    double r2 = 0.0;
-#pragma unroll 1
-    for (int c = lane; c < cells; c += 32) {
-        const double v = residual64(sm, lg, c, ns);
-        r2 = fma(v, v, r2);
-    }
-    return warp_sum(r2) <= stop.limit;
-}
-
-// The 16 x 16 start: the 8 x 8 solution interpolated, in FP64 where that stage
-// was refined, else in FP32.
-__device__ __forceinline__ void interpolate(bool refined, const G8& g8, G16& g16, const Ghost<float>& td,
-                                            const Ghost<double>& bd, W16Smem& sm, int lane) {
-    const int cx = lane & 7, ry = lane >> 3;
-    __syncwarp();
-    if (!refined) {
-        prolong16(g8, g16, td, false, lane);
-#pragma unroll
-        for (int y = 0; y < 4; ++y)
-#pragma unroll
-            for (int x = 0; x < 2; ++x) sm.p[16 * (4 * ry + y) + 2 * cx + x] = widen(g16.p[y][x]);
-        return;
-    }
-    sm.c[lane] = sm.p[lane];
-    sm.c[32 + lane] = sm.p[32 + lane];
-    __syncwarp();
-    const int Iw = cx > 0 ? cx - 1 : cx, Ie = cx < 7 ? cx + 1 : cx;
-#pragma unroll 1
-    for (int y = 0; y < 4; ++y) {
-        const int J = 2 * ry + (y >> 1), Jy = (y & 1) ? J + 1 : J - 1;
-        const bool edge = Jy < 0 || Jy > 7;
-        const double* row = sm.c + 8 * J;
-        const double* oth = sm.c + 8 * (edge ? J : Jy);
-        const double o = row[cx];
-        double l = row[Iw], r = row[Ie], oo = oth[cx], ol = oth[Iw], orr = oth[Ie];
-        if (cx == 0) {
-            l = fma(2.0, bd.w, -o);
-            ol = fma(2.0, bd.w, -oo);
-        }
-        if (cx == 7) {
-            r = fma(2.0, bd.e, -o);
-            orr = fma(2.0, bd.e, -oo);
-        }
-        if (edge && bd.ns) {
-            const double gv = 2.0 * (Jy < 0 ? bd.s : bd.n);
-            oo = gv - oo;
-            ol = gv - ol;
-            orr = gv - orr;
-        }
-        const int c = 16 * (4 * ry + y) + 2 * cx;
-        sm.p[c] = prolong_vals(o, l, oo, ol);
-        sm.p[c + 1] = prolong_vals(o, r, oo, orr);
-    }
-}
-
-// A sample whose V-cycles left the finite numbers: its QoI until the second
-// launch has solved it again with SAFE (a payload no arithmetic makes).
-constexpr long long kAgain = 0x7ff8000057313641ll;
-
-// One sample, by one warp.
-template <bool SAFE>
-__device__ __forceinline__ void solve_sample(const ResidentArgs& a, size_t s, W16Smem& sm, int lane) {
-    const Ghost<float> td{(float)a.bd.w, (float)a.bd.e, (float)a.bd.s, (float)a.bd.n, a.bd.ns};
-    const Ghost<float> zero{0.0f, 0.0f, 0.0f, 0.0f, a.bd.ns};
-    const int bx = lane & 3, by = (lane >> 2) & 3, cx = lane & 7, ry = lane >> 3;
-    const Inner in8{bx > 0, bx < 3, by > 0, by < 3}, in16{cx > 0, cx < 7, ry > 0, ry < 3};
-    const double* K = a.K + s * 256;
-    G8 g8;
-    G16 g16;
-    const double* kc = K + 64 * by + 4 * bx;
-    // grid 4 x 4: exact solve of its stage problem (every fourth cell of the
-    // field); then it carries corrections only (geometric means)
-#pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {
-        const float k = pass ? children_mean(kc, 2) : narrow(__ldg(kc));
-        const float b = coarse_inverse(k, td, sm, lane);
-        if (!pass) prolong8(coarse_solve(b, sm, lane), g8, td, false, lane);
-    }
-    bool ok = true;
-    double q = NAN;
-    int tests[2] = {0, 0}, cycles[2] = {0, 0};
-#pragma unroll 1
-    for (int st = 0; st < 2; ++st) {   // the stages 8 x 8 and 16 x 16
-        // 8 x 8 is refined where Q^c is asked for, else it starts 16 x 16 with nu0 cycles
-        const bool refined = st || a.qc != nullptr;
-        const int lg = 3 + st, cells = 64 << 2 * st;
-        if (st) {
-            interpolate(a.qc != nullptr, g8, g16, td, a.bd, sm, lane);
-            correction8(K, a.bd.ns, sm, lane);
-        } else {
-            stage_faces(K, 3, a.bd.ns, sm, lane);
-        }
-        load8(sm.faces, g8, lane);
-        if (st) {
-            stage_faces(K, 4, a.bd.ns, sm, lane);
-            load16(sm.faces, g16, sm, lane);
-        } else if (refined) {
-            store8(g8, sm, lane);
-        } else {
-            stage_rhs8(sm.faces, g8, td, lane);
-        }
-        const Stop stop = stage_limit(sm, 1 << lg, a.bd, a.tol, lane);
-        double q_prev = NAN;
-        // FP64 residual -> FP32 V-cycles on the correction -> FP64 update
-#pragma unroll 1
-        for (int it = 0;; ++it) {
-            if (refined) {
-                const bool done = residual_test(sm, lg, a.bd.ns, stop, lane);
-                q = qoi(sm, 1 << lg, a.bd, lane);
-                ++tests[st];
-                if (done || (a.qtol > 0 && fabs(q - q_prev) <= a.qtol * fabs(q))) break;
-                q_prev = q;
-                if (it >= a.max_cycles) {
-                    ok = false;
-                    break;
-                }
-                __syncwarp();
-                if (st) {
-#pragma unroll
-                    for (int y = 0; y < 4; ++y) {
-                        const float2 v = *reinterpret_cast<const float2*>(sm.r + 16 * (4 * ry + y) + 2 * cx);
-                        g16.b[y][0] = v.x;
-                        g16.b[y][1] = v.y;
-                        g16.p[y][0] = g16.p[y][1] = 0.0f;
-                    }
-                } else {
-#pragma unroll
-                    for (int y = 0; y < 2; ++y) {
-                        const float2 v = *reinterpret_cast<const float2*>(sm.r + 8 * (2 * by + y) + 2 * bx);
-                        g8.b[y][0] = v.x;
-                        g8.b[y][1] = v.y;
-                        g8.p[y][0] = g8.p[y][1] = 0.0f;
-                    }
-                }
-            } else if (it) {
-                break;
-            }
-            const int n = refined ? a.ir : a.nu0;
-            cycles[st] += n;
-#pragma unroll 1
-            for (int v = 0; v < n; ++v) vcycle<SAFE>(st, g16, g8, in16, in8, sm, a.nu1, a.nu2, zero, lane);
-            if (!refined) continue;
-            __syncwarp();
-            if (st) {
-#pragma unroll
-                for (int y = 0; y < 4; ++y)
-                    *reinterpret_cast<float2*>(sm.r + 16 * (4 * ry + y) + 2 * cx) =
-                        make_float2(g16.p[y][0], g16.p[y][1]);
-            } else if (lane < 16) {
-#pragma unroll
-                for (int y = 0; y < 2; ++y)
-                    *reinterpret_cast<float2*>(sm.r + 8 * (2 * by + y) + 2 * bx) = make_float2(g8.p[y][0], g8.p[y][1]);
-            }
-            __syncwarp();
-            bool finite = true;
-#pragma unroll 2
-            for (int c = lane; c < cells; c += 32) {
-                const float e = sm.r[c];
-                finite = finite && isfinite(e);
-                sm.p[c] += widen(e);
-            }
-            if (!SAFE && !__all_sync(kAll, finite)) {
-                if (lane == 0) a.qf[s] = __longlong_as_double(kAgain);
-                return;
-            }
-            __syncwarp();
-        }
-        if (!st && lane == 0 && a.qc) a.qc[s] = q;
-    }
-    if (lane == 0) {
-        if (a.flops) {   // the counts of fmg_resident.cu
-            const double c[2] = {64.0, 256.0};
-            double work = 0.0, work64 = 0.0, model = 0.0;
-            for (int st = 0; st < 2; ++st) {
-                const double updates = tests[st] ? tests[st] - 1.0 : 0.0;
-                work64 += c[st] * (14.0 * tests[st] + updates);
-                model += c[st] * 20.0 * tests[st] + cycles[st] * vcycle_bytes(4, 1 + st, a.nu1, a.nu2, 4);
-                work += cycles[st] * vcycle_flops(4, 1 + st, a.nu1, a.nu2);
-            }
-            atomicAdd(a.flops, work + work64);
-            atomicAdd(a.flops + 1, work64);
-            atomicAdd(a.flops + 2, model);
-        }
-        a.qf[s] = q;
-        if (a.status) a.status[s] = ok ? FM_OK : FM_ENOTCONV;
-    }
-    if (a.p_out) {
-        double* po = a.p_out + s * 256;
-        for (int c = lane; c < 256; c += 32) po[c] = sm.p[c];
-    }
-    __syncwarp();
-}
-
-}  // namespace
 
 __global__ void __launch_bounds__(32 * kW16Warps, 4) k_fmg_warp16(ResidentArgs a) {
     extern __shared__ __align__(16) unsigned char w16_smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     W16Smem& sm = reinterpret_cast<W16Smem*>(w16_smem)[warp];
+    const Ghost<float> td{(float)a.bd.w, (float)a.bd.e, (float)a.bd.s, (float)a.bd.n, a.bd.ns};
+    const Ghost<float> zero{0.0f, 0.0f, 0.0f, 0.0f, a.bd.ns};
     const size_t stride = (size_t)gridDim.x * kW16Warps;
 #pragma unroll 1
-    for (size_t s = (size_t)blockIdx.x * kW16Warps + warp; s < a.S; s += stride) solve_sample<false>(a, s, sm, lane);
-}
-
-// The samples k_fmg_warp16 left.
-__global__ void __launch_bounds__(32 * kW16Warps) k_fmg_warp16_again(ResidentArgs a) {
-    extern __shared__ __align__(16) unsigned char w16_smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    W16Smem& sm = reinterpret_cast<W16Smem*>(w16_smem)[warp];
-    const size_t stride = (size_t)gridDim.x * kW16Warps * 32;
-#pragma unroll 1
-    for (size_t s0 = ((size_t)blockIdx.x * kW16Warps + warp) * 32; s0 < a.S; s0 += stride) {
-        const size_t s = s0 + lane;
-        unsigned left = __ballot_sync(kAll, s < a.S && __double_as_longlong(a.qf[s]) == kAgain);
-#pragma unroll 1
-        for (; left; left &= left - 1) solve_sample<true>(a, s0 + __ffs(left) - 1, sm, lane);
+    for (size_t s = (size_t)blockIdx.x * kW16Warps + warp; s < a.S; s += stride) {
+        G8 g8;
+        G16 g16;
+        const Stages r = coarse_stages<4>(a, a.K + s * 256, g8, g16, sm, td, zero, lane);
+        if (lane == 0) {
+            if (a.flops && r.finite) {   // the counts of fmg_resident.cu
+                const double c[2] = {64.0, 256.0};
+                double work = 0.0, work64 = 0.0, model = 0.0;
+                for (int st = 0; st < 2; ++st) {
+                    const double updates = r.tests[st] ? r.tests[st] - 1.0 : 0.0;
+                    work64 += c[st] * (14.0 * r.tests[st] + updates);
+                    model += c[st] * 20.0 * r.tests[st] + r.cycles[st] * vcycle_bytes(4, 1 + st, a.nu1, a.nu2, 4);
+                    work += r.cycles[st] * vcycle_flops(4, 1 + st, a.nu1, a.nu2);
+                }
+                atomicAdd(a.flops, work + work64);
+                atomicAdd(a.flops + 1, work64);
+                atomicAdd(a.flops + 2, model);
+            }
+            a.qf[s] = r.finite ? r.q[1] : __longlong_as_double(kAgain);
+            if (a.qc) a.qc[s] = r.q[0];
+            if (a.status) a.status[s] = r.ok ? FM_OK : FM_ENOTCONV;
+        }
+        if (a.p_out) {
+            double* po = a.p_out + s * 256;
+            for (int c = lane; c < 256; c += 32) po[c] = sm.p[c];
+        }
+        __syncwarp();
     }
 }
 
-bool launch_warp16(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st) {
+void launch_warp16(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st) {
     constexpr size_t smem = kW16Warps * sizeof(W16Smem);
     static std::once_flag once;
     std::call_once(once, [] {
         cudaFuncSetAttribute(k_fmg_warp16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaFuncSetAttribute(k_fmg_warp16_again, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     });
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fmg_warp16, 32 * kW16Warps, smem);
     const size_t need = (a.S + kW16Warps - 1) / kW16Warps;
     const size_t grid = std::min<size_t>(need, (size_t)std::max(per_sm, 1) * std::max(ctx->sms, 1));
-    const int pi = prof_start(ctx, kFamResidentFmg, st);
-    ResidentArgs b = a;
-    b.flops = prof_counter(ctx, pi);
-    k_fmg_warp16<<<(unsigned)grid, 32 * kW16Warps, smem, st>>>(b);
-    k_fmg_warp16_again<<<(unsigned)std::min<size_t>((need + 31) / 32, grid), 32 * kW16Warps, smem, st>>>(b);
-    prof_stop(ctx, pi, st, 8.0 * 256 * (double)a.S + 16.0 * a.S, 0.0);
-    return true;
+    k_fmg_warp16<<<(unsigned)grid, 32 * kW16Warps, smem, st>>>(a);
 }
 
 }  // namespace fm
