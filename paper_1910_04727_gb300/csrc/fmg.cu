@@ -20,6 +20,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "fmg_resident.cuh"
 #include "fmg_strip.cuh"
 
 namespace fm {
@@ -1527,11 +1528,31 @@ static void vcycle_tail(const Hierarchy<T>& H, int kt, const fm_solve_params& pr
     a.Ainv = H.AinvC;
     a.active = active;
     a.order = listed ? H.order : nullptr;
-    const size_t smem = tail_smem_bytes<T>(kt, H.n0);
     const double top = (double)H.g[kt].n * H.g[kt].n;
-    FM_TIMED(ctx, kFamVcycleTail, st, (3.0 * cells + 2.0 * top) * sizeof(T) * a.S,
-             (10.0 * (prm.nu1 + prm.nu2) + 18.0) * cells * a.S,
-             k_vcycle_tail<T><<<(unsigned)a.S, kTailThreads, smem, st>>>(a));
+    const double bytes = (3.0 * cells + 2.0 * top) * sizeof(T) * a.S;
+    const double flops = (10.0 * (prm.nu1 + prm.nu2) + 18.0) * cells * a.S;
+    if constexpr (sizeof(T) == 4) {
+        if (kt == 3 && H.n0 == 4) {   // 4, 8, 16, 32: in registers
+            Tail32Args t{};
+            t.nu1 = a.nu1;
+            t.nu2 = a.nu2;
+            t.ns = a.ns;
+            for (int j = 0; j < 3; ++j) {
+                t.Te[j] = a.Te[j + 1];
+                t.Tn[j] = a.Tn[j + 1];
+                t.D[j] = a.D[j + 1];
+            }
+            t.Ainv = a.Ainv;
+            t.b = a.b;
+            t.p = a.p;
+            t.active = a.active;
+            t.order = a.order;
+            FM_TIMED(ctx, kFamVcycleTail, st, bytes, flops, launch_tail32(t, a.S, st));
+            return;
+        }
+    }
+    FM_TIMED(ctx, kFamVcycleTail, st, bytes, flops,
+             k_vcycle_tail<T><<<(unsigned)a.S, kTailThreads, tail_smem_bytes<T>(kt, H.n0), st>>>(a));
 }
 
 // Whether the smoother of correction grid k reads the zero iterate that the

@@ -56,4 +56,16 @@ __device__ __forceinline__ double vcycle_bytes(int n0, int k, int nu1, int nu2, 
 void launch_warp16(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st);
 void launch_team32(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st);
 
+// The level-wise V-cycle from the 32 x 32 correction grid down in registers
+// (fmg_team32.cu): operators of the grids 8, 16, 32, the 4 x 4 inverse, the 32 x 32
+// rhs and result; S CTAs, one a sample (listed by order, if given).
+struct Tail32Args {
+    int nu1, nu2, ns;
+    const float *Te[3], *Tn[3], *D[3];
+    const float *Ainv, *b;
+    float* p;
+    const int32_t *active, *order;
+};
+void launch_tail32(const Tail32Args& a, size_t S, cudaStream_t st);
+
 }  // namespace fm

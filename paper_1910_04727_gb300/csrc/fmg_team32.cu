@@ -24,7 +24,12 @@ namespace {
 constexpr int kTeam = 160;        // threads: four bands and the coarse grids
 constexpr int kBandBarrier = 1;   // named barrier of the bands
 
-struct Team32Smem {
+struct Borders {
+    float top[4][32], bot[4][32];   // border rows of the bands' iterates
+    float c16[256];                 // the 16 x 16 grid's rhs, then its correction
+};
+
+struct Team32Smem : Borders {
     double p[1024], d[1024], te[1024], tn[1024];
     double tw[32], ts[32];
     double f[4][32];
@@ -34,8 +39,6 @@ struct Team32Smem {
         } faces;
         float r[1024];            // residual, then correction
     };
-    float top[4][32], bot[4][32];   // border rows of the bands' iterates
-    float c16[256];                 // the 16 x 16 grid's rhs, then its correction
     Stop stop;
     float rr[4];                    // partial norms
     double r2[4], q;
@@ -53,8 +56,8 @@ __device__ __forceinline__ void band_sync() { asm volatile("bar.sync %0, %1;" ::
 
 __device__ __forceinline__ void all_sync() { asm volatile("bar.sync 0, %0;" ::"n"(kTeam) : "memory"); }
 
-template <int C>
-__device__ __forceinline__ void half_sweep32(Band& g, Team32Smem& sm, int band, int lane) {
+template <Form F, int C>
+__device__ __forceinline__ void half_sweep32(Band& g, Borders& sm, int band, int lane) {
     const int cx = lane & 15;
     const bool up = lane >= 16;   // the band's upper four rows
     float nb[4];
@@ -71,23 +74,24 @@ __device__ __forceinline__ void half_sweep32(Band& g, Team32Smem& sm, int band, 
         acc = x == 0 ? fmaf(g.ei[y], g.p[y][1], acc) : fmaf(g.ee[y], nb[y], acc);
         acc = y == 0 ? fmaf(g.sf[x], lo, acc) : fmaf(g.nf[y > 0 ? y - 1 : 0][x], g.p[y > 0 ? y - 1 : 0][x], acc);
         acc = y == 3 ? fmaf(g.nf[3][x], hi, acc) : fmaf(g.nf[y][x], g.p[y < 3 ? y + 1 : 3][x], acc);
-        g.p[y][x] = quotient(acc, g.d[y][x], g.rd[y][x]);
+        g.p[y][x] = F == kResident32 ? quotient(acc, g.d[y][x], g.rd[y][x]) : __fmul_rn(acc, g.rd[y][x]);
     }
     if (up) sm.top[band][2 * cx + ((3 + C) & 1)] = g.p[3][(3 + C) & 1];
     else sm.bot[band][2 * cx + (C & 1)] = g.p[0][C & 1];
     band_sync();
 }
 
-__device__ __forceinline__ void sweeps32(Band& g, Team32Smem& sm, int n, int band, int lane) {
+template <Form F>
+__device__ __forceinline__ void sweeps32(Band& g, Borders& sm, int n, int band, int lane) {
 #pragma unroll 1
     for (int s = 0; s < n; ++s) {
-        half_sweep32<0>(g, sm, band, lane);
-        half_sweep32<1>(g, sm, band, lane);
+        half_sweep32<F, 0>(g, sm, band, lane);
+        half_sweep32<F, 1>(g, sm, band, lane);
     }
 }
 
 // Both border rows, after the iterate changed as a whole.
-__device__ __forceinline__ void publish(const Band& g, Team32Smem& sm, int band, int lane) {
+__device__ __forceinline__ void publish(const Band& g, Borders& sm, int band, int lane) {
     const int cx = lane & 15;
     if (lane >= 16) *reinterpret_cast<float2*>(&sm.top[band][2 * cx]) = make_float2(g.p[3][0], g.p[3][1]);
     else *reinterpret_cast<float2*>(&sm.bot[band][2 * cx]) = make_float2(g.p[0][0], g.p[0][1]);
@@ -95,7 +99,8 @@ __device__ __forceinline__ void publish(const Band& g, Team32Smem& sm, int band,
 }
 
 // Residual restricted to the 16 x 16 rhs.
-__device__ __forceinline__ void restrict32(const Band& g, Team32Smem& sm, int band, int lane) {
+template <Form F>
+__device__ __forceinline__ void restrict32(const Band& g, Borders& sm, int band, int lane) {
     const int cx = lane & 15;
     const bool up = lane >= 16;
     float W[4], E[4], S[2], N[2];
@@ -117,10 +122,10 @@ __device__ __forceinline__ void restrict32(const Band& g, Team32Smem& sm, int ba
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int y = 2 * h + q, ys = y > 0 ? y - 1 : 0, yn = y < 3 ? y + 1 : 3;
-            r[q][0] = residual<0>(g.d[y][0], g.p[y][0], g.b[y][0], g.w[y], W[y], g.ei[y], g.p[y][1],
+            r[q][0] = residual<F, 0>(g.d[y][0], g.p[y][0], g.b[y][0], g.w[y], W[y], g.ei[y], g.p[y][1],
                                   y == 0 ? g.sf[0] : g.nf[ys][0], y == 0 ? S[0] : g.p[ys][0], g.nf[y][0],
                                   y == 3 ? N[0] : g.p[yn][0]);
-            r[q][1] = residual<1>(g.d[y][1], g.p[y][1], g.b[y][1], g.ei[y], g.p[y][0], g.ee[y], E[y],
+            r[q][1] = residual<F, 1>(g.d[y][1], g.p[y][1], g.b[y][1], g.ei[y], g.p[y][0], g.ee[y], E[y],
                                   y == 0 ? g.sf[1] : g.nf[ys][1], y == 0 ? S[1] : g.p[ys][1], g.nf[y][1],
                                   y == 3 ? N[1] : g.p[yn][1]);
         }
@@ -130,7 +135,7 @@ __device__ __forceinline__ void restrict32(const Band& g, Team32Smem& sm, int ba
 
 // p (+)= P u from the 16 x 16 values in sm.c16 (add: black cells alone where
 // post-smoothing replaces the red ones).
-__device__ __forceinline__ void prolong32(Band& g, const Team32Smem& sm, const Ghost<float>& gh, bool add, bool all,
+__device__ __forceinline__ void prolong32(Band& g, const Borders& sm, const Ghost<float>& gh, bool add, bool all,
                                           int band, int lane) {
     const int I = lane & 15, J0 = 4 * band + 2 * (lane >> 4);
     float o[4], l[4], r[4];   // coarse rows J0 - 1 .. J0 + 2
@@ -165,6 +170,41 @@ __device__ __forceinline__ void prolong32(Band& g, const Team32Smem& sm, const G
         const float vr = x == 0 ? prolong_vals(o[J], l[J], o[K], l[K]) : prolong_vals(o[J], r[J], o[K], r[K]);
         g.p[y][x] = add ? __fadd_rn(g.p[y][x], vr) : vr;
     }
+}
+
+// One V-cycle on the 32 x 32 grid: the bands' part and the fifth warp's.
+template <Form F>
+__device__ __forceinline__ void band_vcycle(Band& g, Borders& sm, int nu1, int nu2, const Ghost<float>& zero, int band,
+                                            int lane) {
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+        if (h) {
+            restrict32<F>(g, sm, band, lane);
+            all_sync();
+            all_sync();   // the correction from 16 x 16 is in
+            prolong32(g, sm, zero, true, nu2 == 0, band, lane);
+            publish(g, sm, band, lane);
+        }
+        sweeps32<F>(g, sm, h ? nu2 : nu1, band, lane);
+    }
+}
+
+template <Form F>
+__device__ __forceinline__ void coarse_vcycle(G16& g16, G8& g8, Borders& sm, CoarseSmem& cs, int nu1, int nu2,
+                                              const Ghost<float>& zero, int lane) {
+    float* const c16 = sm.c16 + 16 * 4 * (lane >> 3) + 2 * (lane & 7);   // the lane's cells
+    all_sync();   // the restricted residual is in
+#pragma unroll
+    for (int y = 0; y < 4; ++y) {
+        const float2 r = *reinterpret_cast<const float2*>(c16 + 16 * y);
+        g16.b[y][0] = r.x;
+        g16.b[y][1] = r.y;
+        g16.p[y][0] = g16.p[y][1] = 0.0f;
+    }
+    vcycle<F>(true, g16, g8, cs, nu1, nu2, zero, lane);
+#pragma unroll
+    for (int y = 0; y < 4; ++y) *reinterpret_cast<float2*>(c16 + 16 * y) = make_float2(g16.p[y][0], g16.p[y][1]);
+    all_sync();
 }
 
 // FP64 faces of a band's rows and their FP32 copies; the edges' faces are 2K (or 0).
@@ -344,19 +384,7 @@ __device__ __forceinline__ void band_role(const ResidentArgs& a, size_t s, const
         }
         publish(g, sm, warp, lane);
 #pragma unroll 1
-        for (int v = 0; v < a.ir; ++v) {
-#pragma unroll 1
-            for (int h = 0; h < 2; ++h) {
-                if (h) {
-                    restrict32(g, sm, warp, lane);
-                    all_sync();
-                    all_sync();   // the correction from 16 x 16 is in
-                    prolong32(g, sm, zero, true, a.nu2 == 0, warp, lane);
-                    publish(g, sm, warp, lane);
-                }
-                sweeps32(g, sm, h ? a.nu2 : a.nu1, warp, lane);
-            }
-        }
+        for (int v = 0; v < a.ir; ++v) band_vcycle<kResident32>(g, sm, a.nu1, a.nu2, zero, warp, lane);
         bool finite = true;
 #pragma unroll
         for (int y = 0; y < 4; ++y) {
@@ -376,13 +404,14 @@ __device__ __forceinline__ void band_role(const ResidentArgs& a, size_t s, const
 __device__ __forceinline__ void coarse_role(const ResidentArgs& a, size_t s, const Ghost<float>& td,
                                             const Ghost<float>& zero, Team32Smem& sm, int lane) {
     const double* K = a.K + s * 1024;
-    float* const c16 = sm.c16 + 16 * 4 * (lane >> 3) + 2 * (lane & 7);   // the lane's cells
     G8 g8;
     G16 g16;
     const Stages low = coarse_stages<5>(a, K, g8, g16, sm.w16, td, zero, lane);
     if (a.qc == nullptr) {
 #pragma unroll
-        for (int y = 0; y < 4; ++y) *reinterpret_cast<float2*>(c16 + 16 * y) = make_float2(g16.p[y][0], g16.p[y][1]);
+        for (int y = 0; y < 4; ++y)
+            *reinterpret_cast<float2*>(sm.c16 + 16 * (4 * (lane >> 3) + y) + 2 * (lane & 7)) =
+                make_float2(g16.p[y][0], g16.p[y][1]);
     }
     all_sync();
     if (lane == 0 && !low.finite) sm.bad = 1;
@@ -399,21 +428,7 @@ __device__ __forceinline__ void coarse_role(const ResidentArgs& a, size_t s, con
         if (stage_done(sm, a, it, l, [] {})) break;
         cycles += a.ir;
 #pragma unroll 1
-        for (int v = 0; v < a.ir; ++v) {
-            all_sync();   // the restricted residual is in
-#pragma unroll
-            for (int y = 0; y < 4; ++y) {
-                const float2 r = *reinterpret_cast<const float2*>(c16 + 16 * y);
-                g16.b[y][0] = r.x;
-                g16.b[y][1] = r.y;
-                g16.p[y][0] = g16.p[y][1] = 0.0f;
-            }
-            vcycle<true>(true, g16, g8, sm.w16, a.nu1, a.nu2, zero, lane);
-#pragma unroll
-            for (int y = 0; y < 4; ++y)
-                *reinterpret_cast<float2*>(c16 + 16 * y) = make_float2(g16.p[y][0], g16.p[y][1]);
-            all_sync();
-        }
+        for (int v = 0; v < a.ir; ++v) coarse_vcycle<kResident32>(g16, g8, sm, sm.w16, a.nu1, a.nu2, zero, lane);
         all_sync();   // the update is done
     }
     if (lane == 0) {
@@ -434,6 +449,66 @@ __device__ __forceinline__ void coarse_role(const ResidentArgs& a, size_t s, con
         a.qf[s] = bad ? __longlong_as_double(kAgain) : l.q;
         if (a.qc) a.qc[s] = low.q[1];
         if (a.status) a.status[s] = l.ok && low.ok ? FM_OK : FM_ENOTCONV;
+    }
+}
+
+struct Tail32Smem : Borders {
+    CoarseSmem coarse;
+};
+
+// A correction operator in memory -> the 16 x 16 and 8 x 8 grids' registers.
+__device__ __forceinline__ void operator16(const float* __restrict__ Te, const float* __restrict__ Tn,
+                                           const float* __restrict__ D, G16& g, CoarseSmem& sm, int lane) {
+    const int cx = lane & 7, ry = lane >> 3;
+#pragma unroll
+    for (int y = 0; y < 4; ++y) {
+        const int j = 4 * ry + y, c = 16 * j + 2 * cx;
+        const float2 e = *reinterpret_cast<const float2*>(Te + c), t = *reinterpret_cast<const float2*>(Tn + c);
+        const float2 d = *reinterpret_cast<const float2*>(D + c);
+        const float w = up1(e.y);
+        sm.df[2 * y][lane] = d.x;
+        sm.df[2 * y + 1][lane] = d.y;
+        g.rd[y][0] = recip(d.x);
+        g.rd[y][1] = recip(d.y);
+        g.w[y] = cx > 0 ? w : 0.0f;
+        g.ei[y] = e.x;
+        g.ee[y] = cx < 7 ? e.y : 0.0f;
+        g.nf[y][0] = j < 15 ? t.x : 0.0f;
+        g.nf[y][1] = j < 15 ? t.y : 0.0f;
+    }
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const float s = __shfl_up_sync(kAll, g.nf[3][x], 8);
+        g.sf[x] = ry > 0 ? s : 0.0f;
+    }
+}
+
+__device__ __forceinline__ void operator8(const float* __restrict__ Te, const float* __restrict__ Tn,
+                                          const float* __restrict__ D, G8& g, int lane) {
+    const int bx = lane & 3, by = (lane >> 2) & 3;
+    float t[2][2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int c = 8 * (2 * by + q) + 2 * bx;
+        const float2 e = *reinterpret_cast<const float2*>(Te + c), n = *reinterpret_cast<const float2*>(Tn + c);
+        const float2 d = *reinterpret_cast<const float2*>(D + c);
+        const float w = lf(e.y);
+        g.w[q] = bx > 0 ? w : 0.0f;
+        g.ei[q] = e.x;
+        g.ee[q] = bx < 3 ? e.y : 0.0f;
+        t[q][0] = n.x;
+        t[q][1] = n.y;
+        g.d[q][0] = d.x;
+        g.d[q][1] = d.y;
+        g.rd[q][0] = recip(d.x);
+        g.rd[q][1] = recip(d.y);
+    }
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const float s = be(t[1][x]);
+        g.sf[x] = by > 0 ? s : 0.0f;
+        g.ni[x] = t[0][x];
+        g.nn[x] = by < 3 ? t[1][x] : 0.0f;
     }
 }
 
@@ -458,6 +533,73 @@ __global__ void __launch_bounds__(kTeam, 3) k_fmg_team32(ResidentArgs a) {
             all_sync();
         }
     }
+}
+
+// The V-cycle of the level-wise schedule from a 32 x 32 correction grid down to
+// 4 x 4, from a zero iterate: k_vcycle_tail's arithmetic, one sample a CTA.  Bound by
+// the chain of half-sweeps (eight of 32 x 32 at a barrier each, as many of each grid
+// below in one warp); the shared-memory form issues nine loads an update.  A solve
+// of 1000 samples of 256 x 256: 62 launches of 25.7 us on average, now 12.5.
+__global__ void __launch_bounds__(kTeam, 3) k_vcycle_tail32(Tail32Args a) {
+    __shared__ Tail32Smem sm;
+    const size_t s = a.order ? (size_t)a.order[blockIdx.x] : blockIdx.x;
+    if (a.active && !a.active[s]) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const Ghost<float> zero{0.0f, 0.0f, 0.0f, 0.0f, a.ns};
+    if (warp == 4) {
+        G8 g8;
+        G16 g16;
+        const float* A = a.Ainv + s * 256;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {   // 16 rows of 16
+            const int e = 4 * (lane + 32 * q);
+            *reinterpret_cast<float4*>(&sm.coarse.ainv[e >> 4][e & 15]) = *reinterpret_cast<const float4*>(A + e);
+        }
+        operator8(a.Te[0] + s * 64, a.Tn[0] + s * 64, a.D[0] + s * 64, g8, lane);
+        operator16(a.Te[1] + s * 256, a.Tn[1] + s * 256, a.D[1] + s * 256, g16, sm.coarse, lane);
+        __syncwarp();
+        coarse_vcycle<kLevelwise>(g16, g8, sm, sm.coarse, a.nu1, a.nu2, zero, lane);
+        return;
+    }
+    const int cx = lane & 15, row0 = 8 * warp + 4 * (lane >> 4);
+    const float* te = a.Te[2] + s * 1024;
+    const float* tn = a.Tn[2] + s * 1024;
+    const float* dd = a.D[2] + s * 1024;
+    Band g;
+#pragma unroll
+    for (int y = 0; y < 4; ++y) {
+        const int j = row0 + y, c = 32 * j + 2 * cx;
+        const float2 e = *reinterpret_cast<const float2*>(te + c), t = *reinterpret_cast<const float2*>(tn + c);
+        const float2 d = *reinterpret_cast<const float2*>(dd + c);
+        const float2 b = *reinterpret_cast<const float2*>(a.b + s * 1024 + c);
+        const float w = up1(e.y);
+        g.d[y][0] = d.x;
+        g.d[y][1] = d.y;
+        g.rd[y][0] = recip(d.x);
+        g.rd[y][1] = recip(d.y);
+        g.b[y][0] = b.x;
+        g.b[y][1] = b.y;
+        g.p[y][0] = g.p[y][1] = 0.0f;
+        g.w[y] = cx > 0 ? w : 0.0f;
+        g.ei[y] = e.x;
+        g.ee[y] = cx < 15 ? e.y : 0.0f;
+        g.nf[y][0] = j < 31 ? t.x : 0.0f;
+        g.nf[y][1] = j < 31 ? t.y : 0.0f;
+        if (y == 0) {
+            const float2 u = j > 0 ? *reinterpret_cast<const float2*>(tn + c - 32) : make_float2(0.0f, 0.0f);
+            g.sf[0] = u.x;
+            g.sf[1] = u.y;
+        }
+    }
+    publish(g, sm, warp, lane);
+    band_vcycle<kLevelwise>(g, sm, a.nu1, a.nu2, zero, warp, lane);
+#pragma unroll
+    for (int y = 0; y < 4; ++y)
+        *reinterpret_cast<float2*>(a.p + s * 1024 + 32 * (row0 + y) + 2 * cx) = make_float2(g.p[y][0], g.p[y][1]);
+}
+
+void launch_tail32(const Tail32Args& a, size_t S, cudaStream_t st) {
+    k_vcycle_tail32<<<(unsigned)S, kTeam, 0, st>>>(a);
 }
 
 void launch_team32(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st) {
