@@ -565,12 +565,14 @@ __global__ void __launch_bounds__(256) k_mlp_out_train(int B, int ldt, const __n
                                                        float* __restrict__ out, float* __restrict__ dout,
                                                        float* __restrict__ sq, const float* __restrict__ Z3,
                                                        __nv_bfloat16* __restrict__ dZ,
-                                                       __nv_bfloat16* __restrict__ dZT) {
+                                                       __nv_bfloat16* __restrict__ dZT, int* step) {
     __shared__ __align__(16) __nv_bfloat16 tr[kH][kOutRows + 8];   // rows of 48 bytes
     constexpr int kPer = kOutRows / 8, kJ = kH / 32;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b0 = blockIdx.x * kOutRows + warp * kPer;   // B is a multiple of 128
     pdl_wait_then_release();
+    // training runs: the batch of this step has been taken in, the next may be chosen
+    if (step && blockIdx.x == 0 && threadIdx.x == 0) step[0] = step[1] + 1;
     float w[kJ], h[kPer][kJ], z[kPer][kJ];
 #pragma unroll
     for (int q = 0; q < kJ; ++q) w[q] = __bfloat162float(w4[lane + 32 * q]);
@@ -674,35 +676,51 @@ __global__ void k_surrogate_value(int n, const float* __restrict__ out, double m
     if (t < n) s[t] = mu + sd * (double)out[t];
 }
 
-// Mini-batch `*step` of a training run: rows perm[(step / spe) * n + (step %
-// spe) * B + b] of xi (FP64 [n][M]) and of the standardised targets tt, as
-// the BF16 operands X [B][D] (zero padded) and XT [D][ldt] and the FP32 t [B].
-__global__ void k_train_batch(int B, int M, int D, int ldt, int n, int spe, const int* __restrict__ step,
-                              const int32_t* __restrict__ perm, const double* __restrict__ xi,
-                              const float* __restrict__ tt, __nv_bfloat16* __restrict__ X,
-                              __nv_bfloat16* __restrict__ XT, float* __restrict__ t) {
+// Mini-batch step[0] of a training run: rows perm[(step / spe) * n + (step % spe)
+// * B + b] of xi (FP64 [n][M]) and of the standardised targets tt, as the BF16
+// operands X [B][D] (zero padded) and XT [D][ldt] and the FP32 t [B].  CTAs take
+// tiles of 32 x 32, transposed through shared memory (2-byte stores of XT a row
+// apart took a sector each).  What the step reads does not depend on the one
+// before, so it is read while that one's Adam update still runs.
+//
+// step[0]: the number the next batch takes; step[1]: of the batch in X.
+__global__ void __launch_bounds__(256) k_train_batch(int B, int M, int D, int ldt, int n, int spe, int* step,
+                                                     const int32_t* __restrict__ perm, const double* __restrict__ xi,
+                                                     const float* __restrict__ tt, __nv_bfloat16* __restrict__ X,
+                                                     __nv_bfloat16* __restrict__ XT, float* __restrict__ t) {
+    __shared__ __nv_bfloat16 tile[32][34];
+    const int tiles = D / 32, b0 = (int)(blockIdx.x / tiles) * 32, k0 = (int)(blockIdx.x % tiles) * 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k = k0 + lane;
+    const int s = __ldcg(step);
+    const size_t first = (size_t)(s / spe) * n + (size_t)(s % spe) * B + b0;
+    size_t row[4];
+    __nv_bfloat16 v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) row[q] = (size_t)perm[first + warp + 8 * q];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = __float2bfloat16_rn((float)(k < M ? xi[row[q] * M + k] : 0.0));
+    const float tv = k0 == 0 && threadIdx.x < 32 ? tt[perm[first + threadIdx.x]] : 0.0f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) tile[lane][warp + 8 * q] = v[q];
+    __syncthreads();
     pdl_wait_then_release();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= B * D) return;
-    const int b = i / D, k = i % D;
-    const int s = *step;
-    const size_t row = (size_t)perm[(size_t)(s / spe) * n + (size_t)(s % spe) * B + b];
-    const __nv_bfloat16 v = __float2bfloat16_rn((float)(k < M ? xi[row * M + k] : 0.0));
-    X[(size_t)b * D + k] = v;
-    XT[(size_t)k * ldt + b] = v;
-    if (k == 0) t[b] = tt[row];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        X[(size_t)(b0 + warp + 8 * q) * D + k] = v[q];
+        XT[(size_t)(k0 + warp + 8 * q) * ldt + b0 + lane] = tile[warp + 8 * q][lane];
+    }
+    if (k0 == 0 && threadIdx.x < 32) t[b0 + threadIdx.x] = tv;
+    if (blockIdx.x == 0 && threadIdx.x == 0) step[1] = s;
 }
 
 // One Adam step (Kingma & Ba) at step number *step of `total`, learning rate
 // lr0 (1 + cos(pi step / total)) / 2, followed by the BF16 operand copies of
-// the updated weights (row-major and, for W2 / W3, transposed); the step
-// counter then advances (`done` counts finished blocks, zero between steps).
+// the updated weights (row-major and, for W2 / W3, transposed).
 struct AdamArgs {
     size_t np;
     float *P, *m, *v;
     const float* g;
-    int* step;
-    int* done;
+    const int* step;
     int total;
     float lr0, b1, b2, eps;
     size_t off[8];
@@ -710,31 +728,17 @@ struct AdamArgs {
     __nv_bfloat16 *W1b, *W2b, *W3b, *W2T, *W3T, *w4b;
 };
 
-// One parameter's Adam update with learning rate lr and bias corrections c1,
-// c2; returns its BF16 operand copy, written row-major.
-__device__ __forceinline__ __nv_bfloat16 adam_update(const AdamArgs& a, size_t t, float lr, float c1, float c2) {
-    const float gt = a.g[t];
-    const float mt = a.b1 * a.m[t] + (1.0f - a.b1) * gt;
-    const float vt = a.b2 * a.v[t] + (1.0f - a.b2) * gt * gt;
-    a.m[t] = mt;
-    a.v[t] = vt;
-    const float p = a.P[t] - lr * (mt / c1) / (sqrtf(vt / c2) + a.eps);
-    a.P[t] = p;
-    const __nv_bfloat16 h = __float2bfloat16_rn(p);
-    if (t < a.off[1]) a.W1b[(t / a.M) * a.D + t % a.M] = h;
-    else if (t >= a.off[2] && t < a.off[3]) a.W2b[t - a.off[2]] = h;
-    else if (t >= a.off[4] && t < a.off[5]) a.W3b[t - a.off[4]] = h;
-    else if (t >= a.off[6] && t < a.off[7]) a.w4b[t - a.off[6]] = h;
-    return h;
-}
-
 // Blocks of 256 parameters; those of W2 and W3 (256 x 256, starting at a
 // multiple of 256) take 16 x 16 tiles, whose transposed operand goes through
 // shared memory in 32-byte rows (2-byte stores a row apart took a sector each).
-__global__ void k_adam_step(AdamArgs a) {
+// Only the gradient is new to the step: parameters, moments, step number and
+// coefficients (once per block) are read and formed while the kernels before
+// still run.  20480 pairs x 20 epochs: 9.5 us a step with everything after the
+// wait and a count of finished blocks (645 atomics on one word) to advance the
+// step, 4.2 us so.
+__global__ void __launch_bounds__(256) k_adam_step(AdamArgs a) {
     __shared__ __align__(16) __nv_bfloat16 tr[16][24];
-    __shared__ float coef[3];   // learning rate and bias corrections of this step, formed once per block
-    pdl_wait_then_release();
+    __shared__ float coef[3];   // learning rate and bias corrections of this step
     size_t t = (size_t)blockIdx.x * 256 + threadIdx.x;
     const size_t o = t < a.off[4] ? a.off[2] : a.off[4];
     const bool tile = (t >= a.off[2] && t < a.off[3]) || (t >= a.off[4] && t < a.off[5]);   // the whole block
@@ -746,35 +750,40 @@ __global__ void k_adam_step(AdamArgs a) {
         tc0 = (q & 15) * 16;
         t = o + (size_t)(tr0 + ty) * kH + tc0 + tx;
     }
-    const int s = *a.step;
+    const bool live = t < a.np;
+    const float m0 = live ? __ldcg(a.m + t) : 0.0f, v0 = live ? __ldcg(a.v + t) : 0.0f;
+    const float p0 = live ? __ldcg(a.P + t) : 0.0f;
     if (threadIdx.x < 3) {
+        const int s = __ldcg(a.step);
         const float k = (float)(s + 1);
         coef[threadIdx.x] = threadIdx.x == 0   ? a.lr0 * 0.5f * (1.0f + cospif((float)s / (float)a.total))
                             : threadIdx.x == 1 ? 1.0f - powf(a.b1, k)
                                                : 1.0f - powf(a.b2, k);
     }
     __syncthreads();
-    if (t < a.np) {
-        const __nv_bfloat16 h = adam_update(a, t, coef[0], coef[1], coef[2]);
+    pdl_wait_then_release();
+    if (live) {   // (contractions spelled out: hoisting the loads changed the compiler's choice)
+        const float gt = a.g[t];
+        const float mt = fmaf(1.0f - a.b1, gt, __fmul_rn(a.b1, m0));
+        const float vt = fmaf(a.b2, v0, __fmul_rn(__fmul_rn(1.0f - a.b2, gt), gt));
+        a.m[t] = mt;
+        a.v[t] = vt;
+        const float p = p0 - coef[0] * (mt / coef[1]) / (sqrtf(vt / coef[2]) + a.eps);
+        a.P[t] = p;
+        const __nv_bfloat16 h = __float2bfloat16_rn(p);
+        if (t < a.off[1]) a.W1b[(t / a.M) * a.D + t % a.M] = h;
+        else if (t >= a.off[2] && t < a.off[3]) a.W2b[t - a.off[2]] = h;
+        else if (t >= a.off[4] && t < a.off[5]) a.W3b[t - a.off[4]] = h;
+        else if (t >= a.off[6] && t < a.off[7]) a.w4b[t - a.off[6]] = h;
         if (tile) tr[tx][ty] = h;
     }
     if (tile) {
         __syncthreads();
         if (threadIdx.x < 32) {   // column tc0 + r, rows tr0 + 8 c ..
-            const int r = threadIdx.x >> 1, c = threadIdx.x & 1;
+            const int q = threadIdx.x >> 1, c = threadIdx.x & 1;
             __nv_bfloat16* WT = o == a.off[2] ? a.W2T : a.W3T;
-            *reinterpret_cast<uint4*>(WT + (size_t)(tc0 + r) * kH + tr0 + 8 * c) =
-                *reinterpret_cast<const uint4*>(&tr[r][8 * c]);
-        }
-    }
-    // the last block to finish advances the step counter (every block has
-    // read it by then) and re-arms the block count for the next step
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        if (atomicAdd(a.done, 1) == (int)gridDim.x - 1) {
-            *a.step = s + 1;
-            *a.done = 0;
+            *reinterpret_cast<uint4*>(WT + (size_t)(tc0 + q) * kH + tr0 + 8 * c) =
+                *reinterpret_cast<const uint4*>(&tr[q][8 * c]);
         }
     }
 }
@@ -845,6 +854,8 @@ struct MlpState {
         double *K = nullptr, *q = nullptr;
         cudaGraph_t graph = nullptr;
         cudaGraphExec_t exec = nullptr;
+        cudaGraph_t graph_many = nullptr;
+        cudaGraphExec_t exec_many = nullptr;
         std::vector<double> hq;        // targets Q_0 on the host
         int n = 0, batch = 0;
         fm_train_report rep{};         // fields known at launch
@@ -1041,7 +1052,7 @@ static void refresh_bf16(fm_ctx* ctx, cudaStream_t st) {
 // GEMMs, the output layer with its gradient, dZ2, dZ1, dW1, Adam with the
 // step counter) instead of 17.  The bias sums run on S->side2, beside both: in
 // line with the weight gradients they made that branch the longer one.
-static void train_step_grads(fm_ctx* ctx, int B, cudaStream_t st, bool pdl = false) {
+static void train_step_grads(fm_ctx* ctx, int B, cudaStream_t st, bool pdl = false, int* step = nullptr) {
     MlpState* S = state(ctx);
     const int D = S->D, L = kMaxBatch;
     constexpr int BN = kTrainBN;
@@ -1056,7 +1067,7 @@ static void train_step_grads(fm_ctx* ctx, int B, cudaStream_t st, bool pdl = fal
     gemm<BN, kEpiFwdGelu>(ctx, S->mH2, S->tW3, B, kH, kH, e, st, pdl);
     // output layer and dZ3 = bf16(dout w4 gelu'(Z3)) on st; gw4 = dout^T H3, gb4 = sum dout beside it
     launch(pdl, k_mlp_out_train, dim3((unsigned)(B / kOutRows)), dim3(256), 0, st, B, L, S->H[2], S->w4b,
-           S->P + S->off[7], S->t, S->out, S->dout, S->sq, S->Z[2], S->dZ[2], S->dZT[2]);
+           S->P + S->off[7], S->t, S->out, S->dout, S->sq, S->Z[2], S->dZ[2], S->dZT[2], step);
     cudaEventRecord(S->ev_fork, st);
     cudaStreamWaitEvent(sd, S->ev_fork, 0);
     cudaStreamWaitEvent(sb, S->ev_fork, 0);
@@ -1320,10 +1331,14 @@ static fm_status train_finish(fm_ctx* ctx, fm_train_report* rep) {
         rep->var_residual = var_res;
         rep->seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - R.t0).count();
     }
-    if (R.exec) cudaGraphExecDestroy(R.exec);
-    if (R.graph) cudaGraphDestroy(R.graph);
-    R.exec = nullptr;
-    R.graph = nullptr;
+    for (cudaGraphExec_t* e : {&R.exec, &R.exec_many}) {
+        if (*e) cudaGraphExecDestroy(*e);
+        *e = nullptr;
+    }
+    for (cudaGraph_t* g : {&R.graph, &R.graph_many}) {
+        if (*g) cudaGraphDestroy(*g);
+        *g = nullptr;
+    }
     R.hq.clear();
     return stt;
 }
@@ -1422,30 +1437,44 @@ extern "C" fm_status surrogate_train(fm_ctx* ctx, const fm_train_opts* opts, fm_
         FM_CUDA_TRY(ctx, cudaMemset(S->step, 0, 8));
         refresh_bf16(ctx, nullptr);
         FM_CUDA_TRY(ctx, cudaDeviceSynchronize());
-        // one training step as a CUDA graph: batch gather, forward, backward,
-        // Adam + BF16 refresh, step counter; replayed `total` times
-        AdamArgs aa{S->np, S->P, S->Am, S->Av, S->G, S->step, S->step + 1, total, (float)opts->lr, 0.9f, 0.999f, 1e-8f,
+        // training steps as CUDA graphs: batch gather, forward, backward, Adam +
+        // BF16 refresh.  One step, replayed first; eight once those are under way
+        // (a graph of one step starts 2.6 us after the one before has drained, inside
+        // a graph a step's batch is read during that one's Adam update).
+        AdamArgs aa{S->np, S->P, S->Am, S->Av, S->G, S->step + 1, total, (float)opts->lr, 0.9f, 0.999f, 1e-8f,
                     {}, M, S->D, S->W1b, S->W2b, S->W3b, S->W2T, S->W3T, S->w4b};
         for (int i = 0; i < 8; ++i) aa.off[i] = S->off[i];
-        const bool prof_on = ctx->prof.active;
-        ctx->prof.active = false;    // no event records inside the captured graph
-        FM_CUDA_TRY(ctx, cudaStreamBeginCapture(ts, cudaStreamCaptureModeThreadLocal));
-        // programmatic dependent launches: every kernel's launch and setup
-        // overlap its predecessor (kernels wait for it before touching data)
-        launch(true, k_train_batch, dim3(nb((size_t)batch * S->D)), dim3(256), 0, ts, batch, M, S->D, kMaxBatch, n,
-               spe, (const int*)S->step, (const int32_t*)R.perm, (const double*)R.xi, (const float*)R.tt, S->X,
-               S->XT, S->t);
-        train_step_grads(ctx, batch, ts, true);
-        launch(true, k_adam_step, dim3(nb(S->np)), dim3(256), 0, ts, aa);
-        const cudaError_t ce = cudaStreamEndCapture(ts, &R.graph);
-        ctx->prof.active = prof_on;
-        FM_CUDA_TRY(ctx, ce);
-        FM_CUDA_TRY(ctx, cudaGraphInstantiate(&R.exec, R.graph, 0));
+        auto capture = [&](int steps, cudaGraph_t* graph, cudaGraphExec_t* exec) {
+            const bool prof_on = ctx->prof.active;
+            ctx->prof.active = false;    // no event records inside the captured graph
+            cudaError_t ce = cudaStreamBeginCapture(ts, cudaStreamCaptureModeThreadLocal);
+            // programmatic dependent launches: every kernel's launch and setup
+            // overlap its predecessor (kernels wait for it before touching what it may write)
+            for (int k = 0; k < steps && ce == cudaSuccess; ++k) {
+                launch(true, k_train_batch, dim3((unsigned)(batch / 32 * (S->D / 32))), dim3(256), 0, ts, batch, M, S->D,
+                       kMaxBatch, n, spe, S->step, (const int32_t*)R.perm, (const double*)R.xi, (const float*)R.tt,
+                       S->X, S->XT, S->t);
+                train_step_grads(ctx, batch, ts, true, S->step);
+                launch(true, k_adam_step, dim3(nb(S->np)), dim3(256), 0, ts, aa);
+            }
+            if (ce == cudaSuccess) ce = cudaStreamEndCapture(ts, graph);
+            ctx->prof.active = prof_on;
+            if (ce == cudaSuccess) ce = cudaGraphInstantiate(exec, *graph, 0);
+            return ce;
+        };
+        constexpr int kMany = 8, kLead = 16;   // steps of the long graph; single steps before it
+        FM_CUDA_TRY(ctx, capture(1, &R.graph, &R.exec));
         const int pidx = prof_start(ctx, kFamMlpTrain, ts);
         FM_CUDA_TRY(ctx, cudaGraphLaunch(R.exec, ts));
         // the first step's batch errors, for the report
         FM_CUDA_TRY(ctx, cudaMemcpyAsync(R.sq0, S->sq, (size_t)batch * 4, cudaMemcpyDeviceToDevice, ts));
-        for (int k = 1; k < total; ++k) FM_CUDA_TRY(ctx, cudaGraphLaunch(R.exec, ts));
+        int k = 1;
+        if (total >= kLead + 4 * kMany) {
+            for (; k < kLead; ++k) FM_CUDA_TRY(ctx, cudaGraphLaunch(R.exec, ts));
+            FM_CUDA_TRY(ctx, capture(kMany, &R.graph_many, &R.exec_many));
+            for (; k + kMany <= total; k += kMany) FM_CUDA_TRY(ctx, cudaGraphLaunch(R.exec_many, ts));
+        }
+        for (; k < total; ++k) FM_CUDA_TRY(ctx, cudaGraphLaunch(R.exec, ts));
         const double D = S->D;
         prof_stop(ctx, pidx, ts, 0.0, (double)total * 2.0 * batch * (2.0 * D * kH + 6.0 * kH * kH));
         FM_CUDA_TRY(ctx, cudaEventRecord(R.trained, ts));
