@@ -101,8 +101,12 @@ __global__ void k_faces(int n, size_t S, int ns, const double* __restrict__ K, T
     const CellAt at = cell_at(t, n);
     const int i = at.i, j = at.j;
     const C k = rounded<C>(K[t]);
-    const C te = (i < n - 1) ? harmonic_mean(k, rounded<C>(K[t + 1])) : C(2) * k;
-    const C tn = (j < n - 1) ? harmonic_mean(k, rounded<C>(K[t + n])) : (ns ? C(2) * k : C(0));
+    // formed everywhere (of k with itself past an edge) and replaced by integers at
+    // the edges: an FP64 product there would take its turn in every warp
+    const C he = harmonic_mean(k, rounded<C>(K[i < n - 1 ? t + 1 : t]));
+    const C hn = harmonic_mean(k, rounded<C>(K[j < n - 1 ? t + n : t]));
+    const C te = (i < n - 1) ? he : twice(k);
+    const C tn = (j < n - 1) ? hn : (ns ? twice(k) : C(0));
     Te[t] = rounded<T>(te);
     Tn[t] = rounded<T>(tn);
     if (Te64) {
@@ -134,7 +138,7 @@ __global__ void k_diagonal(int n, size_t S, int ns, const double* K, const T* __
     };
     auto fe = [&](size_t u) { return face(Te, Te64, u); };
     auto fn = [&](size_t u) { return face(Tn, Tn64, u); };
-    auto edge = [&] { return C(2) * rounded<C>(K[t]); };
+    auto edge = [&] { return twice(rounded<C>(K[t])); };
     const C tw = (i > 0) ? fe(t - 1) : edge();
     const C ts = (j > 0) ? fn(t - n) : (ns ? edge() : C(0));
     const C d = tw + fe(t) + ts + fn(t);
@@ -143,17 +147,36 @@ __global__ void k_diagonal(int n, size_t S, int ns, const double* K, const T* __
     if (rD) rD[t] = T(1) / (T)d;
 }
 
-// Right-hand side of a stage problem: the Dirichlet data moved to the rhs
-// (zero, without a read of K, off the edges).
+// Cell o of the edge of an n x n grid (4 (n - 1) cells).
+__device__ __forceinline__ void ring_cell(int o, int n, int& i, int& j) {
+    const int q = o / (n - 1), e = o % (n - 1);   // side, position along it
+    i = q == 0 ? e : q == 1 ? n - 1 : q == 2 ? n - 1 - e : 0;
+    j = q == 0 ? 0 : q == 1 ? e : q == 2 ? n - 1 : n - 1 - e;
+}
+// Threads for S grids' cells and, after them, their edge cells once more.
+inline size_t ring_threads(size_t S, int n) { return S * ((size_t)n * n + 4 * (size_t)(n - 1)); }
+
+// Right-hand side of a stage problem: the Dirichlet data moved to the rhs.  Zero,
+// without a read of K, off the edges; edge cells on threads of their own (in one
+// pass their FP64 products took their turn in every warp: 288 us for the stages of
+// 5000 FP64 samples of 64 x 64).
 template <typename T>
 __global__ void k_stage_rhs(int n, size_t S, const double* __restrict__ K, Bnd bd, T* __restrict__ b) {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t cells = (size_t)n * n;
-    if (t >= S * cells) return;
-    const CellAt at = cell_at(t, n);
-    const int i = at.i, j = at.j;
-    const bool edge = i == 0 || i == n - 1 || (bd.ns && (j == 0 || j == n - 1));
-    b[t] = edge ? (T)dirichlet_rhs(bd, n, i, j, K[t]) : T(0);
+    if (t < S * cells) {
+        const CellAt at = cell_at(t, n);
+        if (at.i > 0 && at.i < n - 1 && at.j > 0 && at.j < n - 1) b[t] = T(0);
+        return;
+    }
+    const int ring = 4 * (n - 1);
+    const size_t u = t - S * cells, s = u / ring;
+    if (s >= S) return;
+    int i, j;
+    ring_cell((int)(u % ring), n, i, j);
+    const size_t g = s * cells + (size_t)j * n + i;
+    const bool edge = i == 0 || i == n - 1 || bd.ns;
+    b[g] = edge ? (T)dirichlet_rhs(bd, n, i, j, K[g]) : T(0);
 }
 
 // One colour of a red-black Gauss-Seidel sweep: cells with (i + j) % 2 == color.
@@ -471,16 +494,12 @@ __global__ void k_prolong(int nc, size_t S, const U* __restrict__ uc, Ghost<U> g
         const size_t r = t - S * cells;
         s = r / ring;
         if (s >= S || inactive(active, s)) return;
-        const int e = (int)(r % ring), q = e / (nf - 1), o = e % (nf - 1);   // side, position along it
-        i = q == 0 ? o : q == 1 ? nf - 1 : q == 2 ? nf - 1 - o : 0;
-        j = q == 0 ? 0 : q == 1 ? o : q == 2 ? nf - 1 : nf - 1 - o;
+        ring_cell((int)(r % ring), nf, i, j);
         v = prolong_at(nc, uc + s * (size_t)nc * nc, i, j, gh);
     }
     const size_t g = s * cells + (size_t)j * nf + i;
     pf[g] = add ? pf[g] + v : v;
 }
-
-inline size_t prolong_threads(size_t S, int n) { return S * ((size_t)n * n + 4 * (size_t)(n - 1)); }
 
 // Three neighbouring values of a coarse row around column I: its own, west and
 // east; past the Dirichlet edges the error's ghosts, minus its own.
@@ -1702,7 +1721,7 @@ static void vcycles(const Hierarchy<T>& H, int k, int top, const fm_solve_params
         } else {
             const Ghost<T> zg{T(0), T(0), T(0), T(0), ns};
             FM_TIMED(ctx, kFamProlong, st, 2.25 * ts * cells, 8.0 * cells,
-                     k_prolong<T><<<blocks_for(prolong_threads(S, n)), kBlock, 0, st>>>(c.n, S, c.p, zg, 1, cur,
+                     k_prolong<T><<<blocks_for(ring_threads(S, n)), kBlock, 0, st>>>(c.n, S, c.p, zg, 1, cur,
                                                                                         active));
             smooth_with<T>(ctx, tile, threads, n, S, prm.nu2, g.b, Te, Tn, D, rD, cur, g.p, active, st, nullptr, ns);
         }
@@ -1900,12 +1919,12 @@ static fm_status fmg_batch(const Hierarchy<T>& H, const fm_solve_params& prm, do
             const GridBufs<T>& c = H.g[k - 1];
             if (mixed && refined && k == H.m && H.m >= 1 && refine_c) {
                 FM_TIMED(ctx, kFamFmgInterp, st, 10.0 * cells, 8.0 * cells,
-                         k_prolong<double><<<blocks_for(prolong_threads(S, g.n)), kBlock, 0, st>>>(
+                         k_prolong<double><<<blocks_for(ring_threads(S, g.n)), kBlock, 0, st>>>(
                              c.n, S, c.p64, Ghost<double>{bd.g[0], bd.g[1], bd.g[2], bd.g[3], bd.ns}, 0, g.p64,
                              nullptr));
             } else {
                 FM_TIMED(ctx, kFamFmgInterp, st, 1.25 * ts * cells, 8.0 * cells,
-                         k_prolong<T><<<blocks_for(prolong_threads(S, g.n)), kBlock, 0, st>>>(
+                         k_prolong<T><<<blocks_for(ring_threads(S, g.n)), kBlock, 0, st>>>(
                              c.n, S, c.p, Ghost<T>{(T)bd.g[0], (T)bd.g[1], (T)bd.g[2], (T)bd.g[3], bd.ns}, 0,
                              refined ? g.p : start_iterate(H, k, prm, prm.nu0), nullptr));
             }
@@ -1914,7 +1933,7 @@ static fm_status fmg_batch(const Hierarchy<T>& H, const fm_solve_params& prm, do
         // the coarsest grid is solved first)
         if (!(mixed && refined && k > 0))
             FM_TIMED(ctx, kFamStageRhs, st, ts * cells, 2.0 * cells,
-                     k_stage_rhs<T><<<blocks_for(cells), kBlock, 0, st>>>(g.n, S, g.K, bd, g.b));
+                     k_stage_rhs<T><<<blocks_for(ring_threads(S, g.n)), kBlock, 0, st>>>(g.n, S, g.K, bd, g.b));
         if (k == 0) vcycles(H, 0, 0, prm, nullptr, st, 1, false);
         if (!refined) {
             if (k > 0) vcycles(H, k, k, prm, nullptr, st, prm.nu0, false);

@@ -61,6 +61,15 @@ __device__ __forceinline__ T rounded(double x) {
     else return x;
 }
 
+// 2 x, in FP64 by the exponent (outside the FP64 pipe, as narrow and widen).
+static __device__ __noinline__ double twice_rare(double x) { return 2.0 * x; }
+__device__ __forceinline__ float twice(float x) { return 2.0f * x; }
+__device__ __forceinline__ double twice(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x);
+    if (((hi >> 20) & 0x7ffu) - 1u > 2044u) return twice_rare(x);
+    return __hiloint2double((int)(hi + 0x100000u), __double2loint(x));
+}
+
 // Harmonic mean 2ab / (a + b) of two coefficients, the face between them.
 // FP64: the divide of the FP64 pipe (a 58th of the FP32 rate) bounds the
 // set-up of every operator, so the quotient is formed with five operations
@@ -70,7 +79,7 @@ __device__ __forceinline__ T rounded(double x) {
 // one of 8.4e9 random pairs differed from the IEEE quotient, by an ulp.
 __device__ __forceinline__ float harmonic_mean(float a, float b) { return 2.0f * a * b / (a + b); }
 __device__ __forceinline__ double harmonic_mean(double a, double b) {
-    const double n = (a + a) * b, d = a + b;
+    const double n = twice(a) * b, d = a + b;
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
     const double e = fma(-d, r, 1.0);
