@@ -103,6 +103,8 @@ struct StripArgs {
     int n, W, nwin, seg, segs, resident;   // resident: groups in flight on the whole GPU
     int lgn;                               // PACK: log2 n
     size_t S;
+    size_t head;                           // packs in segments of seg rows; those after them in segments of seg2
+    int seg2, segs2;
     const T *b, *Te, *Tn, *D, *rD, *p_in;
     T* p_out;
     const int32_t* active;
@@ -115,6 +117,14 @@ struct StripArgs {
 
 // Halo columns and rows (even: rows and columns go in pairs).
 __host__ __device__ constexpr int strip_halo(int HS, bool fuse) { return fuse ? HS + 2 : HS; }
+
+// Rows of the shortest segments (even, at least 16 or the grid) with which
+// `units` strips of n rows still go into one wave of `resident` groups.
+__host__ __device__ inline int strip_fill(int n, size_t units, size_t resident) {
+    const int k = (int)(resident / (units > 0 ? units : 1));
+    const int seg = k > 1 ? ((n + k - 1) / k + 1) / 2 * 2 : n;
+    return seg < 16 ? (n < 16 ? n : 16) : seg < n ? seg : n;
+}
 
 // Shared memory of one warp.
 template <typename T, int HS, bool FUSE, bool EC>
@@ -156,25 +166,32 @@ __global__ void __launch_bounds__(32 * kStripMaxWarps, (strip_min_blocks<T, HS, 
     // last residual test left, with segments short enough to fill one wave
     // of groups when those samples are few
     const int pk = PACK ? 64 >> a.lgn : 1;
-    size_t S = a.S;
+    size_t S = a.S, head = a.head;
     int seg = a.seg, segs = a.segs;
     if (a.dcount) S = (size_t)*a.dcount;
     const size_t packs = (S + pk - 1) / pk;
-    if (a.dcount && packs * a.nwin < (size_t)a.resident) {
-        int sg = n;
-        while (sg / 2 >= 16 && packs * a.nwin * (size_t)((n + sg / 2 - 1) / (sg / 2)) <= (size_t)a.resident) sg /= 2;
-        seg = sg;
-        segs = (n + sg - 1) / sg;
+    if (a.dcount) {
+        head = packs;
+        if (packs > 0 && packs * a.nwin < (size_t)a.resident) {
+            seg = strip_fill(n, packs * a.nwin, (size_t)a.resident);
+            segs = (n + seg - 1) / seg;
+        }
     }
     const size_t unit = (size_t)blockIdx.x * (blockDim.x / (32 * W)) + grp;
-    if (unit >= packs * (size_t)segs * a.nwin) return;
     const int win = (int)(unit % a.nwin);
-    const size_t rest = unit / a.nwin;
+    size_t rest = unit / a.nwin, pack0 = 0;   // unit of the window's row of packs and segments
+    if (rest >= head * (size_t)segs) {
+        rest -= head * (size_t)segs;
+        pack0 = head;
+        seg = a.seg2;
+        segs = a.segs2;
+        if (rest >= (packs - head) * (size_t)segs) return;
+    }
     const int sy = (int)(rest % segs);
     const int gw = 64 * W;                              // columns of the group's window
     const int wx = win * (gw - 2 * XH);                 // its first column
     const int gx = PACK ? (2 * lane) & (n - 1) : wx + 64 * wig + 2 * lane;   // the lane's first column
-    const size_t si = PACK ? (rest / segs) * pk + ((2 * lane) >> a.lgn) : rest / segs;
+    const size_t si = PACK ? (pack0 + rest / segs) * pk + ((2 * lane) >> a.lgn) : pack0 + rest / segs;
     bool in_x = gx < n;
     size_t s = 0;
     if (PACK) {
@@ -482,21 +499,37 @@ inline void strip_windows(int n, int XH, int* W, int* nwin) {
     }
 }
 
-// Rows per segment: the power-of-two fraction of n (at least 16 rows) that
-// minimises the waves of units over the resident groups times the steps of
-// one unit (segment plus 2 halo rows plus the steps that drain the wavefront).
-inline int strip_segment(int n, size_t units1, int HS, int VH, int resident) {
-    int best = n;
+// How `packs` strips-of-samples of nwin windows are cut into row segments: all into
+// the power-of-two fraction of n (at least 16 rows) that minimises the waves of
+// units over the resident groups times the steps of one unit (segment plus halo
+// rows plus the steps that drain the wavefront), or, where that is less, whole
+// waves of uncut strips and one wave of the rest in segments that just fill it.
+// 1000 samples of 256 x 256, 304 groups resident: four waves of 265 steps, against
+// three and one of 117 (88 samples in three segments); the solve's eight-half-sweep
+// passes 8.4 -> 7.7 ms.
+struct StripCut {
+    size_t head;     // packs in segments of seg rows; the rest in segments of seg2
+    int seg, seg2;
+};
+
+inline StripCut strip_cut(int n, size_t packs, int nwin, int HS, int VH, int resident) {
+    auto steps = [&](int seg) { return std::min(seg + (seg < n ? 2 * VH : 0), n) + HS + 1; };
+    const size_t units1 = packs * nwin, R = (size_t)std::max(1, resident);
+    StripCut best{packs, n, n};
     double best_cost = 1e300;
     for (int seg = n; seg >= 16; seg /= 2) {
         const size_t units = units1 * ((n + seg - 1) / seg);
-        const double waves = std::ceil((double)units / std::max(1, resident));
-        const double cost = waves * (std::min(seg + (seg < n ? 2 * VH : 0), n) + HS + 1);
+        const double cost = std::ceil((double)units / (double)R) * steps(seg);
         if (cost < best_cost * 0.999) {
             best_cost = cost;
-            best = seg;
+            best = {packs, seg, seg};
         }
         if (seg % 4) break;   // segments start on even rows
+    }
+    const size_t waves = units1 / R, head = std::min(packs, waves * R / nwin), rest = packs - head;
+    if (rest > 0 && rest * nwin <= R) {
+        const int seg2 = strip_fill(n, rest * nwin, R);
+        if (waves * (double)steps(n) + steps(seg2) < best_cost * 0.98) best = {head, n, seg2};
     }
     return best;
 }
@@ -539,9 +572,13 @@ struct StripVariant {
         const bool listed = !dev && c.order && c.busy > 0 && c.busy < c.S;
         a.S = listed ? c.busy : c.S;
         const size_t packs = (a.S + pk - 1) / pk;
-        a.seg = strip_segment(c.n, packs * a.nwin, HS, VH, a.resident);
+        const StripCut cut = strip_cut(c.n, packs, a.nwin, HS, VH, a.resident);
+        a.head = cut.head;
+        a.seg = cut.seg;
         a.segs = (c.n + a.seg - 1) / a.seg;
-        size_t units = packs * (size_t)a.nwin * a.segs;
+        a.seg2 = cut.seg2;
+        a.segs2 = (c.n + a.seg2 - 1) / a.seg2;
+        size_t units = (a.head * a.segs + (packs - a.head) * a.segs2) * (size_t)a.nwin;
         if (dev) units = std::max(units, (size_t)a.resident);
         a.b = c.b;
         a.Te = c.Te;
