@@ -48,6 +48,12 @@ constexpr uint32_t kOzABytes = kOzM * kOzK * 2, kOzBBytes = kOzN * kOzK * 2;
 constexpr uint32_t kOzStage = kOzDigits * (kOzABytes + kOzBBytes);
 constexpr size_t kOzSmem = 1024 + kOzStages * kOzStage + 64 * 16 + 128;
 constexpr int kOzNoScale = -(1 << 28);   // exponent of a row that is not split (a value that is not finite, or far out)
+// Largest sum of a pair's scale exponents that is split.  What is left out is
+// relative to the scales, not to the sum, so a large entry that meets a zero
+// coefficient would cost digits (2^40 against 0: 1e-6 of the field); below
+// this line it is under 2^-50 of the field.  Fields reach it only where one mode
+// alone contributes 64 or more to the logarithm (in use the sum is 5 to 7).
+constexpr int kOzMaxScale = 10;
 constexpr size_t kOzMaxBytes = (size_t)4 << 30;   // most digits kept per level
 
 // 2^(j / 64) as the sum of two doubles.
@@ -266,9 +272,9 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                     if (c >= cells || s >= S) continue;
                     const int e = e_c + ex[s];
                     double g;
-                    if (e > -(1 << 20)) {
+                    if (e > -(1 << 20) && e <= kOzMaxScale) {
                         g = oz_join(acc, i, e);
-                    } else {   // a row that is not split: the plain sum
+                    } else {   // a row or a pair that is not split: the plain sum
                         g = 0.0;
                         for (int k = 0; k < M; ++k) g = fma(xi[(size_t)s * M + k], B[(size_t)c * M + k], g);
                     }

@@ -60,6 +60,16 @@ def test_rows_that_are_not_split():
             np.testing.assert_allclose(K[s][fin], ref[s][fin], rtol=1e-13)
 
 
+@pytest.mark.parametrize("scale", [2.0 ** 12, 2.0 ** 40, 2.0 ** 150])
+def test_a_large_entry_against_a_zero_coefficient_costs_no_digits(scale):
+    r = np.random.default_rng(74)
+    B, xi = 0.3 * r.standard_normal((64, 40)), r.standard_normal((33, 40))
+    B[5, 7] = scale
+    xi[:, 7] = 0.0
+    xi[9, 2], B[:, 2] = scale, 0.0
+    _check(_ctx(8, B).kl_field_batch(0, torch.tensor(xi, device="cuda")).cpu().numpy(), B, xi)
+
+
 def test_streams_and_capture():
     r = np.random.default_rng(73)
     B = 0.3 * r.standard_normal((256, 48))
