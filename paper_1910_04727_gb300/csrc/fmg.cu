@@ -144,7 +144,7 @@ __global__ void k_diagonal(int n, size_t S, int ns, const double* K, const T* __
     const C d = tw + fe(t) + ts + fn(t);
     D[t] = rounded<T>(d);
     if (D64) D64[t] = (double)d;
-    if (rD) rD[t] = T(1) / (T)d;
+    if (rD) rD[t] = recip_set((T)d);
 }
 
 // Cell o of the edge of an n x n grid (4 (n - 1) cells).
@@ -2135,7 +2135,7 @@ __global__ void k_tune_fill(size_t count, T* __restrict__ b, T* __restrict__ Te,
     Te[t] = (T)(0.5 + u0);
     Tn[t] = (T)(0.5 + u1);
     D[t] = (T)(4.5 + u2);
-    rD[t] = T(1) / D[t];
+    rD[t] = recip_set(D[t]);
     b[t] = (T)(2.0 * u2 - 1.0);
     p[t] = (T)(2.0 * u0 - 1.0);
 }

@@ -13,7 +13,7 @@
 // coarsest inverse.
 //
 // Bound: the FP64 pipe (2 lanes a clock and SM), 72 % of its rate: six operations a
-// cell and residual, one an update, eight a face.  Conversions, the norm of the
+// cell and residual, one an update, five a face.  Conversions, the norm of the
 // residual and the flop counts stay out of it.  20000 samples:
 // 5.1 ms by the shared-memory form (nine loads an update, one update after the
 // other, 107000 instructions a sample), 2.7 ms with the grids in registers and

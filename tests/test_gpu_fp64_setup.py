@@ -31,6 +31,14 @@ def test_coarse_inverse_and_child_means(n0, case, S):
         _check(c, K, OL.params(bc_case=case, pS=0.3, pN=0.7), n0, kernel=1)
 
 
+@pytest.mark.parametrize("exponent", [480, -481])
+def test_coefficients_on_both_sides_of_the_short_reciprocal(exponent):
+    import paper_1910_04727_gb300 as fm
+    c = fm.Context(1, 16, 8)
+    K = W.smooth_lognormal_field(64, S=5, tag=4500) * 2.0 ** exponent
+    _check(c, K, OL.params(), 4, kernel=1)
+
+
 @pytest.mark.parametrize("n,per_sm,converged", [(16, 8, 0), (32, 4, 0), (64, 1, 0), (64, 4, 1)])
 def test_auto_schedule_on_both_sides_of_its_line(n, per_sm, converged):
     import paper_1910_04727_gb300 as fm
