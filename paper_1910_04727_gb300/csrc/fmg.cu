@@ -1495,12 +1495,16 @@ static T* smooth_with(fm_ctx* ctx, int tile, int threads, int n, size_t S, int n
 static int tune_slot(int n) { return std::min(15, 31 - __builtin_clz((unsigned)n)); }
 
 // Smoother launch shape of grid n.  Untuned defaults (fastest on GB300 for two
-// sweeps): register-blocked regions up to 32 x 32 (FP64 solves of 5000 32 x 32
-// samples 2.37 ms against 2.48 with packed strips), then column strips.  FP64
-// strips against one launch per colour, fixed schedule: 64 x 64, 5000 samples
-// 12.0 / 14.0 ms; 128 x 128, 1000 samples 8.9 / 11.5; 256 x 256, 250 samples
-// 9.2 / 11.8 (before the strips read 1 / D instead of forming it, the FP64
-// divide made colour launches the faster ones).  An fm_autotune or
+// sweeps): column strips from 64 x 64 (FP64 strips against one launch per colour,
+// fixed schedule: 64 x 64, 5000 samples 12.0 / 14.0 ms; 128 x 128, 1000 samples 8.9 /
+// 11.5; 256 x 256, 250 samples 9.2 / 11.8).  32 x 32 and 16 x 16 in FP32: strips too,
+// with several samples in a warp (converged mixed solves, register-blocked regions
+// / strips on both: 64 x 64, 1000 samples 3.88 / 3.47 ms, 5000 12.1 / 10.5; 32 x 32
+// level-wise, 300 samples 1.97 / 1.69, 15000 14.6 / 8.9).  In FP64: one staged
+// region a sample (fixed schedule, register-blocked / staged / strips: 32 x 32, 15000
+// samples 5.00 / 4.72 / 5.03; 64 x 64, 5000 samples 6.25 / 6.12 / 6.40; converged 32 x
+// 32, 15000 samples 28.7 / 26.5 / 28.5; level on a few hundred samples).  Below, and
+// where strips do not fit: one register-blocked region a sample.  An fm_autotune or
 // fm_set_smoother_shape entry for this grid and precision replaces the
 // default.  Tiles and strips need both smoothing phases of the V-cycle (so
 // the iterate goes p -> p2 -> p); tiles need their staged region in shared
@@ -1509,7 +1513,11 @@ template <typename T>
 static void smooth_shape(const fm_ctx* ctx, int n, const fm_solve_params& prm, int* tile, int* threads) {
     const int pi = sizeof(T) == 4 ? 1 : 0, slot = tune_slot(n);
     *threads = 0;
-    *tile = n <= 32 ? 32 : kShapeStrip;   // 32: one register-blocked region per sample
+    *tile = n <= 32 ? 32 : kShapeStrip;   // 32: one region per sample, register-blocked
+    if (n == 16 || n == 32) {
+        if (sizeof(T) == 8) *threads = 8 * n;   // staged
+        else if (strip_fits(n, prm.nu1, prm.nu2)) *tile = kShapeStrip;
+    }
     if (ctx->tune.n[pi][slot] == n) {
         *tile = ctx->tune.tile[pi][slot];
         *threads = ctx->tune.threads[pi][slot];

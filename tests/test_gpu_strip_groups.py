@@ -56,3 +56,21 @@ def test_strip_rows_that_are_no_power_of_two_against_the_oracle():
             of, oc, _, _ = OL.fmg_solve_batch(K, prm, n0=3)
             assert np.max(np.abs(qf.cpu().numpy() - of) / np.abs(of)) < bar, n
             assert np.max(np.abs(qc.cpu().numpy() - oc) / np.abs(oc)) < bar, n
+
+
+@pytest.mark.parametrize("n,S", [(16, 1), (16, 37), (32, 3), (32, 301), (64, 5)])
+@pytest.mark.parametrize("nu1,nu2", [(2, 2), (1, 2), (3, 2)])
+@pytest.mark.parametrize("precision,energy", [(0, False), (1, False), (1, True)])
+def test_default_shapes_of_small_grids_give_the_register_regions_bits(n, S, nu1, nu2, precision, energy):
+    import paper_1910_04727_gb300 as fm
+    K = torch.tensor(W.smooth_lognormal_field(n, S=S, tag=3700 + n), device="cuda")
+    got = []
+    for shape in (None, 32):
+        c = fm.Context(1, n, 8, precision=precision, converged=precision, tol=1e-12, qtol=0.0, max_cycles=100,
+                       energy_step=energy)
+        for g in (16, 32):
+            if shape is not None:
+                c.set_smoother_shape(g, shape, 0, precision)
+        got.append(c.fmg_solve_batch(K, want_p=True, want_status=True, kernel=1, nu1=nu1, nu2=nu2))
+    for x, y in zip(*got):
+        assert torch.equal(x, y)
