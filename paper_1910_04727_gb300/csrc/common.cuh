@@ -126,11 +126,11 @@ struct Ghost {
 // resident kernel the shorter chain of launches, so it runs batches that it
 // takes in about one wave (fixed schedule) or a few (converged, where the
 // level-wise chain is several times longer).  Measured on GB300, ms level-wise
-// / resident, fixed: 16 x 16 0.35 / 0.32 at 1216 samples, 0.41 / 0.45 at 1824,
-// 6.6 / 14.6 at 60000; 32 x 32 0.59 / 0.43 at 608, 0.63 / 0.70 at 760; 64 x 64
-// 0.72 / 0.49 at 152, 0.88 / 0.96 at 200.  Converged: 16 x 16 4.95 / 4.20 at
-// 5000, 14.2 / 14.9 at 20000; 32 x 32 8.7 / 7.5 at 2432, 14.1 / 15.0 at 5000;
-// 64 x 64 13.4 / 12.4 at 608, 16.1 / 16.4 at 912.
+// / resident, fixed: 16 x 16 0.34 / 0.33 at 1216 samples, 0.39 / 0.46 at 1824,
+// 6.6 / 14.6 at 60000; 32 x 32 0.51 / 0.43 at 608, 0.55 / 0.69 at 760; 64 x 64
+// 0.67 / 0.48 at 152, 0.80 / 0.93 at 200.  Converged: 16 x 16 4.0 / 3.7 at
+// 4864, 6.4 / 7.1 at 9728; 32 x 32 4.7 / 3.8 at 1216, 6.6 / 6.9 at 2432;
+// 64 x 64 5.6 / 5.1 at 304, 7.4 / 9.1 at 608.
 // Mixed: resident up to 32 x 32 (grids in registers: 16 x 16 2.2 / 0.27 at 4000,
 // 12.2 / 2.2 at 40000; 32 x 32 2.8 / 0.47 at 1000, 8.6 / 2.5 at 8000), and a converged
 // 64 x 64 batch of at most two samples per SM (2.8 / 2.4 at 300).
@@ -139,7 +139,7 @@ inline bool auto_resident(int n_fine, size_t S, int sms, const fm_solve_params& 
     if (prm.precision == FM_PREC_MIXED)
         return n_fine <= 32 || (prm.converged && n_fine == 64 && S <= 2 * (size_t)sms);
     if (n_fine > 64) return false;
-    const size_t per_sm = prm.converged ? (n_fine <= 16 ? 32 : n_fine <= 32 ? 16 : 4)
+    const size_t per_sm = prm.converged ? (n_fine <= 16 ? 32 : n_fine <= 32 ? 12 : 2)
                                         : (n_fine <= 16 ? 8 : n_fine <= 32 ? 4 : 1);
     return S <= per_sm * (size_t)sms;
 }

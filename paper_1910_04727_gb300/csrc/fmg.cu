@@ -1503,14 +1503,19 @@ static int tune_slot(int n) { return std::min(15, 31 - __builtin_clz((unsigned)n
 // level-wise, 300 samples 1.97 / 1.69, 15000 14.6 / 8.9).  In FP64: one staged
 // region a sample (fixed schedule, register-blocked / staged / strips: 32 x 32, 15000
 // samples 5.00 / 4.72 / 5.03; 64 x 64, 5000 samples 6.25 / 6.12 / 6.40; converged 32 x
-// 32, 15000 samples 28.7 / 26.5 / 28.5; level on a few hundred samples).  Below, and
+// 32, 15000 samples 28.7 / 26.5 / 28.5; level on a few hundred samples).  FP64 grids from 64 x 64
+// of less than 2 Mi cells in the whole batch (1 Mi at 64 x 64): colour launches, since
+// a strip marches its rows one after the other and few strips leave the SMs waiting
+// (fixed schedule, strips / colours: one sample of 256 x 256 1.48 / 1.07 ms, 32 1.93 /
+// 1.72, 64 level; one of 1024 x 1024 3.15 / 2.24, four 3.99 / 3.43 with strips on the
+// finest 3.32; 160 of 64 x 64 0.77 / 0.73, 400 0.95 / 0.99).  Below, and
 // where strips do not fit: one register-blocked region a sample.  An fm_autotune or
 // fm_set_smoother_shape entry for this grid and precision replaces the
 // default.  Tiles and strips need both smoothing phases of the V-cycle (so
 // the iterate goes p -> p2 -> p); tiles need their staged region in shared
 // memory, strips 1 or 2 sweeps.
 template <typename T>
-static void smooth_shape(const fm_ctx* ctx, int n, const fm_solve_params& prm, int* tile, int* threads) {
+static void smooth_shape(const fm_ctx* ctx, int n, size_t S, const fm_solve_params& prm, int* tile, int* threads) {
     const int pi = sizeof(T) == 4 ? 1 : 0, slot = tune_slot(n);
     *threads = 0;
     *tile = n <= 32 ? 32 : kShapeStrip;   // 32: one region per sample, register-blocked
@@ -1518,6 +1523,7 @@ static void smooth_shape(const fm_ctx* ctx, int n, const fm_solve_params& prm, i
         if (sizeof(T) == 8) *threads = 8 * n;   // staged
         else if (strip_fits(n, prm.nu1, prm.nu2)) *tile = kShapeStrip;
     }
+    if (sizeof(T) == 8 && n >= 64 && S * n * n < ((size_t)1 << (n > 64 ? 21 : 20))) *tile = 0;
     if (ctx->tune.n[pi][slot] == n) {
         *tile = ctx->tune.tile[pi][slot];
         *threads = ctx->tune.threads[pi][slot];
@@ -1589,7 +1595,7 @@ static bool reads_zero(const Hierarchy<T>& H, int k, const fm_solve_params& prm)
     if (k == 0) return false;
     if (H.g[k].n <= H.ctx->tail_max && !prm.energy_step) return false;
     int tile, threads;
-    smooth_shape<T>(H.ctx, H.g[k].n, prm, &tile, &threads);
+    smooth_shape<T>(H.ctx, H.g[k].n, H.S, prm, &tile, &threads);
     return tile != kShapeStrip;
 }
 
@@ -1599,7 +1605,7 @@ static bool reads_zero(const Hierarchy<T>& H, int k, const fm_solve_params& prm)
 template <typename T>
 static T* start_iterate(const Hierarchy<T>& H, int k, const fm_solve_params& prm, int count) {
     int tile, threads;
-    smooth_shape<T>(H.ctx, H.g[k].n, prm, &tile, &threads);
+    smooth_shape<T>(H.ctx, H.g[k].n, H.S, prm, &tile, &threads);
     const bool merged = k > 0 && tile == kShapeStrip && count > 1 && strip_merges<T>(prm.nu1, prm.nu2);
     return merged && count % 2 == 0 ? H.g[k].p2 : H.g[k].p;
 }
@@ -1658,7 +1664,7 @@ static void vcycles(const Hierarchy<T>& H, int k, int top, const fm_solve_params
     const size_t cells = S * (size_t)n * n;
     const GridBufs<T>& c = H.g[k - 1];
     int tile, threads;
-    smooth_shape<T>(ctx, n, prm, &tile, &threads);
+    smooth_shape<T>(ctx, n, S, prm, &tile, &threads);
     T* const pc = reads_zero(H, k - 1, prm) ? c.p : nullptr;   // the coarse iterate, where it must be zeroed
     // the V-cycle below: the resident tail for correction grids up to
     // ctx->tail_max, else grid by grid
@@ -1752,7 +1758,7 @@ static void stage_test(const Hierarchy<T>& H, int k, const fm_solve_params& prm,
     const int chunks = test_chunks(g.n);
     const size_t ns = H.listed() ? H.busy : S;
     int tile, threads;
-    smooth_shape<T>(ctx, g.n, prm, &tile, &threads);
+    smooth_shape<T>(ctx, g.n, S, prm, &tile, &threads);
     T* const pT = tile == kShapeStrip ? nullptr : g.p;   // strips start from zero without reading it
     FM_TIMED(ctx, kFamResidualRestrict, st, (mixed ? 48.0 : 40.0) * ns * cells, 12.0 * ns * cells,
              k_stage_partials<T><<<(unsigned)(ns * chunks), kBlock, 0, st>>>(
@@ -2197,7 +2203,7 @@ static fm_status autotune_grid(fm_ctx* ctx, int n, int nsweeps, fm_tune_entry* e
     int def_tile = 0, def_threads = 0;
     const int pi = sizeof(T) == 4 ? 1 : 0, slot = tune_slot(n);
     ctx->tune.n[pi][slot] = 0;   // the untuned default
-    smooth_shape<T>(ctx, n, dp, &def_tile, &def_threads);
+    smooth_shape<T>(ctx, n, S, dp, &def_tile, &def_threads);
     double best = 1e30;
     int bt = def_tile, bth = def_threads;
     e->ms_default = time_shape(def_tile, def_threads);

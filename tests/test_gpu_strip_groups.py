@@ -74,3 +74,20 @@ def test_default_shapes_of_small_grids_give_the_register_regions_bits(n, S, nu1,
         got.append(c.fmg_solve_batch(K, want_p=True, want_status=True, kernel=1, nu1=nu1, nu2=nu2))
     for x, y in zip(*got):
         assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("n,S", [(64, 255), (64, 256), (128, 127), (128, 128), (256, 1)])
+@pytest.mark.parametrize("converged", [0, 1])
+def test_fp64_batches_on_both_sides_of_the_strip_line(n, S, converged):
+    import paper_1910_04727_gb300 as fm
+    K = torch.tensor(W.smooth_lognormal_field(n, S=min(S, 8), tag=3800 + n), device="cuda")
+    K = K.repeat((S + 7) // 8, 1, 1)[:S].contiguous()
+    got = []
+    for shape in (None, -1):
+        c = fm.Context(1, n, 8, converged=converged, tol=1e-10, max_cycles=100)
+        for g in (64, 128, 256):
+            if shape is not None:
+                c.set_smoother_shape(g, shape, 0, 0)
+        got.append(c.fmg_solve_batch(K, want_p=True, want_status=True, kernel=1))
+    for x, y in zip(*got):
+        assert torch.equal(x, y)
