@@ -11,7 +11,7 @@
 // cells across a warp: coalesced), so the next tile's products run under this
 // one's epilogue.  Bound: HBM (the FP64 fields out, the BF16 basis in).  The
 // conversion of exp to FP64 is done in integers: the FP64 pipe, where F2F runs,
-// takes 1.7 us per million.  500 fields of 256 x 256 cells from 256 modes: 85 us
+// takes 1.7 us per million.  500 fields of 256 x 256 cells from 256 modes: 84 us
 // (4.7 TB/s of field, basis and coefficients), 126 with a CTA per tile, two K
 // stages and F2F.
 //
@@ -205,22 +205,57 @@ __global__ void k_nystrom_cross_bf16(int n_ref, size_t r0, size_t rows, int q, i
     o[2 * Kpad + jq] = __double2bfloat16(v - (double)__bfloat162float(hi));
 }
 
-// x [n][M] FP64 -> [n][Kp] BF16 in the split layout (hi, lo, hi) or plain (hi).
+// v -> hi = BF16(v) in the low half, lo = BF16(v - hi) in the high half, each rounded
+// to nearest even.  In integers: the conversions and the subtraction are five operations of
+// the FP64 pipe, which bound the kernel below.
+static __device__ __noinline__ unsigned bf16_split_rare(double v) {
+    const __nv_bfloat16 hi = __double2bfloat16(v), lo = __double2bfloat16(v - (double)__bfloat162float(hi));
+    return (unsigned)__bfloat16_as_ushort(hi) | (unsigned)__bfloat16_as_ushort(lo) << 16;
+}
+__device__ __forceinline__ unsigned bf16_split(double v) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
+    const unsigned sign = (unsigned)(bits >> 48) & 0x8000u;
+    if ((bits << 1) == 0) return sign;
+    const int be = (int)(bits >> 52) & 0x7FF;
+    if ((unsigned)(be - 960) > 189u) return bf16_split_rare(v);   // 2^-63 .. 2^127
+    const unsigned long long m = (bits & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    const unsigned h = (unsigned)((m + ((1ull << 44) - 1 + ((m >> 45) & 1))) >> 45);   // 128 .. 256
+    const long long d = (long long)(m - ((unsigned long long)h << 45));                // v - hi, in units of m
+    const unsigned hi = sign | (((unsigned)(be - 896) << 7) + (h - 128u));
+    if (d == 0) return hi;
+    const int z = __clzll(d < 0 ? -d : d);   // 19 .. 63
+    const unsigned long long u = (unsigned long long)(d < 0 ? -d : d) << z;
+    const unsigned r = (unsigned)(u >> 56);
+    const unsigned long long rem = u << 8;
+    const unsigned up = rem > (1ull << 63) || (rem == (1ull << 63) && (r & 1u)) ? 1u : 0u;
+    const unsigned lo = (((unsigned)(be + 11 - z - 896) << 7) + (r & 0x7Fu) + up) | (d < 0 ? sign ^ 0x8000u : sign);
+    return hi | lo << 16;
+}
+
+// x [n][M] FP64 -> [n][Kp] BF16 in the split layout (hi, lo, hi) or plain (hi).  A warp
+// takes 64 columns of a row at a time (blockIdx.y: further columns of the same rows).
+// Bound: HBM.  With a thread an element, a 64-bit division each and FP64 conversions it
+// took the larger part of calls with many coefficients per cell: 25027 fields of 32 x 32
+// from 584 modes 248 -> 183 us a call, 500 of 256 x 256 from 256 modes 85.7 -> 84.0.
 __global__ void k_xi_to_bf16(size_t n, int M, int Mpad, int split, const double* __restrict__ x,
                              __nv_bfloat16* __restrict__ out) {
-    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n * Mpad) return;
-    const size_t s = t / Mpad;
-    const int k = (int)(t % Mpad);
-    const double v = (k < M) ? x[s * M + k] : 0.0;
-    const __nv_bfloat16 hi = __double2bfloat16(v);
-    const int Kp = split ? 3 * Mpad : Mpad;
-    __nv_bfloat16* o = out + s * Kp;
-    o[k] = hi;
-    if (split) {
-        o[Mpad + k] = __double2bfloat16(v - (double)__bfloat162float(hi));
-        o[2 * Mpad + k] = hi;
+    const size_t s = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (s >= n) return;
+    const double* row = x + s * M;
+    unsigned* o = reinterpret_cast<unsigned*>(out + s * (size_t)(split ? 3 * Mpad : Mpad));
+    for (int k = 64 * blockIdx.y + 2 * (threadIdx.x & 31); k < Mpad; k += 64 * gridDim.y) {
+        const unsigned a = k < M ? bf16_split(row[k]) : 0u, b = k + 1 < M ? bf16_split(row[k + 1]) : 0u;
+        const unsigned hi = __byte_perm(a, b, 0x5410);
+        o[k >> 1] = hi;
+        if (split) {
+            o[(Mpad + k) >> 1] = __byte_perm(a, b, 0x7632);
+            o[(2 * Mpad + k) >> 1] = hi;
+        }
     }
+}
+static void launch_xi_to_bf16(size_t n, int M, int Mpad, int split, const double* x, void* out, cudaStream_t st) {
+    const dim3 grid((unsigned)((n + 7) / 8), n < 4096 ? (unsigned)std::min(Mpad / 64, 65535) : 1u);
+    k_xi_to_bf16<<<grid, 256, 0, st>>>(n, M, Mpad, split, x, (__nv_bfloat16*)out);
 }
 
 // basis [cells][M] FP64 -> [cells][Kp] BF16, split layout (hi, hi, lo).
@@ -333,8 +368,7 @@ fm_status kl_tc_field(fm_ctx* ctx, int level, uint32_t n, const double* d_xi, do
                                               (int)kTcSmem));
         attr = true;
     }
-    k_xi_to_bf16<<<nblk((size_t)n * Mpad), 256, 0, st>>>(n, M, Mpad, ctx->tc.split, d_xi,
-                                                        (__nv_bfloat16*)ctx->tc.xi);
+    launch_xi_to_bf16(n, M, Mpad, ctx->tc.split, d_xi, ctx->tc.xi, st);
     // the coefficient map covers the buffer's capacity; rows >= n are never stored
     const unsigned grid = gemm_grid(ctx, cells, n);
     const double flops = 2.0 * (double)n * cells * Kp;
@@ -382,7 +416,7 @@ fm_status kl_tc_nystrom(fm_ctx* ctx, int q, const double* dVt, const double* d_i
             break;
         }
         // B operand: V^T, split (hi, lo, hi)
-        k_xi_to_bf16<<<nblk((size_t)M * Kpad), 256>>>((size_t)M, nq, Kpad, 1, dVt, (__nv_bfloat16*)B);
+        launch_xi_to_bf16((size_t)M, nq, Kpad, 1, dVt, B, 0);
         CUtensorMap mapB, mapA;
         if (!make_map(&mapB, B, M, Kp, kTcN) || !make_map(&mapA, A, chunk, Kp, kTcM)) {
             set_error(ctx, "kl_basis_build: cuTensorMapEncodeTiled failed");
