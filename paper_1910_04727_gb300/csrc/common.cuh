@@ -119,9 +119,15 @@ struct Ghost {
     int ns;
 };
 
+// Whether the resident kernel takes a grid: its hierarchy (coarsest grid
+// prm.n_coarsest) by powers of two and in shared memory (fmg_resident.cu).
+bool fmg_resident_takes(int n_fine, const fm_solve_params& prm);
+
 // The schedule FM_KERNEL_AUTO takes for S samples of a grid: the resident
 // kernel (one CTA or warp per sample) or the level-wise schedule; the latter
-// always for the energy-optimal step, which the resident kernel lacks.
+// always for the energy-optimal step, which the resident kernel lacks, and for
+// hierarchies it does not take (a caller that gets true here sizes no
+// level-wise scratch).
 // FP64: the level-wise schedule has the higher throughput on every grid, the
 // resident kernel the shorter chain of launches, so it runs batches that it
 // takes in about one wave (fixed schedule) or a few (converged, where the
@@ -135,10 +141,9 @@ struct Ghost {
 // 12.2 / 2.2 at 40000; 32 x 32 2.8 / 0.47 at 1000, 8.6 / 2.5 at 8000), and a converged
 // 64 x 64 batch of at most two samples per SM (2.8 / 2.4 at 300).
 inline bool auto_resident(int n_fine, size_t S, int sms, const fm_solve_params& prm) {
-    if (prm.energy_step) return false;
+    if (prm.energy_step || !fmg_resident_takes(n_fine, prm)) return false;
     if (prm.precision == FM_PREC_MIXED)
         return n_fine <= 32 || (prm.converged && n_fine == 64 && S <= 2 * (size_t)sms);
-    if (n_fine > 64) return false;
     const size_t per_sm = prm.converged ? (n_fine <= 16 ? 32 : n_fine <= 32 ? 12 : 2)
                                         : (n_fine <= 16 ? 8 : n_fine <= 32 ? 4 : 1);
     return S <= per_sm * (size_t)sms;
@@ -427,7 +432,7 @@ fm_status fmg_solve_impl(fm_ctx* ctx, int n_fine, uint32_t S, const double* d_K,
                          const fm_solve_params& prm, double* d_qf, double* d_qc, double* d_p,
                          int32_t* d_status, cudaStream_t stream);
 
-// Sample-resident FMG (fmg_resident.cu); false if the grid does not fit.
+// Sample-resident FMG (fmg_resident.cu); false where fmg_resident_takes is.
 bool fmg_resident_launch(fm_ctx* ctx, int n_fine, int n0, size_t S, const double* d_K,
                          const fm_solve_params& prm, double* qf, double* qc, double* p_out,
                          int32_t* status, cudaStream_t st);

@@ -696,11 +696,24 @@ constexpr size_t kResidentSmemMax = 227 * 1024;
 
 // Grids up to 16 x 16 run one sample per warp (four per CTA, barriers are
 // __syncwarp); larger grids one sample per CTA.
+static int resident_groups(int n_fine) { return n_fine <= 16 ? 4 : 1; }
+static size_t resident_cta_bytes(int n_fine, int n0, bool mixed) {
+    const size_t slot = mixed ? resident_slot_bytes<float>() : resident_slot_bytes<double>();
+    return resident_groups(n_fine) * (slot + resident_smem_bytes(n_fine, n0, mixed, n_fine <= 16));
+}
+
+// Power-of-two hierarchies (shift-and-mask indexing) that fit in shared memory:
+// none above 64 x 64, whose grids the layout's table would not hold either.
+bool fmg_resident_takes(int n_fine, const fm_solve_params& prm) {
+    const int n0 = prm.n_coarsest;
+    return n_fine <= 64 && (n0 & (n0 - 1)) == 0 &&
+           resident_cta_bytes(n_fine, n0, prm.precision == FM_PREC_MIXED) <= kResidentSmemMax;
+}
+
 template <typename T, bool MIXED, bool WARP>
-static bool launch_resident(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st) {
-    const int groups = WARP ? 4 : 1;
-    const size_t smem = groups * (resident_slot_bytes<T>() + resident_smem_bytes(a.n_fine, a.n0, MIXED, WARP));
-    if (smem > kResidentSmemMax) return false;
+static void launch_resident(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st) {
+    const int groups = resident_groups(a.n_fine);
+    const size_t smem = resident_cta_bytes(a.n_fine, a.n0, MIXED);
     // a 32 x 32 sample on 128 threads: four CTAs per SM (shared memory
     // allows four, registers four at 128 threads); measured 1.45x the
     // samples per second of 256 threads (two CTAs per SM), the half-sweeps
@@ -724,13 +737,12 @@ static bool launch_resident(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st)
     }
     k_fmg_resident<T, MIXED, WARP><<<(unsigned)grid, threads, smem, st>>>(b);
     prof_stop(ctx, pi, st, 8.0 * cells + 16.0 * a.S, 0.0);
-    return true;
 }
 
 template <typename T, bool MIXED>
-static bool launch_resident(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st) {
-    if (a.n_fine <= 16) return launch_resident<T, MIXED, true>(ctx, a, st);
-    return launch_resident<T, MIXED, false>(ctx, a, st);
+static void launch_resident(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st) {
+    if (a.n_fine <= 16) launch_resident<T, MIXED, true>(ctx, a, st);
+    else launch_resident<T, MIXED, false>(ctx, a, st);
 }
 
 void resident_init_attributes() {
@@ -747,7 +759,7 @@ void resident_init_attributes() {
 bool fmg_resident_launch(fm_ctx* ctx, int n_fine, int n0, size_t S, const double* d_K,
                          const fm_solve_params& prm, double* qf, double* qc, double* p_out,
                          int32_t* status, cudaStream_t st) {
-    if (n0 & (n0 - 1)) return false;   // power-of-two hierarchies only (shift-and-mask indexing)
+    if (!fmg_resident_takes(n_fine, prm)) return false;
     ResidentArgs a;
     a.n_fine = n_fine;
     a.n0 = n0;
@@ -769,8 +781,9 @@ bool fmg_resident_launch(fm_ctx* ctx, int n_fine, int n0, size_t S, const double
     a.status = status;
     a.again = false;
     a.flops = nullptr;
-    if (prm.precision == FM_PREC_MIXED) return launch_resident<float, true>(ctx, a, st);
-    return launch_resident<double, false>(ctx, a, st);
+    if (prm.precision == FM_PREC_MIXED) launch_resident<float, true>(ctx, a, st);
+    else launch_resident<double, false>(ctx, a, st);
+    return true;
 }
 
 }  // namespace fm
