@@ -133,7 +133,10 @@ typedef struct {
 #define FM_KERNEL_AUTO 0       /* resident where it is the faster schedule (mixed form: up to
                                   32 x 32, and a converged 64 x 64 batch of at most two samples
                                   per SM; FP64: batches up to 64 x 64 of a few samples per SM; not
-                                  with the energy step), else levelwise */
+                                  with the energy step, and only where n_coarsest is 2 or 4), else
+                                  levelwise.  Where the levelwise schedule's scratch finds no room,
+                                  and under a stream capture that would have to allocate it (FP64
+                                  grids up to 16 x 16: under any), resident too where it can */
 #define FM_KERNEL_LEVELWISE 1  /* one kernel per grid operation over all samples */
 #define FM_KERNEL_RESIDENT 2   /* one CTA per sample, hierarchy in shared memory
                                   (n_fine <= 64 in FP64) */

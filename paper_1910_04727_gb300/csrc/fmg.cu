@@ -1330,21 +1330,29 @@ int64_t batch_limit(const fm_ctx* ctx, int n) {
     return std::max<int64_t>(lim, 1);
 }
 
+bool arena_holds(Arena& ar, size_t need) {
+    if (ar.capacity >= need) return true;
+    if (ar.base) cudaFree(ar.base);
+    ar.base = nullptr;
+    ar.capacity = 0;
+    if (cudaMalloc((void**)&ar.base, need) != cudaSuccess) {
+        cudaGetLastError();
+        ar.base = nullptr;
+        return false;
+    }
+    ar.capacity = need;
+    return true;
+}
+
 // Scratch of a level-wise batch of S samples: grows `ar` when it is too small
 // (never while a stream is being captured: callers size it first).
 template <typename T>
 static fm_status carve(fm_ctx* ctx, Arena& ar, Hierarchy<T>& H, int n_fine, int n0, size_t S, const double* d_K,
                        bool mixed, bool converged) {
     const size_t need = hierarchy_bytes(n_fine, n0, S, sizeof(T), mixed, converged);
-    if (ar.capacity < need) {
-        if (ar.base) cudaFree(ar.base);
-        ar.base = nullptr;
-        ar.capacity = 0;
-        if (cudaMalloc((void**)&ar.base, need) != cudaSuccess) {
-            set_error(ctx, "fmg scratch allocation of " + std::to_string(need) + " bytes failed");
-            return FM_ENOMEM;
-        }
-        ar.capacity = need;
+    if (!arena_holds(ar, need)) {
+        set_error(ctx, "fmg scratch allocation of " + std::to_string(need) + " bytes failed");
+        return FM_ENOMEM;
     }
     char* cur = ar.base;
     auto take = [&](size_t bytes) {
@@ -2034,7 +2042,22 @@ fm_status fmg_solve_with(fm_ctx* ctx, Arena& ar, int n_fine, uint32_t S, const d
                  "fmg_solve_batch: the energy-optimal correction step runs in converged mode on the level-wise "
                  "schedule");
     if (S == 0) return FM_OK;
-    if (prm.kernel == FM_KERNEL_RESIDENT || (prm.kernel == FM_KERNEL_AUTO && auto_resident(n_fine, S, ctx->sms, prm))) {
+    bool resident = prm.kernel == FM_KERNEL_RESIDENT;
+    if (prm.kernel == FM_KERNEL_AUTO) {
+        resident = auto_resident(n_fine, S, ctx->sms, prm);
+        // The resident kernel takes no scratch, so it runs what the level-wise schedule
+        // would be faster at but finds no room for: none left, or a stream capture, in
+        // which nothing can be allocated.  FP64 grids up to 16 x 16 take it in every
+        // capture: their graphs keep no address of scratch that a later call may free.
+        if (!resident && !prm.energy_step && fmg_resident_takes(n_fine, prm)) {
+            const size_t need = fmg_levelwise_scratch(ctx, n_fine, S, prm);
+            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+            FM_CUDA_TRY(ctx, cudaStreamIsCapturing(st, &cs));
+            if (cs != cudaStreamCaptureStatusNone) resident = n_fine <= 16 || ar.capacity < need;
+            else resident = !arena_holds(ar, need);
+        }
+    }
+    if (resident) {
         if (fmg_resident_launch(ctx, n_fine, n0, S, d_K, prm, d_qf, d_qc, d_p, d_status, st)) {
             FM_CUDA_TRY(ctx, cudaGetLastError());
             return FM_OK;

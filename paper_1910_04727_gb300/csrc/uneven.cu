@@ -140,21 +140,19 @@ extern "C" fm_status fmg_solve_uneven(fm_ctx* ctx, int32_t n_groups, const fm_ba
     std::vector<cudaStream_t> branch;
     FM_TRY(uneven_prepare(ctx, n_groups, prio, &branch));
     UnevenState* U = uneven_state(ctx);
-    // level-wise scratch is sized before the capture (no allocation inside it)
+    // level-wise scratch is sized before the capture (no allocation inside it); a
+    // group that finds no room for it takes the resident kernel where that can
+    std::vector<char> resident(n_groups, 0);
     for (int g = 0; g < n_groups; ++g) {
         const fm_batch_group& G = groups[g];
-        if (G.count == 0 || resident_grid(ctx, G, *prm)) continue;
+        resident[g] = resident_grid(ctx, G, *prm);
+        if (G.count == 0 || resident[g]) continue;
         const size_t need = fmg_levelwise_scratch(ctx, G.n_fine, G.count, *prm);
-        Arena& a = U->arenas[g];
-        if (a.capacity < need) {
-            if (a.base) cudaFree(a.base);
-            a.base = nullptr;
-            a.capacity = 0;
-            if (cudaMalloc((void**)&a.base, need) != cudaSuccess) {
-                set_error(ctx, "fmg_solve_uneven: scratch allocation of " + std::to_string(need) + " bytes failed");
-                return FM_ENOMEM;
-            }
-            a.capacity = need;
+        if (arena_holds(U->arenas[g], need)) continue;
+        resident[g] = prm->kernel == FM_KERNEL_AUTO && !prm->energy_step && fmg_resident_takes(G.n_fine, *prm);
+        if (!resident[g]) {
+            set_error(ctx, "fmg_solve_uneven: scratch allocation of " + std::to_string(need) + " bytes failed");
+            return FM_ENOMEM;
         }
     }
     FM_CUDA_TRY(ctx, cudaGetLastError());
@@ -170,7 +168,7 @@ extern "C" fm_status fmg_solve_uneven(fm_ctx* ctx, int32_t n_groups, const fm_ba
         if (G.count == 0) continue;
         cudaStreamWaitEvent(branch[g], U->fork, 0);
         fm_solve_params p = *prm;
-        p.kernel = resident_grid(ctx, G, *prm) ? FM_KERNEL_AUTO : FM_KERNEL_LEVELWISE;
+        p.kernel = resident[g] ? FM_KERNEL_RESIDENT : FM_KERNEL_LEVELWISE;
         st = fmg_solve_with(ctx, U->arenas[g], G.n_fine, G.count, G.d_K, p, G.d_qf, G.d_qc, nullptr, G.d_status,
                             branch[g]);
         cudaEventRecord(U->join[g], branch[g]);
@@ -194,7 +192,7 @@ extern "C" fm_status fmg_solve_uneven(fm_ctx* ctx, int32_t n_groups, const fm_ba
     // per group: grid, non-empty, schedule, and whether Q^c is asked for (a
     // converged solve refines its coarse stage only then)
     for (int g = 0; g < n_groups; ++g)
-        key.insert(key.end(), {groups[g].n_fine, groups[g].count > 0, resident_grid(ctx, groups[g], *prm),
+        key.insert(key.end(), {groups[g].n_fine, groups[g].count > 0, resident[g],
                                groups[g].d_qc != nullptr});
     cudaGraphExec_t exec = nullptr;
     for (size_t i = 0; i < U->kept.size() && !exec; ++i) {
