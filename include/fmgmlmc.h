@@ -60,7 +60,8 @@ typedef int32_t fm_status;
 
 /* Arithmetic of the KL field synthesis.
  * AUTO: FP64 in the FP64 form, BF16X3 in the mixed form.
- * FP64: FP64 SIMT contraction.
+ * FP64: split products on the tensor cores, exact below the rounding of their sum,
+ *       up to 512 modes; an FP64 contraction above.
  * BF16: tcgen05 tensor cores, BF16 basis and coefficients, FP32 accumulation
  *       (relative error of g about 2^-8).
  * BF16X3: tcgen05 tensor cores on the split products hi*hi + hi*lo + lo*hi
@@ -251,7 +252,12 @@ fm_status lattice_generating_vector(const fm_ctx* ctx, uint32_t* z);
  * n of a coarser level samples the field at the finest-grid points that
  * injection keeps (cell (i,j) of grid n -> cell (s i, s j) of grid n_ref,
  * s = n_ref / n), so the coarse coefficients of level l and the fine ones of
- * level l-1 coincide.  basis_ref is device memory if on_device, else host. */
+ * level l-1 coincide.  basis_ref is device memory if on_device, else host.
+ * The context holds the basis of every level (8 bytes an entry) and, up to 512
+ * modes, its parts for the tensor cores: in the FP64 mode 18 bytes an entry, modes
+ * rounded up to a multiple of 32 (a level of more than 4 GiB of them, or one that
+ * finds no room, goes without and synthesises in the FP64 pipe); in the BF16 modes
+ * (any number of modes, rounded up to 64) 2, BF16X3 6. */
 fm_status kl_basis_set(fm_ctx* ctx, const double* basis_ref, int32_t on_device);
 
 /* Build the KL basis of the Matern covariance of Sec. 3.1 (smoothness cfg.nu,
@@ -295,7 +301,8 @@ fm_status kl_basis_get(const fm_ctx* ctx, double* basis_ref_out, int32_t on_devi
 /* Field synthesis (Sec. 3.1): d_K[s][c] = exp(sum_k B_l[c][k] d_xi[s*M + k])
  * for the n samples of MLMC level `level` (grid n_level0 << level), in the
  * context's kl_mode; d_K is [n][N_l][N_l] doubles.  The tensor-core forms
- * report a device-side wait that ran out through fm_sync. */
+ * report a device-side wait that ran out through fm_sync.  FP64: a call takes no
+ * scratch and gives the same bits on every stream and under a capture. */
 fm_status kl_field_batch(fm_ctx* ctx, int32_t level, uint32_t n, const double* d_xi,
                          double* d_K, void* stream);
 

@@ -314,14 +314,6 @@ struct OzState {
     void* basis[FM_MAX_LEVELS] = {};   // BF16 digits [cells][9 Mpad] per level
     int* ec[FM_MAX_LEVELS] = {};       // scale exponents of the basis rows
     CUtensorMap mapA[FM_MAX_LEVELS];
-    static constexpr int kStreams = 4;
-    struct Xi {                        // digits of a batch's coefficients, one buffer per stream
-        unsigned long long id = 0;
-        size_t cap = 0;
-        void* digits = nullptr;
-        int* ex = nullptr;
-        CUtensorMap map;
-    } xi[kStreams];
 };
 
 }  // namespace fm

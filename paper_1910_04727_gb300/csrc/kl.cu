@@ -2,8 +2,8 @@
 //
 // kl_field_batch is the contraction K[s][c] = exp(sum_k B[c][k] xi[s][k]):
 // cells x modes by modes x samples.  The FP64 form is a split product on the
-// tensor cores (kl_split.cu) up to 512 modes; above, and where a call cannot
-// take it, the register-tiled SIMT GEMM below, in the FP64 pipe, with the
+// tensor cores (kl_split.cu) up to 512 modes; above, and on levels whose digits
+// find no room, the register-tiled SIMT GEMM below, in the FP64 pipe, with the
 // exponential fused into the epilogue, so g is never written to memory.
 #include <cublas_v2.h>
 #include <cusolverDn.h>

@@ -19,13 +19,20 @@
 // takes M operations per field value and its exponential 21; here the
 // conversion takes 3 and the exponential 11 (fm_exp below), and the 45 M
 // tensor-core products per value run beside it, a tile ahead.  2000 fields of
-// 64 x 64 cells from 128 modes: 283 us (388 with a tile per CTA and two CTAs an
+// 64 x 64 cells from 128 modes: 279 us (388 with a tile per CTA and two CTAs an
 // SM, whose loads and products were not hidden), 2035 by the FP64 contraction (95% of that
 // pipe), with errors against 128-bit arithmetic of 8.2e-17 (rms; at most
-// 4.9e-16) against its 6.9e-16 (6.2e-15).
+// 4.9e-16) against its 6.9e-16 (6.2e-15).  From 256 modes up the products bound
+// it: 100 fields of 256 x 256 from 256 modes 351 us (3791 by the contraction), 500 of 64 x
+// 64 from 512 modes 198 (2134).
 //
 // A tile is 128 cells x 32 samples: eight 128 x 32 accumulators in 256 columns
 // of tensor memory, the digits of 32 modes per stage (64-byte swizzle, 90 KB).
+// The basis is cut once, when it is installed; the coefficients are cut by four
+// warps of every CTA, straight into the operand stage, so that a call keeps
+// nothing: no buffer to size, to share between streams or to hold under a capture.
+// Each tile cuts its 32 rows anew, in integers beside the FP64 pipe (a kernel of
+// its own for them and their digits by TMA took 284 us for the first case above).
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
@@ -41,12 +48,14 @@ constexpr int kOzM = 128;      // cells per tile (MMA M)
 constexpr int kOzN = 32;       // samples per tile (MMA N)
 constexpr int kOzK = 32;       // modes per stage (one 64-byte swizzle row)
 constexpr int kOzEpi = 256;          // threads that drain and store
-constexpr int kOzThreads = kOzEpi + 64;
+constexpr int kOzCut = 128;          // threads that cut the coefficients
+constexpr int kOzThreads = kOzEpi + 64 + kOzCut;
 constexpr int kOzStages = 2;
 constexpr int kOzMaxM = 512;   // 512 modes x 8 pairs x 2^12 = 2^24
 constexpr uint32_t kOzABytes = kOzM * kOzK * 2, kOzBBytes = kOzN * kOzK * 2;
 constexpr uint32_t kOzStage = kOzDigits * (kOzABytes + kOzBBytes);
-constexpr size_t kOzSmem = 1024 + kOzStages * kOzStage + 64 * 16 + 128;
+constexpr int kOzRowSets = 4;  // tiles whose coefficient rows' scales are kept (see the cutting warps)
+constexpr size_t kOzSmem = 1024 + kOzStages * kOzStage + 64 * 16 + kOzRowSets * kOzN * 4 + 192;
 constexpr int kOzNoScale = -(1 << 28);   // exponent of a row that is not split (a value that is not finite, or far out)
 // Largest sum of a pair's scale exponents that is split.  What is left out is
 // relative to the scales, not to the sum, so a large entry that meets a zero
@@ -154,20 +163,53 @@ __device__ __forceinline__ uint64_t sdesc_kmajor_sw64(uint32_t saddr) {
     return d;
 }
 
+// The scale exponent of a row whose largest biased exponent is top: 2^e is at
+// least twice the largest magnitude.  Rows with values that are not finite, or
+// with scales far from 1, are left to the plain sum (kOzNoScale).
+__device__ __forceinline__ int row_scale(int top) {
+    const int e = top - 1023 + 2;
+    if (top == 0) return 0;
+    return top != 0x7FF && e < 200 && e > -200 ? e : kOzNoScale;
+}
+// x below the scale 2^e as a 63-bit fixed-point number (units of 2^(e - 63)).
+__device__ __forceinline__ long long row_fixed(double x, int e) {
+    const long long bits = __double_as_longlong(x);
+    const int be = (int)(bits >> 52) & 0x7FF;
+    if (be == 0 || e == kOzNoScale) return 0;
+    const long long m = (bits & 0xFFFFFFFFFFFFFLL) | (1LL << 52);   // at exponent be - 1075
+    const int sh = be - 1075 - (e - kOzDigits * kOzBits);           // at most 9
+    long long v = 0;
+    if (sh >= 0) v = m << sh;
+    else if (sh > -54) v = (m + (1LL << (-sh - 1))) >> -sh;
+    return bits < 0 ? -v : v;
+}
+// Digit i of v, balanced, cut from the low end (i = kOzDigits - 1 first, 0 last),
+// as the bits of the FP32 number d 2^(-7 i), whose upper half is its BF16.
+__device__ __forceinline__ unsigned next_digit(long long& v, int i) {
+    const int d = i > 0 ? ((int)(v + 64) & 127) - 64 : (int)v;
+    v = (v - d) >> kOzBits;
+    const float f = __uint_as_float(0x4B400000u + (unsigned)d) - 12582912.0f;   // 1.5 2^23 + d
+    return __float_as_uint(f * (1.0f / (float)(1LL << (kOzBits * i))));
+}
+
 // Persistent: CTA b takes tiles b, b + gridDim.x, ... (sample tiles fastest).
-// Warps 0 .. 7 drain, warp 8 (one thread) loads, warp 9 (one thread) issues the
-// products; two stages of operands and two sets of accumulators, so the next
-// tile's products run under this one's epilogue.
+// Warps 0 .. 7 drain, warp 8 (one thread) loads the basis digits, warp 9 (one
+// thread) issues the products, warps 10 .. 13 cut the coefficients; two stages of
+// operands and two sets of accumulators, so the next tile's products run under
+// this one's epilogue.
 __global__ void __launch_bounds__(kOzThreads, 1)
-    k_kl_split(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int cells, int S,
-               int M, int Mpad, const int* __restrict__ ec, const int* __restrict__ ex, const double* __restrict__ B,
-               const double* __restrict__ xi, double* __restrict__ K, int* __restrict__ err) {
+    k_kl_split(const __grid_constant__ CUtensorMap mapA, int cells, int S, int M, int Mpad,
+               const int* __restrict__ ec, const double* __restrict__ B, const double* __restrict__ xi,
+               double* __restrict__ K, int* __restrict__ err) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = tc::smem_u32(smem_raw);
     uint8_t* stage = smem_raw + ((1024 - (raw & 1023)) & 1023);   // per stage: A digits, then B digits
     double2* tab = reinterpret_cast<double2*>(stage + kOzStages * kOzStage);
-    uint64_t* full = reinterpret_cast<uint64_t*>(tab + 64);
-    uint64_t* empty = full + kOzStages;
+    int* ex = reinterpret_cast<int*>(tab + 64);   // the coefficient rows' scales, by tile (kOzRowSets in turn)
+    uint64_t* full = reinterpret_cast<uint64_t*>(ex + kOzRowSets * kOzN);   // basis digits in
+    uint64_t* cut = full + kOzStages;             // coefficient digits in
+    uint64_t* scaled = cut + kOzStages;           // a tile's scales in
+    uint64_t* empty = scaled + kOzRowSets;
     uint64_t* tfull = empty + kOzStages;    // accumulators ready, by set
     uint64_t* tempty = tfull + 2;           // accumulators drained
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
@@ -177,15 +219,16 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     if (threadIdx.x == 0) {
         for (int i = 0; i < kOzStages; ++i) {
             tc::mbar_init(&full[i], 1);
+            tc::mbar_init(&cut[i], kOzCut / 32);
             tc::mbar_init(&empty[i], 1);
         }
+        for (int i = 0; i < kOzRowSets; ++i) tc::mbar_init(&scaled[i], kOzN);
         for (int i = 0; i < 2; ++i) {
             tc::mbar_init(&tfull[i], 1);
             tc::mbar_init(&tempty[i], kOzEpi);
         }
         tc::fence_barrier_init();
         tc::prefetch_tensormap(&mapA);
-        tc::prefetch_tensormap(&mapB);
     }
     if (warp == 0) tc::tmem_alloc(tmem_slot, 2 * kOzAcc * kOzN);
     tc::fence_before_sync();
@@ -198,17 +241,14 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             int q = 0;   // stage loads so far
             bool ok = true;
             for (unsigned tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x) {
-                const int s0 = (int)(tile % stiles) * kOzN, c0 = (int)(tile / stiles) * kOzM;
+                const int c0 = (int)(tile / stiles) * kOzM;
                 for (int kb = 0; kb < kblocks; ++kb) {
                     const int st = q % kOzStages, round = q / kOzStages;
                     if (round > 0 && !(ok = tc::mbar_wait(&empty[st], (round - 1) & 1, err))) break;
                     uint8_t* a = stage + st * kOzStage;
-                    uint8_t* b = a + kOzDigits * kOzABytes;
-                    tc::mbar_arrive_expect_tx(&full[st], kOzStage);
-                    for (int i = 0; i < kOzDigits; ++i) {
+                    tc::mbar_arrive_expect_tx(&full[st], kOzDigits * kOzABytes);
+                    for (int i = 0; i < kOzDigits; ++i)
                         tc::tma_load_2d(a + i * kOzABytes, &mapA, &full[st], i * Mpad + kb * kOzK, c0);
-                        tc::tma_load_2d(b + i * kOzBBytes, &mapB, &full[st], i * Mpad + kb * kOzK, s0);
-                    }
                     ++q;
                 }
             }
@@ -227,20 +267,104 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                 for (int kb = 0; kb < kblocks; ++kb, ++q) {
                     const int st = q % kOzStages;
                     if (!(ok = tc::mbar_wait(&full[st], (q / kOzStages) & 1, err))) break;
+                    if (!(ok = tc::mbar_wait(&cut[st], (q / kOzStages) & 1, err))) break;
                     tc::fence_after_sync();
-                    const uint32_t sa = tc::smem_u32(stage + st * kOzStage), sb = sa + kOzDigits * kOzABytes;
+                    const uint32_t sa = tc::smem_u32(stage + st * kOzStage);
+                    const uint64_t da = sdesc_kmajor_sw64(sa), db = sdesc_kmajor_sw64(sa + kOzDigits * kOzABytes);
+                    // Unrolled, descriptors by constant steps: formed anew for every product,
+                    // their instructions held the tensor cores up (one thread issues, in a warp
+                    // beside three others of its scheduler): 100 fields of 256 x 256 from 256 modes
+                    // 475 us, 351 so.
+#pragma unroll
                     for (int i = 0; i < kOzDigits; ++i)
-                        for (int j = 0; i + j < kOzDigits; ++j) {
+#pragma unroll
+                        for (int j = 0; j < kOzDigits - i; ++j) {
                             const int t = i + j < kOzAcc ? i + j : kOzAcc - 1;
-                            const uint32_t a = sa + i * kOzABytes, b = sb + j * kOzBBytes;
 #pragma unroll
                             for (int k = 0; k < kOzK / 16; ++k)
-                                tc::mma_bf16(acc + t * kOzN, sdesc_kmajor_sw64(a + 32 * k),
-                                             sdesc_kmajor_sw64(b + 32 * k), idesc, (kb | i | k) != 0 || j >= kOzAcc);
+                                tc::mma_bf16(acc + t * kOzN, da + (i * kOzABytes + 32 * k) / 16,
+                                             db + (j * kOzBBytes + 32 * k) / 16, idesc,
+                                             (kb | i | k) != 0 || j >= kOzAcc);
                         }
                     tc::mma_commit(&empty[st]);
                 }
                 tc::mma_commit(&tfull[set]);
+            }
+        }
+    } else if (warp >= 10) {
+        // Eight rows a warp.  The digits of modes 2 p, 2 p + 1 of two rows at a time: lane
+        // 16 h + p has row h, its 4 bytes of the row's 64 at 4 p, whose 16-byte chunk the
+        // swizzle exchanges by bits 7, 8 of the address (the row's bits 1, 2).
+        const int r0 = 8 * (warp - 10), p = lane & 15, half = lane >> 4;
+        int q = 0, it = 0;
+        bool ok = true;
+        for (unsigned tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x, ++it) {
+            const int s0 = (int)(tile % stiles) * kOzN;
+            const double* rows[8];   // rows past the batch: the last one's, cut to zero below and never stored
+            int top[8];              // largest biased exponent of each row
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                rows[r] = xi + (size_t)min(s0 + r0 + r, S - 1) * M;
+                top[r] = 0;
+            }
+#pragma unroll 2
+            for (int k = lane; k < M; k += 32) {   // (sixteen loads in flight)
+#pragma unroll
+                for (int r = 0; r < 8; ++r) top[r] = max(top[r], (__double2hiint(rows[r][k]) >> 20) & 0x7FF);
+            }
+            int e_mine = 0;   // lane r: the scale of row r0 + r
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                const int e = row_scale(__reduce_max_sync(0xffffffffu, top[r]));
+                if (lane == r) e_mine = s0 + r0 + r < S ? e : 0;
+            }
+            for (int kb = 0; kb < kblocks; ++kb, ++q) {
+                const int st = q % kOzStages, round = q / kOzStages, k = kb * kOzK + 2 * p;
+                // cut before the stage is free: between the products that read it last and those
+                // that read it next there are the stores alone
+                unsigned dig[4][kOzDigits];
+                {
+                    double x[4][2];
+#pragma unroll
+                    for (int r2 = 0; r2 < 4; ++r2) {
+                        const int s = s0 + r0 + 2 * r2 + half;
+                        const double* row = xi + (size_t)s * M;
+                        x[r2][0] = s < S && k < M ? row[k] : 0.0;
+                        x[r2][1] = s < S && k + 1 < M ? row[k + 1] : 0.0;
+                    }
+#pragma unroll
+                    for (int r2 = 0; r2 < 4; ++r2) {
+                        const int e = __shfl_sync(0xffffffffu, e_mine, 2 * r2 + half);
+                        long long v0 = row_fixed(x[r2][0], e), v1 = row_fixed(x[r2][1], e);
+#pragma unroll
+                        for (int i = kOzDigits - 1; i >= 0; --i) {
+                            const unsigned d0 = next_digit(v0, i), d1 = next_digit(v1, i);
+                            dig[r2][i] = __byte_perm(d0, d1, 0x7632);
+                        }
+                    }
+                }
+                if (round > 0) {
+                    ok = __all_sync(0xffffffffu, tc::mbar_wait(&empty[st], (round - 1) & 1, err));
+                    if (!ok) break;
+                }
+                // The set of scales of kOzRowSets tiles ago is free: this stage was last read
+                // by products of a tile at most two before this one, and these began once
+                // the tile two before theirs was drained.
+                if (kb == 0 && lane < 8) {
+                    ex[(it % kOzRowSets) * kOzN + r0 + lane] = e_mine;
+                    tc::mbar_arrive(&scaled[it % kOzRowSets]);
+                }
+                uint8_t* b = stage + st * kOzStage + kOzDigits * kOzABytes;
+#pragma unroll
+                for (int r2 = 0; r2 < 4; ++r2) {
+                    const int r = r0 + 2 * r2 + half;
+                    uint8_t* dst = b + 64 * r + (((p >> 2) ^ ((r >> 1) & 3)) << 4) + 4 * (p & 3);
+#pragma unroll
+                    for (int i = 0; i < kOzDigits; ++i) *reinterpret_cast<unsigned*>(dst + i * kOzBBytes) = dig[r2][i];
+                }
+                tc::fence_proxy_async_smem();   // the stores are operands of the tensor cores
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&cut[st]);
             }
         }
     } else {
@@ -251,7 +375,10 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             const int c = c0 + 32 * (warp & 3) + lane;
             const int e_c = c < cells ? ec[c] : 0;
             // all lanes or none (the loads below are warp-wide)
-            const bool ok = __all_sync(0xffffffffu, tc::mbar_wait(&tfull[set], (it >> 1) & 1, err));
+            bool ok = __all_sync(0xffffffffu, tc::mbar_wait(&scaled[it % kOzRowSets], (it / kOzRowSets) & 1, err));
+            if (!ok) break;
+            const int e_row = ex[(it % kOzRowSets) * kOzN + lane];   // lane r: the scale of row r
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(&tfull[set], (it >> 1) & 1, err));
             if (!ok) break;
             tc::fence_after_sync();
             const uint32_t row = tmem + set * (kOzAcc * kOzN) + ((uint32_t)(32 * (warp & 3)) << 16);
@@ -269,8 +396,8 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const int s = s0 + col + i;
+                    const int e = e_c + __shfl_sync(0xffffffffu, e_row, col + i);
                     if (c >= cells || s >= S) continue;
-                    const int e = e_c + ex[s];
                     double g;
                     if (e > -(1 << 20) && e <= kOzMaxScale) {
                         g = oz_join(acc, i, e);
@@ -301,32 +428,14 @@ __global__ void k_split_rows(size_t rows, int M, int Mpad, const double* __restr
     int top = 0;   // largest biased exponent of the row
     for (int k = lane; k < M; k += 32) top = max(top, (__double2hiint(row[k]) >> 20) & 0x7FF);
     top = __reduce_max_sync(0xffffffffu, top);
-    // 2^e is at least twice the largest magnitude; rows with values that are
-    // not finite, or with scales far from 1, are left to the plain sum
-    const int e = top - 1023 + 2;
-    const bool split = top != 0x7FF && e < 200 && (e > -200 || top == 0);
-    if (lane == 0) exps[r] = split ? (top == 0 ? 0 : e) : kOzNoScale;
+    const int e = row_scale(top);
+    if (lane == 0) exps[r] = e;
     __nv_bfloat16* o = out + r * (size_t)(kOzDigits * Mpad);
     for (int k = lane; k < Mpad; k += 32) {
-        long long v = 0;
-        if (k < M && split && top != 0) {
-            const long long bits = __double_as_longlong(row[k]);
-            const int be = (int)(bits >> 52) & 0x7FF;
-            if (be != 0) {
-                // mantissa 2^52 .. 2^53 at exponent be - 1075; in units of 2^(e - 63)
-                const long long m = (bits & 0xFFFFFFFFFFFFFLL) | (1LL << 52);
-                const int sh = be - 1075 - (e - kOzDigits * kOzBits);   // at most 9
-                if (sh >= 0) v = m << sh;
-                else if (sh > -54) v = (m + (1LL << (-sh - 1))) >> -sh;
-                if (bits < 0) v = -v;
-            }
-        }
+        long long v = k < M ? row_fixed(row[k], e) : 0;
 #pragma unroll
-        for (int i = kOzDigits - 1; i >= 0; --i) {
-            const int d = i > 0 ? ((int)(v + 64) & 127) - 64 : (int)v;
-            v = (v - d) >> kOzBits;
-            o[(size_t)i * Mpad + k] = __float2bfloat16_rn((float)d * (1.0f / (float)(1LL << (kOzBits * i))));
-        }
+        for (int i = kOzDigits - 1; i >= 0; --i)
+            o[(size_t)i * Mpad + k] = __ushort_as_bfloat16((unsigned short)(next_digit(v, i) >> 16));
     }
 }
 
@@ -385,63 +494,22 @@ void kl_split_free(fm_ctx* ctx) {
         cudaFree(ctx->oz.basis[l]);
         cudaFree(ctx->oz.ec[l]);
     }
-    for (OzState::Xi& x : ctx->oz.xi) {
-        cudaFree(x.digits);
-        cudaFree(x.ex);
-    }
 }
 
-// Fields of n samples of `level` into d_K; false: the caller's FP64
-// contraction serves this call (no digits of this level, a stream beyond the
-// kept buffers, or a stream capture, whose graph would keep a buffer's address).
+// Fields of n samples of `level` into d_K; false: no digits of this level are
+// installed, and the caller's FP64 contraction serves the call.
 bool kl_split_field(fm_ctx* ctx, int level, uint32_t n, const double* d_xi, double* d_K, cudaStream_t st,
                     fm_status* status) {
     OzState& z = ctx->oz;
     *status = FM_OK;
     if (!z.have[level]) return false;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    unsigned long long id = 0;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone ||
-        cudaStreamGetId(st, &id) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    // the digits of xi: one buffer per stream (calls on other streams may
-    // overlap this one), up to kStreams of them
-    OzState::Xi* x = nullptr;
-    for (OzState::Xi& c : z.xi)
-        if (c.cap && c.id == id) x = &c;
-    for (OzState::Xi& c : z.xi)
-        if (!x && !c.cap) x = &c;
-    if (!x) return false;
-    if (x->cap < n) {
-        cudaFree(x->digits);
-        cudaFree(x->ex);
-        x->digits = nullptr;
-        x->ex = nullptr;
-        x->cap = 0;
-        if (cudaMalloc(&x->digits, (size_t)n * kOzDigits * z.Mpad * 2) != cudaSuccess ||
-            cudaMalloc((void**)&x->ex, (size_t)n * sizeof(int)) != cudaSuccess ||
-            !oz_map(&x->map, x->digits, n, (uint64_t)kOzDigits * z.Mpad, kOzN)) {
-            cudaGetLastError();
-            cudaFree(x->digits);
-            cudaFree(x->ex);
-            x->digits = nullptr;
-            x->ex = nullptr;
-            return false;
-        }
-        x->cap = n;
-        x->id = id;
-    }
     const int N = grid_of_level(ctx, level), cells = N * N, M = ctx->cfg.M;
-    k_split_rows<<<warps_grid(n), 256, 0, st>>>(n, M, z.Mpad, d_xi, (__nv_bfloat16*)x->digits, x->ex);
     const size_t tiles = (size_t)((n + kOzN - 1) / kOzN) * ((cells + kOzM - 1) / kOzM);
     const unsigned grid = (unsigned)std::min<size_t>(tiles, (size_t)std::max(ctx->sms, 1));
     FM_TIMED(ctx, kFamKlGemm, st, 8.0 * ((double)n * M + (double)cells * M + (double)n * cells),
              2.0 * n * (double)cells * M,
-             k_kl_split<<<grid, kOzThreads, kOzSmem, st>>>(z.mapA[level], x->map, cells, (int)n, M, z.Mpad,
-                                                           z.ec[level], x->ex, ctx->d_basis[level], d_xi, d_K,
-                                                           ctx->tc.err));
+             k_kl_split<<<grid, kOzThreads, kOzSmem, st>>>(z.mapA[level], cells, (int)n, M, z.Mpad, z.ec[level],
+                                                           ctx->d_basis[level], d_xi, d_K, ctx->tc.err));
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_error(ctx, std::string("kl_field_batch: ") + cudaGetErrorString(e));
