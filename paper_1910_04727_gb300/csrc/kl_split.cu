@@ -19,7 +19,7 @@
 // takes M operations per field value and its exponential 21; here the
 // conversion takes 3 and the exponential 11 (fm_exp below), and the 45 M
 // tensor-core products per value run beside it, a tile ahead.  2000 fields of
-// 64 x 64 cells from 128 modes: 279 us (388 with a tile per CTA and two CTAs an
+// 64 x 64 cells from 128 modes: 275 us (388 with a tile per CTA and two CTAs an
 // SM, whose loads and products were not hidden), 2035 by the FP64 contraction (95% of that
 // pipe), with errors against 128-bit arithmetic of 8.2e-17 (rms; at most
 // 4.9e-16) against its 6.9e-16 (6.2e-15).  From 256 modes up the products bound
@@ -57,12 +57,16 @@ constexpr uint32_t kOzStage = kOzDigits * (kOzABytes + kOzBBytes);
 constexpr int kOzRowSets = 4;  // tiles whose coefficient rows' scales are kept (see the cutting warps)
 constexpr size_t kOzSmem = 1024 + kOzStages * kOzStage + 64 * 16 + kOzRowSets * kOzN * 4 + 192;
 constexpr int kOzNoScale = -(1 << 28);   // exponent of a row that is not split (a value that is not finite, or far out)
-// Largest sum of a pair's scale exponents that is split.  What is left out is
-// relative to the scales, not to the sum, so a large entry that meets a zero
-// coefficient would cost digits (2^40 against 0: 1e-6 of the field); below
-// this line it is under 2^-50 of the field.  Fields reach it only where one mode
-// alone contributes 64 or more to the logarithm (in use the sum is 5 to 7).
-constexpr int kOzMaxScale = 10;
+// Largest sum of a pair's scale exponents that is split whatever the sum of its
+// products.  What is left out is relative to the scales (below 2^-60 of their
+// product), not to the sum, so a large entry that meets a zero coefficient would
+// cost digits (2^40 against 0: 1e-6 of the field); up to this line it is under
+// 2^-50 of the field.  The line is on the product of the two rows' largest
+// magnitudes, whichever modes hold them.  Past it a pair is split where its sum g is
+// as large as kOzSumBits allow: the part left out is then below half an ulp of g.
+// (A constant of -120 in the logarithm takes every pair past the line: 2000 fields of
+// 64 x 64 from 128 modes 4.02 ms by plain sums, 2.05 by the FP64 contraction, 0.28 so.)
+constexpr int kOzMaxScale = 10, kOzSumBits = 6, kOzFarScale = 400;
 constexpr size_t kOzMaxBytes = (size_t)4 << 30;   // most digits kept per level
 
 // 2^(j / 64) as the sum of two doubles.
@@ -398,10 +402,13 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                     const int s = s0 + col + i;
                     const int e = e_c + __shfl_sync(0xffffffffu, e_row, col + i);
                     if (c >= cells || s >= S) continue;
-                    double g;
-                    if (e > -(1 << 20) && e <= kOzMaxScale) {
+                    double g = 0.0;
+                    bool split = e > -(1 << 20) && e <= kOzFarScale;
+                    if (split) {
                         g = oz_join(acc, i, e);
-                    } else {   // a row or a pair that is not split: the plain sum
+                        split = e <= kOzMaxScale || e <= ((__double2hiint(g) >> 20) & 0x7FF) - 1023 + kOzSumBits;
+                    }
+                    if (!split) {   // a row or a pair that is not split: the plain sum
                         g = 0.0;
                         for (int k = 0; k < M; ++k) g = fma(xi[(size_t)s * M + k], B[(size_t)c * M + k], g);
                     }
