@@ -302,7 +302,11 @@ fm_status kl_basis_get(const fm_ctx* ctx, double* basis_ref_out, int32_t on_devi
  * for the n samples of MLMC level `level` (grid n_level0 << level), in the
  * context's kl_mode; d_K is [n][N_l][N_l] doubles.  The tensor-core forms
  * report a device-side wait that ran out through fm_sync.  FP64: a call takes no
- * scratch and gives the same bits on every stream and under a capture. */
+ * scratch and gives the same bits on every stream and under a capture.  BF16,
+ * BF16X3: calls share a buffer of the context that grows with the largest n; calls on
+ * several streams wait for one another on the device.  A captured call uses the
+ * buffer of its capture: make one call of the largest n first, and order the graph's
+ * launches with the context's other field calls. */
 fm_status kl_field_batch(fm_ctx* ctx, int32_t level, uint32_t n, const double* d_xi,
                          double* d_K, void* stream);
 

@@ -91,6 +91,11 @@ extern "C" fm_status fm_create(const fm_config* cfg, fm_ctx** out) {
         }
         ctx->h_lattice_z = *z;
     }
+    if (ctx->tc.xi_order.create() != cudaSuccess) {
+        fm_destroy(ctx);
+        set_error(nullptr, "fm_create: event creation failed");
+        return FM_ECUDA;
+    }
     cudaDeviceGetStreamPriorityRange(&ctx->prio_lo, &ctx->prio_hi);
     ctx->prio_lo = std::min(ctx->prio_lo, ctx->prio_hi + fm_ctx::kPrioLevels - 1);
     for (int p = ctx->prio_hi; p <= ctx->prio_lo; ++p) {
@@ -128,6 +133,7 @@ extern "C" void fm_destroy(fm_ctx* ctx) {
         if (s) cudaStreamDestroy(s);
     for (int l = 0; l < FM_MAX_LEVELS; ++l) cudaFree(ctx->tc.basis[l]);
     cudaFree(ctx->tc.xi);
+    ctx->tc.xi_order.free();
     cudaFree(ctx->tc.err);
     kl_split_free(ctx);
     delete ctx;

@@ -288,6 +288,37 @@ struct Arena {
     size_t used = 0;
 };
 
+// Order of the calls that share a buffer of the context: a call waits, on its own
+// stream, for the one before, whichever stream that ran on.  Calls under a stream
+// capture are left out (an event of another stream cannot be waited for there): their
+// graphs' launches are the caller's to order.
+struct StreamOrder {
+    cudaEvent_t done = nullptr;
+    bool used = false;
+    bool skip = false;      // this call is being captured
+    bool on_null = false;   // the call before ran on the legacy stream (the one that is never another)
+    cudaError_t create() { return cudaEventCreateWithFlags(&done, cudaEventDisableTiming); }
+    cudaError_t begin(cudaStream_t st) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        const cudaError_t e = cudaStreamIsCapturing(st, &cs);
+        skip = cs != cudaStreamCaptureStatusNone;
+        if (e != cudaSuccess || skip || !used || (on_null && !st)) return e;
+        return cudaStreamWaitEvent(st, done, 0);
+    }
+    cudaError_t end(cudaStream_t st) {
+        if (skip) return cudaSuccess;
+        const cudaError_t e = cudaEventRecord(done, st);
+        used = used || e == cudaSuccess;
+        on_null = !st;
+        return e;
+    }
+    void free() {
+        if (done) cudaEventDestroy(done);
+        done = nullptr;
+        used = false;
+    }
+};
+
 // Smoother launch shape per (precision, grid): chosen by fm_autotune.
 struct TuneTable {
     int32_t n[2][16] = {};        // grid the entry was tuned for (0: none)
@@ -304,6 +335,7 @@ struct TcState {
     CUtensorMap mapB;
     void* xi = nullptr;                // BF16 [capacity][Kp]
     size_t xi_capacity = 0, mapB_rows = 0;
+    StreamOrder xi_order;              // calls on several streams share xi
     int* err = nullptr;                // device flag: a bounded wait ran out
 };
 

@@ -368,6 +368,7 @@ fm_status kl_tc_field(fm_ctx* ctx, int level, uint32_t n, const double* d_xi, do
                                               (int)kTcSmem));
         attr = true;
     }
+    FM_CUDA_TRY(ctx, ctx->tc.xi_order.begin(st));
     launch_xi_to_bf16(n, M, Mpad, ctx->tc.split, d_xi, ctx->tc.xi, st);
     // the coefficient map covers the buffer's capacity; rows >= n are never stored
     const unsigned grid = gemm_grid(ctx, cells, n);
@@ -378,6 +379,7 @@ fm_status kl_tc_field(fm_ctx* ctx, int level, uint32_t n, const double* d_xi, do
                                                         ctx->tc.mapB, cells, (int)n,
                                                         Kp / kTcK, d_K, ctx->tc.err, nullptr));
     FM_CUDA_TRY(ctx, cudaGetLastError());
+    FM_CUDA_TRY(ctx, ctx->tc.xi_order.end(st));
     return FM_OK;
 }
 
