@@ -327,7 +327,9 @@ fm_status kl_field_batch(fm_ctx* ctx, int32_t level, uint32_t n, const double* d
  * tolerance, not bit for bit.  d_p (nullable) the finest solution
  * [n][n_fine][n_fine]; d_status (nullable) per-sample FM_OK / FM_ENOTCONV.
  * n_fine must be n_coarsest times a power of two.  Scratch is owned by the
- * context.  prm->kernel picks the schedule: the resident one (the whole
+ * context: levelwise calls on several streams share it and wait for one another
+ * on the device (captured ones excepted: order their graphs' launches, and let no
+ * later call need more scratch).  prm->kernel picks the schedule: the resident one (the whole
  * hierarchy of a sample in shared memory, n_fine <= 64) or the level-wise
  * one (any n_fine up to 8192); both run FP64 and mixed, fixed and converged
  * (the energy step: level-wise only). */

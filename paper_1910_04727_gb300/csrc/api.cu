@@ -91,7 +91,7 @@ extern "C" fm_status fm_create(const fm_config* cfg, fm_ctx** out) {
         }
         ctx->h_lattice_z = *z;
     }
-    if (ctx->tc.xi_order.create() != cudaSuccess) {
+    if (ctx->tc.xi_order.create() != cudaSuccess || ctx->arena_order.create() != cudaSuccess) {
         fm_destroy(ctx);
         set_error(nullptr, "fm_create: event creation failed");
         return FM_ECUDA;
@@ -119,6 +119,7 @@ extern "C" void fm_destroy(fm_ctx* ctx) {
     cudaFree(ctx->d_sobol_V);
     cudaFree(ctx->d_lattice_z);
     cudaFree(ctx->arena.base);
+    ctx->arena_order.free();
     cudaFree(ctx->d_xi);
     cudaFree(ctx->d_K);
     cudaFree(ctx->d_q);

@@ -366,6 +366,7 @@ struct fm_ctx {
     std::vector<uint32_t> h_lattice_z;
     // scratch
     fm::Arena arena;
+    fm::StreamOrder arena_order;     // calls on several streams share arena
     double* d_xi = nullptr;          // points of the current batch
     size_t xi_capacity = 0;
     double* d_K = nullptr;           // fields of the current batch

@@ -2066,9 +2066,15 @@ fm_status fmg_solve_with(fm_ctx* ctx, Arena& ar, int n_fine, uint32_t S, const d
                      "fmg_solve_batch: the resident schedule needs the hierarchy in shared memory "
                      "(n_fine <= 64) and a power-of-two coarsest grid (2 or 4)");
     }
-    if (prm.precision == FM_PREC_MIXED)
-        return levelwise<float>(ctx, ar, n_fine, n0, S, d_K, prm, d_qf, d_qc, d_p, d_status, st);
-    return levelwise<double>(ctx, ar, n_fine, n0, S, d_K, prm, d_qf, d_qc, d_p, d_status, st);
+    // the context's own scratch serves calls on any stream, one after the other
+    // (branches of an uneven batch have scratch of their own)
+    const bool shared = &ar == &ctx->arena;
+    if (shared) FM_CUDA_TRY(ctx, ctx->arena_order.begin(st));
+    const fm_status rs = prm.precision == FM_PREC_MIXED
+                             ? levelwise<float>(ctx, ar, n_fine, n0, S, d_K, prm, d_qf, d_qc, d_p, d_status, st)
+                             : levelwise<double>(ctx, ar, n_fine, n0, S, d_K, prm, d_qf, d_qc, d_p, d_status, st);
+    if (shared) FM_CUDA_TRY(ctx, ctx->arena_order.end(st));
+    return rs;
 }
 
 // ------------------------------------------------------------------ allocation-free variant

@@ -40,3 +40,18 @@ def test_tensor_core_fields(kl_mode):
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(out, want[1])
+
+
+@pytest.mark.parametrize("n,S,kw", [(16, 4000, {}), (64, 600, {}), (64, 400, dict(kernel=1)),
+                                    (128, 40, dict(precision=1, converged=1, tol=1e-10, max_cycles=100))])
+def test_level_wise_solves(n, S, kw):
+    import paper_1910_04727_gb300 as fm
+    import workloads as W
+    c = fm.Context(1, n, 8)
+    Ks = [torch.tensor(W.smooth_lognormal_field(n, S=8, tag=5600 + n + q), device="cuda").repeat(S // 8 - q, 1, 1)
+          for q in range(4)]
+    want = [c.fmg_solve_batch(K, want_p=True, **kw) for K in Ks]
+    for w, outs in zip(want, _overlapped(lambda K: c.fmg_solve_batch(K, want_p=True, **kw), Ks, rounds=3)):
+        for out in outs:
+            for x, y in zip(w, out):
+                assert torch.equal(x, y)
