@@ -19,11 +19,11 @@
 // takes M operations per field value and its exponential 21; here the
 // conversion takes 3 and the exponential 11 (fm_exp below), and the 45 M
 // tensor-core products per value run beside it, a tile ahead.  2000 fields of
-// 64 x 64 cells from 128 modes: 275 us (388 with a tile per CTA and two CTAs an
+// 64 x 64 cells from 128 modes: 272 us (388 with a tile per CTA and two CTAs an
 // SM, whose loads and products were not hidden), 2035 by the FP64 contraction (95% of that
 // pipe), with errors against 128-bit arithmetic of 8.2e-17 (rms; at most
 // 4.9e-16) against its 6.9e-16 (6.2e-15).  From 256 modes up the products bound
-// it: 100 fields of 256 x 256 from 256 modes 351 us (3791 by the contraction), 500 of 64 x
+// it: 100 fields of 256 x 256 from 256 modes 336 us (3791 by the contraction), 500 of 64 x
 // 64 from 512 modes 198 (2134).
 //
 // A tile is 128 cells x 32 samples: eight 128 x 32 accumulators in 256 columns
@@ -51,6 +51,7 @@ constexpr int kOzEpi = 256;          // threads that drain and store
 constexpr int kOzCut = 128;          // threads that cut the coefficients
 constexpr int kOzThreads = kOzEpi + 64 + kOzCut;
 constexpr int kOzStages = 2;
+constexpr unsigned kOzBand = 8;      // cell tiles of a band (4 .. 32 within 1% of one another)
 constexpr int kOzMaxM = 512;   // 512 modes x 8 pairs x 2^12 = 2^24
 constexpr uint32_t kOzABytes = kOzM * kOzK * 2, kOzBBytes = kOzN * kOzK * 2;
 constexpr uint32_t kOzStage = kOzDigits * (kOzABytes + kOzBBytes);
@@ -196,7 +197,7 @@ __device__ __forceinline__ unsigned next_digit(long long& v, int i) {
     return __float_as_uint(f * (1.0f / (float)(1LL << (kOzBits * i))));
 }
 
-// Persistent: CTA b takes tiles b, b + gridDim.x, ... (sample tiles fastest).
+// Persistent: CTA b takes tiles b, b + gridDim.x, ...
 // Warps 0 .. 7 drain, warp 8 (one thread) loads the basis digits, warp 9 (one
 // thread) issues the products, warps 10 .. 13 cut the coefficients; two stages of
 // operands and two sets of accumulators, so the next tile's products run under
@@ -218,7 +219,21 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     uint64_t* tempty = tfull + 2;           // accumulators drained
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned stiles = (unsigned)(S + kOzN - 1) / kOzN, tiles = stiles * ((unsigned)(cells + kOzM - 1) / kOzM);
+    const unsigned stiles = (unsigned)(S + kOzN - 1) / kOzN, ctiles = (unsigned)(cells + kOzM - 1) / kOzM;
+    const unsigned tiles = stiles * ctiles;
+    // Tile t: bands of kOzBand cell tiles, in a band the cell tiles of one sample tile
+    // after the other.  CTAs that run side by side share operands and write runs of 8 KB
+    // of a field.  Sample tiles fastest, they wrote 1 KB of every field at a stride of a
+    // field: once tiles of unlike length (a last one of few samples) had set the CTAs
+    // apart, 817 fields of 256 x 256 from 108 modes took 1.82 ms, 1.65 so.
+    struct At {
+        int s0, c0;
+    };
+    auto at = [&](unsigned t) {
+        const unsigned band = t / (stiles * kOzBand), r = t - band * stiles * kOzBand;
+        const unsigned w = min(kOzBand, ctiles - band * kOzBand);
+        return At{(int)(r / w) * kOzN, (int)(band * kOzBand + r % w) * kOzM};
+    };
     if (threadIdx.x < 64) tab[threadIdx.x] = kExpTable[threadIdx.x];
     if (threadIdx.x == 0) {
         for (int i = 0; i < kOzStages; ++i) {
@@ -245,7 +260,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             int q = 0;   // stage loads so far
             bool ok = true;
             for (unsigned tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x) {
-                const int c0 = (int)(tile / stiles) * kOzM;
+                const int c0 = at(tile).c0;
                 for (int kb = 0; kb < kblocks; ++kb) {
                     const int st = q % kOzStages, round = q / kOzStages;
                     if (round > 0 && !(ok = tc::mbar_wait(&empty[st], (round - 1) & 1, err))) break;
@@ -303,7 +318,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         int q = 0, it = 0;
         bool ok = true;
         for (unsigned tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x, ++it) {
-            const int s0 = (int)(tile % stiles) * kOzN;
+            const int s0 = at(tile).s0;
             const double* rows[8];   // rows past the batch: the last one's, cut to zero below and never stored
             int top[8];              // largest biased exponent of each row
 #pragma unroll
@@ -314,7 +329,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 #pragma unroll 2
             for (int k = lane; k < M; k += 32) {   // (sixteen loads in flight)
 #pragma unroll
-                for (int r = 0; r < 8; ++r) top[r] = max(top[r], (__double2hiint(rows[r][k]) >> 20) & 0x7FF);
+                for (int r = 0; r < 8; ++r) top[r] = max(top[r], (__double2hiint(__ldcg(rows[r] + k)) >> 20) & 0x7FF);
             }
             int e_mine = 0;   // lane r: the scale of row r0 + r
 #pragma unroll
@@ -333,8 +348,8 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                     for (int r2 = 0; r2 < 4; ++r2) {
                         const int s = s0 + r0 + 2 * r2 + half;
                         const double* row = xi + (size_t)s * M;
-                        x[r2][0] = s < S && k < M ? row[k] : 0.0;
-                        x[r2][1] = s < S && k + 1 < M ? row[k + 1] : 0.0;
+                        x[r2][0] = s < S && k < M ? __ldcg(row + k) : 0.0;
+                        x[r2][1] = s < S && k + 1 < M ? __ldcg(row + k + 1) : 0.0;
                     }
 #pragma unroll
                     for (int r2 = 0; r2 < 4; ++r2) {
@@ -375,7 +390,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         int it = 0;
         for (unsigned tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++it) {
             const int set = it & 1;
-            const int s0 = (int)(tile % stiles) * kOzN, c0 = (int)(tile / stiles) * kOzM;
+            const int s0 = at(tile).s0, c0 = at(tile).c0;
             const int c = c0 + 32 * (warp & 3) + lane;
             const int e_c = c < cells ? ec[c] : 0;
             // all lanes or none (the loads below are warp-wide)
@@ -412,7 +427,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                         g = 0.0;
                         for (int k = 0; k < M; ++k) g = fma(xi[(size_t)s * M + k], B[(size_t)c * M + k], g);
                     }
-                    K[(size_t)s * cells + c] = fm_exp(g, tab);
+                    __stcs(K + (size_t)s * cells + c, fm_exp(g, tab));   // streamed past the operands in L2
                 }
             }
         }
