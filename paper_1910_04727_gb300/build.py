@@ -38,7 +38,7 @@ def _sources():
 
 
 def _headers():
-    return glob.glob(os.path.join(_SRC, "*.cuh")) + glob.glob(os.path.join(_INC, "*.h"))
+    return glob.glob(os.path.join(_SRC, "*.cuh")) + glob.glob(os.path.join(_SRC, "*.h")) + glob.glob(os.path.join(_INC, "*.h"))
 
 
 def _stale(obj, deps):

@@ -106,9 +106,10 @@ extern "C" fm_status fm_create(const fm_config* cfg, fm_ctx** out) {
             return FM_ECUDA;
         }
     }
-    fmg_init_attributes();
-    resident_init_attributes();
+    fmg_init_attributes(ctx->device);
+    resident_init_attributes(ctx->device);
     kl_split_init_attributes();
+    kl_tc_init_attributes();
     *out = ctx;
     return FM_OK;
 }

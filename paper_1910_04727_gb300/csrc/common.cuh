@@ -451,8 +451,8 @@ fm_status fmg_solve_with(fm_ctx* ctx, Arena& ar, int n_fine, uint32_t S, const d
 size_t fmg_levelwise_scratch(const fm_ctx* ctx, int n_fine, uint32_t S, const fm_solve_params& prm);
 // Grows `ar` to `need` bytes (contents lost); false, with an empty arena, where there is no room.
 bool arena_holds(Arena& ar, size_t need);
-void fmg_init_attributes();
-void resident_init_attributes();
+void fmg_init_attributes(int device);
+void resident_init_attributes(int device);
 void uneven_free(fm_ctx* ctx);
 void batched_free(fm_ctx* ctx);
 fm_status fmg_solve_impl(fm_ctx* ctx, int n_fine, uint32_t S, const double* d_K,
@@ -472,7 +472,8 @@ fm_status kl_split_install(fm_ctx* ctx);
 bool kl_split_field(fm_ctx* ctx, int level, uint32_t n, const double* d_xi, double* d_K, cudaStream_t st,
                     fm_status* status);
 void kl_split_free(fm_ctx* ctx);
-void kl_split_init_attributes();
+void kl_split_init_attributes();   // on the current device
+void kl_tc_init_attributes();      // likewise
 // Nystrom interpolation of the KL basis on the tensor cores (kl_tc.cu).
 fm_status kl_tc_nystrom(fm_ctx* ctx, int q, const double* dVt, const double* d_inv_sqrt_theta, double* d_out);
 

@@ -22,6 +22,7 @@
 #include "common.cuh"
 #include "fmg_resident.cuh"
 #include "fmg_strip.cuh"
+#include "once_per_device.h"
 
 namespace fm {
 
@@ -1411,20 +1412,21 @@ static fm_status carve(fm_ctx* ctx, Arena& ar, Hierarchy<T>& H, int n_fine, int 
 
 constexpr size_t kMaxSmem = 200 * 1024;   // dynamic shared memory of the tile smoother
 
-// Kernel attributes and occupancies, set once per process before any launch
-// or capture.
-void fmg_init_attributes() {
-    static std::once_flag once;
-    std::call_once(once, [] {
+// Kernel attributes and occupancies, set once on every device before any launch
+// or capture there.
+void fmg_init_attributes(int device) {
+    static OncePerDevice once;
+    once.run(device, [&] {
         cudaFuncSetAttribute(k_rbgs_tile<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
         cudaFuncSetAttribute(k_rbgs_tile<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
         cudaFuncSetAttribute(k_vcycle_tail<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)tail_smem_max<float>());
         cudaFuncSetAttribute(k_vcycle_tail<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)tail_smem_max<double>());
-        int dev = 0, sms = 1;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        warp16_init();
+        team32_init();
+        int sms = 1;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
         strip_init<float>(sms);
         strip_init<double>(sms);
         cudaGetLastError();

@@ -27,11 +27,11 @@
 // infinity or a NaN there.
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 
 #include "common.cuh"
 #include "fmg_resident.cuh"
 #include "fmg_strip.cuh"
+#include "once_per_device.h"
 
 namespace fm {
 
@@ -745,9 +745,9 @@ static void launch_resident(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st)
     else launch_resident<T, MIXED, false>(ctx, a, st);
 }
 
-void resident_init_attributes() {
-    static std::once_flag once;
-    std::call_once(once, [] {
+void resident_init_attributes(int device) {
+    static OncePerDevice once;
+    once.run(device, [] {
         const int m = (int)kResidentSmemMax;
         cudaFuncSetAttribute(k_fmg_resident<float, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, m);
         cudaFuncSetAttribute(k_fmg_resident<float, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, m);

@@ -53,6 +53,9 @@ __device__ __forceinline__ double vcycle_bytes(int n0, int k, int nu1, int nu2, 
 // The converged mixed form with grids in registers: 16 x 16, one sample per warp
 // (fmg_warp16.cu), and 32 x 32, one per five warps (fmg_team32.cu), coarsest grid
 // 4 x 4.  Samples that leave the finite numbers come back as kAgain in qf.
+// (..._init: kernel attributes on the current device.)
+void warp16_init();
+void team32_init();
 void launch_warp16(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st);
 void launch_team32(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st);
 

@@ -195,7 +195,7 @@ inline bool strip_merges(int nu1, int nu2) {
     return sizeof(T) == 4 && nu1 == nu2;
 }
 
-// Kernel attributes and occupancies, once per process.
+// Kernel attributes on the current device, and occupancies.
 template <typename T>
 void strip_init(int sms);
 

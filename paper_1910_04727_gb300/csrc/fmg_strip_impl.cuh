@@ -549,7 +549,8 @@ struct StripVariant {
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k, 32 * W * strip_groups(W), smem(W)) !=
                 cudaSuccess)
                 blocks = 1;
-            resident[W] = std::max(1, blocks) * strip_groups(W) * std::max(1, sms);
+            // (the first device's count serves all: the library is built for one kind)
+            if (!resident[W]) resident[W] = std::max(1, blocks) * strip_groups(W) * std::max(1, sms);
         }
     }
     static void launch(fm_ctx* ctx, const StripCall<T>& c, cudaStream_t st) {

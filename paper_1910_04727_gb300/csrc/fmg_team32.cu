@@ -13,7 +13,6 @@
 // threads), 2.5 ms so; 1000 samples 1.73 and 0.47 ms.
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 
 #include "fmg_warp.cuh"
 
@@ -602,12 +601,13 @@ void launch_tail32(const Tail32Args& a, size_t S, cudaStream_t st) {
     k_vcycle_tail32<<<(unsigned)S, kTeam, 0, st>>>(a);
 }
 
+void team32_init() {
+    constexpr size_t smem = sizeof(Team32Smem);
+    cudaFuncSetAttribute(k_fmg_team32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
 void launch_team32(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st) {
     constexpr size_t smem = sizeof(Team32Smem);
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(k_fmg_team32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    });
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fmg_team32, kTeam, smem);
     const size_t grid = std::min<size_t>(a.S, (size_t)std::max(per_sm, 1) * std::max(ctx->sms, 1));

@@ -20,7 +20,6 @@
 // everything inlined (instruction fetch), 1.3 ms so.
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 
 #include "fmg_warp.cuh"
 
@@ -66,12 +65,13 @@ __global__ void __launch_bounds__(32 * kW16Warps, 4) k_fmg_warp16(ResidentArgs a
     }
 }
 
+void warp16_init() {
+    constexpr size_t smem = kW16Warps * sizeof(W16Smem);
+    cudaFuncSetAttribute(k_fmg_warp16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
 void launch_warp16(fm_ctx* ctx, const ResidentArgs& a, cudaStream_t st) {
     constexpr size_t smem = kW16Warps * sizeof(W16Smem);
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(k_fmg_warp16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    });
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fmg_warp16, 32 * kW16Warps, smem);
     const size_t need = (a.S + kW16Warps - 1) / kW16Warps;

@@ -311,6 +311,13 @@ static unsigned gemm_grid(const fm_ctx* ctx, int cells, uint32_t n) {
     return (unsigned)std::min<size_t>(tiles, (size_t)std::max(ctx->sms, 1));
 }
 
+// On the current device (kernel attributes are not the process's).
+void kl_tc_init_attributes() {
+    cudaFuncSetAttribute(k_kl_gemm_tc<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
+    cudaFuncSetAttribute(k_kl_gemm_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
+    cudaGetLastError();
+}
+
 fm_status kl_tc_install(fm_ctx* ctx, int split) {
     const int M = ctx->cfg.M, Mpad = (M + kTcK - 1) / kTcK * kTcK, Kp = split ? 3 * Mpad : Mpad;
     ctx->tc.split = split;
@@ -360,14 +367,6 @@ fm_status kl_tc_field(fm_ctx* ctx, int level, uint32_t n, const double* d_xi, do
         FM_CUDA_TRY(ctx, cudaMalloc((void**)&ctx->tc.err, sizeof(int)));
         FM_CUDA_TRY(ctx, cudaMemset(ctx->tc.err, 0, sizeof(int)));
     }
-    static bool attr = false;
-    if (!attr) {
-        FM_CUDA_TRY(ctx, cudaFuncSetAttribute(k_kl_gemm_tc<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)kTcSmem));
-        FM_CUDA_TRY(ctx, cudaFuncSetAttribute(k_kl_gemm_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)kTcSmem));
-        attr = true;
-    }
     FM_CUDA_TRY(ctx, ctx->tc.xi_order.begin(st));
     launch_xi_to_bf16(n, M, Mpad, ctx->tc.split, d_xi, ctx->tc.xi, st);
     // the coefficient map covers the buffer's capacity; rows >= n are never stored
@@ -404,12 +403,6 @@ fm_status kl_tc_nystrom(fm_ctx* ctx, int q, const double* dVt, const double* d_i
     if (!ctx->tc.err) {
         FM_CUDA_TRY(ctx, cudaMalloc((void**)&ctx->tc.err, sizeof(int)));
         FM_CUDA_TRY(ctx, cudaMemset(ctx->tc.err, 0, sizeof(int)));
-    }
-    static bool attr = false;
-    if (!attr) {
-        FM_CUDA_TRY(ctx, cudaFuncSetAttribute(k_kl_gemm_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)kTcSmem));
-        attr = true;
     }
     do {
         if (cudaMalloc(&A, chunk * Kp * 2) != cudaSuccess || cudaMalloc(&B, (size_t)M * Kp * 2) != cudaSuccess) {
