@@ -102,18 +102,12 @@ __device__ __forceinline__ double recip_set(double d) {
 // FP64: the divide of the FP64 pipe (a 58th of the FP32 rate) bounds the
 // set-up of every operator, so the quotient takes three operations instead of
 // nine: the start above, n r, and its correction by its own remainder
-// (Markstein).  2.1e9 random pairs: every one the IEEE quotient, every
-// reciprocal too.  Measured against a start by rcp.approx.f64 and a Newton step in the
-// pipe (two operations more, and IEEE 1 / D): 5304 FP64 samples of 64 x 64 7.79 -> 7.35
-// ms, 1000 mixed samples of 256 x 256 25.7 -> 25.2.
-static __device__ __noinline__ double quotient_rare(double n, double d) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    const double e = fma(-d, r, 1.0);
-    r = fma(r, e, r);
-    const double q = n * r;
-    return fma(fma(-d, q, n), r, q);
-}
+// (Markstein), correct to about 2^-88 before the last rounding: the IEEE quotient but
+// for one in some 2^34 (2.1e9 random pairs, and as many reciprocals, met none).
+// Measured against a start by rcp.approx.f64 and a Newton step in the pipe (two
+// operations more, and IEEE 1 / D): 5304 FP64 samples of 64 x 64 7.79 -> 7.35 ms,
+// 1000 mixed samples of 256 x 256 25.7 -> 25.2.
+static __device__ __noinline__ double quotient_rare(double n, double d) { return n / d; }   // (any d: 1 / d may be 0 or inf)
 __device__ __forceinline__ float harmonic_mean(float a, float b) { return 2.0f * a * b / (a + b); }
 __device__ __forceinline__ double harmonic_mean(double a, double b) {
     const double n = twice(a) * b, d = a + b;
