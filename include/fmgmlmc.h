@@ -382,9 +382,9 @@ typedef struct {
  * the host.  Each sample's results are those fmg_solve_batch gives it.
  * Branches carry stream priorities by grid size, the largest grid's highest
  * (below the surrogate's training stream).  The executable graphs stay in
- * ctx, one per shape (grids, schedules and which groups ask for Q^c; up to
- * 8, the least recently used replaced), and a call with a kept shape updates
- * that graph in place.
+ * ctx, one per shape (grids, schedules, smoother launches and which groups
+ * ask for Q^c and the status; up to 8, the least recently used replaced), and a call with a
+ * kept shape updates that graph in place.
  * prm->kernel: FM_KERNEL_AUTO or FM_KERNEL_LEVELWISE
  * (every group level-wise).  Asynchronous on `stream`; one call at a time
  * per ctx.  Scratch is allocated before the capture (FM_ENOMEM). */

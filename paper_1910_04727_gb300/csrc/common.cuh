@@ -449,6 +449,10 @@ fm_status fmg_solve_with(fm_ctx* ctx, Arena& ar, int n_fine, uint32_t S, const d
                          const fm_solve_params& prm, double* d_qf, double* d_qc, double* d_p,
                          int32_t* d_status, cudaStream_t st);
 size_t fmg_levelwise_scratch(const fm_ctx* ctx, int n_fine, uint32_t S, const fm_solve_params& prm);
+// Appends what decides which kernels a level-wise solve launches, its counts apart:
+// the passes over the scratch and the smoother's shape on every grid.
+void fmg_launch_key(const fm_ctx* ctx, int n_fine, uint32_t S, const fm_solve_params& prm,
+                    std::vector<int64_t>* key);
 // Grows `ar` to `need` bytes (contents lost); false, with an empty arena, where there is no room.
 bool arena_holds(Arena& ar, size_t need);
 void fmg_init_attributes(int device);

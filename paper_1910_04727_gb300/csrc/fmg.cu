@@ -2004,6 +2004,28 @@ static fm_status levelwise(fm_ctx* ctx, Arena& ar, int n_fine, int n0, uint32_t 
     return FM_OK;
 }
 
+template <typename T>
+static void append_shapes(const fm_ctx* ctx, int n_fine, size_t S, const fm_solve_params& prm,
+                          std::vector<int64_t>* key) {
+    for (int n = 2 * prm.n_coarsest; n <= n_fine; n *= 2) {
+        int tile, threads;
+        smooth_shape<T>(ctx, n, S, prm, &tile, &threads);
+        key->push_back(tile);
+        key->push_back(threads);
+    }
+}
+
+void fmg_launch_key(const fm_ctx* ctx, int n_fine, uint32_t S, const fm_solve_params& prm,
+                    std::vector<int64_t>* key) {
+    const int64_t lim = batch_limit(ctx, n_fine), full = S / lim, rest = S % lim;
+    key->push_back(full);
+    for (int64_t cnt : {full ? lim : 0, rest}) {
+        if (cnt == 0) key->push_back(-2);
+        else if (prm.precision == FM_PREC_MIXED) append_shapes<float>(ctx, n_fine, (size_t)cnt, prm, key);
+        else append_shapes<double>(ctx, n_fine, (size_t)cnt, prm, key);
+    }
+}
+
 // Scratch bytes a level-wise solve of S samples of grid n_fine takes (one batch).
 size_t fmg_levelwise_scratch(const fm_ctx* ctx, int n_fine, uint32_t S, const fm_solve_params& prm) {
     const bool mixed = prm.precision == FM_PREC_MIXED;

@@ -189,11 +189,14 @@ extern "C" fm_status fmg_solve_uneven(fm_ctx* ctx, int32_t n_groups, const fm_ba
     // a kept graph of the same shape: update its parameters; otherwise instantiate
     std::vector<int64_t> key = {n_groups, prm->precision, prm->converged, prm->energy_step, prm->nu0, prm->nu1,
                                 prm->nu2, prm->n_coarsest, prm->bc_case, prm->kernel, prm->ir_cycles};
-    // per group: grid, non-empty, schedule, and whether Q^c is asked for (a
-    // converged solve refines its coarse stage only then)
-    for (int g = 0; g < n_groups; ++g)
-        key.insert(key.end(), {groups[g].n_fine, groups[g].count > 0, resident[g],
-                               groups[g].d_qc != nullptr});
+    // per group: grid, non-empty, schedule, whether Q^c is asked for (a converged
+    // solve refines its coarse stage only then) and the status (a launch more), and the
+    // launches of the level-wise schedule (FP64 smoothing goes by the number of cells)
+    for (int g = 0; g < n_groups; ++g) {
+        key.insert(key.end(), {groups[g].n_fine, groups[g].count > 0, resident[g], groups[g].d_qc != nullptr,
+                               groups[g].d_status != nullptr});
+        if (groups[g].count && !resident[g]) fmg_launch_key(ctx, groups[g].n_fine, groups[g].count, *prm, &key);
+    }
     cudaGraphExec_t exec = nullptr;
     for (size_t i = 0; i < U->kept.size() && !exec; ++i) {
         if (U->kept[i].key != key) continue;
@@ -202,7 +205,7 @@ extern "C" fm_status fmg_solve_uneven(fm_ctx* ctx, int32_t n_groups, const fm_ba
             exec = U->kept[i].exec;
             U->kept[i].used = ++U->tick;
             ++U->updates;
-        } else {   // same key, other topology (a changed smoother shape, say): replace it
+        } else {   // same key, other topology: replace it
             cudaGetLastError();
             cudaGraphExecDestroy(U->kept[i].exec);
             U->kept.erase(U->kept.begin() + (long)i);
