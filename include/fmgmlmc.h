@@ -415,14 +415,15 @@ typedef struct {
  * at 128 or 256 threads) for the grids n_min, 2 n_min, ..., <= n_max on a
  * synthetic batch of about 64 Mi cells per grid, and keeps the fastest in
  * ctx for that precision (FM_PREC_FP64: the FP64 grids; FM_PREC_MIXED: the
- * FP32 ones).  Every later solve on ctx uses the choice; the sweeps' results
- * are the same whichever shape runs.  Synchronous; entries (nullable) gets up
+ * FP32 ones).  Every later solve on ctx uses the choice (FP64 column strips give
+ * way to colour launches for batches of few cells, as the built-in default's do);
+ * the sweeps' results are the same whichever shape runs.  Synchronous; entries (nullable) gets up
  * to max_entries rows. */
 fm_status fm_autotune(fm_ctx* ctx, int32_t precision, int32_t nsweeps, int32_t n_min, int32_t n_max,
                       fm_tune_entry* entries, int32_t max_entries, int32_t* n_entries);
 
 /* Sets the smoother launch shape of grid n (a power of two) for one
- * precision, as fm_autotune would set it: tile = 0 one launch per colour
+ * precision, for batches of every size: tile = 0 one launch per colour
  * and sweep; -1 column strips (one warp per 64-column strip marching up the
  * rows, 1 or 2 sweeps); 8, 16, 32 or 64 tiles with threads = 0
  * (register-blocked) or 128 / 256 (staged in shared memory); tile = -2

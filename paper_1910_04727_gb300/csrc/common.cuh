@@ -319,11 +319,12 @@ struct StreamOrder {
     }
 };
 
-// Smoother launch shape per (precision, grid): chosen by fm_autotune.
+// Smoother launch shape per (precision, grid): chosen by fm_autotune or by hand.
 struct TuneTable {
     int32_t n[2][16] = {};        // grid the entry was tuned for (0: none)
     int32_t tile[2][16] = {};     // tile interior (0: one launch per colour, -1: column strips)
     int32_t threads[2][16] = {};
+    bool by_hand[2][16] = {};     // set by fm_set_smoother_shape
 };
 
 // Tensor-core KL synthesis state (kl_tc.cu).

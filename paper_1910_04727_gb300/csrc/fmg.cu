@@ -1521,7 +1521,8 @@ static int tune_slot(int n) { return std::min(15, 31 - __builtin_clz((unsigned)n
 // finest 3.32; 160 of 64 x 64 0.77 / 0.73, 400 0.95 / 0.99).  Below, and
 // where strips do not fit: one register-blocked region a sample.  An fm_autotune or
 // fm_set_smoother_shape entry for this grid and precision replaces the
-// default.  Tiles and strips need both smoothing phases of the V-cycle (so
+// default; the tuner times 64 Mi cells, so strips it has chosen give way to colour
+// launches below the same lines, and those set by hand do not.  Tiles and strips need both smoothing phases of the V-cycle (so
 // the iterate goes p -> p2 -> p); tiles need their staged region in shared
 // memory, strips 1 or 2 sweeps.
 template <typename T>
@@ -1533,11 +1534,15 @@ static void smooth_shape(const fm_ctx* ctx, int n, size_t S, const fm_solve_para
         if (sizeof(T) == 8) *threads = 8 * n;   // staged
         else if (strip_fits(n, prm.nu1, prm.nu2)) *tile = kShapeStrip;
     }
-    if (sizeof(T) == 8 && n >= 64 && S * n * n < ((size_t)1 << (n > 64 ? 21 : 20))) *tile = 0;
-    if (ctx->tune.n[pi][slot] == n) {
+    const bool entry = ctx->tune.n[pi][slot] == n;
+    if (entry) {
         *tile = ctx->tune.tile[pi][slot];
         *threads = ctx->tune.threads[pi][slot];
     }
+    const bool by_hand = entry && ctx->tune.by_hand[pi][slot];
+    if (sizeof(T) == 8 && n >= 64 && *tile == kShapeStrip && !by_hand &&
+        S * n * n < ((size_t)1 << (n > 64 ? 21 : 20)))
+        *tile = 0;
     if (*tile > 0 && (prm.nu1 < 1 || prm.nu2 < 1 ||
                       tile_smem_bytes(*tile, n, std::max(prm.nu1, prm.nu2), sizeof(T)) > kMaxSmem))
         *tile = 0;
@@ -2288,6 +2293,7 @@ static fm_status autotune_grid(fm_ctx* ctx, int n, int nsweeps, fm_tune_entry* e
     ctx->tune.n[pi][slot] = n;
     ctx->tune.tile[pi][slot] = bt;
     ctx->tune.threads[pi][slot] = bth;
+    ctx->tune.by_hand[pi][slot] = false;
     e->n = n;
     e->tile = bt;
     e->threads = bth;
@@ -2345,6 +2351,7 @@ extern "C" fm_status fm_set_smoother_shape(fm_ctx* ctx, int32_t precision, int32
     ctx->tune.n[pi][slot] = n;
     ctx->tune.tile[pi][slot] = tile;
     ctx->tune.threads[pi][slot] = threads;
+    ctx->tune.by_hand[pi][slot] = true;
     return FM_OK;
 }
 
