@@ -30,10 +30,11 @@
 //
 // Arithmetic as in the colour kernel: p = (b + W + E + S + N) (1 / D) with
 // the reciprocal of D (FP32: rcp.approx and one Newton step, which gives the
-// correctly rounded 1 / D for every mantissa and every exponent from 2^-126
-// to 2^125, checked exhaustively; FP64: read from rD, formed once at set-up,
-// since an FP64 reciprocal costs more than a half-sweep's five FP64
-// operations), so the sweeps are bit-identical to the other shapes.
+// correctly rounded 1 / D for every D from 2^-126 up to 2^126, as
+// tests/test_gpu_short_functions.py walks through; FP64: read from rD, formed
+// once at set-up, since an FP64 reciprocal costs more than a half-sweep's five
+// FP64 operations), so the sweeps are bit-identical to the other shapes (FP32 diagonals
+// outside that range, where 1 / D is no normal number, or D none, excepted).
 //
 // FUSE: the warp also forms the residual b - A p of each final row once the
 // row above it is final, and its restriction: the lane's column pair is one
