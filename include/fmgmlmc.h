@@ -26,6 +26,9 @@
  *     default stream) are asynchronous on that stream; the return status
  *     covers argument checks and launch errors only.
  *   - A context is not thread-safe; use one per host thread.
+ *   - A context's calls share its buffers.  kl_field_batch and fmg_solve_batch may be
+ *     made on several streams (they say what they wait for), and point generation uses
+ *     no buffer; order the other calls of one context among streams yourself.
  *   - No C++ exception crosses this interface.
  */
 #ifndef FMGMLMC_H

@@ -35,7 +35,7 @@ namespace fm {
 constexpr int kH = 256;          // hidden width
 constexpr int kGm = 128;         // GEMM tile rows (MMA M)
 constexpr int kGk = 64;          // K per stage
-// Operand stages of a GEMM: the training GEMMs (N tile 64) are chains of
+// Operand stages of a GEMM: the training GEMMs (N tile 32) are chains of
 // latencies, so all four K blocks of a 256-wide layer are in flight at once
 // (with two stages the weight gradients' 16 blocks cost a round trip to L2
 // each pair); the inference GEMMs keep two, for two CTAs an SM.
@@ -761,7 +761,7 @@ struct MlpState {
     CUtensorMap fW1, fW2, fW3;         // the weights in 128-row boxes (fused inference)
     double mu = 0.0, sd = 1.0;
     int* err = nullptr;
-    int* step = nullptr;               // device step counter of a training run; step[1]: Adam's block count
+    int* step = nullptr;               // training run, on the device: [0] the number the next batch takes, [1] of the batch in X
     cudaStream_t st = nullptr;         // training stream (graph capture)
     // the weight- and bias-gradient kernels of a step run on `side`, beside
     // the back-propagation chain on the step's stream (fork / join events)
